@@ -212,7 +212,7 @@ ig_status collect_info(ig_mesh* mesh, int k, ig_solve_info* info) {
     info->iterations = s.iter;
     info->refinements = s.refine;
     for (int c = 0; c < kMaxK; ++c) {
-      info->rel_residual[c] = c < k ? s.relres[c] : 0.0;
+      info->rel_residual[c] = c < k ? std::sqrt(s.relres2[c]) : 0.0;
       info->true_rel_residual[c] = c < k ? s.trueres[c] : 0.0;
     }
   }
@@ -447,8 +447,8 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
   // slices of its first and last row of vertices are narrower), all slices get that width and
   // the SpMV computes a slice's offset instead of loading it.
   int sell_w = 0;
+  long wmax = 0;
   {
-    long wmax = 0;
     for (int w : widths) wmax = w > wmax ? w : wmax;
     const long padded = wmax * (long)nsl;
     if (nsl > 0 && padded <= (long)nnz_sell + (long)nnz_sell / 64 && padded < (long)INT32_MAX) {
@@ -516,7 +516,20 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
     tile_rows = (int)best_rows;
     ntiles = (int)(((long)ni + best_rows - 1) / best_rows);
   };
-  choose_tiles64(ctx->solver_slots, md.tile_rows, md.ntiles);
+  // A mesh whose rows fit on chip (kResMaxRows per SM) is solved by one CTA per SM with one tile each
+  // (ig_resident.cu). Small meshes spread over fewer SMs: 128 rows are one warp per SM sub-partition,
+  // below which an iteration gets no shorter (2,025 rows, k = 3: 6.8 us an iteration in tiles of 128,
+  // 7.8 in tiles of 64, 7.9 in tiles of 256). Above kResSmall rows the tiles have 256 rows at least,
+  // for the sake of the batches, whose CTAs take 256 rows at a time (5,917 rows, k = 3: 9.0 us in
+  // tiles of 256 against 8.2 in tiles of 128).
+  const bool resident = ctx->num_sms >= 1 && ctx->num_sms <= kResMaxCtas && ni <= (long)ctx->num_sms * kResMaxRows;
+  if (resident) {
+    const int rows = (ni + ctx->num_sms - 1) / ctx->num_sms;
+    md.tile_rows = ni <= kResSmall ? 128 : (std::max(rows, kResMinRows) + 31) / 32 * 32;
+    md.ntiles = (ni + md.tile_rows - 1) / md.tile_rows;
+  } else {
+    choose_tiles64(ctx->solver_slots, md.tile_rows, md.ntiles);
+  }
   choose_tiles(ctx->solver_slots32, kTileRows, md.tile_rows32, md.ntiles32);
   if (ni >= kBigRows) {
     choose_tiles(ctx->solver_slots32, kMaxTileRows32, md.tile_rows32u, md.ntiles32u);
@@ -526,6 +539,7 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
   }
   md.nnz_sell = nnz_sell;
   md.sell_w = sell_w;
+  md.sell_wmax = (int)(wmax / 32);
   md.sell_ptr = sell_ptr;
   md.sell_col = sell_col;
   md.F = F;
@@ -536,9 +550,10 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
   md.inc = inc;
   md.err = err;
   const size_t nv = (size_t)n * kMaxK;
-  // partial sums: the loop kernels' tiles (twice over for the cluster loop of small meshes, which
-  // keeps the SpMV's and the update's partials apart), and the VJP's per-face-tile sums of dl/dt
-  const size_t npart = std::max(std::max((size_t)md.ntiles, (size_t)md.ntiles32) * 2 * kPartStride,
+  // partial sums: the loop kernels' tiles (and the geodesic warm start's, of kTileRows rows), and the
+  // VJP's per-face-tile sums of dl/dt
+  const size_t npart = std::max(std::max(std::max((size_t)md.ntiles, (size_t)md.ntiles32),
+                                         (size_t)(ni + kTileRows - 1) / kTileRows) * kPartStride,
                                 (size_t)(mi + 255) / 256) + 8;
   UP_CK(mesh_alloc(M, &md.facew, 4 * (size_t)m), "alloc");
   UP_CK(mesh_alloc(M, &md.A, (size_t)nnz_sell), "alloc");
@@ -555,6 +570,12 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
   UP_CK(mesh_alloc(M, &md.gface, 9 * (size_t)m), "alloc");
   UP_CK(mesh_alloc(M, &md.part, npart), "alloc");
   UP_CK(mesh_alloc(M, &md.s, 1), "alloc");
+  if (resident) {
+    unsigned char* meet = nullptr;
+    UP_CK(mesh_alloc(M, &meet, meet_bytes(md.ntiles)), "alloc");
+    UP_CK(cudaMemsetAsync(meet, 0, meet_bytes(md.ntiles), st), "memset");
+    md.meet = meet;
+  }
   UP_CK(cudaMemsetAsync(md.s, 0, sizeof(SolveScal), st), "memset");
   UP_CK(cudaMemsetAsync(md.p, 0, sizeof(double) * nv, st), "memset");
   UP_CK(cudaMemsetAsync(md.q, 0, sizeof(double) * nv, st), "memset");

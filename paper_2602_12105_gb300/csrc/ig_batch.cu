@@ -87,7 +87,7 @@ ig_status batch_info(ig_batch* b, int k, ig_solve_info* infos) {
       inf.iterations = ss[i].iter;
       inf.refinements = ss[i].refine;
       for (int c = 0; c < k; ++c) {
-        inf.rel_residual[c] = ss[i].relres[c];
+        inf.rel_residual[c] = std::sqrt(ss[i].relres2[c]);
         inf.true_rel_residual[c] = ss[i].trueres[c];
       }
     }

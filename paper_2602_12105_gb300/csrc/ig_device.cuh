@@ -8,6 +8,8 @@
 namespace ig {
 namespace {
 
+constexpr int kWarps = kBlock / 32;
+
 template <int K>
 struct KP {
   static constexpr int v = (K == 3) ? 4 : K;
@@ -19,39 +21,6 @@ __device__ __forceinline__ bool positive_finite(double x) {
 }
 __device__ __forceinline__ bool is_finite(double x) {
   return (__double_as_longlong(x) & 0x7ff0000000000000ll) != 0x7ff0000000000000ll;
-}
-
-// Thread j of the CTA adds the partials of tiles j, j + kBlock, j + 2 kBlock, ... in that order
-// (the association is fixed by the tile count alone, so the result is deterministic). Loads go in
-// batches of 4 tiles so that a thread has several L2 requests in flight.
-template <int NV>
-__device__ __noinline__ void gather_partials_impl(const double* __restrict__ part, int ntiles, double* out) {
-  double v[NV];
-#pragma unroll
-  for (int i = 0; i < NV; ++i) v[i] = 0.0;
-  for (int t = threadIdx.x; t < ntiles; t += 4 * kBlock) {
-    // four tiles' loads in flight together; a tile past the end reads as +0, which leaves the
-    // sum unchanged
-    double b[4][NV];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int tu = t + u * kBlock;
-#pragma unroll
-      for (int i = 0; i < NV; ++i) b[u][i] = tu < ntiles ? __ldcg(part + tu * kPartStride + i) : 0.0;
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-#pragma unroll
-      for (int i = 0; i < NV; ++i) v[i] += b[u][i];
-  }
-#pragma unroll
-  for (int i = 0; i < NV; ++i) out[i] = v[i];
-}
-
-// (kept out of line: only the last CTA of a reduction runs it)
-template <int NV>
-__device__ __forceinline__ void gather_partials(const double* __restrict__ part, int ntiles, double (&v)[NV]) {
-  gather_partials_impl<NV>(part, ntiles, v);
 }
 
 // Sum v[0..NV) over the CTA; thread 0 receives the totals. sh holds NV*kBlock doubles.
@@ -74,37 +43,15 @@ __device__ __forceinline__ void block_sum(double (&v)[NV], double* sh) {
   __syncthreads();
 }
 
-// Block-sum v, publish the tile's partials, and return true in the last CTA of the mesh, whose
-// thread 0 then holds the mesh totals (partials added in tile order, so the result does not
-// depend on which CTA finished last).
-template <int NV>
-__device__ __forceinline__ bool reduce_tiles(double (&v)[NV], double* part, int tile, int ntiles, unsigned int* cnt,
-                                             double* sh) {
-  __shared__ int s_last;
-  block_sum<NV>(v, sh);
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int i = 0; i < NV; ++i) part[tile * kPartStride + i] = v[i];
-    __threadfence();
-    const unsigned prev = atomicAdd(cnt, 1u);
-    s_last = (prev == (unsigned)ntiles - 1u);
-  }
-  __syncthreads();
-  if (!s_last) return false;
-  __threadfence();
-  gather_partials<NV>(part, ntiles, v);
-  block_sum<NV>(v, sh);
-  if (threadIdx.x == 0) *cnt = 0u;
-  return true;
-}
-
+// Row load and store of a padded [n][KP] vector (rows 32-byte aligned for K = 3 and 4): one access
+// per row. A gather touches one 32-byte sector per row either way, but two 16-byte loads look their
+// lines up in L1 twice, which bound the resident product on meshes in scattered order.
 template <int K>
 __device__ __forceinline__ void load_row(const double* __restrict__ p, long row, double (&v)[K]) {
   if constexpr (K == 3 || K == 4) {
-    const double2* q = reinterpret_cast<const double2*>(p + row * KP<K>::v);
-    const double2 a = q[0], b = q[1];
-    v[0] = a.x; v[1] = a.y; v[2] = b.x;
-    if constexpr (K == 4) v[3] = b.y;
+    const double4_32a a = reinterpret_cast<const double4_32a*>(p)[row];
+    v[0] = a.x; v[1] = a.y; v[2] = a.z;
+    if constexpr (K == 4) v[3] = a.w;
   } else if constexpr (K == 2) {
     const double2 a = reinterpret_cast<const double2*>(p + row * 2)[0];
     v[0] = a.x; v[1] = a.y;
@@ -113,14 +60,14 @@ __device__ __forceinline__ void load_row(const double* __restrict__ p, long row,
   }
 }
 
-// Row store into a padded [n][KP] vector (16-byte stores where the row allows).
 template <int K>
 __device__ __forceinline__ void store_row(double* __restrict__ p, long row, const double (&v)[K]) {
   if constexpr (K == 3 || K == 4) {
-    double2* q = reinterpret_cast<double2*>(p + row * KP<K>::v);
-    q[0] = make_double2(v[0], v[1]);
-    if constexpr (K == 4) q[1] = make_double2(v[2], v[3]);
-    else p[row * 4 + 2] = v[2];
+    double4_32a a;
+    a.x = v[0]; a.y = v[1]; a.z = v[2];
+    if constexpr (K == 4) a.w = v[3];
+    else a.w = 0.0;  // a whole sector
+    reinterpret_cast<double4_32a*>(p)[row] = a;
   } else if constexpr (K == 2) {
     reinterpret_cast<double2*>(p + row * 2)[0] = make_double2(v[0], v[1]);
   } else {
@@ -254,18 +201,20 @@ struct GatherAoS64 {
 // Transposed warp sum. In a plain butterfly every lane adds every value at each of the five
 // levels; here, at the first levels, a lane keeps half of its values and sends the other half to
 // its partner, so NV <= 8 values cost 9 shuffles and 9 adds per lane (NV <= 4: 6 and 6) instead of
-// 5 NV of each. Afterwards lane L holds the warp total of value warp_sum_index<NV>(L), and the
+// 5 NV of each (NV = 2: 5 and 5). Afterwards lane L holds the warp total of value warp_sum_index<NV>(L), and the
 // lanes selected by warp_sum_writer<NV>(L) hold each total once. The additions are in a fixed
 // order, so the sums are deterministic. (FP64 adds are scarce on this GPU: 2 per clock per SM.)
 template <int NV>
 __device__ __forceinline__ int warp_sum_index(int lane) {
-  if constexpr (NV <= 2) return 0;
+  if constexpr (NV <= 1) return 0;
+  else if constexpr (NV <= 2) return (lane >> 4) & 1;
   else if constexpr (NV <= 4) return ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
   else return ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
 }
 template <int NV>
 __device__ __forceinline__ bool warp_sum_writer(int lane) {
-  if constexpr (NV <= 2) return lane == 0;
+  if constexpr (NV <= 1) return lane == 0;
+  else if constexpr (NV <= 2) return (lane & 15) == 0;
   else if constexpr (NV <= 4) return (lane & 0x13) == 0;
   else return (lane & 3) == 0;
 }
@@ -273,13 +222,19 @@ __device__ __forceinline__ bool warp_sum_writer(int lane) {
 template <int NV, typename T>
 __device__ __forceinline__ T warp_sum_transposed(T (&v)[NV], int lane) {
   static_assert(NV >= 1 && NV <= 8, "at most 8 values");
-  if constexpr (NV <= 2) {
-    // plain butterfly on the (one or two) values; lane 0 returns value 0 and v[] holds both totals
+  if constexpr (NV == 1) {
+    T a = v[0];
 #pragma unroll
-    for (int i = 0; i < NV; ++i)
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    return a;
+  } else if constexpr (NV == 2) {
+    const bool h16 = (lane & 16) != 0;
+    const T keep = h16 ? v[1] : v[0];
+    const T send = h16 ? v[0] : v[1];
+    T a = keep + __shfl_xor_sync(0xffffffffu, send, 16);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
-    return v[0];
+    for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    return a;
   } else if constexpr (NV <= 4) {
     T a[4];
 #pragma unroll
@@ -333,33 +288,121 @@ __device__ __forceinline__ T warp_sum_transposed(T (&v)[NV], int lane) {
   }
 }
 
-constexpr int kWarps = kBlock / 32;
-
-// Sum the per-thread values v[0..NV) over the CTA: each warp adds its lanes (in T: FP32 for the
-// mixed-precision kernels, FP64 otherwise), then threads 0..NV-1 add the kWarps warp totals in FP64
-// in warp order and write them to out[0..NV). red holds NV * kWarps doubles; a caller that sums
-// consecutive tiles alternates between two such buffers, so that one barrier per tile suffices
-// (a warp can reach the buffer again only after the next tile's barrier, which the readers of
-// this tile pass after their reads).
+// Sums over the CTA, in two halves. First each warp adds its lanes' values (in T: FP32 for the
+// mixed-precision kernels, FP64 otherwise) and writes the totals to red (8 * kWarps doubles); after
+// a barrier, warp 0 adds the kWarps warp totals of every value in FP64: four lanes per value take
+// two warps each and add in a butterfly, three additions deep. An FP64 instruction occupies its SM
+// sub-partition for 64 cycles whatever the number of active lanes, so the number of instructions on
+// the path counts, not that of additions: the serial sum of 8 totals took 512 cycles.
 template <int NV, typename T>
-__device__ __forceinline__ void tile_reduce(T (&v)[NV], double* red, double* out) {
+__device__ __forceinline__ void warp_totals(T (&v)[NV], double* red) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const T w = warp_sum_transposed<NV>(v, lane);
-  if constexpr (NV <= 2) {
-    if (lane == 0)
+  const int idx = warp_sum_index<NV>(lane);
+  if (warp_sum_writer<NV>(lane) && idx < NV) red[idx * kWarps + warp] = (double)w;
+}
+// On one warp: lanes 4 v .. 4 v + 3 return the sum of value v's warp totals (v < NV; 0 for the rest).
+template <int NV>
+__device__ __forceinline__ double add_warps(const double* red) {
+  static_assert(kWarps == 8 && NV <= 8, "four lanes per value, two warps each");
+  const int lane = threadIdx.x & 31, v = lane >> 2, j = lane & 3;
+  double a = v < NV ? red[v * kWarps + j] + red[v * kWarps + j + 4] : 0.0;
+  a += __shfl_xor_sync(0xffffffffu, a, 1);
+  a += __shfl_xor_sync(0xffffffffu, a, 2);
+  return a;
+}
+// The same sum on one thread, without the warp's shuffles (which cost the loop kernels spills).
+__device__ __forceinline__ double add_warps_of(const double* red) {
+  return ((red[0] + red[4]) + (red[1] + red[5])) + ((red[2] + red[6]) + (red[3] + red[7]));
+}
+template <int NV>
+__device__ __forceinline__ void add_warps_to(const double* red, double* out) {
+  const double a = add_warps<NV>(red);
+  const int lane = threadIdx.x & 31, v = lane >> 2;
+  if ((lane & 3) == 0 && v < NV) out[v] = a;
+}
+
+// Sum the per-thread values v[0..NV) over the CTA into out[0..NV). A caller that sums consecutive
+// tiles alternates between two red buffers, so that one barrier per tile suffices (a warp can reach
+// the buffer again only after the next tile's barrier, which warp 0 passes after its reads).
+template <int NV, typename T>
+__device__ __forceinline__ void tile_reduce(T (&v)[NV], double* red, double* out) {
+  warp_totals<NV>(v, red);
+  __syncthreads();
+  if (threadIdx.x < NV) out[threadIdx.x] = add_warps_of(red + threadIdx.x * kWarps);
+}
+
+// How a CTA adds the partial sums of a mesh's tiles: VP lanes (the power of two above NV) take one
+// tile's values, so that a warp covers 32 / VP tiles with each load and its lanes are all busy; warp w
+// starts at tile w * 32 / VP, a lane adds its tiles in order, the lanes of one value add in a
+// butterfly and the warps as above. The association depends on the tile count alone.
+template <int NV>
+struct PartialMap {
+  static constexpr int VP = NV <= 1 ? 1 : (NV <= 2 ? 2 : (NV <= 4 ? 4 : 8));
+  static constexpr int kTiles = 32 / VP;            // tiles per warp and step
+  static constexpr int kStride = kTiles * kWarps;   // tiles per CTA and step
+  __device__ static __forceinline__ int value(int lane) { return lane % VP; }
+  __device__ static __forceinline__ int first(int warp, int lane) { return warp * kTiles + lane / VP; }
+  // the lane sums a of this warp, added over its tiles, to red
+  __device__ static __forceinline__ void to_warp_total(double a, double* red) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-      for (int i = 0; i < NV; ++i) red[i * kWarps + warp] = (double)v[i];
-  } else {
-    const int idx = warp_sum_index<NV>(lane);
-    if (warp_sum_writer<NV>(lane) && idx < NV) red[idx * kWarps + warp] = (double)w;
+    for (int o = VP; o < 32; o <<= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+    if (lane < NV) red[lane * kWarps + warp] = a;
+  }
+};
+
+// tot[0..NV) = the sums of the tiles' partials, on warp 0 (the others may go on; red must not be in
+// use by any warp). Kept out of line: only the last CTA of a reduction runs it.
+template <int NV>
+__device__ __noinline__ void combine_partials(const double* __restrict__ part, int ntiles, double* red,
+                                                 double* tot) {
+  using Map = PartialMap<NV>;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, v = Map::value(lane);
+  double a = 0.0;
+  for (int t = Map::first(warp, lane); t < ntiles; t += 4 * Map::kStride) {
+    double b[4];  // four steps' loads in flight; a tile past the end adds +0
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int tu = t + u * Map::kStride;
+      b[u] = tu < ntiles && v < NV ? __ldcg(part + (long)tu * kPartStride + v) : 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (t + u * Map::kStride < ntiles) a += b[u];
+  }
+  Map::to_warp_total(a, red);
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    add_warps_to<NV>(red, tot);
+    __syncwarp();
+  }
+}
+
+// Sum v over the tile, publish the tile's partials, and return true in the last CTA of the mesh,
+// which then holds the mesh totals in v (every thread).
+template <int NV>
+__device__ __forceinline__ bool reduce_tiles(double (&v)[NV], double* part, int tile, int ntiles, unsigned int* cnt) {
+  __shared__ double red[8 * kWarps];
+  __shared__ double tot[8];
+  __shared__ int s_last;
+  tile_reduce<NV>(v, red, part + (long)tile * kPartStride);
+  if (threadIdx.x < 32) __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    const unsigned prev = atomicAdd(cnt, 1u);
+    s_last = (prev == (unsigned)ntiles - 1u);
   }
   __syncthreads();
-  if (threadIdx.x < NV) {
-    double a = red[threadIdx.x * kWarps];
+  if (!s_last) return false;
+  __threadfence();
+  combine_partials<NV>(part, ntiles, red, tot);
+  __syncthreads();
 #pragma unroll
-    for (int j = 1; j < kWarps; ++j) a += red[threadIdx.x * kWarps + j];
-    out[threadIdx.x] = a;
-  }
+  for (int i = 0; i < NV; ++i) v[i] = tot[i];
+  if (threadIdx.x == 0) *cnt = 0u;
+  return true;
 }
 
 // ------------------------------------------------------------------------------- persistent tiles
@@ -413,6 +456,24 @@ __device__ __forceinline__ void load_mesh(const MeshDev* __restrict__ mds, int i
   __syncthreads();
 }
 
+// What the CTA that completes a mesh does: add the partials and run the finish step. Out of line,
+// with its own registers.
+template <int NV, typename Finish>
+__device__ __noinline__ void complete_mesh(TileCtx& tc, int ntiles, unsigned int* cnt, const Finish& finish) {
+  __threadfence();
+  // the mesh's scalars are read into shared memory while the partials are gathered, so that
+  // the finish step does not wait on one global load after another
+  static_assert(sizeof(SolveScal) % 4 == 0 && sizeof(SolveScal) / 4 <= kBlock, "SolveScal copy");
+  if (threadIdx.x < (int)(sizeof(SolveScal) / 4))
+    reinterpret_cast<unsigned*>(&tc.cur)[threadIdx.x] =
+        __ldcg(reinterpret_cast<const unsigned*>(tc.md.s) + threadIdx.x);
+  combine_partials<NV>(tc.md.part, ntiles, tc.red[0], tc.tot);  // its barrier also publishes cur
+  if (threadIdx.x < 32) {
+    if (threadIdx.x == 0) *cnt = 0u;
+    finish(tc.md, tc.cur, tc.tot);
+  }
+}
+
 // The loop kernels run one CTA per resident slot; CTA b takes the flat tiles b, b + G, b + 2G, ...
 // (G = gridDim.x). A tile's sums go to the mesh's part[tile]; each CTA counts the tiles it did
 // per run of consecutive tiles of one mesh and adds that count to the mesh's counter with one
@@ -424,7 +485,7 @@ __device__ __forceinline__ void flush_tiles(TileCtx& tc, int tiling, unsigned ru
                                             const Finish& finish) {
   const int ntiles = tile_count(tc.md, tiling);
   unsigned int* cnt = &tc.md.s->cnt[cnt_idx];
-  if (threadIdx.x < NV) __threadfence();  // the tile sums this thread wrote, before the count
+  if (threadIdx.x < 32) __threadfence();  // the tile sums this warp wrote, before the count
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -432,23 +493,7 @@ __device__ __forceinline__ void flush_tiles(TileCtx& tc, int tiling, unsigned ru
     tc.last = (prev + run == (unsigned)ntiles);
   }
   __syncthreads();
-  if (tc.last) {
-    __threadfence();
-    // the mesh's scalars are read into shared memory while the partials are gathered, so that
-    // the finish step does not wait on one global load after another
-    static_assert(sizeof(SolveScal) % 4 == 0 && sizeof(SolveScal) / 4 <= kBlock, "SolveScal copy");
-    if (threadIdx.x < (int)(sizeof(SolveScal) / 4))
-      reinterpret_cast<unsigned*>(&tc.cur)[threadIdx.x] =
-          __ldcg(reinterpret_cast<const unsigned*>(tc.md.s) + threadIdx.x);
-    double v[NV];
-    gather_partials<NV>(tc.md.part, ntiles, v);
-    tile_reduce<NV>(v, tc.red[0], tc.tot);
-    __syncthreads();
-    if (threadIdx.x < 32) {
-      if (threadIdx.x == 0) *cnt = 0u;
-      finish(tc.md, tc.cur, tc.tot);
-    }
-  }
+  if (tc.last) complete_mesh<NV>(tc, ntiles, cnt, finish);
   __syncthreads();
 }
 
@@ -805,6 +850,90 @@ __device__ __noinline__ void finish_spmv(SolveScal* s, const SolveScal& cur, int
     s->status = IG_ERR_NONFINITE;
     s->done = 1;
   }
+}
+
+// ------------------------------------------------------------------------------- last-CTA steps
+// The per-mesh scalar updates run on one thread of the last CTA of a reduction. They are kept
+// out of line (and count active columns explicitly) so that this bookkeeping is compiled on its
+// own, apart from the unrolled arithmetic of the kernels.
+__device__ __noinline__ void finish_init(SolveScal* s, int k, const double* acc, double tol, int max_iter) {
+  int nact = 0, bad = 0;
+  for (int c = 0; c < kMaxK; ++c) {
+    const double rz = c < k ? acc[c] : 0.0;
+    const double bb = c < k ? acc[k + c] : 0.0;
+    if (c < k && (!is_finite(bb) || !is_finite(rz))) bad = 1;
+    const int act = (c < k && positive_finite(bb)) ? 1 : 0;
+    s->rz[c] = rz;
+    s->bnorm2[c] = bb;
+    s->rhs2[c] = bb;
+    s->active[c] = act;
+    s->relres2[c] = act ? 1.0 : 0.0;
+    s->alpha[c] = 0.0;
+    s->beta[c] = 0.0;
+    s->scale[c] = 1.0;
+    s->trueres[c] = -1.0;
+    nact += act;
+  }
+  s->k = k;
+  s->cnt[0] = 0u;
+  s->cnt[1] = 0u;
+  s->iter = 0;
+  s->refine = 0;
+  s->phase = 0;
+  s->tol = tol;
+  s->max_iter = max_iter;
+  s->status = bad ? IG_ERR_NONFINITE : IG_OK;
+  s->done = (bad != 0 || nact == 0) ? 1 : 0;
+}
+
+// Convergence test per column (recursive residual), beta_c = rz_new / rz, iteration count. Runs on
+// warp 0 of the CTA that completes the mesh: lane c takes column c, lane 0 the mesh's fields.
+// Returns (on lane 0) whether the mesh is now done. The test compares squares (the root of the
+// reported residual is taken on the host), and its division runs beside that of beta, on lanes
+// 8 .. 8 + k: a division takes about 500 cycles and a root 700 for any number of lanes.
+__device__ __noinline__ int finish_update(SolveScal* s, const SolveScal& cur, int k, const double* acc) {
+  const int c = threadIdx.x & 31, col = c & 7;
+  int act = 0, bad = 0;
+  const double* den = c < 8 ? cur.rz : cur.bnorm2;
+  const double* num = c < 8 ? acc : acc + k;
+  double quot = 0.0;
+  if (col < k && c < 16) quot = num[col] / den[col];
+  const double rel2 = __shfl_down_sync(0xffffffffu, quot, 8);
+  if (c < k && cur.active[c] != 0) {
+    const double rzn = acc[c], rr = acc[k + c];
+    if (!is_finite(rzn) || !is_finite(rr)) {
+      bad = 1;
+    } else {
+      const double bta = quot;
+      s->relres2[c] = rel2;
+      if (rel2 <= cur.tol * cur.tol) {
+        s->active[c] = 0;
+        s->beta[c] = 0.0;
+      } else {
+        s->beta[c] = bta;
+        s->rz[c] = rzn;
+        act = 1;
+      }
+    }
+  }
+  const int nact = __popc(__ballot_sync(0xffffffffu, act));
+  const int anybad = __any_sync(0xffffffffu, bad);
+  int done = 0;
+  if (c == 0) {
+    const int it = cur.iter + 1;
+    s->iter = it;
+    if (anybad) {
+      s->status = IG_ERR_NONFINITE;
+      done = 1;
+    } else if (nact == 0) {
+      done = 1;
+    } else if (it >= cur.max_iter) {
+      s->status = IG_ERR_NOT_CONVERGED;
+      done = 1;
+    }
+    if (done) s->done = 1;
+  }
+  return done;
 }
 
 // ------------------------------------------------------------------------------- finalize

@@ -21,7 +21,6 @@ __global__ void __launch_bounds__(kBlock) mnorm_kernel(const MeshDev* __restrict
                                                        const double* __restrict__ U,
                                                        const double* __restrict__ T, double* __restrict__ G,
                                                        double* __restrict__ w, double* __restrict__ loss) {
-  __shared__ double sh[kBlock];
   const int2 tl = tiles[blockIdx.x];
   const MeshDev& md = mds[tl.x];
   const long nn = md.n;
@@ -40,7 +39,7 @@ __global__ void __launch_bounds__(kBlock) mnorm_kernel(const MeshDev* __restrict
     w[row] = 0.5 * e;
     acc[0] = fma(m, 0.5 * e, acc[0]);
   }
-  if (reduce_tiles<1>(acc, md.part, tl.y, md.ntiles, &md.s->cnt[2], sh) && threadIdx.x == 0) *loss = acc[0];
+  if (reduce_tiles<1>(acc, md.part, tl.y, md.ntiles, &md.s->cnt[2]) && threadIdx.x == 0) *loss = acc[0];
 }
 
 // V <- V - eta g over 3n values.

@@ -40,7 +40,12 @@ constexpr int kMaxTileRows32 = 64 * kTileRows;      // the largest mixed-precisi
 constexpr int kMaxPasses64 = 8;      // FP64 solver tiles: at most 8 passes of kBlock rows
 constexpr int kTileRows64 = kBlock * kMaxPasses64;
 constexpr int kMaxK = 4;
-constexpr int kSmallTiles = 16;      // a single mesh of at most this many FP64 tiles loops in one cluster
+// Resident solves (ig_resident.cu): one tile per CTA, one CTA per SM
+constexpr int kResMaxCtas = 160;     // most CTAs
+constexpr int kResMinRows = 256;     // fewest rows of a tile of more than kResSmall rows
+constexpr int kResSmall = 2048;      // meshes up to this size: tiles of 128 rows
+constexpr int kResMaxRows = 1216;    // most rows of a tile (227 KB of shared memory at 188 bytes a row)
+constexpr int kClusterTiles = 16;    // up to this many tiles meet as one thread-block cluster
 constexpr int kPartStride = 8;       // doubles per tile in the partial-sum arrays
 
 // Device error word bits (OR-ed by kernels, decoded on the host).
@@ -88,12 +93,11 @@ struct SolveScal {
   double beta[kMaxK];
   double bnorm2[kMaxK];  // ||rhs||^2 of the system being iterated
   double rhs2[kMaxK];    // ||rhs||^2 of the outer (FP64) system
-  double relres[kMaxK];  // last relative residual seen by the stopping test
+  double relres2[kMaxK]; // square of the last relative residual seen by the stopping test
   double trueres[kMaxK]; // FP64 recomputed relative residual (filled on request)
   double scale[kMaxK];   // mixed precision: norm of the residual the inner system was scaled by
   int active[kMaxK];     // columns still iterating (the inner FP32 system in mixed precision)
   int active64[kMaxK];   // mixed precision: columns whose FP64 residual is still above tol
-  double relres_inner[kMaxK];
   int inner_iter;        // mixed precision: iterations of the current inner solve
   int inner_cap;         // mixed precision: cap on iterations of one inner solve
   int k;
@@ -123,6 +127,7 @@ struct MeshDev {
   int ntiles32u, tile_rows32u;  // the mixed-precision update's tiles (one wave on meshes of kBigRows or more)
   int nnz_sell;            // stored entries of the sliced layout (0: A is plain CSR on rowptr/col)
   int sell_w;              // every slice has this many entries per row (0: widths differ)
+  int sell_wmax;           // the widest slice's entries per row
   const int* sell_ptr;     // [ceil(n/32)+1] slice offsets, or null for plain CSR
   const int* sell_col;     // [nnz_sell]
   // mixed precision: the columns as 16-bit offsets from each slice's first row, kept when every
@@ -161,6 +166,7 @@ struct MeshDev {
   double* lam;             // adjoint solution [n][k]
   double* gface;           // per-face gradient contributions [m][9]
   double* part;            // [ntiles][kPartStride] partial sums
+  void* meet;              // resident solves: meet_bytes(ntiles) bytes, zeroed at upload (null: not one)
   SolveScal* s;
   int* err;
   // FP32 face geometry (IG_PRECISION_MIXED_GEOM32): when geom32 is set the operator is the FP32
@@ -415,6 +421,12 @@ cudaError_t launch_operator_csr(const MeshDev& md, double* Acsr, cudaStream_t st
 cudaError_t launch_operator32_csr(const MeshDev& md, float* Acsr, cudaStream_t st);
 
 // ig_pcg.cu: see Group above
+
+// ig_resident.cu: a whole FP64 solve of a group of one mesh in one launch; false, with nothing
+// launched, when the mesh does not qualify or the device refuses the launch
+bool launch_resident(Group& g, int k, const double* in, double* out, int rhs_mass, const ig_solve_opts& o,
+                     cudaStream_t st);
+size_t meet_bytes(int ntiles);
 
 // ig_eigs.cu: shift-invert subspace iteration (workspace of eig_workspace_doubles(n) doubles)
 size_t eig_workspace_doubles(long n);

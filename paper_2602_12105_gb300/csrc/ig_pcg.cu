@@ -28,91 +28,12 @@ namespace ig {
 
 namespace {
 
-// ------------------------------------------------------------------------------- last-CTA steps
-// The per-mesh scalar updates run on one thread of the last CTA of a reduction. They are kept
-// out of line (and count active columns explicitly) so that this bookkeeping is compiled on its
-// own, apart from the unrolled arithmetic of the kernels.
-__device__ __noinline__ void finish_init(SolveScal* s, int k, const double* acc, double tol, int max_iter) {
-  int nact = 0, bad = 0;
-  for (int c = 0; c < kMaxK; ++c) {
-    const double rz = c < k ? acc[c] : 0.0;
-    const double bb = c < k ? acc[k + c] : 0.0;
-    if (c < k && (!is_finite(bb) || !is_finite(rz))) bad = 1;
-    const int act = (c < k && positive_finite(bb)) ? 1 : 0;
-    s->rz[c] = rz;
-    s->bnorm2[c] = bb;
-    s->rhs2[c] = bb;
-    s->active[c] = act;
-    s->relres[c] = act ? 1.0 : 0.0;
-    s->alpha[c] = 0.0;
-    s->beta[c] = 0.0;
-    s->scale[c] = 1.0;
-    s->trueres[c] = -1.0;
-    nact += act;
-  }
-  s->k = k;
-  s->cnt[0] = 0u;
-  s->cnt[1] = 0u;
-  s->iter = 0;
-  s->refine = 0;
-  s->phase = 0;
-  s->tol = tol;
-  s->max_iter = max_iter;
-  s->status = bad ? IG_ERR_NONFINITE : IG_OK;
-  s->done = (bad != 0 || nact == 0) ? 1 : 0;
-}
-
-// Convergence test per column (recursive residual), beta_c = rz_new / rz, iteration count. Runs on
-// warp 0 of the CTA that completes the mesh: lane c takes column c, lane 0 the mesh's fields.
-// Returns (on lane 0) whether the mesh is now done.
-__device__ __noinline__ int finish_update(SolveScal* s, const SolveScal& cur, int k, const double* acc) {
-  const int c = threadIdx.x & 31;
-  int act = 0, bad = 0;
-  if (c < k && cur.active[c] != 0) {
-    const double rzn = acc[c], rr = acc[k + c];
-    if (!is_finite(rzn) || !is_finite(rr)) {
-      bad = 1;
-    } else {
-      const double rel = sqrt(rr / cur.bnorm2[c]);
-      const double bta = rzn / cur.rz[c];  // computed alongside rel, kept only if not converged
-      s->relres[c] = rel;
-      if (rel <= cur.tol) {
-        s->active[c] = 0;
-        s->beta[c] = 0.0;
-      } else {
-        s->beta[c] = bta;
-        s->rz[c] = rzn;
-        act = 1;
-      }
-    }
-  }
-  const int nact = __popc(__ballot_sync(0xffffffffu, act));
-  const int anybad = __any_sync(0xffffffffu, bad);
-  int done = 0;
-  if (c == 0) {
-    const int it = cur.iter + 1;
-    s->iter = it;
-    if (anybad) {
-      s->status = IG_ERR_NONFINITE;
-      done = 1;
-    } else if (nact == 0) {
-      done = 1;
-    } else if (it >= cur.max_iter) {
-      s->status = IG_ERR_NOT_CONVERGED;
-      done = 1;
-    }
-    if (done) s->done = 1;
-  }
-  return done;
-}
-
 // ------------------------------------------------------------------------------- init
 // rhs = M * in (rhs_mass) or in; x = 0; r = rhs; z = D^-1 r; p = q = 0; per mesh: rz, ||rhs||^2.
 template <int K>
 __global__ void __launch_bounds__(kBlock) init_kernel(const MeshDev* __restrict__ mds, const int2* __restrict__ tiles,
                                                       IoTable io, int rhs_mass, LoopCtl* ctl, double tol,
                                                       int max_iter, int cap) {
-  __shared__ double sh[2 * K * kBlock];
   const int2 tl = tiles[blockIdx.x];
   const MeshDev& md = mds[tl.x];
   const long nn = md.n;
@@ -146,7 +67,7 @@ __global__ void __launch_bounds__(kBlock) init_kernel(const MeshDev* __restrict_
       acc[K + c] = fma(b, b, acc[K + c]);
     }
   }
-  if (reduce_tiles<2 * K>(acc, md.part, tl.y, md.ntiles, &md.s->cnt[2], sh) && threadIdx.x == 0)
+  if (reduce_tiles<2 * K>(acc, md.part, tl.y, md.ntiles, &md.s->cnt[2]) && threadIdx.x == 0)
     finish_init(md.s, K, acc, tol, max_iter);
 }
 
@@ -182,10 +103,11 @@ __device__ __forceinline__ void spmv_tile(const MeshDev& md, int tile, const Sca
       const double b = sn.beta[c];
       const double pn = fma(b, pi[c], zi[c]);
       const double qn = fma(b, qi[c], w[c]);
-      p[row * KP<K>::v + c] = pn;
+      pi[c] = pn;
       q[c * nn + row] = qn;
       pq[c] = fma(pn, qn, pq[c]);
     }
+    store_row<K>(p, row, pi);
   }
   tile_reduce<K>(pq, red, out);
 }
@@ -282,116 +204,11 @@ __global__ void __launch_bounds__(kBlock, 4) update_kernel(const MeshDev* __rest
   }
 }
 
-// ------------------------------------------------------------------------------- small meshes
-// The whole iteration loop of a small single mesh (at most kSmallTiles FP64 tiles) in one
-// thread-block cluster with one CTA per tile. A CTA runs its tile through the tile bodies of the
-// multi-CTA kernels and publishes the tile's partial sums; after a cluster barrier every CTA adds
-// all the partials in tile order and runs the finish step on its own shared-memory copy of the
-// solve state (the same inputs and arithmetic in every CTA, so the copies stay equal), and goes
-// on. Two cluster barriers per iteration replace the kernel boundaries, the last-CTA hand-offs
-// and the graph loop's node transitions, which make up most of an iteration of a mesh of a few
-// tiles. The arithmetic and its order are those of the multi-CTA path: the same bits. The SpMV's
-// and the update's partials live in separate halves of the partial buffer, so a CTA that runs
-// ahead never overwrites partials that another CTA is still adding.
-__device__ __forceinline__ void cluster_sync_all() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-template <int NV, typename Finish>
-__device__ __forceinline__ void finish_cluster(TileCtx& tc, SolveScal& st, const double* part, int nt,
-                                               const Finish& finish) {
-  double v[NV];
-  gather_partials<NV>(part, nt, v);
-  if (threadIdx.x < (int)(sizeof(SolveScal) / 4))
-    reinterpret_cast<unsigned*>(&tc.cur)[threadIdx.x] = reinterpret_cast<const unsigned*>(&st)[threadIdx.x];
-  tile_reduce<NV>(v, tc.red[0], tc.tot);
-  __syncthreads();
-  if (threadIdx.x < 32) finish(&st, tc.cur, tc.tot);
-  __syncthreads();
-}
-
-template <int K>
-__global__ void __launch_bounds__(kBlock) solve_cluster_kernel(const MeshDev* __restrict__ mds, LoopCtl* ctl) {
-  __shared__ TileCtx tc;
-  __shared__ SolveScal st;
-  load_mesh(mds, 0, tc);
-  const int nt = tc.md.ntiles, tile = blockIdx.x;
-  static_assert(sizeof(SolveScal) % 4 == 0 && sizeof(SolveScal) / 4 <= kBlock, "SolveScal copy");
-  if (threadIdx.x < (int)(sizeof(SolveScal) / 4))
-    reinterpret_cast<unsigned*>(&st)[threadIdx.x] = __ldcg(reinterpret_cast<const unsigned*>(tc.md.s) + threadIdx.x);
-  __syncthreads();
-  double* part_spmv = tc.md.part;
-  double* part_upd = tc.md.part + (long)nt * kPartStride;
-  const int cap = __ldcg(&ctl->cap);
-  int it = 0;
-  for (; it < cap && !st.done; ++it) {
-    if (threadIdx.x < kMaxK) tc.sn.beta[threadIdx.x] = st.beta[threadIdx.x];
-    __syncthreads();
-    spmv_tile<K>(tc.md, tile, tc.sn, tc.red[1], part_spmv + (long)tile * kPartStride);
-    cluster_sync_all();
-    finish_cluster<K>(tc, st, part_spmv, nt,
-                      [](SolveScal* s, const SolveScal& cur, const double* v) { finish_spmv(s, cur, K, v); });
-    if (threadIdx.x < kMaxK) tc.sn.alpha[threadIdx.x] = st.alpha[threadIdx.x];
-    __syncthreads();
-    update_tile<K>(tc.md, tile, tc.sn, tc.red[1], part_upd + (long)tile * kPartStride);
-    cluster_sync_all();
-    finish_cluster<2 * K>(tc, st, part_upd, nt,
-                          [](SolveScal* s, const SolveScal& cur, const double* v) { finish_update(s, cur, K, v); });
-  }
-  if (blockIdx.x == 0) {
-    if (threadIdx.x < (int)(sizeof(SolveScal) / 4))
-      reinterpret_cast<unsigned*>(tc.md.s)[threadIdx.x] = reinterpret_cast<const unsigned*>(&st)[threadIdx.x];
-    if (threadIdx.x == 0) {
-      ctl->iter = it;
-      ctl->all_done = 1;
-    }
-  }
-}
-
-// Launch of the cluster loop: one cluster of ntiles CTAs (non-portable sizes above 8 allowed).
-// Returns false, with nothing launched, when the device refuses that cluster.
-template <int K>
-bool launch_cluster_loop(Group& g, cudaStream_t st) {
-  const int nt = g.host_mds[0].ntiles;
-  static bool attr_set = false;
-  if (!attr_set) {
-    if (cudaFuncSetAttribute(solve_cluster_kernel<K>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-        cudaSuccess) {
-      cudaGetLastError();
-      return false;
-    }
-    attr_set = true;
-  }
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(nt, 1, 1);
-  cfg.blockDim = dim3(kBlock, 1, 1);
-  cfg.dynamicSmemBytes = 0;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = nt;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  int clusters = 0;
-  if (cudaOccupancyMaxActiveClusters(&clusters, solve_cluster_kernel<K>, &cfg) != cudaSuccess || clusters < 1) {
-    cudaGetLastError();
-    return false;
-  }
-  if (cudaLaunchKernelEx(&cfg, solve_cluster_kernel<K>, (const MeshDev*)g.mds, g.ctl) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return true;
-}
-
 // ------------------------------------------------------------------------------- true residual
 // trueres = ||rhs - A x|| / ||rhs|| per column with x = io.out (the written solution).
 template <int K>
 __global__ void __launch_bounds__(kBlock) residual_kernel(const MeshDev* __restrict__ mds,
                                                           const int2* __restrict__ tiles, IoTable io, int rhs_mass) {
-  __shared__ double sh[K * kBlock];
   const int2 tl = tiles[blockIdx.x];
   const MeshDev& md = mds[tl.x];
   const long nn = md.n;
@@ -414,7 +231,7 @@ __global__ void __launch_bounds__(kBlock) residual_kernel(const MeshDev* __restr
       acc[c] = fma(res, res, acc[c]);
     }
   }
-  if (reduce_tiles<K>(acc, md.part, tl.y, md.ntiles, &md.s->cnt[2], sh) && threadIdx.x == 0) {
+  if (reduce_tiles<K>(acc, md.part, tl.y, md.ntiles, &md.s->cnt[2]) && threadIdx.x == 0) {
     for (int c = 0; c < K; ++c) {
       const double r2 = md.s->rhs2[c];
       md.s->trueres[c] = r2 > 0.0 ? sqrt(acc[c] / r2) : sqrt(acc[c]);
@@ -503,9 +320,6 @@ cudaError_t host_loop_k(Group& g, int max_it, int poll, cudaStream_t st) {
 
 template <int K>
 cudaError_t loop_k(Group& g, const ig_solve_opts& o, cudaStream_t st) {
-  if (o.launch == IG_LAUNCH_GRAPH && !prof_on() && g.nmesh == 1 && g.host_mds[0].ntiles <= kSmallTiles &&
-      launch_cluster_loop<K>(g, st))
-    return cudaSuccess;
   if (o.launch == IG_LAUNCH_GRAPH && !prof_on()) {
     SolvePlan& pl = g.plans[0][K];
     if (!pl.exec) {
@@ -526,6 +340,8 @@ cudaError_t end_k(Group& g, const IoTable& io, cudaStream_t st) {
 
 template <int K>
 cudaError_t solve_k(Group& g, const IoTable& io, int rhs_mass, const ig_solve_opts& o, cudaStream_t st) {
+  if (o.launch == IG_LAUNCH_GRAPH && !prof_on() && launch_resident(g, K, io.in[0], io.out[0], rhs_mass, o, st))
+    return cudaSuccess;
   cudaError_t e = begin_k<K>(g, io, rhs_mass, o, st);
   if (e == cudaSuccess) e = loop_k<K>(g, o, st);
   if (e == cudaSuccess) e = end_k<K>(g, io, st);
@@ -957,7 +773,7 @@ extern "C" ig_status ig_solve_csr_noalloc(const int32_t* rowptr_dev, const int32
   info->k = k;
   info->iterations = s.iter;
   for (int c = 0; c < k; ++c) {
-    info->rel_residual[c] = s.relres[c];
+    info->rel_residual[c] = sqrt(s.relres2[c]);
     info->true_rel_residual[c] = s.trueres[c];
   }
   return (ig_status)info->status;

@@ -54,8 +54,7 @@ __device__ __noinline__ void finish_init_mixed(SolveScal* s, int k, const double
     s->bnorm2[c] = 0.0;
     s->active64[c] = act;
     s->active[c] = 0;
-    s->relres[c] = act ? 1.0 : 0.0;
-    s->relres_inner[c] = 0.0;
+    s->relres2[c] = act ? 1.0 : 0.0;
     s->scale[c] = act ? sqrt(bb) : 1.0;
     s->rz[c] = 0.0;
     s->alpha[c] = 0.0;
@@ -93,9 +92,9 @@ __device__ __noinline__ void finish_residual(SolveScal* s, const SolveScal& cur,
     if (!is_finite(res2[c])) {
       bad = 1;
     } else {
-      const double rel = sqrt(res2[c] / cur.rhs2[c]);
-      s->relres[c] = rel;
-      if (rel <= cur.tol || !positive_finite(res2[c])) {
+      const double rel2 = res2[c] / cur.rhs2[c];  // squares, as in finish_update
+      s->relres2[c] = rel2;
+      if (rel2 <= cur.tol * cur.tol || !positive_finite(res2[c])) {
         s->active64[c] = 0;
       } else {
         s->scale[c] = sqrt(res2[c]);
@@ -132,7 +131,6 @@ __device__ __noinline__ int finish_restart(SolveScal* s, const SolveScal& cur, i
     s->bnorm2[c] = acc[k + c];
     s->alpha[c] = 0.0;
     s->beta[c] = 0.0;
-    s->relres_inner[c] = act ? 1.0 : 0.0;
   }
   const int nact = __popc(__ballot_sync(0xffffffffu, act));
   const int phase = nact ? kPhaseInner : kPhaseApply;
@@ -146,17 +144,20 @@ __device__ __noinline__ int finish_restart(SolveScal* s, const SolveScal& cur, i
 // Inner FP32 iteration: inner convergence test, beta, switch to Apply when the inner solve is done.
 // Returns (on lane 0) the phase after it, or -1 when the mesh is done (a non-finite sum).
 __device__ __noinline__ int finish_update_mixed(SolveScal* s, const SolveScal& cur, int k, const double* acc) {
-  const int c = threadIdx.x & 31;
+  const int c = threadIdx.x & 31, col = c & 7;
   int act = 0, bad = 0;
+  const double* den = c < 8 ? cur.rz : cur.bnorm2;  // the divisions side by side, the test on squares (finish_update)
+  const double* num = c < 8 ? acc : acc + k;
+  double quot = 0.0;
+  if (col < k && c < 16) quot = num[col] / den[col];
+  const double rel2 = __shfl_down_sync(0xffffffffu, quot, 8);
   if (c < k && cur.active[c] != 0) {
     const double rzn = acc[c], rr = acc[k + c];
     if (!is_finite(rzn) || !is_finite(rr)) {
       bad = 1;
     } else {
-      const double rel = sqrt(rr / cur.bnorm2[c]);
-      const double bta = rzn / cur.rz[c];  // computed alongside rel, kept only if not converged
-      s->relres_inner[c] = rel;
-      if (rel <= cur.inner_tol || !positive_finite(rzn)) {
+      const double bta = quot;
+      if (rel2 <= cur.inner_tol * cur.inner_tol || !positive_finite(rzn)) {
         s->active[c] = 0;
         s->beta[c] = 0.0;
       } else {
@@ -191,7 +192,6 @@ __global__ void __launch_bounds__(kBlock) init_mixed_kernel(const MeshDev* __res
                                                             const int2* __restrict__ tiles, IoTable io, int rhs_mass,
                                                             LoopCtl* ctl, double tol, double inner_tol, int max_iter,
                                                             int max_refine, int cap) {
-  __shared__ double sh[K * kBlock];
   const int2 tl = tiles[blockIdx.x];
   const MeshDev& md = mds[tl.x];
   const long nn = md.n;
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(kBlock) init_mixed_kernel(const MeshDev* __res
       }
     }
   }
-  if (reduce_tiles<K>(acc, md.part, tl.y, md.ntiles32, &md.s->cnt[2], sh) && threadIdx.x == 0)
+  if (reduce_tiles<K>(acc, md.part, tl.y, md.ntiles32, &md.s->cnt[2]) && threadIdx.x == 0)
     finish_init_mixed(md.s, K, acc, tol, inner_tol, max_iter, max_refine);
 }
 

@@ -1,0 +1,517 @@
+// ig_resident.cu -- the FP64 conjugate-gradient solve of a single mesh in one launch, with the mesh's
+// rows held in shared memory (the solve of ig_pcg.cu: the same row arithmetic, tiles and order of the
+// sums, so the same bits).
+//
+// A mesh of at most kResMaxRows rows per SM gets one tile per CTA and at most one CTA per SM
+// (choose_tiles64 in ig_api.cu). Its CTAs keep their rows' operator, direction, residual and solution
+// on chip through the whole solve; only z = D^-1 r, which the neighbours' rows gather, goes through
+// global memory (L2). Per iteration the CTAs meet twice, to add p.q and then r.z and r.r; every CTA adds
+// all the tiles' partials in tile order and runs the finish step on its own copy of the solve state,
+// so no step waits for one last CTA, and no kernel boundary or graph node lies in the loop.
+//
+// Measured, per iteration (the two-kernel graph loop before, and this): 163,842 rows k = 3 41 -> 26 us
+// and k = 4 47 -> 31 us, 66,049 rows k = 1 23 -> 8.5 us, 5,917 rows k = 1 20.6 -> 8.5 us, 642 rows k = 3
+// (a cluster of 6 CTAs; three CTAs of 256 rows before) 10 -> 6 us.
+//
+// What bounds it: on large meshes FP64 instructions and the gathers of z together. A warp's FP64
+// instruction occupies its SM sub-partition for 64 cycles (16 per SM), so the 45 per row and iteration
+// (three columns) take 11.7 us on 163,842 rows; eight row warps are enough to issue them, and fewer
+// threads leave fewer sums to add (the sums of 32 warps would take 2.2 us of FP64 issue in the
+// update alone, those of 8 a quarter). On small meshes the chain of an iteration: two gathers, two
+// meetings of about 1 us (a store to L2, then a load that sees it), and sums and divisions whose every
+// FP64 step costs 64 cycles.
+#include "ig_device.cuh"
+
+namespace ig {
+
+namespace {
+
+// One posted value: the number of the meeting beside it, written and read as one 16-byte word, so
+// that a reader that sees the number has the value. Slots alternate between two buffers: a CTA
+// posts for meeting i + 2 only after meeting i + 1, for which every CTA had read the slots of i.
+struct __align__(16) Slot {
+  double value;
+  unsigned long long number;
+};
+constexpr int kSpinLimit = 1 << 21;  // polls of one wait (about a second); then the solve fails
+
+__device__ __forceinline__ void post(Slot* s, double value, unsigned long long number) {
+  asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(s),
+               "l"(__double_as_longlong(value)), "l"(number)
+               : "memory");
+}
+// ACQUIRE: with the value comes what its CTA released (an acquire load per slot: a fence after
+// relaxed loads took the geodesic case from 8.3 to 9.6 us an iteration).
+template <bool ACQUIRE>
+__device__ __forceinline__ bool peek(const Slot* s, unsigned long long number, double& value) {
+  unsigned long long a, b;
+  if constexpr (ACQUIRE)
+    asm volatile("{\n\t.reg .b128 t;\n\tld.acquire.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+                 : "=l"(a), "=l"(b)
+                 : "l"(s)
+                 : "memory");
+  else
+    asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+                 : "=l"(a), "=l"(b)
+                 : "l"(s)
+                 : "memory");
+  value = __longlong_as_double((long long)a);
+  return b == number;
+}
+__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ double peer_load(const double* p, int rank) {
+  unsigned a = (unsigned)__cvta_generic_to_shared(p), r;
+  double v;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+  asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(r) : "memory");
+  return v;
+}
+
+// What the host lays out in dynamic shared memory: rows of rp entries; aw slots of the operator (a
+// wider slice's further slots are read from global memory), and the solution when it fits.
+struct ResLayout {
+  int rp;      // rows per CTA
+  int aw;      // operator slots per row on chip
+  int x_on;    // the solution is on chip
+  int bytes;
+};
+
+struct ResShared {
+  MeshDev md;
+  SolveScal st;
+  double red[8 * kWarps];
+  double red2[8 * kWarps];
+  double tot[8];
+  double box[2][8];          // cluster: this CTA's posted sums, by parity of the meeting
+  int width[kResMaxRows / 32];
+};
+
+constexpr int kResThreads = kBlock + 32;  // eight warps take the rows; the ninth posts and finishes
+
+// Where the CTAs meet. CLUSTER: all of them form one thread-block cluster (at most 16 CTAs).
+//
+// A meeting adds per-thread sums over all tiles, in three steps between CTA barriers: the row warps
+// leave their warps' totals in red; the ninth warp adds them and posts the tile's sums; the row warps
+// collect every tile's sums, a few per lane, into red2. The caller's ninth warp then adds red2.
+template <bool CLUSTER>
+struct Meeting {
+  Slot* slots;
+  int nct;
+  unsigned long long number;
+
+  // ninth warp: the tile's sums, posted. RELEASE: what the CTA wrote to global memory before is
+  // visible to the CTAs that collect them. (The product's meeting needs no order beyond its data:
+  // its sums depend on every z the CTA gathered, and the z written next depends on the sums.)
+  template <int NV, bool RELEASE>
+  __device__ __forceinline__ void post_sums(ResShared& sh) {
+    const int lane = threadIdx.x & 31;
+    const double a = add_warps<NV>(sh.red);
+    const bool writer = (lane & 3) == 0 && (lane >> 2) < NV;
+    if constexpr (CLUSTER) {
+      if (writer) sh.box[number & 1][lane >> 2] = a;
+    } else {
+      if (RELEASE) fence_gpu();
+      if (writer) post(slots + (number & 1) * (8 * (size_t)nct) + 8 * (size_t)blockIdx.x + (lane >> 2), a, number);
+    }
+  }
+
+  // row warps: every tile's sums into red2 (ACQUIRE: with what their CTAs released). Returns true
+  // when a wait ran out.
+  template <int NV, bool ACQUIRE>
+  __device__ __forceinline__ bool collect(ResShared& sh) {
+    using Map = PartialMap<NV>;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, val = Map::value(lane);
+    const int first = Map::first(warp, lane);
+    double a = 0.0;
+    bool late = false;
+    if constexpr (CLUSTER) {
+      for (int t = first; t < nct; t += Map::kStride)
+        if (val < NV) a += peer_load(&sh.box[number & 1][val], t);
+    } else {
+      const Slot* buf = slots + (number & 1) * (8 * (size_t)nct) + val;
+      constexpr int J = (kResMaxCtas + Map::kStride - 1) / Map::kStride;
+      double b[J];
+      unsigned want = 0;
+#pragma unroll
+      for (int j = 0; j < J; ++j) {
+        b[j] = 0.0;
+        if (val < NV && first + j * Map::kStride < nct) want |= 1u << j;
+      }
+      for (int spins = 0; want != 0 && !late; late = ++spins > kSpinLimit) {
+#pragma unroll
+        for (int j = 0; j < J; ++j)
+          if (want >> j & 1) {
+            double x;
+            if (peek<ACQUIRE>(buf + 8 * (size_t)(first + j * Map::kStride), number, x)) {
+              b[j] = x;
+              want &= ~(1u << j);
+            }
+          }
+      }
+      const int steps = (nct + Map::kStride - 1) / Map::kStride;
+#pragma unroll
+      for (int j = 0; j < J; ++j)
+        if (j < steps) a += b[j];
+    }
+    Map::to_warp_total(a, sh.red2);
+    return late;
+  }
+
+  // One meeting up to the barrier after which red2 is complete; true when a wait ran out.
+  template <int NV, bool RELEASE>
+  __device__ __forceinline__ bool meet(ResShared& sh, double (&v)[NV], bool row_warp, bool has_rows) {
+    ++number;
+    if (row_warp) {
+      if (has_rows) warp_totals<NV>(v, sh.red);
+      else if ((threadIdx.x & 31) < NV) sh.red[(threadIdx.x & 31) * kWarps + (threadIdx.x >> 5)] = 0.0;
+    }
+    __syncthreads();
+    if (!row_warp) post_sums<NV, RELEASE>(sh);
+    if constexpr (CLUSTER) cluster_sync_all();
+    bool late = false;
+    if (row_warp) late = collect<NV, RELEASE>(sh);
+    return __syncthreads_or(late) != 0;
+  }
+};
+
+// Four operator slots of one row: values and the gathered rows of z.
+template <int K>
+struct Slots4 {
+  double a[4], v[4][K];
+  __device__ __forceinline__ void load(const MeshDev& md, const double* sa, const int* sc, int rp, int i, int j0,
+                                       int on) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (j0 + u < on) {
+        a[u] = sa[(j0 + u) * rp + i];
+        const int col = sc[(j0 + u) * rp + i];
+        load_row<K>(md.z, IG_IN_RANGE(col, md.n, md.err) ? col : 0, v[u]);
+      }
+  }
+  __device__ __forceinline__ void add_to(double (&w)[K], int j0, int on) const {
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (j0 + u < on) {
+#pragma unroll
+        for (int c = 0; c < K; ++c) w[c] = fma(a[u], v[u][c], w[c]);
+      }
+  }
+};
+
+// The slots from the ninth on of a wide row: on chip up to `on`, the rest from global memory.
+template <int K>
+__device__ __forceinline__ void wide_slots(const MeshDev& md, const double* sa, const int* sc, int rp, int i, int on,
+                                           int width, long row, double (&w)[K]) {
+  for (int j = 8; j < on; ++j) {
+    const int col = sc[j * rp + i];
+    double v[K];
+    load_row<K>(md.z, IG_IN_RANGE(col, md.n, md.err) ? col : 0, v);
+#pragma unroll
+    for (int c = 0; c < K; ++c) w[c] = fma(sa[j * rp + i], v[c], w[c]);
+  }
+  const long e = __ldg(md.sell_ptr + (row >> 5)) + (row & 31);
+  for (int j = on; j < width; ++j) {
+    const double a = __ldg(md.A + e + 32 * j);
+    const int col = __ldg(md.sell_col + e + 32 * j);
+    double v[K];
+    load_row<K>(md.z, IG_IN_RANGE(col, md.n, md.err) ? col : 0, v);
+#pragma unroll
+    for (int c = 0; c < K; ++c) w[c] = fma(a, v[c], w[c]);
+  }
+}
+
+template <int K, bool CLUSTER>
+__global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const MeshDev* __restrict__ mds,
+                                                                        const double* __restrict__ in,
+                                                                        double* __restrict__ out, int rhs_mass,
+                                                                        double tol, int max_iter, int cap,
+                                                                        ResLayout lay) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ ResShared sh;
+  {
+    static_assert(sizeof(MeshDev) % 4 == 0 && sizeof(SolveScal) % 4 == 0, "copied as 4-byte words");
+    const unsigned* src = reinterpret_cast<const unsigned*>(mds);
+    for (int j = threadIdx.x; j < (int)(sizeof(MeshDev) / 4); j += kResThreads)
+      reinterpret_cast<unsigned*>(&sh.md)[j] = __ldg(src + j);
+    __syncthreads();
+    for (int j = threadIdx.x; j < (int)(sizeof(SolveScal) / 4); j += kResThreads)
+      reinterpret_cast<unsigned*>(&sh.st)[j] = __ldcg(reinterpret_cast<const unsigned*>(sh.md.s) + j);
+  }
+  const MeshDev& md = sh.md;
+  const int tid = threadIdx.x;
+  const bool row_warp = tid < kBlock;
+  const long nn = md.n;
+  const long t0 = (long)blockIdx.x * md.tile_rows;
+  // the ninth warp has no rows
+  const int rows = !row_warp ? 0 : (int)(nn - t0 < md.tile_rows ? nn - t0 : md.tile_rows);
+  const bool has_rows = (tid & ~31) < rows;  // this warp has a row
+  const int rp = lay.rp, aw = lay.aw;
+  double* q = reinterpret_cast<double*>(dyn);
+  double* p = q + K * rp;
+  double* r = p + K * rp;
+  double* dinv = r + K * rp;
+  double* sa = dinv + rp;
+  double* xs = sa + (size_t)aw * rp;
+  int* sc = reinterpret_cast<int*>(xs + (lay.x_on ? K * rp : 0));
+  double* x = lay.x_on ? xs : md.x + t0;   // component c of row i at x[c * xn + i]
+  const long xn = lay.x_on ? rp : nn;
+  double* z = md.z;
+
+  // the rows' operator on chip; slices of 32 rows, one per warp and step
+  for (int i = tid; i < rows; i += kBlock) {
+    const long row = t0 + i;
+    const int sl = (int)(row >> 5);
+    const int b0 = __ldg(md.sell_ptr + sl), w = (__ldg(md.sell_ptr + sl + 1) - b0) >> 5;
+    if ((i & 31) == 0) sh.width[i >> 5] = w;
+    const long e = b0 + (row & 31);
+    for (int j = 0; j < (w < aw ? w : aw); ++j) {
+      sa[j * rp + i] = __ldg(md.A + e + 32 * j);
+      sc[j * rp + i] = __ldg(md.sell_col + e + 32 * j);
+    }
+    dinv[i] = md.Dinv[row];
+  }
+
+  Meeting<CLUSTER> mt;
+  mt.slots = reinterpret_cast<Slot*>(md.meet) + 1;
+  mt.nct = gridDim.x;
+  // numbers of this launch: above those of every launch before it (the word ahead of the slots
+  // counts launches; CTA 0 advances it at the end, when every CTA has long read it)
+  unsigned long long launches = 0;
+  if constexpr (!CLUSTER) launches = __ldcg(reinterpret_cast<const unsigned long long*>(md.meet));
+  mt.number = launches << 32;
+
+  // start: rhs = M * in or in; r = rhs, z = D^-1 r, p = q = x = 0; r.z and |rhs|^2
+  bool late;
+  {
+    double acc[2 * K];
+#pragma unroll
+    for (int c = 0; c < 2 * K; ++c) acc[c] = 0.0;
+    for (int i = tid; i < rows; i += kBlock) {
+      const long row = t0 + i;
+      const double d = dinv[i];
+      const double mass = rhs_mass ? md.M[row] : 1.0;
+      double zo[K];
+#pragma unroll
+      for (int c = 0; c < K; ++c) {
+        const double b = rhs_mass ? mass * in[row * K + c] : in[row * K + c];
+        zo[c] = d * b;
+        x[c * xn + i] = 0.0;
+        p[c * rp + i] = 0.0;
+        q[c * rp + i] = 0.0;
+        r[c * rp + i] = b;
+        acc[c] = fma(b, zo[c], acc[c]);
+        acc[K + c] = fma(b, b, acc[K + c]);
+      }
+      store_row<K>(z, row, zo);
+    }
+    late = mt.template meet<2 * K, true>(sh, acc, row_warp, has_rows);
+    if (!row_warp) {
+      add_warps_to<2 * K>(sh.red2, sh.tot);
+      __syncwarp();
+      if (tid == kBlock) finish_init(&sh.st, K, sh.tot, tol, max_iter);
+    }
+  }
+
+  for (int it = 0; it < cap && !late; ++it) {
+    // p = z + beta p, q = A z + beta q, p.q. A row's product needs only z, which is there: the row
+    // warps start on their first row's while the ninth warp finishes the meeting before (beta, done).
+    {
+      double beta[K], pq[K];
+#pragma unroll
+      for (int c = 0; c < K; ++c) {
+        beta[c] = 0.0;
+        pq[c] = 0.0;
+      }
+      // The slots are taken four at a time, and the loads run ahead of the arithmetic: the second
+      // four are under way while the first are added, the next row's first four while the rest of
+      // this row is. Two warps share a sub-partition's FP64 unit and would otherwise wait for their
+      // loads together.
+      bool waiting = true;
+      Slots4<K> s0, s1;
+      int width = 0, on = 0;
+      if ((tid & ~31) < rows) {
+        width = sh.width[tid >> 5];
+        on = width < aw ? width : aw;
+        s0.load(md, sa, sc, rp, tid < rows ? tid : rows - 1, 0, on);
+      }
+      for (int i = tid; (i & ~31) < rows; i += kBlock) {  // whole warps: a barrier is inside
+        const int ii = i < rows ? i : rows - 1;
+        double w[K];
+#pragma unroll
+        for (int c = 0; c < K; ++c) w[c] = 0.0;
+        double zi[K];
+        s1.load(md, sa, sc, rp, ii, 4, on);
+        load_row<K>(z, t0 + ii, zi);
+        s0.add_to(w, 0, on);
+        const int on_i = on, width_i = width, next = i + kBlock;
+        if ((next & ~31) < rows) {
+          width = sh.width[next >> 5];
+          on = width < aw ? width : aw;
+          s0.load(md, sa, sc, rp, next < rows ? next : rows - 1, 0, on);
+        }
+        s1.add_to(w, 4, on_i);
+        if (width_i > 8 || on_i < width_i) wide_slots<K>(md, sa, sc, rp, ii, on_i, width_i, t0 + i, w);
+        if (waiting) {
+          waiting = false;
+          __syncthreads();
+          if (sh.st.done) break;
+#pragma unroll
+          for (int c = 0; c < K; ++c) beta[c] = sh.st.beta[c];
+        }
+        if (i < rows) {
+#pragma unroll
+          for (int c = 0; c < K; ++c) {
+            const double pn = fma(beta[c], p[c * rp + i], zi[c]);
+            const double qn = fma(beta[c], q[c * rp + i], w[c]);
+            p[c * rp + i] = pn;
+            q[c * rp + i] = qn;
+            pq[c] = fma(pn, qn, pq[c]);
+          }
+        }
+      }
+      if (waiting) __syncthreads();
+      if (sh.st.done) break;
+      late = mt.template meet<K, false>(sh, pq, row_warp, has_rows);
+      if (late) break;
+      if (!row_warp) {
+        add_warps_to<K>(sh.red2, sh.tot);
+        __syncwarp();
+        finish_spmv(&sh.st, sh.st, K, sh.tot);
+      }
+      __syncthreads();
+    }
+    // x += alpha p, r -= alpha q, z = D^-1 r, r.z and r.r
+    {
+      double alpha[K], acc[2 * K];
+#pragma unroll
+      for (int c = 0; c < K; ++c) {
+        alpha[c] = sh.st.alpha[c];
+        acc[c] = 0.0;
+        acc[K + c] = 0.0;
+      }
+      for (int i = tid; i < rows; i += kBlock) {
+        const double d = dinv[i];
+        double rn[K], zo[K];
+#pragma unroll
+        for (int c = 0; c < K; ++c) {
+          rn[c] = fma(-alpha[c], q[c * rp + i], r[c * rp + i]);
+          zo[c] = d * rn[c];
+          r[c * rp + i] = rn[c];
+        }
+        store_row<K>(z, t0 + i, zo);
+#pragma unroll
+        for (int c = 0; c < K; ++c) {
+          x[c * xn + i] = fma(alpha[c], p[c * rp + i], x[c * xn + i]);
+          acc[c] = fma(rn[c], zo[c], acc[c]);
+          acc[K + c] = fma(rn[c], rn[c], acc[K + c]);
+        }
+      }
+      late = mt.template meet<2 * K, true>(sh, acc, row_warp, has_rows);
+      if (late) break;
+      if (!row_warp) {
+        add_warps_to<2 * K>(sh.red2, sh.tot);
+        __syncwarp();
+        finish_update(&sh.st, sh.st, K, sh.tot);
+      }
+    }
+  }
+  for (int i = tid; i < rows; i += kBlock) {
+#pragma unroll
+    for (int c = 0; c < K; ++c) out[(t0 + i) * K + c] = x[c * xn + i];
+  }
+  if (late && tid == kBlock) {  // a CTA stayed away past the limit: report a failed solve
+    sh.st.status = IG_ERR_CUDA;
+    sh.st.done = 1;
+  }
+  __syncthreads();
+  if (blockIdx.x == 0) {
+    for (int j = tid; j < (int)(sizeof(SolveScal) / 4); j += kResThreads)
+      reinterpret_cast<unsigned*>(md.s)[j] = reinterpret_cast<const unsigned*>(&sh.st)[j];
+    if (!CLUSTER && tid == 0) *reinterpret_cast<unsigned long long*>(md.meet) = launches + 1;
+  }
+  if constexpr (CLUSTER) cluster_sync_all();  // no CTA leaves while another reads its sums
+}
+
+// Shared memory of a CTA of rp rows: everything, less the solution, then less operator slots, as far
+// as the SM's 227 KB demand.
+template <int K>
+ResLayout layout(int rp, int wmax) {
+  const int room = 227 * 1024 - (int)sizeof(ResShared) - 256;
+  const int fixed = rp * 8 * (3 * K + 1);
+  ResLayout l{};
+  l.rp = rp;
+  l.x_on = fixed + rp * 8 * K + 12 * rp * wmax <= room;
+  const int left = room - fixed - (l.x_on ? rp * 8 * K : 0);
+  l.aw = left / (12 * rp) < wmax ? left / (12 * rp) : wmax;
+  l.bytes = fixed + (l.x_on ? rp * 8 * K : 0) + 12 * rp * l.aw;
+  return l;
+}
+
+template <int K, bool CLUSTER>
+bool launch_k(Group& g, const double* in, double* out, int rhs_mass, const ig_solve_opts& o, cudaStream_t st) {
+  const MeshDev& md = g.host_mds[0];
+  auto kern = solve_resident_kernel<K, CLUSTER>;
+  const ResLayout lay = layout<K>(md.tile_rows, md.sell_wmax);
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, lay.bytes) != cudaSuccess ||
+      (CLUSTER && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
+    cudaGetLastError();
+    return false;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(md.ntiles, 1, 1);
+  cfg.blockDim = dim3(kResThreads, 1, 1);
+  cfg.dynamicSmemBytes = lay.bytes;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  if (CLUSTER) {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = md.ntiles;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+  } else {
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (CLUSTER) {
+    int clusters = 0;
+    if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters < 1) {
+      cudaGetLastError();
+      return false;
+    }
+  }
+  if (cudaLaunchKernelEx(&cfg, kern, (const MeshDev*)g.mds, in, out, rhs_mass, o.rel_tol, o.max_iter, o.max_iter + 2,
+                         lay) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return true;
+}
+
+template <int K>
+bool launch(Group& g, const double* in, double* out, int rhs_mass, const ig_solve_opts& o, cudaStream_t st) {
+  if (g.host_mds[0].ntiles <= kClusterTiles && launch_k<K, true>(g, in, out, rhs_mass, o, st)) return true;
+  return launch_k<K, false>(g, in, out, rhs_mass, o, st);
+}
+
+}  // namespace
+
+size_t meet_bytes(int ntiles) { return sizeof(Slot) * (1 + 2 * 8 * (size_t)ntiles); }
+
+bool launch_resident(Group& g, int k, const double* in, double* out, int rhs_mass, const ig_solve_opts& o,
+                     cudaStream_t st) {
+  if (g.nmesh != 1 || !g.host_mds[0].meet) return false;
+  switch (k) {
+    case 1: return launch<1>(g, in, out, rhs_mass, o, st);
+    case 2: return launch<2>(g, in, out, rhs_mass, o, st);
+    case 3: return launch<3>(g, in, out, rhs_mass, o, st);
+    case 4: return launch<4>(g, in, out, rhs_mass, o, st);
+    default: return false;
+  }
+}
+
+}  // namespace ig

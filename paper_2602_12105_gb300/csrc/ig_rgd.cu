@@ -486,7 +486,6 @@ __global__ void __launch_bounds__(kBlock) rgd_gdface_kernel(const MeshDev* __res
 __global__ void __launch_bounds__(kBlock) rgd_warm_kernel(const MeshDev* __restrict__ mds, const double* __restrict__ b,
                                                           const double* __restrict__ u, double* __restrict__ rhs,
                                                           double* ratio) {
-  __shared__ double sh[2 * kBlock];
   const MeshDev& md = mds[0];
   const long n = md.n;
   const int ntile = (int)((n + kTileRows - 1) / kTileRows);
@@ -503,7 +502,7 @@ __global__ void __launch_bounds__(kBlock) rgd_warm_kernel(const MeshDev* __restr
       acc[1] = fma(r, r, acc[1]);
     }
   }
-  if (reduce_tiles<2>(acc, md.part, blockIdx.x, ntile, &md.s->cnt[2], sh) && threadIdx.x == 0)
+  if (reduce_tiles<2>(acc, md.part, blockIdx.x, ntile, &md.s->cnt[2]) && threadIdx.x == 0)
     *ratio = acc[1] > 0.0 ? sqrt(acc[0] / acc[1]) : 1e300;
 }
 
