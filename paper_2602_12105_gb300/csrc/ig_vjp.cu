@@ -12,6 +12,14 @@
 // cot_c = -dot_c / s) and P = -sum_c omega_c dot_c, E_f = P / s + w_a s / 2 and
 //   grad_{p_c} E_f = [ -omega_c (d_{c+2} - d_{c+1}) + (omega_{c+1} - omega_{c+2}) d_c ] / s
 //                    + (w_a / 2 - P / s^2) (N x d_c) / s.
+// N x d_c = dot_{c+2} d_{c+2} - dot_{c+1} d_{c+1}, and d_c = -d_{c+1} - d_{c+2}, so with
+// W_c = omega_c / s and k_c = (w_a / 2 - P / s^2) dot_c / s each corner's gradient is a combination of
+// two edges,
+//   grad_{p_c} E_f = (W_c + e_c - k_{c+1}) d_{c+1} + (e_c - W_c + k_{c+2}) d_{c+2},
+//   e_c = W_{c+2} - W_{c+1},
+// and the third is minus the sum of the other two (E_f does not change when the face moves). The
+// FP64 kernel is bound by FP64 instructions (2 per clock per SM): this form takes about 104 per face
+// (k = 3) where the cross products corner by corner took about 140.
 // (The CPU oracle reaches the same numbers through the per-corner cotangent gradients.)
 //
 // A loss may also depend on V through the mass directly (the M-norm loss of the inverse-fairing
@@ -92,7 +100,7 @@ __global__ void __launch_bounds__(256) vjp_face_kernel(const MeshDev* __restrict
     // per-vertex <Lambda_v, B_v - U_v> and the per-corner <dLambda, dU>; with mass weights w,
     // d(sum_i M_i w_i)/dV adds sum_f ((1/3) sum_{v in f} w_v) grad area_f, i.e. w_v to the sum
     double wa = 0.0;
-    double omega[3] = {0.0, 0.0, 0.0};
+    double W[3] = {0.0, 0.0, 0.0};  // omega_c / s
     if constexpr (MODE != 2) {
       // <Lambda_v, B_v - U_v> of the three vertices, formed once per vertex by vjp_vertex_kernel
       wa = (__ldg(wvert + vid[0]) + __ldg(wvert + vid[1])) + __ldg(wvert + vid[2]);
@@ -105,42 +113,39 @@ __global__ void __launch_bounds__(256) vjp_face_kernel(const MeshDev* __restrict
           Uv[c][k] = U[(long)vid[c] * K + k];
         }
       }
-      const double mt2 = -0.5 * tval;
+      const double mt2 = -0.5 * tval * inv_s;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         const int a = (c + 1) % 3, b = (c + 2) % 3;
-        double lu = 0.0;
+        double lu = (L[a][0] - L[b][0]) * (Uv[a][0] - Uv[b][0]);
 #pragma unroll
-        for (int k = 0; k < K; ++k) lu = fma(L[a][k] - L[b][k], Uv[a][k] - Uv[b][k], lu);
+        for (int k = 1; k < K; ++k) lu = fma(L[a][k] - L[b][k], Uv[a][k] - Uv[b][k], lu);
         // dl/dt = -<Lambda, L U> = -sum_c (cot_c / 2) lu_c = sum_c (dot_c / s / 2) lu_c
         if (CLAMP && clamp_on && -dot[c] * inv_s < clamp_min) {
           // a clamped corner holds cot = clamp_min: no term in dl/dV, clamp_min in dl/dt
-          omega[c] = 0.0;
+          W[c] = 0.0;
           if (gt) gt_part = fma(-0.5 * clamp_min, lu, gt_part);
         } else {
-          omega[c] = mt2 * lu;
+          W[c] = mt2 * lu;
           if (gt) gt_part = fma(0.5 * dot[c] * inv_s, lu, gt_part);
         }
       }
     }
     if constexpr (MODE != 0) wa += (__ldg(cl.wm + vid[0]) + __ldg(cl.wm + vid[1])) + __ldg(cl.wm + vid[2]);
-    wa *= (1.0 / 3.0);
-    const double Pv = -(omega[0] * dot[0] + omega[1] * dot[1] + omega[2] * dot[2]);
-    const double coef = (0.5 * wa - Pv * inv_s * inv_s) * inv_s;
+    wa *= (1.0 / 6.0);  // w_a / 2
+    const double S = fma(W[0], dot[0], fma(W[1], dot[1], W[2] * dot[2]));
+    const double coef = inv_s * fma(inv_s, S, wa);
     double g[9];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
+    for (int c = 0; c < 2; ++c) {
       const int a = (c + 1) % 3, b = (c + 2) % 3;
-      const double om = omega[c] * inv_s;
-      const double dom = (omega[a] - omega[b]) * inv_s;
-      double nxd[3];
-      nxd[0] = N[1] * dd[c][2] - N[2] * dd[c][1];
-      nxd[1] = N[2] * dd[c][0] - N[0] * dd[c][2];
-      nxd[2] = N[0] * dd[c][1] - N[1] * dd[c][0];
+      const double e = W[b] - W[a];
+      const double ca = fma(-coef, dot[a], W[c] + e), cb = fma(coef, dot[b], e - W[c]);
 #pragma unroll
-      for (int d = 0; d < 3; ++d)
-        g[3 * c + d] = fma(coef, nxd[d], fma(dom, dd[c][d], -om * (dd[b][d] - dd[a][d])));
+      for (int d = 0; d < 3; ++d) g[3 * c + d] = fma(ca, dd[a][d], cb * dd[b][d]);
     }
+#pragma unroll
+    for (int d = 0; d < 3; ++d) g[6 + d] = -(g[d] + g[3 + d]);
     double* out = md.gface + 9 * (long)f;
 #pragma unroll
     for (int i = 0; i < 9; ++i) out[i] = g[i];
