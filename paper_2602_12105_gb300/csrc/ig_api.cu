@@ -464,6 +464,18 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
   UP_CK(mesh_alloc(M, &sell_col, (size_t)nnz_sell), "alloc sell");
   UP_CK(launch_sell_fill(rowptr, col, ni, sell_ptr, sell_col, st), "sell fill");
 
+  // the column pattern that most slices share, if any
+  int host_pat[2 + kPatW] = {};  // found, offsets, slices that follow it
+  unsigned* patbit = nullptr;
+  {
+    int* pat = nullptr;
+    UP_CK(tmp.get(&pat, 2 + kPatW), "alloc tmp");
+    UP_CK(mesh_alloc(M, &patbit, (size_t)(nsl + 31) / 32), "alloc pattern");
+    UP_CK(launch_sell_pattern(sell_ptr, sell_col, rowptr, ni, pat, patbit, pat + 1 + kPatW, st), "sell pattern");
+    UP_CK(cudaMemcpyAsync(host_pat, pat, sizeof(host_pat), cudaMemcpyDeviceToHost, st), "read pattern");
+    UP_CK(cudaStreamSynchronize(st), "sell pattern");
+  }
+
   // operator and solver workspace
   MeshDev& md = M->md;
   std::memset(&md, 0, sizeof(md));
@@ -474,9 +486,9 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
   // never on a batch.
   // Mixed precision: 256..max_rows rows; a mesh that fills the GPU gets a tile count that is a
   // whole multiple of the resident CTA slots S of the solver kernels, so every launch ends in full
-  // waves. The SpMV and the p-update take one pass (kTileRows rows) per tile: a big mesh's tiles
-  // are dealt cyclically, so CTAs at work at the same time cover neighbouring rows and share the
-  // gathered p lines in L2. The update gathers nothing; on a big mesh it takes one wave of large
+  // waves. The p-update and the residual (and the SpMV, see below) take one pass (kTileRows rows) per tile: a
+  // big mesh's tiles are dealt cyclically, so CTAs at work at the same time cover neighbouring rows and
+  // share gathered lines in L2. The update gathers nothing; on a big mesh it takes one wave of large
   // tiles (up to kMaxTileRows32 rows, in passes of kTileRows), which costs far fewer barriers and
   // partial sums (one-wave tiles measured 139.9 -> 113.7 us per update launch on the 4096 x 2048
   // grid, and 139.2 -> 159.5 us per SpMV launch, hence the two tilings).
@@ -537,6 +549,33 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
     md.tile_rows32u = md.tile_rows32;
     md.ntiles32u = md.ntiles32;
   }
+  const bool patterned = host_pat[0] != 0 && 2 * (long)host_pat[1 + kPatW] >= nsl;
+  if (patterned) {
+    md.pat_on = 1;
+    for (int u = 0; u < kPatW; ++u) md.pat[u] = host_pat[1 + u];
+    md.patbit = patbit;
+  }
+  // Mixed-precision SpMV: on a large mesh with a column pattern (a grid), a tile is a block of grid
+  // lines, tile_rows32 rows wide and as many lines high as make one wave: the rows of p that a line
+  // gathers are those its neighbours in the block gather too, and stay in L1 (rows in order fetch
+  // each row of p three times from L2). In a copy of the kernel between copies of the other two,
+  // 4096 x 2048: 106 us a launch with rows in order, 98 in blocks; 2047 x 1531: 48 and 40. The line
+  // length comes from the pattern's largest offset; where it is too far from a multiple of the width
+  // (a line's neighbours would lie three eighths beside the block's next line), rows go in order.
+  // A block's products are added line by line as those of the tiles in order are (same FP32 sums).
+  md.s32_h = 1;
+  md.s32_ncb = md.ntiles32s = md.ntiles32;
+  if (ni >= kBigRows && patterned) {
+    long far = 0;
+    for (int u = 0; u < kPatW; ++u) far = std::max<long>(far, host_pat[1 + u]);
+    const long w = md.tile_rows32, ncb = std::max(1l, (far + w / 2) / w);
+    if (8 * std::labs(far - 1 - ncb * w) <= 3 * w && ncb <= md.ntiles32 / 2) {
+      const long lines = (md.ntiles32 + ncb - 1) / ncb, S = std::max(1, ctx->solver_slots32);
+      md.s32_ncb = (int)ncb;
+      md.s32_h = (int)std::min<long>(128, (lines * ncb + S - 1) / S);
+      md.ntiles32s = (int)(((lines + md.s32_h - 1) / md.s32_h) * ncb);
+    }
+  }
   md.nnz_sell = nnz_sell;
   md.sell_w = sell_w;
   md.sell_wmax = (int)(wmax / 32);
@@ -552,7 +591,7 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
   const size_t nv = (size_t)n * kMaxK;
   // partial sums: the loop kernels' tiles (and the geodesic warm start's, of kTileRows rows), and the
   // VJP's per-face-tile sums of dl/dt
-  const size_t npart = std::max(std::max(std::max((size_t)md.ntiles, (size_t)md.ntiles32),
+  const size_t npart = std::max(std::max(std::max((size_t)md.ntiles, (size_t)std::max(md.ntiles32, md.ntiles32s)),
                                          (size_t)(ni + kTileRows - 1) / kTileRows) * kPartStride,
                                 (size_t)(mi + 255) / 256) + 8;
   UP_CK(mesh_alloc(M, &md.facew, 4 * (size_t)m), "alloc");

@@ -10,6 +10,15 @@ namespace {
 
 constexpr int kWarps = kBlock / 32;
 
+// A pointer read from a mesh descriptor, known to be to global memory (the descriptors lie in shared
+// memory, so the compiler cannot tell and would use generic accesses, which may alias the descriptor
+// itself).
+template <typename T>
+__device__ __forceinline__ T* as_global(T* p) {
+  __builtin_assume(__isGlobal(p));
+  return p;
+}
+
 template <int K>
 struct KP {
   static constexpr int v = (K == 3) ? 4 : K;
@@ -110,40 +119,6 @@ __device__ __forceinline__ void row_product(const MeshDev& md, const TA* __restr
     }
     const int base = b0 + (int)(row & 31);
     const int* __restrict__ sc = md.sell_col;
-    if constexpr (sizeof(TX) == 4) {
-      // FP32: up to 8 slots at once (a mesh row has ~7): all column/value loads, then the gathers.
-      // A mesh whose columns all fit reads them as 16-bit offsets from the slice's first row.
-      const bool c16 = md.sell_c16 != nullptr;
-      const short* __restrict__ s16 = md.sell_c16;
-      const int rbase = sl << 5;
-      for (int j0 = 0; j0 < w; j0 += 8) {
-        int cj[8];
-        TA aj[8];
-        if (c16) {
-#pragma unroll
-          for (int u = 0; u < 8; ++u)
-            if (j0 + u < w) {
-              cj[u] = rbase + (int)__ldg(s16 + base + 32 * (j0 + u));
-              aj[u] = __ldg(A + base + 32 * (j0 + u));
-            }
-        } else {
-#pragma unroll
-          for (int u = 0; u < 8; ++u)
-            if (j0 + u < w) {
-              cj[u] = __ldg(sc + base + 32 * (j0 + u));
-              aj[u] = __ldg(A + base + 32 * (j0 + u));
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (j0 + u < w) {
-            TX v[K];
-            gather(IG_IN_RANGE(cj[u], md.n, md.err) ? cj[u] : 0, v);
-#pragma unroll
-            for (int c = 0; c < K; ++c) acc[c] = fma_t((TX)aj[u], v[c], acc[c]);
-          }
-      }
-    } else {
 #pragma unroll 4
       for (int j = 0; j < w; ++j) {
         const int e = base + 32 * j;
@@ -154,7 +129,6 @@ __device__ __forceinline__ void row_product(const MeshDev& md, const TA* __restr
 #pragma unroll
         for (int c = 0; c < K; ++c) acc[c] = fma_t(a, v[c], acc[c]);
       }
-    }
   } else {
     const int e0 = __ldg(md.rowptr + row), e1 = __ldg(md.rowptr + row + 1);
     for (int e = e0; e < e1; ++e) {
@@ -168,16 +142,93 @@ __device__ __forceinline__ void row_product(const MeshDev& md, const TA* __restr
   }
 }
 
+// Streams that are read once per launch leave L1 to the gathered vector.
+__device__ __forceinline__ float load_stream(const float* a) {
+  float v;
+  asm("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(a));
+  return v;
+}
+__device__ __forceinline__ int load_stream(const short* a) {
+  short v;
+  asm("ld.global.nc.L1::no_allocate.s16 %0, [%1];" : "=h"(v) : "l"(a));
+  return v;
+}
+__device__ __forceinline__ int load_stream(const int* a) {
+  int v;
+  asm("ld.global.nc.L1::no_allocate.s32 %0, [%1];" : "=r"(v) : "l"(a));
+  return v;
+}
+
+// FP32 product of one row (lane `row & 31` of slice sl) of the sliced layout with the padded vector
+// p. A slice that follows the mesh's column pattern (pat) reads no columns, and all its loads are under
+// way together; otherwise the columns and values of up to eight slots come first, then their rows of p.
+template <int K>
+__device__ __forceinline__ void row_product32(const MeshDev& md, const float* __restrict__ A,
+                                              const float* __restrict__ p, int sl, int row, bool pat,
+                                              float (&acc)[K]) {
+#pragma unroll
+  for (int c = 0; c < K; ++c) acc[c] = 0.f;
+  int b0, w;
+  if (md.sell_w) {  // slices of one width: the offset is computed, not loaded
+    w = md.sell_w;
+    b0 = sl * 32 * w;
+  } else {
+    b0 = __ldg(md.sell_ptr + sl);
+    w = (__ldg(md.sell_ptr + sl + 1) - b0) >> 5;
+  }
+  const float* __restrict__ a = A + b0 + (row & 31);
+  if (pat) {
+    float aj[kPatW], v[kPatW][K];
+#pragma unroll
+    for (int u = 0; u < kPatW; ++u) aj[u] = load_stream(a + 32 * u);
+#pragma unroll
+    for (int u = 0; u < kPatW; ++u) {
+      const int cj = row + md.pat[u];
+      load_row32<K>(p, IG_IN_RANGE(cj, md.n, md.err) ? cj : 0, v[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < kPatW; ++u)
+#pragma unroll
+      for (int c = 0; c < K; ++c) acc[c] = fmaf(aj[u], v[u][c], acc[c]);
+    return;
+  }
+  const bool c16 = md.sell_c16 != nullptr;
+  const int base = b0 + (row & 31);
+  for (int j0 = 0; j0 < w; j0 += 8) {
+    int cj[8];
+    float aj[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (j0 + u < w) {
+        cj[u] = c16 ? (row & ~31) + load_stream(md.sell_c16 + base + 32 * (j0 + u))
+                    : load_stream(md.sell_col + base + 32 * (j0 + u));
+        aj[u] = load_stream(a + 32 * (j0 + u));
+      }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (j0 + u < w) {
+        float v[K];
+        load_row32<K>(p, IG_IN_RANGE(cj[u], md.n, md.err) ? cj[u] : 0, v);
+#pragma unroll
+        for (int c = 0; c < K; ++c) acc[c] = fmaf(aj[u], v[c], acc[c]);
+      }
+  }
+}
+
+// Which of the slices s0 .. s0 + 31 follow the mesh's column pattern (bit i: slice s0 + i); 0 past the
+// last slice's word, and on meshes without a pattern.
+__device__ __forceinline__ unsigned pattern_bits(const MeshDev& md, int s0, int nsl) {
+  if (!md.pat_on || s0 >= nsl) return 0u;
+  const int w0 = s0 >> 5, last = (nsl - 1) >> 5;
+  const unsigned a = __ldg(md.patbit + w0), b = w0 < last ? __ldg(md.patbit + w0 + 1) : 0u;
+  return __funnelshift_r(a, b, s0 & 31);
+}
+
 // Gathers: rows of the padded p vectors, columns of an [K][n] vector, rows of an [n][K] vector.
 template <int K>
 struct GatherP64 {
   const double* p;
   __device__ __forceinline__ void operator()(int j, double (&v)[K]) const { load_row<K>(p, j, v); }
-};
-template <int K>
-struct GatherP32 {
-  const float* p;
-  __device__ __forceinline__ void operator()(int j, float (&v)[K]) const { load_row32<K>(p, j, v); }
 };
 template <int K>
 struct GatherSoA64 {
@@ -311,9 +362,15 @@ __device__ __forceinline__ double add_warps(const double* red) {
   a += __shfl_xor_sync(0xffffffffu, a, 2);
   return a;
 }
-// The same sum on one thread, without the warp's shuffles (which cost the loop kernels spills).
+// The same sum on one thread, without the warp's shuffles (which cost the loop kernels spills), or the
+// sum in warp order.
+template <bool TREE>
 __device__ __forceinline__ double add_warps_of(const double* red) {
-  return ((red[0] + red[4]) + (red[1] + red[5])) + ((red[2] + red[6]) + (red[3] + red[7]));
+  if constexpr (TREE) return ((red[0] + red[4]) + (red[1] + red[5])) + ((red[2] + red[6]) + (red[3] + red[7]));
+  double a = red[0];
+#pragma unroll
+  for (int j = 1; j < kWarps; ++j) a += red[j];
+  return a;
 }
 template <int NV>
 __device__ __forceinline__ void add_warps_to(const double* red, double* out) {
@@ -322,14 +379,20 @@ __device__ __forceinline__ void add_warps_to(const double* red, double* out) {
   if ((lane & 3) == 0 && v < NV) out[v] = a;
 }
 
+// The two orders of the FP64 sums over warps and tiles. The FP64 solver adds in trees (the resident
+// solve runs these sums in every CTA, where they count). The mixed-precision solver keeps its sums in
+// warp and tile order: the scale of its inner right-hand sides comes from them, and FP32 face
+// geometry rounds what depends on that scale, so that one bit of it shows in the gradient.
+constexpr bool kTree = true, kInOrder = false;
+
 // Sum the per-thread values v[0..NV) over the CTA into out[0..NV). A caller that sums consecutive
 // tiles alternates between two red buffers, so that one barrier per tile suffices (a warp can reach
 // the buffer again only after the next tile's barrier, which warp 0 passes after its reads).
-template <int NV, typename T>
+template <int NV, bool TREE, typename T>
 __device__ __forceinline__ void tile_reduce(T (&v)[NV], double* red, double* out) {
   warp_totals<NV>(v, red);
   __syncthreads();
-  if (threadIdx.x < NV) out[threadIdx.x] = add_warps_of(red + threadIdx.x * kWarps);
+  if (threadIdx.x < NV) out[threadIdx.x] = add_warps_of<TREE>(red + threadIdx.x * kWarps);
 }
 
 // How a CTA adds the partial sums of a mesh's tiles: VP lanes (the power of two above NV) take one
@@ -379,14 +442,62 @@ __device__ __noinline__ void combine_partials(const double* __restrict__ part, i
   }
 }
 
-// Sum v over the tile, publish the tile's partials, and return true in the last CTA of the mesh,
-// which then holds the mesh totals in v (every thread).
+// In tile order: thread j of the CTA adds tiles j, j + kBlock, ... into out[0..NV) (the CTA then adds
+// its threads' sums by warp and in warp order). Loads go in batches of four tiles; kept out of line:
+// only the last CTA of a reduction runs it.
 template <int NV>
+__device__ __noinline__ void gather_in_order(const double* __restrict__ part, int ntiles, double* out) {
+  double v[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) v[i] = 0.0;
+  for (int t = threadIdx.x; t < ntiles; t += 4 * kBlock) {
+    double b[4][NV];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int i = 0; i < NV; ++i)
+        b[u][i] = t + u * kBlock < ntiles ? __ldcg(part + (long)(t + u * kBlock) * kPartStride + i) : 0.0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (t + u * kBlock < ntiles) {  // warps past the last tile add nothing
+#pragma unroll
+        for (int i = 0; i < NV; ++i) v[i] += b[u][i];
+      }
+  }
+#pragma unroll
+  for (int i = 0; i < NV; ++i) out[i] = v[i];
+}
+
+// Sum v over the tile, publish the tile's partials, and return true in the last CTA of the mesh,
+// which then holds the mesh totals in v (every thread; thread 0 with in-order sums).
+template <int NV, bool TREE>
 __device__ __forceinline__ bool reduce_tiles(double (&v)[NV], double* part, int tile, int ntiles, unsigned int* cnt) {
   __shared__ double red[8 * kWarps];
   __shared__ double tot[8];
   __shared__ int s_last;
-  tile_reduce<NV>(v, red, part + (long)tile * kPartStride);
+  if constexpr (!TREE) {
+    // in order within the CTA too: column by column over the warps, then over the lanes
+    __shared__ double sh[NV * kBlock];
+    block_sum<NV>(v, sh);
+    if (threadIdx.x == 0) {
+#pragma unroll
+      for (int i = 0; i < NV; ++i) part[(long)tile * kPartStride + i] = v[i];
+      __threadfence();
+      s_last = atomicAdd(cnt, 1u) == (unsigned)ntiles - 1u;
+    }
+    __syncthreads();
+    if (!s_last) return false;
+    __threadfence();
+#pragma unroll
+    for (int i = 0; i < NV; ++i) v[i] = 0.0;
+    for (int t = threadIdx.x; t < ntiles; t += kBlock)
+#pragma unroll
+      for (int i = 0; i < NV; ++i) v[i] += __ldcg(part + (long)t * kPartStride + i);
+    block_sum<NV>(v, sh);
+    if (threadIdx.x == 0) *cnt = 0u;
+    return true;
+  }
+  tile_reduce<NV, TREE>(v, red, part + (long)tile * kPartStride);
   if (threadIdx.x < 32) __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -406,11 +517,12 @@ __device__ __forceinline__ bool reduce_tiles(double (&v)[NV], double* part, int 
 }
 
 // ------------------------------------------------------------------------------- persistent tiles
-// The tilings of a mesh: 0 the FP64 solver's, 1 the mixed-precision SpMV's and p-update's, 2 the
-// mixed-precision update's (one wave of large tiles on meshes of at least kBigRows rows, the
-// tiling 1 otherwise, so that the chunked lists of smaller meshes serve both).
+// The tilings of a mesh: 0 the FP64 solver's, 1 the mixed-precision p-update's and residual's, 2 the
+// mixed-precision update's (one wave of large tiles on meshes of at least kBigRows rows) and 3 the
+// mixed-precision SpMV's (blocks of grid lines on such meshes); 2 and 3 are the tiling 1 on
+// smaller meshes, so that their chunked lists serve all.
 __device__ __forceinline__ int tile_count(const MeshDev& md, int tiling) {
-  return tiling == 0 ? md.ntiles : (tiling == 1 ? md.ntiles32 : md.ntiles32u);
+  return tiling == 0 ? md.ntiles : (tiling == 1 ? md.ntiles32 : (tiling == 2 ? md.ntiles32u : md.ntiles32s));
 }
 
 // Per-CTA view of the mesh whose tiles the CTA is working on: a copy of its MeshDev and of the
@@ -424,6 +536,7 @@ struct ScalSnap {
   int act64[kMaxK];
   int done;
   int phase;
+  int inner_iter;
 };
 
 struct TileCtx {
@@ -445,6 +558,7 @@ __device__ __forceinline__ void load_mesh(const MeshDev* __restrict__ mds, int i
     const SolveScal* s = mds[i].s;
     tc.sn.done = s->done;
     tc.sn.phase = s->phase;
+    tc.sn.inner_iter = s->inner_iter;
 #pragma unroll
     for (int c = 0; c < kMaxK; ++c) {
       tc.sn.alpha[c] = s->alpha[c];
@@ -456,31 +570,13 @@ __device__ __forceinline__ void load_mesh(const MeshDev* __restrict__ mds, int i
   __syncthreads();
 }
 
-// What the CTA that completes a mesh does: add the partials and run the finish step. Out of line,
-// with its own registers.
-template <int NV, typename Finish>
-__device__ __noinline__ void complete_mesh(TileCtx& tc, int ntiles, unsigned int* cnt, const Finish& finish) {
-  __threadfence();
-  // the mesh's scalars are read into shared memory while the partials are gathered, so that
-  // the finish step does not wait on one global load after another
-  static_assert(sizeof(SolveScal) % 4 == 0 && sizeof(SolveScal) / 4 <= kBlock, "SolveScal copy");
-  if (threadIdx.x < (int)(sizeof(SolveScal) / 4))
-    reinterpret_cast<unsigned*>(&tc.cur)[threadIdx.x] =
-        __ldcg(reinterpret_cast<const unsigned*>(tc.md.s) + threadIdx.x);
-  combine_partials<NV>(tc.md.part, ntiles, tc.red[0], tc.tot);  // its barrier also publishes cur
-  if (threadIdx.x < 32) {
-    if (threadIdx.x == 0) *cnt = 0u;
-    finish(tc.md, tc.cur, tc.tot);
-  }
-}
-
 // The loop kernels run one CTA per resident slot; CTA b takes the flat tiles b, b + G, b + 2G, ...
 // (G = gridDim.x). A tile's sums go to the mesh's part[tile]; each CTA counts the tiles it did
 // per run of consecutive tiles of one mesh and adds that count to the mesh's counter with one
 // atomic. The CTA whose addition completes the mesh adds the partials in tile order
 // (deterministic, independent of G and of any batch) and calls finish(md, scalars, totals) on
 // warp 0, with a shared-memory copy of the mesh's scalars to read (writes go to md.s).
-template <int NV, typename Finish>
+template <int NV, bool TREE, typename Finish>
 __device__ __forceinline__ void flush_tiles(TileCtx& tc, int tiling, unsigned run, int cnt_idx,
                                             const Finish& finish) {
   const int ntiles = tile_count(tc.md, tiling);
@@ -493,7 +589,28 @@ __device__ __forceinline__ void flush_tiles(TileCtx& tc, int tiling, unsigned ru
     tc.last = (prev + run == (unsigned)ntiles);
   }
   __syncthreads();
-  if (tc.last) complete_mesh<NV>(tc, ntiles, cnt, finish);
+  if (tc.last) {
+    __threadfence();
+    // the mesh's scalars are read into shared memory while the partials are gathered, so that
+    // the finish step does not wait on one global load after another
+    static_assert(sizeof(SolveScal) % 4 == 0 && sizeof(SolveScal) / 4 <= kBlock, "SolveScal copy");
+    if (threadIdx.x < (int)(sizeof(SolveScal) / 4))
+      reinterpret_cast<unsigned*>(&tc.cur)[threadIdx.x] =
+          __ldcg(reinterpret_cast<const unsigned*>(tc.md.s) + threadIdx.x);
+    // (the barriers in here also publish cur)
+    if constexpr (TREE) {
+      combine_partials<NV>(tc.md.part, ntiles, tc.red[0], tc.tot);
+    } else {
+      double v[NV];
+      gather_in_order<NV>(tc.md.part, ntiles, v);
+      tile_reduce<NV, TREE>(v, tc.red[0], tc.tot);
+      __syncthreads();
+    }
+    if (threadIdx.x < 32) {
+      if (threadIdx.x == 0) *cnt = 0u;
+      finish(tc.md, tc.cur, tc.tot);
+    }
+  }
   __syncthreads();
 }
 
@@ -699,9 +816,9 @@ struct TileWalk {
 };
 
 // body(md, tile, red, out) does the tile's work and sums its NV values into out with
-// tile_reduce(v, red, out); active(sn) says whether a mesh takes part in this launch (uniform per
+// tile_reduce(v, red, out) (TREE: the order of the sums over warps and tiles); active(sn) says whether a mesh takes part in this launch (uniform per
 // CTA). tiling: see tile_count; cnt_idx selects the mesh counter.
-template <int NV, typename Active, typename Body, typename Finish>
+template <int NV, bool TREE, typename Active, typename Body, typename Finish>
 __device__ __forceinline__ void tile_loop(const MeshDev* __restrict__ mds, const ListRef& L, int tiling, int cnt_idx,
                                           TileCtx& tc, const Active& active, const Body& body,
                                           const Finish& finish) {
@@ -711,7 +828,7 @@ __device__ __forceinline__ void tile_loop(const MeshDev* __restrict__ mds, const
   unsigned run = 0;
   while (w.more()) {
     if (w.mi != cur) {
-      if (run) flush_tiles<NV>(tc, tiling, run, cnt_idx, finish);
+      if (run) flush_tiles<NV, TREE>(tc, tiling, run, cnt_idx, finish);
       cur = w.mi;
       run = 0;
       load_mesh(mds, cur, tc);
@@ -725,7 +842,7 @@ __device__ __forceinline__ void tile_loop(const MeshDev* __restrict__ mds, const
     }
     w.next(L, nt);
   }
-  if (run) flush_tiles<NV>(tc, tiling, run, cnt_idx, finish);
+  if (run) flush_tiles<NV, TREE>(tc, tiling, run, cnt_idx, finish);
 }
 
 // Tile loop without sums.
@@ -827,6 +944,15 @@ __device__ __forceinline__ void load_row32(const float* __restrict__ p, long row
   } else {
     v[0] = p[row];
   }
+}
+
+// Row store into a padded [n][KP] float vector, the pad of K = 3 with it (one 16-byte store).
+template <int K>
+__device__ __forceinline__ void store_row32(float* __restrict__ p, long row, const float (&v)[K]) {
+  if constexpr (K == 3) reinterpret_cast<float4*>(p)[row] = make_float4(v[0], v[1], v[2], 0.f);
+  else if constexpr (K == 4) reinterpret_cast<float4*>(p)[row] = make_float4(v[0], v[1], v[2], v[3]);
+  else if constexpr (K == 2) reinterpret_cast<float2*>(p)[row] = make_float2(v[0], v[1]);
+  else p[row] = v[0];
 }
 
 // alpha_c = rz_c / (p_c . q_c) for active columns. The finish steps run on the 32 lanes of warp 0

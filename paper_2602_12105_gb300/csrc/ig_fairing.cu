@@ -39,7 +39,7 @@ __global__ void __launch_bounds__(kBlock) mnorm_kernel(const MeshDev* __restrict
     w[row] = 0.5 * e;
     acc[0] = fma(m, 0.5 * e, acc[0]);
   }
-  if (reduce_tiles<1>(acc, md.part, tl.y, md.ntiles, &md.s->cnt[2]) && threadIdx.x == 0) *loss = acc[0];
+  if (reduce_tiles<1, kTree>(acc, md.part, tl.y, md.ntiles, &md.s->cnt[2]) && threadIdx.x == 0) *loss = acc[0];
 }
 
 // V <- V - eta g over 3n values.

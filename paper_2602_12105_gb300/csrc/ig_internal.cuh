@@ -46,6 +46,7 @@ constexpr int kResMinRows = 256;     // fewest rows of a tile of more than kResS
 constexpr int kResSmall = 2048;      // meshes up to this size: tiles of 128 rows
 constexpr int kResMaxRows = 1216;    // most rows of a tile (227 KB of shared memory at 188 bytes a row)
 constexpr int kClusterTiles = 16;    // up to this many tiles meet as one thread-block cluster
+constexpr int kPatW = 7;             // entries of a column pattern (MeshDev::pat): the regular vertex of valence 6
 constexpr int kPartStride = 8;       // doubles per tile in the partial-sum arrays
 
 // Device error word bits (OR-ed by kernels, decoded on the host).
@@ -125,6 +126,9 @@ struct MeshDev {
   int tile_rows;           // rows per FP64 solver tile (<= kTileRows64, a multiple of 32), chosen at upload
   int ntiles32, tile_rows32;  // the same for the mixed-precision kernels (their own occupancy)
   int ntiles32u, tile_rows32u;  // the mixed-precision update's tiles (one wave on meshes of kBigRows or more)
+  // the mixed-precision SpMV's tiles: with the tiles of tile_rows32 rows in lines of s32_ncb, one of
+  // its tiles is s32_h of them below each other (see ig_mesh_upload); in order: s32_h = 1
+  int ntiles32s, s32_h, s32_ncb;
   int nnz_sell;            // stored entries of the sliced layout (0: A is plain CSR on rowptr/col)
   int sell_w;              // every slice has this many entries per row (0: widths differ)
   int sell_wmax;           // the widest slice's entries per row
@@ -134,6 +138,12 @@ struct MeshDev {
   // stored column lies within +-32767 of its slice's first row (null otherwise); the FP32 SpMV
   // then reads these instead of sell_col
   const short* sell_c16;   // [nnz_sell] or null
+  // Slices whose rows all have six neighbours at the same column offsets (an unbroken stretch of a
+  // grid line): when at least half of a mesh's slices share one such pattern, the FP32 SpMV takes
+  // their columns from it and reads none.
+  int pat_on;
+  int pat[kPatW];          // column minus row of each slot
+  const unsigned* patbit;  // [ceil(nslices/32)] bit s: slice s follows the pattern
   int k;
   double t;
   const int* F;
@@ -409,6 +419,10 @@ cudaError_t launch_pattern_rows(const int* F, int n, const int* incptr, int* inc
 cudaError_t launch_pattern_cols(const int* F, int n, const int* incptr, const int* inc_fc, const int* nbr,
                                 const int* rowptr, int* col, int* diagpos, int2* inc, int* err, cudaStream_t st);
 cudaError_t launch_sell_width(const int* rowptr, int n, int* width32, cudaStream_t st);
+// a column pattern of the mesh: pat[0] = whether there is one, pat[1..kPatW] = its offsets; bits and
+// *count: the slices that follow it
+cudaError_t launch_sell_pattern(const int* sell_ptr, const int* sell_col, const int* rowptr, int n, int* pat,
+                                unsigned* bits, int* count, cudaStream_t st);
 cudaError_t launch_sell_c16(const int* sell_ptr, const int* sell_col, int n, short* c16, int* nfar,
                             cudaStream_t st);
 cudaError_t launch_sell_fill(const int* rowptr, const int* col, int n, const int* sell_ptr, int* sell_col,

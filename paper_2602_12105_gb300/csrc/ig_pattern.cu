@@ -269,6 +269,67 @@ __global__ void __launch_bounds__(256) sell_c16_kernel(const int* __restrict__ s
   if (!__all_sync(0xffffffffu, fits) && lane == 0) atomicAdd(nfar, 1);
 }
 
+// Whether slice sl has kPatW entries in each of its 32 rows and slot j of every row at the same offset
+// from the row; off[j] = that offset (one warp).
+__device__ __forceinline__ bool slice_pattern(const int* __restrict__ sell_ptr, const int* __restrict__ sell_col,
+                                              const int* __restrict__ rowptr, int n, int sl, int lane,
+                                              int (&off)[kPatW]) {
+  const int b0 = sell_ptr[sl], w = (sell_ptr[sl + 1] - b0) >> 5;
+  const int row = sl * 32 + lane;
+  bool same = w == kPatW && row < n && rowptr[row + 1] - rowptr[row] == kPatW;
+  if (!__all_sync(0xffffffffu, same)) return false;
+#pragma unroll
+  for (int j = 0; j < kPatW; ++j) {
+    const int d = sell_col[b0 + 32 * j + lane] - row;
+    off[j] = __shfl_sync(0xffffffffu, d, 0);
+    same = same && d == off[j];
+  }
+  return __all_sync(0xffffffffu, same);
+}
+
+// One warp: the pattern of the first of 32 slices spread over the mesh that has one, the middle first
+// (at odd places, which are not all at the ends of grid lines).
+__global__ void __launch_bounds__(32) sell_pick_kernel(const int* __restrict__ sell_ptr, const int* __restrict__ sell_col,
+                                                       const int* __restrict__ rowptr, int n, int* __restrict__ pat,
+                                                       int* __restrict__ count) {
+  const int nsl = (n + 31) / 32;
+  bool found = false;
+  int off[kPatW] = {};
+  for (int t = 0; t < 32 && !found; ++t)
+    found = slice_pattern(sell_ptr, sell_col, rowptr, n, (int)(((long)nsl * (32 + 37 * t) / 64 + 7 * t + 3) % nsl), threadIdx.x,
+                          off);
+  if (threadIdx.x == 0) {
+    pat[0] = found;
+#pragma unroll
+    for (int u = 0; u < kPatW; ++u) pat[1 + u] = off[u];
+    *count = 0;
+  }
+}
+
+// One warp per 32 slices: which of them follow the pattern.
+__global__ void __launch_bounds__(256) sell_mark_kernel(const int* __restrict__ sell_ptr, const int* __restrict__ sell_col,
+                                                        const int* __restrict__ rowptr, int n, const int* __restrict__ pat,
+                                                        unsigned* __restrict__ bits, int* __restrict__ count) {
+  const int nsl = (n + 31) / 32;
+  const int word = (int)(((long)blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (word * 32 >= nsl) return;  // whole warps leave together
+  unsigned b = 0;
+  if (pat[0]) {
+    for (int i = 0; i < 32 && word * 32 + i < nsl; ++i) {
+      int off[kPatW];
+      if (!slice_pattern(sell_ptr, sell_col, rowptr, n, word * 32 + i, lane, off)) continue;
+      bool same = true;
+#pragma unroll
+      for (int u = 0; u < kPatW; ++u) same = same && off[u] == pat[1 + u];
+      if (same) b |= 1u << i;
+    }
+  }
+  if (lane == 0) {
+    bits[word] = b;
+    if (b) atomicAdd(count, __popc(b));
+  }
+}
+
 inline int blocks_for(long work) { return (int)((work + 255) / 256); }
 
 }  // namespace
@@ -298,6 +359,14 @@ cudaError_t launch_pattern_cols(const int* F, int n, const int* incptr, const in
 
 cudaError_t launch_sell_width(const int* rowptr, int n, int* width32, cudaStream_t st) {
   sell_width_kernel<<<blocks_for((n + 31) / 32), 256, 0, st>>>(rowptr, n, width32);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_sell_pattern(const int* sell_ptr, const int* sell_col, const int* rowptr, int n, int* pat,
+                                unsigned* bits, int* count, cudaStream_t st) {
+  sell_pick_kernel<<<1, 32, 0, st>>>(sell_ptr, sell_col, rowptr, n, pat, count);
+  const long nsl = (n + 31) / 32;
+  sell_mark_kernel<<<blocks_for((nsl + 31) / 32 * 32), 256, 0, st>>>(sell_ptr, sell_col, rowptr, n, pat, bits, count);
   return cudaGetLastError();
 }
 

@@ -9,7 +9,7 @@
 //            r64 = rhs - A64 x64 in FP64; stop when ||r64|| / ||rhs|| <= rel_tol
 //
 // It runs inside the same three-kernel iteration as the FP64 solver, with a per-mesh phase:
-//   Inner   : spmv q32 = A32 p32 | update x32, r32, (r.z, r.r) | pupdate p32
+//   Inner   : spmv q32 = A32 p32 | update r32, (r.z, r.r) | pupdate x32, p32
 //   Apply   : set by update when the inner solve converged; pupdate adds ||r64|| d into x64
 //   (next)  : spmv computes r64 = rhs - A64 x64 and its norms (the refinement residual)
 //   Restart : update forms r32 = r64 / ||r64||, d = 0; pupdate sets p32 = z32
@@ -226,42 +226,51 @@ __global__ void __launch_bounds__(kBlock) init_mixed_kernel(const MeshDev* __res
       }
     }
   }
-  if (reduce_tiles<K>(acc, md.part, tl.y, md.ntiles32, &md.s->cnt[2]) && threadIdx.x == 0)
+  if (reduce_tiles<K, kInOrder>(acc, md.part, tl.y, md.ntiles32, &md.s->cnt[2]) && threadIdx.x == 0)
     finish_init_mixed(md.s, K, acc, tol, inner_tol, max_iter, max_refine);
 }
 
 template <int K>
 __global__ void __launch_bounds__(kBlock, 4) spmv_mixed_kernel(const MeshDev* __restrict__ mds, LoopCtl* ctl, ListRef L) {
   __shared__ TileCtx tc;
-  tile_loop<K>(
-      mds, L, 1, 0, tc, [](const ScalSnap& x) { return !x.done && x.phase == kPhaseInner; },
+  tile_loop<K, kInOrder>(
+      mds, L, 3, 0, tc, [](const ScalSnap& x) { return !x.done && x.phase == kPhaseInner; },
       [&](const MeshDev& md, int tile, double* red, double* out) {
-        const long nn = md.n;
-        const long t0 = (long)tile * md.tile_rows32;
-        const long t1 = t0 + md.tile_rows32 < nn ? t0 + md.tile_rows32 : nn;
-        const float* __restrict__ A = md.A32;
-        const float* __restrict__ p = md.p32;
-        float* __restrict__ q32 = md.q32;
-        float pq[K];
+        const int n = md.n, nsl = (n + 31) >> 5, lane = threadIdx.x & 31;
+        const int rb = tile / md.s32_ncb, cb = tile - rb * md.s32_ncb;
+        const float* __restrict__ A = as_global(md.A32);
+        const float* __restrict__ p = as_global(md.p32);
+        float* __restrict__ q32 = as_global(md.q32);
+        // This warp's slices of the block, line by line. A line's products are added in FP32 over the
+        // warp, the lines in FP64.
+        const int warp = threadIdx.x >> 5, w = md.tile_rows32 >> 5;
+        double sum = 0.0;
+        for (int l = rb * md.s32_h; l < (rb + 1) * md.s32_h; ++l) {
+          const int s0 = (l * md.s32_ncb + cb) * w;
+          if (s0 >= nsl) break;
+          const unsigned bits = pattern_bits(md, s0, nsl);
+          float pq[K];
 #pragma unroll
-        for (int c = 0; c < K; ++c) pq[c] = 0.f;
-        // the SpMV's tiles have at most kTileRows rows: one pass
+          for (int k = 0; k < K; ++k) pq[k] = 0.f;
+          for (int c = warp; c < w; c += kWarps) {
+            const int sl = s0 + c, row = sl * 32 + lane;
+            if (row < n) {
+              float q[K];
+              row_product32<K>(md, A, p, sl, row, (bits >> c & 1u) != 0, q);
+              float pi[K];
+              load_row32<K>(p, row, pi);
 #pragma unroll
-        for (int rr = 0; rr < kRowsPerThread; ++rr) {
-          const long row = t0 + rr * kBlock + threadIdx.x;
-          if (row < t1) {
-            float q[K];
-            row_product<K>(md, A, row, GatherP32<K>{p}, q);
-            float pi[K];
-            load_row32<K>(p, row, pi);
-#pragma unroll
-            for (int c = 0; c < K; ++c) {
-              q32[c * nn + row] = q[c];
-              pq[c] = fmaf(pi[c], q[c], pq[c]);
+              for (int k = 0; k < K; ++k) {
+                q32[(long)k * n + row] = q[k];
+                pq[k] = fmaf(pi[k], q[k], pq[k]);
+              }
             }
           }
+          sum += (double)warp_sum_transposed<K>(pq, lane);
         }
-        tile_reduce<K>(pq, red, out);
+        if (warp_sum_writer<K>(lane) && warp_sum_index<K>(lane) < K) red[warp_sum_index<K>(lane) * kWarps + warp] = sum;
+        __syncthreads();
+        if (threadIdx.x < K) out[threadIdx.x] = add_warps_of<kInOrder>(red + threadIdx.x * kWarps);
       },
       [](const MeshDev& md, const SolveScal& cur, const double* v) { finish_spmv(md.s, cur, K, v); });
 }
@@ -270,16 +279,16 @@ __global__ void __launch_bounds__(kBlock, 4) spmv_mixed_kernel(const MeshDev* __
 // Kept out of the FP32 SpMV kernel so that the hot FP32 kernel stays small; it walks the Apply
 // list (the meshes in that phase), which the previous update launch built.
 template <int K>
-__global__ void __launch_bounds__(kBlock) resid_mixed_kernel(const MeshDev* __restrict__ mds, LoopCtl* ctl, ListRef L) {
+__global__ void __launch_bounds__(kBlock, 4) resid_mixed_kernel(const MeshDev* __restrict__ mds, LoopCtl* ctl, ListRef L) {
   __shared__ TileCtx tc;
   if (!ctl->any_apply) return;  // no mesh of the group is in the Apply phase
-  tile_loop<K>(
+  tile_loop<K, kInOrder>(
       mds, L, 1, 0, tc, [](const ScalSnap& x) { return !x.done && x.phase == kPhaseApply; },
       [&](const MeshDev& md, int tile, double* red, double* out) {
         const long nn = md.n;
         const long t0 = (long)tile * md.tile_rows32;
         const long t1 = t0 + md.tile_rows32 < nn ? t0 + md.tile_rows32 : nn;
-        const double* __restrict__ x = md.x;
+        const double* __restrict__ x = as_global(md.x);
         const bool geom32 = md.geom32 != 0;  // the operator is the FP32 one: its values, exactly
         double acc[K];
 #pragma unroll
@@ -300,13 +309,14 @@ __global__ void __launch_bounds__(kBlock) resid_mixed_kernel(const MeshDev* __re
             }
           }
         }
-        tile_reduce<K>(acc, red, out);
+        tile_reduce<K, kInOrder>(acc, red, out);
       },
       [](const MeshDev& md, const SolveScal& cur, const double* v) { finish_residual(md.s, cur, K, v); });
 }
 
-// Inner phase: x32 += alpha p32, r32 -= alpha q32 and the tile's sums r.z, r.r; all loads of a
-// thread's rows are issued before its stores. Restart phase: r32 = r64 / ||r64||, x32 = 0.
+// Inner phase: r32 -= alpha q32 and the tile's sums r.z, r.r (x32 += alpha p32 waits for the p-update,
+// which reads p32 anyway: 16 bytes a row less per iteration); all loads of a thread's rows are issued
+// before its stores. Restart phase: r32 = r64 / ||r64||, x32 = 0.
 template <int K>
 __global__ void __launch_bounds__(kBlock, 4) update_mixed_kernel(const MeshDev* __restrict__ mds, LoopCtl* ctl, ListRef L,
     cudaGraphConditionalHandle handle, int use_graph) {
@@ -326,7 +336,7 @@ __global__ void __launch_bounds__(kBlock, 4) update_mixed_kernel(const MeshDev* 
     }
   }
   __syncthreads();
-  tile_loop<2 * K>(
+  tile_loop<2 * K, kInOrder>(
       mds, L, 2, 1, tc,
       [](const ScalSnap& x) { return !x.done && x.phase != kPhaseApply; },
       [&](const MeshDev& md, int tile, double* red, double* out) {
@@ -334,50 +344,43 @@ __global__ void __launch_bounds__(kBlock, 4) update_mixed_kernel(const MeshDev* 
         const long t0 = (long)tile * md.tile_rows32u;
         const long t1 = t0 + md.tile_rows32u < nn ? t0 + md.tile_rows32u : nn;
         PassSum<2 * K> sum;
-        const float* __restrict__ D32 = md.Dinv32;
-        float* __restrict__ x32 = md.x32;
-        float* __restrict__ r32 = md.r32;
+        const float* __restrict__ D32 = as_global(md.Dinv32);
+        float* __restrict__ x32 = as_global(md.x32);
+        float* __restrict__ r32 = as_global(md.r32);
         if (tc.sn.phase == kPhaseInner) {
-          const float* __restrict__ p32 = md.p32;
-          const float* __restrict__ q32 = md.q32;
+          const float* __restrict__ q32 = as_global(md.q32);
           const int n32 = md.n;
           float alpha[K];
 #pragma unroll
           for (int c = 0; c < K; ++c) alpha[c] = (float)tc.sn.alpha[c];
-          constexpr int RB = 2;
           for (long base = t0; base < t1; base += kTileRows) {
             float acc[2 * K];
 #pragma unroll
             for (int i = 0; i < 2 * K; ++i) acc[i] = 0.f;
+            constexpr int RB = kRowsPerThread;
+            float d[RB], qs[RB][K], rs[RB][K];
 #pragma unroll
-            for (int r0 = 0; r0 < kRowsPerThread; r0 += RB) {
-              float d[RB], pi[RB][K], xs[RB][K], qs[RB][K], rs[RB][K];
+            for (int u = 0; u < RB; ++u) {
+              const int row = (int)base + u * kBlock + threadIdx.x;
+              if (row < (int)t1) {
+                d[u] = D32[row];
 #pragma unroll
-              for (int u = 0; u < RB; ++u) {
-                const int row = (int)base + (r0 + u) * kBlock + threadIdx.x;
-                if (row < (int)t1) {
-                  d[u] = D32[row];
-                  load_row32<K>(p32, row, pi[u]);
-#pragma unroll
-                  for (int c = 0; c < K; ++c) {
-                    xs[u][c] = x32[(long)c * n32 + row];
-                    qs[u][c] = q32[(long)c * n32 + row];
-                    rs[u][c] = r32[(long)c * n32 + row];
-                  }
+                for (int c = 0; c < K; ++c) {
+                  qs[u][c] = q32[(long)c * n32 + row];
+                  rs[u][c] = r32[(long)c * n32 + row];
                 }
               }
+            }
 #pragma unroll
-              for (int u = 0; u < RB; ++u) {
-                const int row = (int)base + (r0 + u) * kBlock + threadIdx.x;
-                if (row < (int)t1) {
+            for (int u = 0; u < RB; ++u) {
+              const int row = (int)base + u * kBlock + threadIdx.x;
+              if (row < (int)t1) {
 #pragma unroll
-                  for (int c = 0; c < K; ++c) {
-                    const float rv = fmaf(-alpha[c], qs[u][c], rs[u][c]);
-                    x32[(long)c * n32 + row] = fmaf(alpha[c], pi[u][c], xs[u][c]);
-                    r32[(long)c * n32 + row] = rv;
-                    acc[c] = fmaf(rv, d[u] * rv, acc[c]);
-                    acc[K + c] = fmaf(rv, rv, acc[K + c]);
-                  }
+                for (int c = 0; c < K; ++c) {
+                  const float rv = fmaf(-alpha[c], qs[u][c], rs[u][c]);
+                  r32[(long)c * n32 + row] = rv;
+                  acc[c] = fmaf(rv, d[u] * rv, acc[c]);
+                  acc[K + c] = fmaf(rv, rv, acc[K + c]);
                 }
               }
             }
@@ -392,7 +395,7 @@ __global__ void __launch_bounds__(kBlock, 4) update_mixed_kernel(const MeshDev* 
             act[c] = tc.sn.act64[c];
             inv[c] = 1.0 / tc.sn.scale[c];
           }
-          const double* __restrict__ r64 = md.r;
+          const double* __restrict__ r64 = as_global(md.r);
           for (long base = t0; base < t1; base += kTileRows) {
             float acc[2 * K];
 #pragma unroll
@@ -415,7 +418,7 @@ __global__ void __launch_bounds__(kBlock, 4) update_mixed_kernel(const MeshDev* 
             sum.add(acc);
           }
         }
-        tile_reduce<2 * K>(sum.s, red, out);
+        tile_reduce<2 * K, kInOrder>(sum.s, red, out);
       },
       [&](const MeshDev& md, const SolveScal& cur, const double* v) {
         const int phase = cur.phase == kPhaseInner ? finish_update_mixed(md.s, cur, K, v)
@@ -437,8 +440,8 @@ __global__ void __launch_bounds__(kBlock, 4) update_mixed_kernel(const MeshDev* 
   }
 }
 
-// Inner phase: p32 = D^-1 r32 + beta p32 (loads of a thread's rows before its stores). Apply
-// phase: x64 += ||r64|| x32.
+// x32 += alpha p32, then in the Inner phase p32 = D^-1 r32 + beta p32 (loads of a thread's rows before
+// its stores), in the Apply phase x64 += ||r64|| x32.
 template <int K>
 // In the graph loop of a single mesh (use_graph), CTA 0 also sets the condition of the IF node that
 // holds the next iteration's residual kernel: whether the mesh recomputes its FP64 residual then
@@ -456,47 +459,67 @@ __global__ void __launch_bounds__(kBlock, 4) pupdate_mixed_kernel(const MeshDev*
                     const long nn = md.n;
                     const long t0 = (long)tile * md.tile_rows32;
                     const long t1 = t0 + md.tile_rows32 < nn ? t0 + md.tile_rows32 : nn;
+                    // x32 += alpha p32 of this slot's iteration (none when it restarted)
+                    const bool step = tc.sn.inner_iter > 0;
+                    float alpha[K];
+#pragma unroll
+                    for (int c = 0; c < K; ++c) alpha[c] = (float)tc.sn.alpha[c];
+                    float* __restrict__ x32 = as_global(md.x32);
+                    float* __restrict__ p32 = as_global(md.p32);
                     if (tc.sn.phase == kPhaseInner) {
                       float beta[K];
 #pragma unroll
                       for (int c = 0; c < K; ++c) beta[c] = (float)tc.sn.beta[c];
-                      const float* __restrict__ D32 = md.Dinv32;
-                      const float* __restrict__ r32 = md.r32;
-                      float* __restrict__ p32 = md.p32;
-                      constexpr int R = kRowsPerThread;  // one pass: tiles of at most kTileRows rows
-                      float d[R], pi[R][K], rs[R][K];
+                      const float* __restrict__ D32 = as_global(md.Dinv32);
+                      const float* __restrict__ r32 = as_global(md.r32);
+                      constexpr int R = 2;  // rows in flight
 #pragma unroll
-                      for (int u = 0; u < R; ++u) {
-                        const long row = t0 + u * kBlock + threadIdx.x;
-                        if (row < t1) {
-                          d[u] = D32[row];
-                          load_row32<K>(p32, row, pi[u]);
+                      for (int r0 = 0; r0 < kRowsPerThread; r0 += R) {
+                        float d[R], pi[R][K], rs[R][K], xs[R][K];
 #pragma unroll
-                          for (int c = 0; c < K; ++c) rs[u][c] = r32[c * nn + row];
+                        for (int u = 0; u < R; ++u) {
+                          const long row = t0 + (r0 + u) * kBlock + threadIdx.x;
+                          if (row < t1) {
+                            d[u] = D32[row];
+                            load_row32<K>(p32, row, pi[u]);
+#pragma unroll
+                            for (int c = 0; c < K; ++c) {
+                              rs[u][c] = r32[c * nn + row];
+                              if (step) xs[u][c] = x32[c * nn + row];
+                            }
+                          }
                         }
-                      }
 #pragma unroll
-                      for (int u = 0; u < R; ++u) {
-                        const long row = t0 + u * kBlock + threadIdx.x;
-                        if (row < t1) {
+                        for (int u = 0; u < R; ++u) {
+                          const long row = t0 + (r0 + u) * kBlock + threadIdx.x;
+                          if (row < t1) {
+                            float pn[K];
 #pragma unroll
-                          for (int c = 0; c < K; ++c)
-                            p32[row * KPm<K>::v + c] = fmaf(beta[c], pi[u][c], d[u] * rs[u][c]);
+                            for (int c = 0; c < K; ++c) {
+                              if (step) x32[c * nn + row] = fmaf(alpha[c], pi[u][c], xs[u][c]);
+                              pn[c] = fmaf(beta[c], pi[u][c], d[u] * rs[u][c]);
+                            }
+                            store_row32<K>(p32, row, pn);
+                          }
                         }
                       }
                     } else {
                       double sc[K];
 #pragma unroll
                       for (int c = 0; c < K; ++c) sc[c] = tc.sn.scale[c];
-                      const float* __restrict__ x32 = md.x32;
-                      double* __restrict__ x = md.x;
+                      double* __restrict__ x = as_global(md.x);
 #pragma unroll
                       for (int rr = 0; rr < kRowsPerThread; ++rr) {
                         const long row = t0 + rr * kBlock + threadIdx.x;
                         if (row < t1) {
+                          float pi[K];
+                          if (step) load_row32<K>(p32, row, pi);
 #pragma unroll
-                          for (int c = 0; c < K; ++c)
-                            x[c * nn + row] = fma(sc[c], (double)x32[c * nn + row], x[c * nn + row]);
+                          for (int c = 0; c < K; ++c) {
+                            float xv = x32[c * nn + row];
+                            if (step) xv = fmaf(alpha[c], pi[c], xv);
+                            x[c * nn + row] = fma(sc[c], (double)xv, x[c * nn + row]);
+                          }
                         }
                       }
                     }

@@ -502,7 +502,7 @@ __global__ void __launch_bounds__(kBlock) rgd_warm_kernel(const MeshDev* __restr
       acc[1] = fma(r, r, acc[1]);
     }
   }
-  if (reduce_tiles<2>(acc, md.part, blockIdx.x, ntile, &md.s->cnt[2]) && threadIdx.x == 0)
+  if (reduce_tiles<2, kTree>(acc, md.part, blockIdx.x, ntile, &md.s->cnt[2]) && threadIdx.x == 0)
     *ratio = acc[1] > 0.0 ? sqrt(acc[0] / acc[1]) : 1e300;
 }
 
