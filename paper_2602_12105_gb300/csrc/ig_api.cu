@@ -609,17 +609,20 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
   UP_CK(mesh_alloc(M, &md.gface, 9 * (size_t)m), "alloc");
   UP_CK(mesh_alloc(M, &md.part, npart), "alloc");
   UP_CK(mesh_alloc(M, &md.s, 1), "alloc");
-  if (resident) {
+  md.resident = resident;
+  const bool gang = (md.ntiles32 + 3) / 4 <= ctx->num_sms && 4 * md.tile_rows32 <= kGangMaxRows;
+  if (resident || gang) {
+    const size_t bytes = meet_bytes(std::max(resident ? md.ntiles : 0, gang ? (md.ntiles32 + 3) / 4 : 0));
     unsigned char* meet = nullptr;
-    UP_CK(mesh_alloc(M, &meet, meet_bytes(md.ntiles)), "alloc");
-    UP_CK(cudaMemsetAsync(meet, 0, meet_bytes(md.ntiles), st), "memset");
+    UP_CK(mesh_alloc(M, &meet, bytes), "alloc");
+    UP_CK(cudaMemsetAsync(meet, 0, bytes, st), "memset");
     md.meet = meet;
   }
   UP_CK(cudaMemsetAsync(md.s, 0, sizeof(SolveScal), st), "memset");
   UP_CK(cudaMemsetAsync(md.p, 0, sizeof(double) * nv, st), "memset");
   UP_CK(cudaMemsetAsync(md.q, 0, sizeof(double) * nv, st), "memset");
   UP_CK(cudaMemsetAsync(md.z, 0, sizeof(double) * nv, st), "memset");
-  UP_CK(group_init(M->group, &md, 1, ctx->solver_slots, ctx->solver_slots32, st), "group");
+  UP_CK(group_init(M->group, &md, 1, ctx->solver_slots, ctx->solver_slots32, ctx->num_sms, st), "group");
   UP_CK(cudaStreamSynchronize(st), "upload");
 #undef UP_CK
   ctx->live_meshes += 1;

@@ -249,6 +249,14 @@ struct GatherAoS64 {
 };
 
 // ------------------------------------------------------------------------------- warp and tile sums
+// The orders of the FP64 sums over warps and tiles. The FP64 solver adds in trees (the resident solves
+// run these sums in every CTA, where each FP64 step counts). The mixed-precision solver's products and
+// updates do too, with the tiles in groups of four (a CTA of its resident solve takes four at a time).
+// Its residual norms are added in warp and tile order: the scale of the inner right-hand sides comes
+// from them, and FP32 face geometry rounds what depends on that scale, so that one bit of it shows
+// in the gradient.
+enum SumOrder { kTree, kGroups, kInOrder };
+
 // Transposed warp sum. In a plain butterfly every lane adds every value at each of the five
 // levels; here, at the first levels, a lane keeps half of its values and sends the other half to
 // its partner, so NV <= 8 values cost 9 shuffles and 9 adds per lane (NV <= 4: 6 and 6) instead of
@@ -364,9 +372,9 @@ __device__ __forceinline__ double add_warps(const double* red) {
 }
 // The same sum on one thread, without the warp's shuffles (which cost the loop kernels spills), or the
 // sum in warp order.
-template <bool TREE>
+template <SumOrder ORDER>
 __device__ __forceinline__ double add_warps_of(const double* red) {
-  if constexpr (TREE) return ((red[0] + red[4]) + (red[1] + red[5])) + ((red[2] + red[6]) + (red[3] + red[7]));
+  if constexpr (ORDER != kInOrder) return ((red[0] + red[4]) + (red[1] + red[5])) + ((red[2] + red[6]) + (red[3] + red[7]));
   double a = red[0];
 #pragma unroll
   for (int j = 1; j < kWarps; ++j) a += red[j];
@@ -379,20 +387,14 @@ __device__ __forceinline__ void add_warps_to(const double* red, double* out) {
   if ((lane & 3) == 0 && v < NV) out[v] = a;
 }
 
-// The two orders of the FP64 sums over warps and tiles. The FP64 solver adds in trees (the resident
-// solve runs these sums in every CTA, where they count). The mixed-precision solver keeps its sums in
-// warp and tile order: the scale of its inner right-hand sides comes from them, and FP32 face
-// geometry rounds what depends on that scale, so that one bit of it shows in the gradient.
-constexpr bool kTree = true, kInOrder = false;
-
 // Sum the per-thread values v[0..NV) over the CTA into out[0..NV). A caller that sums consecutive
 // tiles alternates between two red buffers, so that one barrier per tile suffices (a warp can reach
 // the buffer again only after the next tile's barrier, which warp 0 passes after its reads).
-template <int NV, bool TREE, typename T>
+template <int NV, SumOrder ORDER, typename T>
 __device__ __forceinline__ void tile_reduce(T (&v)[NV], double* red, double* out) {
   warp_totals<NV>(v, red);
   __syncthreads();
-  if (threadIdx.x < NV) out[threadIdx.x] = add_warps_of<TREE>(red + threadIdx.x * kWarps);
+  if (threadIdx.x < NV) out[threadIdx.x] = add_warps_of<ORDER>(red + threadIdx.x * kWarps);
 }
 
 // How a CTA adds the partial sums of a mesh's tiles: VP lanes (the power of two above NV) take one
@@ -415,24 +417,36 @@ struct PartialMap {
   }
 };
 
+// The sum of one value over a group of four tiles (a tile past the end adds +0).
+__device__ __forceinline__ double add_group(double a, double b, double c, double d) { return (a + b) + (c + d); }
+
 // tot[0..NV) = the sums of the tiles' partials, on warp 0 (the others may go on; red must not be in
 // use by any warp). Kept out of line: only the last CTA of a reduction runs it.
-template <int NV>
-__device__ __noinline__ void combine_partials(const double* __restrict__ part, int ntiles, double* red,
-                                                 double* tot) {
+template <int NV, SumOrder ORDER>
+__device__ __noinline__ void combine_partials(const double* __restrict__ part, int ntiles, double* red, double* tot) {
   using Map = PartialMap<NV>;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, v = Map::value(lane);
   double a = 0.0;
-  for (int t = Map::first(warp, lane); t < ntiles; t += 4 * Map::kStride) {
-    double b[4];  // four steps' loads in flight; a tile past the end adds +0
+  if constexpr (ORDER == kGroups) {
+    for (int g = Map::first(warp, lane); 4 * g < ntiles; g += Map::kStride) {
+      double b[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int tu = t + u * Map::kStride;
-      b[u] = tu < ntiles && v < NV ? __ldcg(part + (long)tu * kPartStride + v) : 0.0;
+      for (int u = 0; u < 4; ++u)
+        b[u] = 4 * g + u < ntiles && v < NV ? __ldcg(part + (long)(4 * g + u) * kPartStride + v) : 0.0;
+      a += add_group(b[0], b[1], b[2], b[3]);
     }
+  } else {
+    for (int t = Map::first(warp, lane); t < ntiles; t += 4 * Map::kStride) {
+      double b[4];  // four steps' loads in flight; a tile past the end adds +0
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (t + u * Map::kStride < ntiles) a += b[u];
+      for (int u = 0; u < 4; ++u) {
+        const int tu = t + u * Map::kStride;
+        b[u] = tu < ntiles && v < NV ? __ldcg(part + (long)tu * kPartStride + v) : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (t + u * Map::kStride < ntiles) a += b[u];
+    }
   }
   Map::to_warp_total(a, red);
   __syncthreads();
@@ -470,12 +484,12 @@ __device__ __noinline__ void gather_in_order(const double* __restrict__ part, in
 
 // Sum v over the tile, publish the tile's partials, and return true in the last CTA of the mesh,
 // which then holds the mesh totals in v (every thread; thread 0 with in-order sums).
-template <int NV, bool TREE>
+template <int NV, SumOrder ORDER>
 __device__ __forceinline__ bool reduce_tiles(double (&v)[NV], double* part, int tile, int ntiles, unsigned int* cnt) {
   __shared__ double red[8 * kWarps];
   __shared__ double tot[8];
   __shared__ int s_last;
-  if constexpr (!TREE) {
+  if constexpr (ORDER == kInOrder) {
     // in order within the CTA too: column by column over the warps, then over the lanes
     __shared__ double sh[NV * kBlock];
     block_sum<NV>(v, sh);
@@ -497,7 +511,7 @@ __device__ __forceinline__ bool reduce_tiles(double (&v)[NV], double* part, int 
     if (threadIdx.x == 0) *cnt = 0u;
     return true;
   }
-  tile_reduce<NV, TREE>(v, red, part + (long)tile * kPartStride);
+  tile_reduce<NV, ORDER>(v, red, part + (long)tile * kPartStride);
   if (threadIdx.x < 32) __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -508,7 +522,7 @@ __device__ __forceinline__ bool reduce_tiles(double (&v)[NV], double* part, int 
   __syncthreads();
   if (!s_last) return false;
   __threadfence();
-  combine_partials<NV>(part, ntiles, red, tot);
+  combine_partials<NV, ORDER>(part, ntiles, red, tot);
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < NV; ++i) v[i] = tot[i];
@@ -576,7 +590,7 @@ __device__ __forceinline__ void load_mesh(const MeshDev* __restrict__ mds, int i
 // atomic. The CTA whose addition completes the mesh adds the partials in tile order
 // (deterministic, independent of G and of any batch) and calls finish(md, scalars, totals) on
 // warp 0, with a shared-memory copy of the mesh's scalars to read (writes go to md.s).
-template <int NV, bool TREE, typename Finish>
+template <int NV, SumOrder ORDER, typename Finish>
 __device__ __forceinline__ void flush_tiles(TileCtx& tc, int tiling, unsigned run, int cnt_idx,
                                             const Finish& finish) {
   const int ntiles = tile_count(tc.md, tiling);
@@ -598,12 +612,12 @@ __device__ __forceinline__ void flush_tiles(TileCtx& tc, int tiling, unsigned ru
       reinterpret_cast<unsigned*>(&tc.cur)[threadIdx.x] =
           __ldcg(reinterpret_cast<const unsigned*>(tc.md.s) + threadIdx.x);
     // (the barriers in here also publish cur)
-    if constexpr (TREE) {
-      combine_partials<NV>(tc.md.part, ntiles, tc.red[0], tc.tot);
+    if constexpr (ORDER != kInOrder) {
+      combine_partials<NV, ORDER>(tc.md.part, ntiles, tc.red[0], tc.tot);
     } else {
       double v[NV];
       gather_in_order<NV>(tc.md.part, ntiles, v);
-      tile_reduce<NV, TREE>(v, tc.red[0], tc.tot);
+      tile_reduce<NV, ORDER>(v, tc.red[0], tc.tot);
       __syncthreads();
     }
     if (threadIdx.x < 32) {
@@ -816,9 +830,9 @@ struct TileWalk {
 };
 
 // body(md, tile, red, out) does the tile's work and sums its NV values into out with
-// tile_reduce(v, red, out) (TREE: the order of the sums over warps and tiles); active(sn) says whether a mesh takes part in this launch (uniform per
+// tile_reduce(v, red, out) (ORDER: of the sums over warps and tiles); active(sn) says whether a mesh takes part in this launch (uniform per
 // CTA). tiling: see tile_count; cnt_idx selects the mesh counter.
-template <int NV, bool TREE, typename Active, typename Body, typename Finish>
+template <int NV, SumOrder ORDER, typename Active, typename Body, typename Finish>
 __device__ __forceinline__ void tile_loop(const MeshDev* __restrict__ mds, const ListRef& L, int tiling, int cnt_idx,
                                           TileCtx& tc, const Active& active, const Body& body,
                                           const Finish& finish) {
@@ -828,7 +842,7 @@ __device__ __forceinline__ void tile_loop(const MeshDev* __restrict__ mds, const
   unsigned run = 0;
   while (w.more()) {
     if (w.mi != cur) {
-      if (run) flush_tiles<NV, TREE>(tc, tiling, run, cnt_idx, finish);
+      if (run) flush_tiles<NV, ORDER>(tc, tiling, run, cnt_idx, finish);
       cur = w.mi;
       run = 0;
       load_mesh(mds, cur, tc);
@@ -842,7 +856,7 @@ __device__ __forceinline__ void tile_loop(const MeshDev* __restrict__ mds, const
     }
     w.next(L, nt);
   }
-  if (run) flush_tiles<NV, TREE>(tc, tiling, run, cnt_idx, finish);
+  if (run) flush_tiles<NV, ORDER>(tc, tiling, run, cnt_idx, finish);
 }
 
 // Tile loop without sums.

@@ -45,6 +45,7 @@ constexpr int kResMaxCtas = 160;     // most CTAs
 constexpr int kResMinRows = 256;     // fewest rows of a tile of more than kResSmall rows
 constexpr int kResSmall = 2048;      // meshes up to this size: tiles of 128 rows
 constexpr int kResMaxRows = 1216;    // most rows of a tile (227 KB of shared memory at 188 bytes a row)
+constexpr int kGangMaxRows = 2336;   // most rows of a CTA of a mixed-precision gang (ig_resident32.cu)
 constexpr int kClusterTiles = 16;    // up to this many tiles meet as one thread-block cluster
 constexpr int kPatW = 7;             // entries of a column pattern (MeshDev::pat): the regular vertex of valence 6
 constexpr int kPartStride = 8;       // doubles per tile in the partial-sum arrays
@@ -176,7 +177,8 @@ struct MeshDev {
   double* lam;             // adjoint solution [n][k]
   double* gface;           // per-face gradient contributions [m][9]
   double* part;            // [ntiles][kPartStride] partial sums
-  void* meet;              // resident solves: meet_bytes(ntiles) bytes, zeroed at upload (null: not one)
+  void* meet;              // resident solves: meet_bytes() bytes, zeroed at upload (null: too large for one)
+  int resident;            // the FP64 solve is a resident one (one tile per CTA)
   SolveScal* s;
   int* err;
   // FP32 face geometry (IG_PRECISION_MIXED_GEOM32): when geom32 is set the operator is the FP32
@@ -341,6 +343,10 @@ struct Group {
   LoopCtl* ctl = nullptr;         // device
   int* act_buf = nullptr;         // device storage of the active list and start tables (LoopCtl)
   ListRef list64{}, list32{}, listapp{};  // what the FP64, mixed and residual loop kernels walk
+  int num_sms = 0;                // SMs of the device (resident solves: at most one CTA on each)
+  int4* gang_plan = nullptr;      // device: the gangs of a mixed-precision solve (null: not one), in mesh order of size
+  int gang_tickets = 0;
+  unsigned* gang_ticket = nullptr;
   int* done_host = nullptr;       // pinned host word for the host-driven loop
   SolvePlan plans[2][kMaxK + 1];  // [mixed][k]
   cudaStream_t capture_stream = nullptr;
@@ -360,7 +366,8 @@ inline bool group_any_clamp(const Group& g) {
     if (md.clamp_on) return true;
   return false;
 }
-cudaError_t group_init(Group& g, const MeshDev* host_mds, int nmesh, int slots64, int slots32, cudaStream_t st);
+cudaError_t group_init(Group& g, const MeshDev* host_mds, int nmesh, int slots64, int slots32, int num_sms,
+                       cudaStream_t st);
 cudaError_t group_upload_mds(Group& g, cudaStream_t st);
 cudaError_t group_set_calls(Group& g, const CallDev* calls, cudaStream_t st);
 void group_destroy(Group& g);
@@ -440,7 +447,12 @@ cudaError_t launch_operator32_csr(const MeshDev& md, float* Acsr, cudaStream_t s
 // launched, when the mesh does not qualify or the device refuses the launch
 bool launch_resident(Group& g, int k, const double* in, double* out, int rhs_mass, const ig_solve_opts& o,
                      cudaStream_t st);
-size_t meet_bytes(int ntiles);
+size_t meet_bytes(int parts);  // for meetings that post up to `parts` partial sums
+// ig_resident32.cu: the loop of a mixed-precision solve of a whole group in one launch (between its
+// init and finalize kernels); false, with nothing launched, when the group does not qualify or the
+// device refuses the launch
+bool launch_gang(Group& g, int k, int cap, cudaStream_t st);
+std::vector<int4> gang_plan(const MeshDev* mds, int nmesh, int num_sms, int* tickets);
 
 // ig_eigs.cu: shift-invert subspace iteration (workspace of eig_workspace_doubles(n) doubles)
 size_t eig_workspace_doubles(long n);

@@ -441,8 +441,10 @@ int solver_blocks_per_sm() {
   return m > 0 ? m : 1;
 }
 
-cudaError_t group_init(Group& g, const MeshDev* host_mds, int nmesh, int slots64, int slots32, cudaStream_t st) {
+cudaError_t group_init(Group& g, const MeshDev* host_mds, int nmesh, int slots64, int slots32, int num_sms,
+                       cudaStream_t st) {
   g.nmesh = nmesh;
+  g.num_sms = num_sms;
   g.host_mds.assign(host_mds, host_mds + nmesh);
   std::vector<int2> tiles, tiles32, ftiles, rtiles;
   for (int i = 0; i < nmesh; ++i) {
@@ -510,6 +512,14 @@ cudaError_t group_init(Group& g, const MeshDev* host_mds, int nmesh, int slots64
     g.listapp = ListRef{c.app_start32, c.app_mesh, c.app_big, &g.ctl->napp_big};
     if ((e = cudaMemcpyAsync(g.ctl, &c, sizeof(LoopCtl), cudaMemcpyHostToDevice, st)) != cudaSuccess) return e;
   }
+  const std::vector<int4> plan = gang_plan(host_mds, nmesh, num_sms, &g.gang_tickets);
+  if (!plan.empty()) {  // the ticket counter lies behind the plan
+    if ((e = cudaMalloc(&g.gang_plan, sizeof(int4) * (plan.size() + 1))) != cudaSuccess) return e;
+    if ((e = cudaMemcpyAsync(g.gang_plan, plan.data(), sizeof(int4) * plan.size(), cudaMemcpyHostToDevice, st)) !=
+        cudaSuccess)
+      return e;
+    g.gang_ticket = reinterpret_cast<unsigned*>(g.gang_plan + plan.size());
+  }
   if ((e = cudaStreamCreateWithFlags(&g.capture_stream, cudaStreamNonBlocking)) != cudaSuccess) return e;
   if ((e = cudaEventRecord(g.calls_ev, st)) != cudaSuccess) return e;
   return cudaStreamSynchronize(st);
@@ -546,6 +556,7 @@ void group_destroy(Group& g) {
   if (g.row_tiles) cudaFree(g.row_tiles);
   if (g.ctl) cudaFree(g.ctl);
   if (g.act_buf) cudaFree(g.act_buf);
+  if (g.gang_plan) cudaFree(g.gang_plan);
   if (g.calls_dev) cudaFree(g.calls_dev);
   if (g.calls_host) cudaFreeHost(g.calls_host);
   if (g.done_host) cudaFreeHost(g.done_host);

@@ -15,16 +15,11 @@
 //   Restart : update forms r32 = r64 / ||r64||, d = 0; pupdate sets p32 = z32
 // so a refinement costs one iteration slot whose SpMV runs in FP64, and no extra launches.
 // FP64 arithmetic is used only for the residual SpMV, the x64 update and the reductions.
-#include "ig_device.cuh"
+#include "ig_mixed.cuh"
 
 namespace ig {
 
 namespace {
-
-template <int K>
-struct KPm {
-  static constexpr int v = (K == 3) ? 4 : K;
-};
 
 // The mixed-precision kernels take a tile in passes of kTileRows rows (kRowsPerThread per thread);
 // a thread adds its rows' FP32 products across the passes of a tile (at most 64 passes, 256
@@ -41,150 +36,6 @@ struct PassSum {
     for (int i = 0; i < NV; ++i) s[i] += x[i];
   }
 };
-
-// ------------------------------------------------------------------------------- bookkeeping
-__device__ __noinline__ void finish_init_mixed(SolveScal* s, int k, const double* acc, double tol, double inner_tol,
-                                               int max_iter, int max_refine) {
-  int nact = 0, bad = 0;
-  for (int c = 0; c < kMaxK; ++c) {
-    const double bb = c < k ? acc[c] : 0.0;
-    if (c < k && !is_finite(bb)) bad = 1;
-    const int act = (c < k && positive_finite(bb)) ? 1 : 0;
-    s->rhs2[c] = bb;
-    s->bnorm2[c] = 0.0;
-    s->active64[c] = act;
-    s->active[c] = 0;
-    s->relres2[c] = act ? 1.0 : 0.0;
-    s->scale[c] = act ? sqrt(bb) : 1.0;
-    s->rz[c] = 0.0;
-    s->alpha[c] = 0.0;
-    s->beta[c] = 0.0;
-    s->trueres[c] = -1.0;
-    nact += act;
-  }
-  s->k = k;
-  s->cnt[0] = 0u;
-  s->cnt[1] = 0u;
-  s->iter = 0;
-  s->refine = 0;
-  s->inner_iter = 0;
-  s->inner_cap = max_iter < 4000 ? max_iter : 4000;
-  s->phase = kPhaseRestart;
-  s->tol = tol;
-  s->inner_tol = inner_tol;
-  s->max_iter = max_iter;
-  s->max_refine = max_refine;
-  s->status = bad ? IG_ERR_NONFINITE : IG_OK;
-  s->done = (bad || nact == 0) ? 1 : 0;
-}
-
-// The finish steps below run on the 32 lanes of warp 0 of the CTA that completes a mesh: lane c
-// handles column c, lane 0 the mesh's own fields (written after the warp's votes). They read the
-// scalars from cur, a shared-memory copy, and write them to s.
-
-// After r64 = rhs - A64 x64: FP64 convergence test per column, the scale of the next inner
-// right-hand side, and the refinement cap.
-__device__ __noinline__ void finish_residual(SolveScal* s, const SolveScal& cur, int k, const double* res2) {
-  const int c = threadIdx.x & 31;
-  const int refine = cur.refine + 1;
-  int act = 0, bad = 0;
-  if (c < k && cur.active64[c] != 0) {
-    if (!is_finite(res2[c])) {
-      bad = 1;
-    } else {
-      const double rel2 = res2[c] / cur.rhs2[c];  // squares, as in finish_update
-      s->relres2[c] = rel2;
-      if (rel2 <= cur.tol * cur.tol || !positive_finite(res2[c])) {
-        s->active64[c] = 0;
-      } else {
-        s->scale[c] = sqrt(res2[c]);
-        act = 1;
-      }
-    }
-  }
-  const int nact = __popc(__ballot_sync(0xffffffffu, act));
-  const int anybad = __any_sync(0xffffffffu, bad);
-  if (c == 0) {
-    s->refine = refine;
-    if (anybad) {
-      s->status = IG_ERR_NONFINITE;
-      s->done = 1;
-    } else if (nact == 0) {
-      s->done = 1;
-    } else if (refine >= cur.max_refine || cur.iter >= cur.max_iter) {
-      s->status = IG_ERR_NOT_CONVERGED;
-      s->done = 1;
-    } else {
-      s->phase = kPhaseRestart;
-    }
-  }
-}
-
-// After forming r32 = r64 / scale: start a new inner solve. Returns (on lane 0) the new phase.
-__device__ __noinline__ int finish_restart(SolveScal* s, const SolveScal& cur, int k, const double* acc) {
-  const int c = threadIdx.x & 31;
-  int act = 0;
-  if (c < k) {
-    act = (cur.active64[c] && positive_finite(acc[k + c])) ? 1 : 0;
-    s->active[c] = act;
-    s->rz[c] = acc[c];
-    s->bnorm2[c] = acc[k + c];
-    s->alpha[c] = 0.0;
-    s->beta[c] = 0.0;
-  }
-  const int nact = __popc(__ballot_sync(0xffffffffu, act));
-  const int phase = nact ? kPhaseInner : kPhaseApply;
-  if (c == 0) {
-    s->inner_iter = 0;
-    s->phase = phase;
-  }
-  return phase;
-}
-
-// Inner FP32 iteration: inner convergence test, beta, switch to Apply when the inner solve is done.
-// Returns (on lane 0) the phase after it, or -1 when the mesh is done (a non-finite sum).
-__device__ __noinline__ int finish_update_mixed(SolveScal* s, const SolveScal& cur, int k, const double* acc) {
-  const int c = threadIdx.x & 31, col = c & 7;
-  int act = 0, bad = 0;
-  const double* den = c < 8 ? cur.rz : cur.bnorm2;  // the divisions side by side, the test on squares (finish_update)
-  const double* num = c < 8 ? acc : acc + k;
-  double quot = 0.0;
-  if (col < k && c < 16) quot = num[col] / den[col];
-  const double rel2 = __shfl_down_sync(0xffffffffu, quot, 8);
-  if (c < k && cur.active[c] != 0) {
-    const double rzn = acc[c], rr = acc[k + c];
-    if (!is_finite(rzn) || !is_finite(rr)) {
-      bad = 1;
-    } else {
-      const double bta = quot;
-      if (rel2 <= cur.inner_tol * cur.inner_tol || !positive_finite(rzn)) {
-        s->active[c] = 0;
-        s->beta[c] = 0.0;
-      } else {
-        s->beta[c] = bta;
-        s->rz[c] = rzn;
-        act = 1;
-      }
-    }
-  }
-  const int nact = __popc(__ballot_sync(0xffffffffu, act));
-  const int anybad = __any_sync(0xffffffffu, bad);
-  int phase = kPhaseInner;
-  if (c == 0) {
-    const int it = cur.iter + 1, inner = cur.inner_iter + 1;
-    s->iter = it;
-    s->inner_iter = inner;
-    if (anybad) {
-      s->status = IG_ERR_NONFINITE;
-      s->done = 1;
-      phase = -1;
-    } else if (nact == 0 || inner >= cur.inner_cap || it >= cur.max_iter) {
-      s->phase = kPhaseApply;
-      phase = kPhaseApply;
-    }
-  }
-  return phase;
-}
 
 // ------------------------------------------------------------------------------- kernels
 template <int K>
@@ -233,7 +84,7 @@ __global__ void __launch_bounds__(kBlock) init_mixed_kernel(const MeshDev* __res
 template <int K>
 __global__ void __launch_bounds__(kBlock, 4) spmv_mixed_kernel(const MeshDev* __restrict__ mds, LoopCtl* ctl, ListRef L) {
   __shared__ TileCtx tc;
-  tile_loop<K, kInOrder>(
+  tile_loop<K, kGroups>(
       mds, L, 3, 0, tc, [](const ScalSnap& x) { return !x.done && x.phase == kPhaseInner; },
       [&](const MeshDev& md, int tile, double* red, double* out) {
         const int n = md.n, nsl = (n + 31) >> 5, lane = threadIdx.x & 31;
@@ -270,7 +121,7 @@ __global__ void __launch_bounds__(kBlock, 4) spmv_mixed_kernel(const MeshDev* __
         }
         if (warp_sum_writer<K>(lane) && warp_sum_index<K>(lane) < K) red[warp_sum_index<K>(lane) * kWarps + warp] = sum;
         __syncthreads();
-        if (threadIdx.x < K) out[threadIdx.x] = add_warps_of<kInOrder>(red + threadIdx.x * kWarps);
+        if (threadIdx.x < K) out[threadIdx.x] = add_warps_of<kGroups>(red + threadIdx.x * kWarps);
       },
       [](const MeshDev& md, const SolveScal& cur, const double* v) { finish_spmv(md.s, cur, K, v); });
 }
@@ -336,7 +187,7 @@ __global__ void __launch_bounds__(kBlock, 4) update_mixed_kernel(const MeshDev* 
     }
   }
   __syncthreads();
-  tile_loop<2 * K, kInOrder>(
+  tile_loop<2 * K, kGroups>(
       mds, L, 2, 1, tc,
       [](const ScalSnap& x) { return !x.done && x.phase != kPhaseApply; },
       [&](const MeshDev& md, int tile, double* red, double* out) {
@@ -418,7 +269,7 @@ __global__ void __launch_bounds__(kBlock, 4) update_mixed_kernel(const MeshDev* 
             sum.add(acc);
           }
         }
-        tile_reduce<2 * K, kInOrder>(sum.s, red, out);
+        tile_reduce<2 * K, kGroups>(sum.s, red, out);
       },
       [&](const MeshDev& md, const SolveScal& cur, const double* v) {
         const int phase = cur.phase == kPhaseInner ? finish_update_mixed(md.s, cur, K, v)
@@ -596,12 +447,20 @@ cudaError_t build_plan_mixed(Group& g, SolvePlan& pl) {
   return cudaSuccess;
 }
 
+int slot_cap(const ig_solve_opts& o) { return o.max_iter + 3 * o.max_refine + 4; }
+
+template <int K>
+cudaError_t init_mixed_k(Group& g, const IoTable& io, int rhs_mass, const ig_solve_opts& o, cudaStream_t st) {
+  init_mixed_kernel<K><<<g.ntiles32, kBlock, 0, st>>>(g.mds, g.tiles32, io, rhs_mass, g.ctl, o.rel_tol, o.inner_tol,
+                                                      o.max_iter, o.max_refine, slot_cap(o));
+  return cudaGetLastError();
+}
+
 template <int K>
 cudaError_t begin_mixed_k(Group& g, const IoTable& io, int rhs_mass, const ig_solve_opts& o, cudaStream_t st) {
-  const int cap = o.max_iter + 3 * o.max_refine + 4;
   IG_PROF("pcg_init", st);
-  init_mixed_kernel<K><<<g.ntiles32, kBlock, 0, st>>>(g.mds, g.tiles32, io, rhs_mass, g.ctl, o.rel_tol, o.inner_tol,
-                                                      o.max_iter, o.max_refine, cap);
+  cudaError_t e = init_mixed_k<K>(g, io, rhs_mass, o, st);
+  if (e != cudaSuccess) return e;
   list_kernel<<<1, kBlock, 0, st>>>(g.mds, g.ctl);
   return cudaGetLastError();
 }
@@ -641,9 +500,18 @@ cudaError_t host_loop_mixed_k(Group& g, int max_it, int poll, cudaStream_t st) {
 
 template <int K>
 cudaError_t solve_mixed_k(Group& g, const IoTable& io, int rhs_mass, const ig_solve_opts& o, cudaStream_t st) {
-  cudaError_t e = begin_mixed_k<K>(g, io, rhs_mass, o, st);
+  const bool graph = o.launch == IG_LAUNCH_GRAPH && !prof_on();
+  cudaError_t e;
+  if (graph && g.gang_plan) {
+    if ((e = init_mixed_k<K>(g, io, rhs_mass, o, st)) != cudaSuccess) return e;
+    if (launch_gang(g, K, slot_cap(o), st)) {
+      finalize_kernel<K><<<g.ntiles, kBlock, 0, st>>>(g.mds, g.tiles, io);
+      return cudaGetLastError();
+    }
+  }
+  e = begin_mixed_k<K>(g, io, rhs_mass, o, st);
   if (e != cudaSuccess) return e;
-  if (o.launch == IG_LAUNCH_GRAPH && !prof_on()) {
+  if (graph) {
     SolvePlan& pl = g.plans[1][K];
     if (!pl.exec) {
       e = build_plan_mixed<K>(g, pl);
@@ -651,7 +519,7 @@ cudaError_t solve_mixed_k(Group& g, const IoTable& io, int rhs_mass, const ig_so
     }
     e = cudaGraphLaunch(pl.exec, st);
   } else {
-    e = host_loop_mixed_k<K>(g, o.max_iter + 3 * o.max_refine + 4, 16, st);
+    e = host_loop_mixed_k<K>(g, slot_cap(o), 16, st);
   }
   if (e != cudaSuccess) return e;
   IG_PROF("pcg_finalize", st);

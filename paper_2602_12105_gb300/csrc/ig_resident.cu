@@ -20,45 +20,12 @@
 // update alone, those of 8 a quarter). On small meshes the chain of an iteration: two gathers, two
 // meetings of about 1 us (a store to L2, then a load that sees it), and sums and divisions whose every
 // FP64 step costs 64 cycles.
-#include "ig_device.cuh"
+#include "ig_meet.cuh"
 
 namespace ig {
 
 namespace {
 
-// One posted value: the number of the meeting beside it, written and read as one 16-byte word, so
-// that a reader that sees the number has the value. Slots alternate between two buffers: a CTA
-// posts for meeting i + 2 only after meeting i + 1, for which every CTA had read the slots of i.
-struct __align__(16) Slot {
-  double value;
-  unsigned long long number;
-};
-constexpr int kSpinLimit = 1 << 21;  // polls of one wait (about a second); then the solve fails
-
-__device__ __forceinline__ void post(Slot* s, double value, unsigned long long number) {
-  asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(s),
-               "l"(__double_as_longlong(value)), "l"(number)
-               : "memory");
-}
-// ACQUIRE: with the value comes what its CTA released (an acquire load per slot: a fence after
-// relaxed loads took the geodesic case from 8.3 to 9.6 us an iteration).
-template <bool ACQUIRE>
-__device__ __forceinline__ bool peek(const Slot* s, unsigned long long number, double& value) {
-  unsigned long long a, b;
-  if constexpr (ACQUIRE)
-    asm volatile("{\n\t.reg .b128 t;\n\tld.acquire.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
-                 : "=l"(a), "=l"(b)
-                 : "l"(s)
-                 : "memory");
-  else
-    asm volatile("{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
-                 : "=l"(a), "=l"(b)
-                 : "l"(s)
-                 : "memory");
-  value = __longlong_as_double((long long)a);
-  return b == number;
-}
-__device__ __forceinline__ void fence_gpu() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
@@ -123,38 +90,14 @@ struct Meeting {
   template <int NV, bool ACQUIRE>
   __device__ __forceinline__ bool collect(ResShared& sh) {
     using Map = PartialMap<NV>;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, val = Map::value(lane);
-    const int first = Map::first(warp, lane);
     double a = 0.0;
     bool late = false;
     if constexpr (CLUSTER) {
-      for (int t = first; t < nct; t += Map::kStride)
+      const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, val = Map::value(lane);
+      for (int t = Map::first(warp, lane); t < nct; t += Map::kStride)
         if (val < NV) a += peer_load(&sh.box[number & 1][val], t);
     } else {
-      const Slot* buf = slots + (number & 1) * (8 * (size_t)nct) + val;
-      constexpr int J = (kResMaxCtas + Map::kStride - 1) / Map::kStride;
-      double b[J];
-      unsigned want = 0;
-#pragma unroll
-      for (int j = 0; j < J; ++j) {
-        b[j] = 0.0;
-        if (val < NV && first + j * Map::kStride < nct) want |= 1u << j;
-      }
-      for (int spins = 0; want != 0 && !late; late = ++spins > kSpinLimit) {
-#pragma unroll
-        for (int j = 0; j < J; ++j)
-          if (want >> j & 1) {
-            double x;
-            if (peek<ACQUIRE>(buf + 8 * (size_t)(first + j * Map::kStride), number, x)) {
-              b[j] = x;
-              want &= ~(1u << j);
-            }
-          }
-      }
-      const int steps = (nct + Map::kStride - 1) / Map::kStride;
-#pragma unroll
-      for (int j = 0; j < J; ++j)
-        if (j < steps) a += b[j];
+      a = collect_sum<NV, ACQUIRE>(slots + (number & 1) * (8 * (size_t)nct), nct, number, kSpinLimit, late);
     }
     Map::to_warp_total(a, sh.red2);
     return late;
@@ -500,11 +443,11 @@ bool launch(Group& g, const double* in, double* out, int rhs_mass, const ig_solv
 
 }  // namespace
 
-size_t meet_bytes(int ntiles) { return sizeof(Slot) * (1 + 2 * 8 * (size_t)ntiles); }
+size_t meet_bytes(int parts) { return sizeof(Slot) * (1 + 2 * 8 * (size_t)parts); }
 
 bool launch_resident(Group& g, int k, const double* in, double* out, int rhs_mass, const ig_solve_opts& o,
                      cudaStream_t st) {
-  if (g.nmesh != 1 || !g.host_mds[0].meet) return false;
+  if (g.nmesh != 1 || !g.host_mds[0].resident) return false;
   switch (k) {
     case 1: return launch<1>(g, in, out, rhs_mass, o, st);
     case 2: return launch<2>(g, in, out, rhs_mass, o, st);

@@ -1,0 +1,470 @@
+// ig_resident32.cu -- the mixed-precision solve (ig_pcg_mixed.cu) of the meshes of a group in one launch,
+// each mesh by a gang of CTAs that hold its rows on chip: the FP32 operator, residual, product and
+// solution of a CTA's tiles stay in shared memory through the whole solve, and only p, which the
+// neighbours' rows gather, and the FP64 vectors of the refinement go through global memory. The row
+// arithmetic, the tiles and the order of the sums are those of the multi-CTA kernels: the same bits,
+// alone and in any batch.
+//
+// One CTA per SM. The CTAs draw tickets; the tickets of a mesh are consecutive, the largest meshes
+// first, so that a CTA that is done with a mesh goes on to the next one without waiting for the rest
+// of the group: a batch takes no launch, and no idle CTA, per iteration, where the multi-CTA loop took
+// four launches per iteration of its slowest mesh. A CTA that draws a ticket waits for the rest of its
+// gang: those CTAs are at work on meshes drawn before, and the lowest gang that is not complete always
+// gets the next tickets, so every wait ends.
+//
+// Per iteration a gang meets three times: for p.q, for r.z and r.r, and after p is written (see
+// ig_meet.cuh). Each CTA has four workers of kBlock threads, which take its tiles four at a time; the
+// sums of such a group of four are posted together.
+#include <algorithm>
+
+#include "ig_meet.cuh"
+#include "ig_mixed.cuh"
+
+namespace ig {
+
+namespace {
+
+constexpr int kGangThreads = 4 * kBlock;
+
+constexpr int kGangGroups = 2;                       // most groups of four tiles a CTA holds
+constexpr int kGangBytes = 227 * 1024 - 8 * 1024;    // dynamic shared memory: all but GangShared's part
+
+// Operator slots per row that fit on chip beside three K-vectors and the preconditioner.
+__host__ __device__ inline int gang_slots(int rows, int k, int wmax) {
+  const int fit = (kGangBytes / rows - 4 * (3 * k + 1)) / 8;
+  return fit < wmax ? fit : wmax;
+}
+
+struct GangShared {
+  MeshDev md;
+  SolveScal st;
+  double red[kGangGroups][4][8 * kWarps];  // warp totals of each group's four tiles
+  double red2[8 * kWarps];
+  double tot[8];
+  int ticket;
+  int width[kGangMaxRows / 32];
+};
+
+struct GangRows {  // what a CTA holds of its mesh, in dynamic shared memory
+  int rp;          // rows held (a multiple of 32)
+  int aw;          // operator slots per row on chip; a wider slice's further slots are read from global memory
+  float *a, *r, *x, *q, *d;
+  int* c;
+};
+
+struct Gang {
+  Slot* slots;
+  int member, nct;       // this CTA, and the CTAs of the gang
+  int first, ngroups;    // this CTA's first group of four tiles and their number
+  int total;             // groups of the mesh
+  int groups_per_cta;
+  unsigned long long number;
+  long long patience;    // polls before a wait is given up
+
+  __device__ __forceinline__ Slot* buffer() const { return slots + (number & 1) * (8 * (size_t)total); }
+
+  // Groups' sums (warp totals in sh.red), posted and collected: afterwards the mesh's totals are in
+  // sh.tot on warp 0. False in every thread when a wait ran out.
+  template <int NV>
+  __device__ __forceinline__ bool meet_sums(GangShared& sh) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    ++number;
+    __syncthreads();
+    if (warp < ngroups) {  // one warp per group: lane = value * 4 + tile, then over the four tiles
+      const int v = lane >> 2, t = lane & 3;
+      double s = v < NV ? add_warps_of<kGroups>(&sh.red[warp][t][v * kWarps]) : 0.0;
+      s += __shfl_xor_sync(0xffffffffu, s, 1);
+      s += __shfl_xor_sync(0xffffffffu, s, 2);
+      if (t == 0 && v < NV) post(buffer() + 8 * (size_t)(first + warp) + v, s, number);
+    }
+    bool late = false;
+    if (warp < kWarps)
+      PartialMap<NV>::to_warp_total(collect_sum<NV, false>(buffer(), total, number, patience, late), sh.red2);
+    if (__syncthreads_or(late)) return false;
+    if (warp == 0) {
+      add_warps_to<NV>(sh.red2, sh.tot);
+      __syncwarp();
+    }
+    return true;
+  }
+
+  // A meeting without values: what any CTA of the gang wrote to global memory before is visible to
+  // all of them after. False in every thread when a wait ran out.
+  __device__ __forceinline__ bool meet_writes() {
+    ++number;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      fence_gpu();
+      post(buffer() + 8 * (size_t)first, 0.0, number);
+    }
+    bool late = false;
+    if ((int)threadIdx.x < nct) {
+      const Slot* theirs = buffer() + 8 * (size_t)(threadIdx.x * groups_per_cta);
+      double x;
+      for (long long spins = 0; !peek<true>(theirs, number, x) && !late; late = ++spins > patience) {
+      }
+    }
+    return __syncthreads_or(late) == 0;
+  }
+};
+
+// The tile of worker `worker` in round `round` of this CTA, and its rows.
+struct GangTile {
+  int tile, t0, rows, local;  // rows t0 .. t0 + rows of the mesh, local .. of the CTA
+};
+__device__ __forceinline__ GangTile gang_tile(const MeshDev& md, int first_tile, int round, int worker) {
+  GangTile g;
+  const int i = 4 * round + worker;
+  g.tile = first_tile + i;
+  g.local = i * md.tile_rows32;
+  g.t0 = g.tile * md.tile_rows32;
+  g.rows = g.tile < md.ntiles32 ? min(md.tile_rows32, md.n - g.t0) : 0;
+  return g;
+}
+
+// One slot's loop of a mesh's solve by its gang: see ig_pcg_mixed.cu for the phases.
+template <int K>
+__device__ __forceinline__ bool gang_solve(GangShared& sh, const GangRows& gr, Gang& gang, int cap) {
+  const MeshDev& md = sh.md;
+  const int worker = threadIdx.x / kBlock, tid = threadIdx.x % kBlock, warp = tid >> 5, lane = tid & 31;
+  const int n = md.n, rp = gr.rp, first_tile = 4 * gang.first;
+  const long nn = n;
+  float* p = as_global(md.p32);
+  double* x64 = as_global(md.x);
+  double* r64 = as_global(md.r);
+
+  for (int it = 0; it < cap && !sh.st.done; ++it) {
+    if (sh.st.phase == kPhaseApply) {
+      // r64 = rhs - A x64 and its norms, once every CTA's x64 is there; the sums in tile order
+      if (!gang.meet_writes()) return false;
+      for (int g = 0; g < gang.ngroups; ++g) {
+        const GangTile t = gang_tile(md, first_tile, g, worker);
+        double acc[K];
+#pragma unroll
+        for (int c = 0; c < K; ++c) acc[c] = 0.0;
+        for (int o = tid; o < t.rows; o += kBlock) {
+          const long row = t.t0 + o;
+          double ax[K];
+          if (md.geom32) row_product<K>(md, md.A32, row, GatherSoA64<K>{md.x, nn}, ax);
+          else row_product<K>(md, md.A, row, GatherSoA64<K>{md.x, nn}, ax);
+#pragma unroll
+          for (int c = 0; c < K; ++c) {
+            const double res = md.rhs[c * nn + row] - ax[c];
+            r64[c * nn + row] = res;
+            acc[c] = fma(res, res, acc[c]);
+          }
+        }
+        const double w = warp_sum_transposed<K>(acc, lane);
+        const int idx = warp_sum_index<K>(lane);
+        if (warp_sum_writer<K>(lane) && idx < K) sh.red[g][worker][idx * kWarps + warp] = w;
+      }
+      __syncthreads();
+      for (int g = 0; g < gang.ngroups; ++g) {
+        const GangTile t = gang_tile(md, first_tile, g, worker);
+        if (tid < K && t.rows > 0)
+          __stcg(md.part + (long)t.tile * kPartStride + tid, add_warps_of<kInOrder>(&sh.red[g][worker][tid * kWarps]));
+      }
+      if (!gang.meet_writes()) return false;
+      double v[K];
+      if (worker == 0) {
+        gather_in_order<K>(md.part, md.ntiles32, v);
+        warp_totals<K>(v, sh.red2);
+      }
+      __syncthreads();
+      if (threadIdx.x < 32) {
+        if (threadIdx.x < K) sh.tot[threadIdx.x] = add_warps_of<kInOrder>(sh.red2 + threadIdx.x * kWarps);
+        __syncwarp();
+        finish_residual(&sh.st, sh.st, K, sh.tot);
+      }
+      __syncthreads();
+      if (sh.st.done) break;
+    }
+    if (sh.st.phase == kPhaseInner) {
+      // q = A p and p.q
+      for (int g = 0; g < gang.ngroups; ++g) {
+        const GangTile t = gang_tile(md, first_tile, g, worker);
+        float pq[K];
+#pragma unroll
+        for (int c = 0; c < K; ++c) pq[c] = 0.f;
+        for (int o = tid; o < t.rows; o += kBlock) {
+          const int i = t.local + o, row = t.t0 + o;
+          const int width = sh.width[i >> 5], on = width < gr.aw ? width : gr.aw;
+          float q[K];
+#pragma unroll
+          for (int c = 0; c < K; ++c) q[c] = 0.f;
+          for (int j0 = 0; j0 < on; j0 += 4) {
+            float v[4][K];
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (j0 + u < on) {
+                const int col = gr.c[(j0 + u) * rp + i];
+                load_row32<K>(p, IG_IN_RANGE(col, n, md.err) ? col : 0, v[u]);
+              }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (j0 + u < on) {
+                const float a = gr.a[(j0 + u) * rp + i];
+#pragma unroll
+                for (int c = 0; c < K; ++c) q[c] = fmaf(a, v[u][c], q[c]);
+              }
+          }
+          if (on < width) {  // slots that did not fit on chip
+            const long e = __ldg(md.sell_ptr + (row >> 5)) + (row & 31);
+            for (int j = on; j < width; ++j) {
+              const float a = __ldg(md.A32 + e + 32 * j);
+              const int col = __ldg(md.sell_col + e + 32 * j);
+              float v[K];
+              load_row32<K>(p, IG_IN_RANGE(col, n, md.err) ? col : 0, v);
+#pragma unroll
+              for (int c = 0; c < K; ++c) q[c] = fmaf(a, v[c], q[c]);
+            }
+          }
+          float pi[K];
+          load_row32<K>(p, row, pi);
+#pragma unroll
+          for (int c = 0; c < K; ++c) {
+            gr.q[c * rp + i] = q[c];
+            pq[c] = fmaf(pi[c], q[c], pq[c]);
+          }
+        }
+        const float w = warp_sum_transposed<K>(pq, lane);
+        const int idx = warp_sum_index<K>(lane);
+        if (warp_sum_writer<K>(lane) && idx < K) sh.red[g][worker][idx * kWarps + warp] = (double)w;
+      }
+      if (!gang.meet_sums<K>(sh)) return false;
+      if (threadIdx.x < 32) finish_spmv(&sh.st, sh.st, K, sh.tot);
+      __syncthreads();
+      if (sh.st.done) break;
+    }
+    // Inner: r -= alpha q; Restart: r = r64 / ||r64||, x = 0; r.z and r.r
+    const bool inner = sh.st.phase == kPhaseInner;
+    {
+      float alpha[K];
+      double inv[K];
+#pragma unroll
+      for (int c = 0; c < K; ++c) {
+        alpha[c] = (float)sh.st.alpha[c];
+        inv[c] = inner ? 0.0 : 1.0 / sh.st.scale[c];
+      }
+      for (int g = 0; g < gang.ngroups; ++g) {
+        const GangTile t = gang_tile(md, first_tile, g, worker);
+        float acc[2 * K];
+#pragma unroll
+        for (int i = 0; i < 2 * K; ++i) acc[i] = 0.f;
+        for (int o = tid; o < t.rows; o += kBlock) {
+          const int i = t.local + o;
+          const float d = gr.d[i];
+#pragma unroll
+          for (int c = 0; c < K; ++c) {
+            float rv;
+            if (inner) {
+              rv = fmaf(-alpha[c], gr.q[c * rp + i], gr.r[c * rp + i]);
+            } else {
+              rv = sh.st.active64[c] ? (float)(r64[c * nn + t.t0 + o] * inv[c]) : 0.f;
+              gr.x[c * rp + i] = 0.f;
+            }
+            gr.r[c * rp + i] = rv;
+            acc[c] = fmaf(rv, d * rv, acc[c]);
+            acc[K + c] = fmaf(rv, rv, acc[K + c]);
+          }
+        }
+        const float w = warp_sum_transposed<2 * K>(acc, lane);
+        const int idx = warp_sum_index<2 * K>(lane);
+        if (warp_sum_writer<2 * K>(lane) && idx < 2 * K) sh.red[g][worker][idx * kWarps + warp] = (double)w;
+      }
+    }
+    if (!gang.meet_sums<2 * K>(sh)) return false;
+    if (threadIdx.x < 32) {
+      if (inner) finish_update_mixed(&sh.st, sh.st, K, sh.tot);
+      else finish_restart(&sh.st, sh.st, K, sh.tot);
+    }
+    __syncthreads();
+    if (sh.st.done) break;
+    // x += alpha p (after an iteration); Inner: p = D^-1 r + beta p; Apply: x64 += ||r64|| x
+    {
+      const bool step = sh.st.inner_iter > 0, next = sh.st.phase == kPhaseInner;
+      float alpha[K], beta[K];
+      double sc[K];
+#pragma unroll
+      for (int c = 0; c < K; ++c) {
+        alpha[c] = (float)sh.st.alpha[c];
+        beta[c] = (float)sh.st.beta[c];
+        sc[c] = sh.st.scale[c];
+      }
+      for (int g = 0; g < gang.ngroups; ++g) {
+        const GangTile t = gang_tile(md, first_tile, g, worker);
+        for (int o = tid; o < t.rows; o += kBlock) {
+          const int i = t.local + o;
+          const long row = t.t0 + o;
+          float pi[K], pn[K];
+          load_row32<K>(p, row, pi);
+          const float d = gr.d[i];
+#pragma unroll
+          for (int c = 0; c < K; ++c) {
+            float xv = gr.x[c * rp + i];
+            if (step) {
+              xv = fmaf(alpha[c], pi[c], xv);
+              gr.x[c * rp + i] = xv;
+            }
+            if (next) pn[c] = fmaf(beta[c], pi[c], d * gr.r[c * rp + i]);
+            else x64[c * nn + row] = fma(sc[c], (double)xv, x64[c * nn + row]);
+          }
+          if (next) store_row32<K>(p, row, pn);
+        }
+      }
+      if (next && !gang.meet_writes()) return false;
+    }
+  }
+  return true;
+}
+
+template <int K>
+__global__ void __launch_bounds__(kGangThreads, 1) solve_gang_kernel(const MeshDev* __restrict__ mds,
+                                                                     const int4* __restrict__ plan, int nplan,
+                                                                     int tickets, unsigned* ticket, int cap) {
+  extern __shared__ __align__(16) unsigned char dyn[];
+  __shared__ GangShared sh;
+  for (;;) {
+    __syncthreads();  // every thread is done with the mesh before
+    if (threadIdx.x == 0) sh.ticket = (int)atomicAdd(ticket, 1u);
+    __syncthreads();
+    if (sh.ticket >= tickets) return;
+    int lo = 0, hi = nplan - 1;  // the last entry whose first ticket is not above this one
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (__ldg(&plan[mid].y) <= sh.ticket) lo = mid;
+      else hi = mid - 1;
+    }
+    const int4 e = __ldg(plan + lo);  // mesh, first ticket, CTAs, groups per CTA
+    for (int j = threadIdx.x; j < (int)(sizeof(MeshDev) / 4); j += kGangThreads)
+      reinterpret_cast<unsigned*>(&sh.md)[j] = __ldg(reinterpret_cast<const unsigned*>(mds + e.x) + j);
+    __syncthreads();
+    const MeshDev& md = sh.md;
+    for (int j = threadIdx.x; j < (int)(sizeof(SolveScal) / 4); j += kGangThreads)
+      reinterpret_cast<unsigned*>(&sh.st)[j] = __ldcg(reinterpret_cast<const unsigned*>(md.s) + j);
+    Gang gang;
+    gang.member = sh.ticket - e.y;
+    gang.nct = e.z;
+    gang.groups_per_cta = e.w;
+    gang.total = (md.ntiles32 + 3) / 4;
+    gang.first = gang.member * e.w;
+    gang.ngroups = min(e.w, gang.total - gang.first);
+    gang.slots = reinterpret_cast<Slot*>(md.meet) + 1;
+    const unsigned long long launches = __ldcg(reinterpret_cast<const unsigned long long*>(md.meet));
+    gang.number = launches << 32;
+    // a wait for the rest of the gang lasts as long as the solve of a mesh drawn before
+    gang.patience = kSpinLimit + 256ll * cap;
+
+    // the rows on chip
+    GangRows gr;
+    const int first_row = 4 * gang.first * md.tile_rows32;
+    const int held = min(4 * gang.ngroups * md.tile_rows32, md.n - first_row);
+    gr.rp = 4 * e.w * md.tile_rows32;
+    gr.aw = gang_slots(gr.rp, K, md.sell_wmax);
+    gr.r = reinterpret_cast<float*>(dyn);
+    gr.x = gr.r + K * gr.rp;
+    gr.q = gr.x + K * gr.rp;
+    gr.d = gr.q + K * gr.rp;
+    gr.a = gr.d + gr.rp;
+    gr.c = reinterpret_cast<int*>(gr.a + gr.aw * gr.rp);
+    for (int i = threadIdx.x; i < held; i += kGangThreads) {
+      const int row = first_row + i, sl = row >> 5;
+      const int b0 = __ldg(md.sell_ptr + sl), w = (__ldg(md.sell_ptr + sl + 1) - b0) >> 5;
+      if ((i & 31) == 0) sh.width[i >> 5] = w;
+      const int at = b0 + (row & 31);
+      for (int j = 0; j < (w < gr.aw ? w : gr.aw); ++j) {
+        gr.a[j * gr.rp + i] = __ldg(md.A32 + at + 32 * j);
+        gr.c[j * gr.rp + i] = __ldg(md.sell_col + at + 32 * j);
+      }
+      gr.d[i] = __ldg(md.Dinv32 + row);
+    }
+    __syncthreads();
+
+    const bool met = gang_solve<K>(sh, gr, gang, cap);
+    __syncthreads();
+    if (gang.member == 0) {
+      if (threadIdx.x == 0 && !met) {  // a CTA stayed away past the limit: report a failed solve
+        sh.st.status = IG_ERR_CUDA;
+        sh.st.done = 1;
+      }
+      __syncthreads();
+      for (int j = threadIdx.x; j < (int)(sizeof(SolveScal) / 4); j += kGangThreads)
+        reinterpret_cast<unsigned*>(md.s)[j] = reinterpret_cast<const unsigned*>(&sh.st)[j];
+      if (threadIdx.x == 0) *reinterpret_cast<unsigned long long*>(md.meet) = launches + 1;
+    }
+  }
+}
+
+static_assert(sizeof(GangShared) <= 8 * 1024 - 256, "shared memory of a gang CTA");
+
+template <int K>
+bool launch(Group& g, int cap, cudaStream_t st) {
+  auto kern = solve_gang_kernel<K>;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGangBytes) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (cudaMemsetAsync(g.gang_ticket, 0, sizeof(unsigned), st) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(g.gang_tickets < g.num_sms ? g.gang_tickets : g.num_sms, 1, 1);
+  cfg.blockDim = dim3(kGangThreads, 1, 1);
+  cfg.dynamicSmemBytes = kGangBytes;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, kern, (const MeshDev*)g.mds, (const int4*)g.gang_plan, g.nmesh, g.gang_tickets,
+                         g.gang_ticket, cap) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return true;
+}
+
+}  // namespace
+
+// The gangs of a group: mesh, first ticket, CTAs and groups of tiles per CTA, the largest first. One
+// group of tiles per CTA when the whole group of meshes then fits on the SMs at once, else two
+// (where they fit on chip): fewer CTAs per mesh leave less of an iteration to its meetings, and more
+// meshes run beside each other. Empty when some mesh is too large.
+std::vector<int4> gang_plan(const MeshDev* mds, int nmesh, int num_sms, int* tickets) {
+  std::vector<int4> plan;
+  long groups = 0;
+  for (int i = 0; i < nmesh; ++i) {
+    const int g = (mds[i].ntiles32 + 3) / 4;
+    if (!mds[i].meet || g > num_sms || g > kResMaxCtas || 4 * mds[i].tile_rows32 > kGangMaxRows) return {};
+    groups += g;
+  }
+  for (int i = 0; i < nmesh; ++i) {
+    const int g = (mds[i].ntiles32 + 3) / 4;
+    const int per = groups > num_sms && 4 * kGangGroups * mds[i].tile_rows32 <= kGangMaxRows ? kGangGroups : 1;
+    plan.push_back(make_int4(i, 0, (g + per - 1) / per, per));
+  }
+  std::stable_sort(plan.begin(), plan.end(),
+                   [mds](const int4& a, const int4& b) { return mds[a.x].n > mds[b.x].n; });
+  int t = 0;
+  for (int4& e : plan) {
+    e.y = t;
+    t += e.z;
+  }
+  *tickets = t;
+  return plan;
+}
+
+bool launch_gang(Group& g, int k, int cap, cudaStream_t st) {
+  if (!g.gang_plan) return false;
+  switch (k) {
+    case 1: return launch<1>(g, cap, st);
+    case 2: return launch<2>(g, cap, st);
+    case 3: return launch<3>(g, cap, st);
+    case 4: return launch<4>(g, cap, st);
+    default: return false;
+  }
+}
+
+}  // namespace ig
