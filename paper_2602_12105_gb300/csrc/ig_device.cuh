@@ -10,6 +10,27 @@ namespace {
 
 constexpr int kWarps = kBlock / 32;
 
+// a / b to within one unit in the last place for operands of ordinary magnitude: a third-order
+// (hyperpower) iteration on the hardware's reciprocal estimate (about 20 bits, whose error e becomes
+// e^3), then one correction of the quotient by its residual. Six FP64 instructions in line, about 450
+// cycles; the compiler's division, a call, took 660 to 1,650 in the finish steps, which every CTA of
+// a resident solve waits for. Other operands (zero, subnormal, infinite, NaN, or 2^400 from 1) take the
+// plain division.
+__device__ __forceinline__ double quotient(double a, double b) {
+  const unsigned ea = ((unsigned)__double2hiint(a) >> 20) & 0x7ffu, eb = ((unsigned)__double2hiint(b) >> 20) & 0x7ffu;
+  if (ea - 623u > 800u || eb - 623u > 800u) return a / b;
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+  const double e = fma(-b, y, 1.0);
+  y = fma(y, fma(e, e, e), y);
+  const double q = a * y;
+  return fma(fma(-b, q, a), y, q);
+}
+// x <= y for x, y >= 0 or NaN x (false): by their bits.
+__device__ __forceinline__ bool not_above(double x, double y) {
+  return __double_as_longlong(x) <= __double_as_longlong(y);
+}
+
 // A pointer read from a mesh descriptor, known to be to global memory (the descriptors lie in shared
 // memory, so the compiler cannot tell and would use generic accesses, which may alias the descriptor
 // itself).
@@ -353,12 +374,14 @@ __device__ __forceinline__ T warp_sum_transposed(T (&v)[NV], int lane) {
 // two warps each and add in a butterfly, three additions deep. An FP64 instruction occupies its SM
 // sub-partition for 64 cycles whatever the number of active lanes, so the number of instructions on
 // the path counts, not that of additions: the serial sum of 8 totals took 512 cycles.
+__device__ __forceinline__ double to_double(double x) { return x; }
+__device__ __forceinline__ double to_double(float x) { return f32_to_f64_exact(x); }
 template <int NV, typename T>
 __device__ __forceinline__ void warp_totals(T (&v)[NV], double* red) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const T w = warp_sum_transposed<NV>(v, lane);
   const int idx = warp_sum_index<NV>(lane);
-  if (warp_sum_writer<NV>(lane) && idx < NV) red[idx * kWarps + warp] = (double)w;
+  if (warp_sum_writer<NV>(lane) && idx < NV) red[idx * kWarps + warp] = to_double(w);
 }
 // On one warp: lanes 4 v .. 4 v + 3 return the sum of value v's warp totals (v < NV; 0 for the rest).
 template <int NV>
@@ -543,9 +566,13 @@ __device__ __forceinline__ int tile_count(const MeshDev& md, int tiling) {
 // scalars the kernels read, taken once per mesh switch. Every CTA of a launch reads the same few
 // scalars; reading them through one thread per CTA keeps them off a single hot L2 line, and the
 // copy in shared memory keeps the mesh's pointers out of the way of the kernels' global stores.
+// The FP32 kernels take alpha and beta as floats, rounded here once: a conversion instruction issues at
+// the FP64 rate, and those of every warp and tile took the p-update of 8.4M rows 20 us of FP64 issue.
 struct ScalSnap {
   double alpha[kMaxK];
   double beta[kMaxK];
+  float alpha32[kMaxK];
+  float beta32[kMaxK];
   double scale[kMaxK];
   int act64[kMaxK];
   int done;
@@ -577,6 +604,8 @@ __device__ __forceinline__ void load_mesh(const MeshDev* __restrict__ mds, int i
     for (int c = 0; c < kMaxK; ++c) {
       tc.sn.alpha[c] = s->alpha[c];
       tc.sn.beta[c] = s->beta[c];
+      tc.sn.alpha32[c] = f64_to_f32_rn(tc.sn.alpha[c]);
+      tc.sn.beta32[c] = f64_to_f32_rn(tc.sn.beta[c]);
       tc.sn.scale[c] = s->scale[c];
       tc.sn.act64[c] = s->active64[c];
     }
@@ -969,11 +998,12 @@ __device__ __forceinline__ void store_row32(float* __restrict__ p, long row, con
   else p[row] = v[0];
 }
 
-// alpha_c = rz_c / (p_c . q_c) for active columns. The finish steps run on the 32 lanes of warp 0
+// alpha_c = rz_c / (p_c . q_c) for active columns. (Each finish step has an inline form for the resident
+// solves, whose state lies in shared memory, and an out-of-line one.) The finish steps run on the 32 lanes of warp 0
 // of the CTA that completes a mesh: lane c handles column c (its divisions and square roots
 // run side by side instead of one after another on one thread), lane 0 the mesh's own fields.
 // They read the scalars from cur (a copy in shared memory) and write them to s.
-__device__ __noinline__ void finish_spmv(SolveScal* s, const SolveScal& cur, int k, const double* pq) {
+__device__ __forceinline__ void finish_spmv_step(SolveScal* s, const SolveScal& cur, int k, const double* pq) {
   const int c = threadIdx.x & 31;
   int bad = 0;
   if (c < k) {
@@ -983,13 +1013,16 @@ __device__ __noinline__ void finish_spmv(SolveScal* s, const SolveScal& cur, int
       s->alpha[c] = 0.0;
       bad = 1;
     } else {
-      s->alpha[c] = cur.rz[c] / pq[c];
+      s->alpha[c] = quotient(cur.rz[c], pq[c]);
     }
   }
   if (__any_sync(0xffffffffu, bad) && c == 0) {
     s->status = IG_ERR_NONFINITE;
     s->done = 1;
   }
+}
+__device__ __noinline__ void finish_spmv(SolveScal* s, const SolveScal& cur, int k, const double* pq) {
+  finish_spmv_step(s, cur, k, pq);
 }
 
 // ------------------------------------------------------------------------------- last-CTA steps
@@ -1020,7 +1053,7 @@ __device__ __noinline__ void finish_init(SolveScal* s, int k, const double* acc,
   s->iter = 0;
   s->refine = 0;
   s->phase = 0;
-  s->tol = tol;
+  s->tol2 = tol * tol;
   s->max_iter = max_iter;
   s->status = bad ? IG_ERR_NONFINITE : IG_OK;
   s->done = (bad != 0 || nact == 0) ? 1 : 0;
@@ -1030,14 +1063,14 @@ __device__ __noinline__ void finish_init(SolveScal* s, int k, const double* acc,
 // warp 0 of the CTA that completes the mesh: lane c takes column c, lane 0 the mesh's fields.
 // Returns (on lane 0) whether the mesh is now done. The test compares squares (the root of the
 // reported residual is taken on the host), and its division runs beside that of beta, on lanes
-// 8 .. 8 + k: a division takes about 500 cycles and a root 700 for any number of lanes.
-__device__ __noinline__ int finish_update(SolveScal* s, const SolveScal& cur, int k, const double* acc) {
+// 8 .. 8 + k: it costs the same for any number of lanes.
+__device__ __forceinline__ int finish_update_step(SolveScal* s, const SolveScal& cur, int k, const double* acc) {
   const int c = threadIdx.x & 31, col = c & 7;
   int act = 0, bad = 0;
   const double* den = c < 8 ? cur.rz : cur.bnorm2;
   const double* num = c < 8 ? acc : acc + k;
   double quot = 0.0;
-  if (col < k && c < 16) quot = num[col] / den[col];
+  if (col < k && c < 16) quot = quotient(num[col], den[col]);
   const double rel2 = __shfl_down_sync(0xffffffffu, quot, 8);
   if (c < k && cur.active[c] != 0) {
     const double rzn = acc[c], rr = acc[k + c];
@@ -1046,7 +1079,7 @@ __device__ __noinline__ int finish_update(SolveScal* s, const SolveScal& cur, in
     } else {
       const double bta = quot;
       s->relres2[c] = rel2;
-      if (rel2 <= cur.tol * cur.tol) {
+      if (not_above(rel2, cur.tol2)) {
         s->active[c] = 0;
         s->beta[c] = 0.0;
       } else {
@@ -1074,6 +1107,9 @@ __device__ __noinline__ int finish_update(SolveScal* s, const SolveScal& cur, in
     if (done) s->done = 1;
   }
   return done;
+}
+__device__ __noinline__ int finish_update(SolveScal* s, const SolveScal& cur, int k, const double* acc) {
+  return finish_update_step(s, cur, k, acc);
 }
 
 // ------------------------------------------------------------------------------- finalize

@@ -63,4 +63,11 @@ __device__ __forceinline__ double f32_to_f64(float f) {
   return __longlong_as_double((long long)(sign | (eo << 52) | ((unsigned long long)(u & 0x7fffffu) << 29)));
 }
 
+// The FP64 value of a float, exactly, denormals included (those and NaN by the hardware conversion).
+__device__ __forceinline__ double f32_to_f64_exact(float f) {
+  const unsigned u = __float_as_uint(f), e = (u >> 23) & 0xffu;
+  if (e - 1u >= 254u) return u << 1 ? (double)f : __hiloint2double((int)u, 0);
+  return __hiloint2double((int)((u & 0x80000000u) | ((u >> 3) & 0x0fffffffu) + 0x38000000u), (int)(u << 29));
+}
+
 }  // namespace ig

@@ -109,7 +109,7 @@ struct SolveScal {
   int refine;            // mixed precision: refinements so far
   int phase;             // mixed precision: kPhaseInner / kPhaseApply / kPhaseRestart
   int max_iter, max_refine;
-  double tol, inner_tol;
+  double tol2, inner_tol2;  // squares of the tolerances
   unsigned int cnt[4];   // last-CTA counters (spmv, update, init/residual, vjp)
 };
 
@@ -345,7 +345,7 @@ struct Group {
   ListRef list64{}, list32{}, listapp{};  // what the FP64, mixed and residual loop kernels walk
   int num_sms = 0;                // SMs of the device (resident solves: at most one CTA on each)
   int4* gang_plan = nullptr;      // device: the gangs of a mixed-precision solve (null: not one), in mesh order of size
-  int gang_tickets = 0;
+  int gang_tickets = 0, gang_workers = 4;
   unsigned* gang_ticket = nullptr;
   int* done_host = nullptr;       // pinned host word for the host-driven loop
   SolvePlan plans[2][kMaxK + 1];  // [mixed][k]
@@ -452,7 +452,8 @@ size_t meet_bytes(int parts);  // for meetings that post up to `parts` partial s
 // init and finalize kernels); false, with nothing launched, when the group does not qualify or the
 // device refuses the launch
 bool launch_gang(Group& g, int k, int cap, cudaStream_t st);
-std::vector<int4> gang_plan(const MeshDev* mds, int nmesh, int num_sms, int* tickets);
+std::vector<int4> gang_plan(const MeshDev* mds, const double* t, int nmesh, int num_sms, int* tickets, int* workers);
+cudaError_t group_order_gangs(Group& g, const double* t, cudaStream_t st);  // for these time steps (null: equal)
 
 // ig_eigs.cu: shift-invert subspace iteration (workspace of eig_workspace_doubles(n) doubles)
 size_t eig_workspace_doubles(long n);

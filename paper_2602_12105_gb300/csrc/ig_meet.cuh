@@ -54,15 +54,20 @@ __device__ __forceinline__ double collect_sum(const Slot* buf, int count, unsign
     b[j] = 0.0;
     if (val < NV && first + j * Map::kStride < count) want |= 1u << j;
   }
+  // all the missing slots of a round are loaded before any is looked at
   for (long long spins = 0; want != 0 && !late; late = ++spins > patience) {
+    double x[J];
+    bool there[J];
+#pragma unroll
+    for (int j = 0; j < J; ++j) {
+      const bool ask = (want >> j & 1u) != 0;
+      there[j] = peek<ACQUIRE>(buf + (ask ? 8 * (size_t)(first + j * Map::kStride) + val : 0), number, x[j]) && ask;
+    }
 #pragma unroll
     for (int j = 0; j < J; ++j)
-      if (want >> j & 1) {
-        double x;
-        if (peek<ACQUIRE>(buf + 8 * (size_t)(first + j * Map::kStride) + val, number, x)) {
-          b[j] = x;
-          want &= ~(1u << j);
-        }
+      if (there[j]) {
+        b[j] = x[j];
+        want &= ~(1u << j);
       }
   }
   const int steps = (count + Map::kStride - 1) / Map::kStride;

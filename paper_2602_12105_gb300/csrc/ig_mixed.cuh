@@ -35,8 +35,8 @@ __device__ __noinline__ void finish_init_mixed(SolveScal* s, int k, const double
   s->inner_iter = 0;
   s->inner_cap = max_iter < 4000 ? max_iter : 4000;
   s->phase = kPhaseRestart;
-  s->tol = tol;
-  s->inner_tol = inner_tol;
+  s->tol2 = tol * tol;
+  s->inner_tol2 = inner_tol * inner_tol;
   s->max_iter = max_iter;
   s->max_refine = max_refine;
   s->status = bad ? IG_ERR_NONFINITE : IG_OK;
@@ -57,9 +57,9 @@ __device__ __noinline__ void finish_residual(SolveScal* s, const SolveScal& cur,
     if (!is_finite(res2[c])) {
       bad = 1;
     } else {
-      const double rel2 = res2[c] / cur.rhs2[c];  // squares, as in finish_update
+      const double rel2 = quotient(res2[c], cur.rhs2[c]);  // squares, as in finish_update
       s->relres2[c] = rel2;
-      if (rel2 <= cur.tol * cur.tol || !positive_finite(res2[c])) {
+      if (not_above(rel2, cur.tol2) || !positive_finite(res2[c])) {
         s->active64[c] = 0;
       } else {
         s->scale[c] = sqrt(res2[c]);
@@ -86,7 +86,7 @@ __device__ __noinline__ void finish_residual(SolveScal* s, const SolveScal& cur,
 }
 
 // After forming r32 = r64 / scale: start a new inner solve. Returns (on lane 0) the new phase.
-__device__ __noinline__ int finish_restart(SolveScal* s, const SolveScal& cur, int k, const double* acc) {
+__device__ __forceinline__ int finish_restart_step(SolveScal* s, const SolveScal& cur, int k, const double* acc) {
   const int c = threadIdx.x & 31;
   int act = 0;
   if (c < k) {
@@ -105,16 +105,19 @@ __device__ __noinline__ int finish_restart(SolveScal* s, const SolveScal& cur, i
   }
   return phase;
 }
+__device__ __noinline__ int finish_restart(SolveScal* s, const SolveScal& cur, int k, const double* acc) {
+  return finish_restart_step(s, cur, k, acc);
+}
 
 // Inner FP32 iteration: inner convergence test, beta, switch to Apply when the inner solve is done.
 // Returns (on lane 0) the phase after it, or -1 when the mesh is done (a non-finite sum).
-__device__ __noinline__ int finish_update_mixed(SolveScal* s, const SolveScal& cur, int k, const double* acc) {
+__device__ __forceinline__ int finish_update_mixed_step(SolveScal* s, const SolveScal& cur, int k, const double* acc) {
   const int c = threadIdx.x & 31, col = c & 7;
   int act = 0, bad = 0;
   const double* den = c < 8 ? cur.rz : cur.bnorm2;  // the divisions side by side, the test on squares (finish_update)
   const double* num = c < 8 ? acc : acc + k;
   double quot = 0.0;
-  if (col < k && c < 16) quot = num[col] / den[col];
+  if (col < k && c < 16) quot = quotient(num[col], den[col]);
   const double rel2 = __shfl_down_sync(0xffffffffu, quot, 8);
   if (c < k && cur.active[c] != 0) {
     const double rzn = acc[c], rr = acc[k + c];
@@ -122,7 +125,7 @@ __device__ __noinline__ int finish_update_mixed(SolveScal* s, const SolveScal& c
       bad = 1;
     } else {
       const double bta = quot;
-      if (rel2 <= cur.inner_tol * cur.inner_tol || !positive_finite(rzn)) {
+      if (not_above(rel2, cur.inner_tol2) || !positive_finite(rzn)) {
         s->active[c] = 0;
         s->beta[c] = 0.0;
       } else {
@@ -149,6 +152,9 @@ __device__ __noinline__ int finish_update_mixed(SolveScal* s, const SolveScal& c
     }
   }
   return phase;
+}
+__device__ __noinline__ int finish_update_mixed(SolveScal* s, const SolveScal& cur, int k, const double* acc) {
+  return finish_update_mixed_step(s, cur, k, acc);
 }
 
 }  // namespace

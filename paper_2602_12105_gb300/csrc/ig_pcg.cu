@@ -512,17 +512,24 @@ cudaError_t group_init(Group& g, const MeshDev* host_mds, int nmesh, int slots64
     g.listapp = ListRef{c.app_start32, c.app_mesh, c.app_big, &g.ctl->napp_big};
     if ((e = cudaMemcpyAsync(g.ctl, &c, sizeof(LoopCtl), cudaMemcpyHostToDevice, st)) != cudaSuccess) return e;
   }
-  const std::vector<int4> plan = gang_plan(host_mds, nmesh, num_sms, &g.gang_tickets);
-  if (!plan.empty()) {  // the ticket counter lies behind the plan
-    if ((e = cudaMalloc(&g.gang_plan, sizeof(int4) * (plan.size() + 1))) != cudaSuccess) return e;
-    if ((e = cudaMemcpyAsync(g.gang_plan, plan.data(), sizeof(int4) * plan.size(), cudaMemcpyHostToDevice, st)) !=
-        cudaSuccess)
-      return e;
-    g.gang_ticket = reinterpret_cast<unsigned*>(g.gang_plan + plan.size());
-  }
+  if ((e = group_order_gangs(g, nullptr, st)) != cudaSuccess) return e;
   if ((e = cudaStreamCreateWithFlags(&g.capture_stream, cudaStreamNonBlocking)) != cudaSuccess) return e;
   if ((e = cudaEventRecord(g.calls_ev, st)) != cudaSuccess) return e;
   return cudaStreamSynchronize(st);
+}
+
+// The gangs of the group's mixed-precision solves, in the order of these time steps (the ticket counter
+// lies behind the plan).
+cudaError_t group_order_gangs(Group& g, const double* t, cudaStream_t st) {
+  const std::vector<int4> plan =
+      gang_plan(g.host_mds.data(), t, g.nmesh, g.num_sms, &g.gang_tickets, &g.gang_workers);
+  if (plan.empty()) return cudaSuccess;
+  if (!g.gang_plan) {
+    cudaError_t e = cudaMalloc(&g.gang_plan, sizeof(int4) * (plan.size() + 1));
+    if (e != cudaSuccess) return e;
+    g.gang_ticket = reinterpret_cast<unsigned*>(g.gang_plan + plan.size());
+  }
+  return cudaMemcpyAsync(g.gang_plan, plan.data(), sizeof(int4) * plan.size(), cudaMemcpyHostToDevice, st);
 }
 
 // Refresh the device copy of the mesh descriptors from g.host_mds.

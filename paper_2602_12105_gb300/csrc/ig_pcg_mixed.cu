@@ -117,7 +117,8 @@ __global__ void __launch_bounds__(kBlock, 4) spmv_mixed_kernel(const MeshDev* __
               }
             }
           }
-          sum += (double)warp_sum_transposed<K>(pq, lane);
+          const double line = to_double(warp_sum_transposed<K>(pq, lane));
+          sum = l == rb * md.s32_h ? line : sum + line;
         }
         if (warp_sum_writer<K>(lane) && warp_sum_index<K>(lane) < K) red[warp_sum_index<K>(lane) * kWarps + warp] = sum;
         __syncthreads();
@@ -203,7 +204,7 @@ __global__ void __launch_bounds__(kBlock, 4) update_mixed_kernel(const MeshDev* 
           const int n32 = md.n;
           float alpha[K];
 #pragma unroll
-          for (int c = 0; c < K; ++c) alpha[c] = (float)tc.sn.alpha[c];
+          for (int c = 0; c < K; ++c) alpha[c] = tc.sn.alpha32[c];
           for (long base = t0; base < t1; base += kTileRows) {
             float acc[2 * K];
 #pragma unroll
@@ -314,13 +315,13 @@ __global__ void __launch_bounds__(kBlock, 4) pupdate_mixed_kernel(const MeshDev*
                     const bool step = tc.sn.inner_iter > 0;
                     float alpha[K];
 #pragma unroll
-                    for (int c = 0; c < K; ++c) alpha[c] = (float)tc.sn.alpha[c];
+                    for (int c = 0; c < K; ++c) alpha[c] = tc.sn.alpha32[c];
                     float* __restrict__ x32 = as_global(md.x32);
                     float* __restrict__ p32 = as_global(md.p32);
                     if (tc.sn.phase == kPhaseInner) {
                       float beta[K];
 #pragma unroll
-                      for (int c = 0; c < K; ++c) beta[c] = (float)tc.sn.beta[c];
+                      for (int c = 0; c < K; ++c) beta[c] = tc.sn.beta32[c];
                       const float* __restrict__ D32 = as_global(md.Dinv32);
                       const float* __restrict__ r32 = as_global(md.r32);
                       constexpr int R = 2;  // rows in flight

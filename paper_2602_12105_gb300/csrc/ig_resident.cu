@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
       if (!row_warp) {
         add_warps_to<K>(sh.red2, sh.tot);
         __syncwarp();
-        finish_spmv(&sh.st, sh.st, K, sh.tot);
+        finish_spmv_step(&sh.st, sh.st, K, sh.tot);
       }
       __syncthreads();
     }
@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
       if (!row_warp) {
         add_warps_to<2 * K>(sh.red2, sh.tot);
         __syncwarp();
-        finish_update(&sh.st, sh.st, K, sh.tot);
+        finish_update_step(&sh.st, sh.st, K, sh.tot);
       }
     }
   }

@@ -5,16 +5,24 @@
 // arithmetic, the tiles and the order of the sums are those of the multi-CTA kernels: the same bits,
 // alone and in any batch.
 //
-// One CTA per SM. The CTAs draw tickets; the tickets of a mesh are consecutive, the largest meshes
+// The CTAs draw tickets; the tickets of a mesh are consecutive, the longest solves
 // first, so that a CTA that is done with a mesh goes on to the next one without waiting for the rest
 // of the group: a batch takes no launch, and no idle CTA, per iteration, where the multi-CTA loop took
 // four launches per iteration of its slowest mesh. A CTA that draws a ticket waits for the rest of its
 // gang: those CTAs are at work on meshes drawn before, and the lowest gang that is not complete always
 // gets the next tickets, so every wait ends.
 //
-// Per iteration a gang meets three times: for p.q, for r.z and r.r, and after p is written (see
-// ig_meet.cuh). Each CTA has four workers of kBlock threads, which take its tiles four at a time; the
-// sums of such a group of four are posted together.
+// A CTA holds a group of four tiles and posts their sums together. Per iteration a gang meets three
+// times: for p.q, for r.z and r.r, and after p is written (see ig_meet.cuh); each meeting takes about
+// 1.2 us for the exchange alone. A single mesh takes CTAs of four workers of kBlock threads, one per
+// SM; a batch of small tiles takes CTAs of two workers, two per SM, so that one computes while the other
+// meets.
+//
+// Measured: 256 icospheres of 162 to 40,962 vertices (a forward and an adjoint solve of the batch), 21
+// and 23 ms in the multi-CTA loop, 11.1 and 11.4 ms here (13.3 and 13.5 with one CTA per SM and the
+// meshes in order of size); a grid of 251,819 vertices 45 -> 17 us an iteration. What bounds it: the
+// chain of an iteration (three meetings, their FP64 sums and divisions), then the latency of the
+// gathers; the L1 data path is busy 36% of the time, DRAM not at all.
 #include <algorithm>
 
 #include "ig_meet.cuh"
@@ -24,23 +32,25 @@ namespace ig {
 
 namespace {
 
-constexpr int kGangThreads = 4 * kBlock;
 
-constexpr int kGangGroups = 2;                       // most groups of four tiles a CTA holds
-constexpr int kGangBytes = 227 * 1024 - 8 * 1024;    // dynamic shared memory: all but GangShared's part
+// Dynamic shared memory of a CTA of W workers: what GangShared leaves of an SM's 227 KB, or of half of
+// them.
+template <int W>
+constexpr int kGangBytes = W == 4 ? 222 * 1024 : 108 * 1024;
 
 // Operator slots per row that fit on chip beside three K-vectors and the preconditioner.
-__host__ __device__ inline int gang_slots(int rows, int k, int wmax) {
-  const int fit = (kGangBytes / rows - 4 * (3 * k + 1)) / 8;
+__host__ __device__ inline int gang_slots(int bytes, int rows, int k, int wmax) {
+  const int fit = (bytes / rows - 4 * (3 * k + 1)) / 8;
   return fit < wmax ? fit : wmax;
 }
 
 struct GangShared {
   MeshDev md;
   SolveScal st;
-  double red[kGangGroups][4][8 * kWarps];  // warp totals of each group's four tiles
+  double red[4][8 * kWarps];               // warp totals of the four tiles
   double red2[8 * kWarps];
   double tot[8];
+  float alpha[kMaxK], beta[kMaxK];         // as floats (a conversion in every warp costs FP64 issue)
   int ticket;
   int width[kGangMaxRows / 32];
 };
@@ -54,32 +64,34 @@ struct GangRows {  // what a CTA holds of its mesh, in dynamic shared memory
 
 struct Gang {
   Slot* slots;
-  int member, nct;       // this CTA, and the CTAs of the gang
-  int first, ngroups;    // this CTA's first group of four tiles and their number
-  int total;             // groups of the mesh
-  int groups_per_cta;
+  int member, nct;     // this CTA and the CTAs of the gang: as many as the mesh has groups of four tiles
   unsigned long long number;
-  long long patience;    // polls before a wait is given up
+  long long patience;  // polls before a wait is given up
 
-  __device__ __forceinline__ Slot* buffer() const { return slots + (number & 1) * (8 * (size_t)total); }
+  __device__ __forceinline__ Slot* buffer() const { return slots + (number & 1) * (8 * (size_t)nct); }
 
-  // Groups' sums (warp totals in sh.red), posted and collected: afterwards the mesh's totals are in
-  // sh.tot on warp 0. False in every thread when a wait ran out.
+  // A meeting for sums. First those of this CTA's four tiles (warp totals in sh.red) are posted ...
   template <int NV>
-  __device__ __forceinline__ bool meet_sums(GangShared& sh) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  __device__ __forceinline__ void post_sums(GangShared& sh) {
+    const int lane = threadIdx.x & 31;
     ++number;
     __syncthreads();
-    if (warp < ngroups) {  // one warp per group: lane = value * 4 + tile, then over the four tiles
+    if (threadIdx.x < 32) {  // lane = value * 4 + tile, then over the four tiles
       const int v = lane >> 2, t = lane & 3;
-      double s = v < NV ? add_warps_of<kGroups>(&sh.red[warp][t][v * kWarps]) : 0.0;
+      double s = v < NV ? add_warps_of<kGroups>(&sh.red[t][v * kWarps]) : 0.0;
       s += __shfl_xor_sync(0xffffffffu, s, 1);
       s += __shfl_xor_sync(0xffffffffu, s, 2);
-      if (t == 0 && v < NV) post(buffer() + 8 * (size_t)(first + warp) + v, s, number);
+      if (t == 0 && v < NV) post(buffer() + 8 * (size_t)member + v, s, number);
     }
+  }
+  // ... then all groups' are collected: the mesh's totals are in sh.tot on warp 0. False in every
+  // thread when a wait ran out.
+  template <int NV>
+  __device__ __forceinline__ bool collect_sums(GangShared& sh) {
+    const int warp = threadIdx.x >> 5;
     bool late = false;
     if (warp < kWarps)
-      PartialMap<NV>::to_warp_total(collect_sum<NV, false>(buffer(), total, number, patience, late), sh.red2);
+      PartialMap<NV>::to_warp_total(collect_sum<NV, false>(buffer(), nct, number, patience, late), sh.red2);
     if (__syncthreads_or(late)) return false;
     if (warp == 0) {
       add_warps_to<NV>(sh.red2, sh.tot);
@@ -95,11 +107,11 @@ struct Gang {
     __syncthreads();
     if (threadIdx.x == 0) {
       fence_gpu();
-      post(buffer() + 8 * (size_t)first, 0.0, number);
+      post(buffer() + 8 * (size_t)member, 0.0, number);
     }
     bool late = false;
     if ((int)threadIdx.x < nct) {
-      const Slot* theirs = buffer() + 8 * (size_t)(threadIdx.x * groups_per_cta);
+      const Slot* theirs = buffer() + 8 * (size_t)threadIdx.x;
       double x;
       for (long long spins = 0; !peek<true>(theirs, number, x) && !late; late = ++spins > patience) {
       }
@@ -108,14 +120,13 @@ struct Gang {
   }
 };
 
-// The tile of worker `worker` in round `round` of this CTA, and its rows.
+// Tile i of a CTA's four, and its rows.
 struct GangTile {
   int tile, t0, rows, local;  // rows t0 .. t0 + rows of the mesh, local .. of the CTA
 };
-__device__ __forceinline__ GangTile gang_tile(const MeshDev& md, int first_tile, int round, int worker) {
+__device__ __forceinline__ GangTile gang_tile(const MeshDev& md, int member, int i) {
   GangTile g;
-  const int i = 4 * round + worker;
-  g.tile = first_tile + i;
+  g.tile = 4 * member + i;
   g.local = i * md.tile_rows32;
   g.t0 = g.tile * md.tile_rows32;
   g.rows = g.tile < md.ntiles32 ? min(md.tile_rows32, md.n - g.t0) : 0;
@@ -123,11 +134,11 @@ __device__ __forceinline__ GangTile gang_tile(const MeshDev& md, int first_tile,
 }
 
 // One slot's loop of a mesh's solve by its gang: see ig_pcg_mixed.cu for the phases.
-template <int K>
+template <int K, int W>
 __device__ __forceinline__ bool gang_solve(GangShared& sh, const GangRows& gr, Gang& gang, int cap) {
   const MeshDev& md = sh.md;
   const int worker = threadIdx.x / kBlock, tid = threadIdx.x % kBlock, warp = tid >> 5, lane = tid & 31;
-  const int n = md.n, rp = gr.rp, first_tile = 4 * gang.first;
+  const int n = md.n, rp = gr.rp;
   const long nn = n;
   float* p = as_global(md.p32);
   double* x64 = as_global(md.x);
@@ -137,8 +148,8 @@ __device__ __forceinline__ bool gang_solve(GangShared& sh, const GangRows& gr, G
     if (sh.st.phase == kPhaseApply) {
       // r64 = rhs - A x64 and its norms, once every CTA's x64 is there; the sums in tile order
       if (!gang.meet_writes()) return false;
-      for (int g = 0; g < gang.ngroups; ++g) {
-        const GangTile t = gang_tile(md, first_tile, g, worker);
+      for (int i4 = worker; i4 < 4; i4 += W) {
+        const GangTile t = gang_tile(md, gang.member, i4);
         double acc[K];
 #pragma unroll
         for (int c = 0; c < K; ++c) acc[c] = 0.0;
@@ -156,13 +167,13 @@ __device__ __forceinline__ bool gang_solve(GangShared& sh, const GangRows& gr, G
         }
         const double w = warp_sum_transposed<K>(acc, lane);
         const int idx = warp_sum_index<K>(lane);
-        if (warp_sum_writer<K>(lane) && idx < K) sh.red[g][worker][idx * kWarps + warp] = w;
+        if (warp_sum_writer<K>(lane) && idx < K) sh.red[i4][idx * kWarps + warp] = w;
       }
       __syncthreads();
-      for (int g = 0; g < gang.ngroups; ++g) {
-        const GangTile t = gang_tile(md, first_tile, g, worker);
+      for (int i4 = worker; i4 < 4; i4 += W) {
+        const GangTile t = gang_tile(md, gang.member, i4);
         if (tid < K && t.rows > 0)
-          __stcg(md.part + (long)t.tile * kPartStride + tid, add_warps_of<kInOrder>(&sh.red[g][worker][tid * kWarps]));
+          __stcg(md.part + (long)t.tile * kPartStride + tid, add_warps_of<kInOrder>(&sh.red[i4][tid * kWarps]));
       }
       if (!gang.meet_writes()) return false;
       double v[K];
@@ -181,8 +192,8 @@ __device__ __forceinline__ bool gang_solve(GangShared& sh, const GangRows& gr, G
     }
     if (sh.st.phase == kPhaseInner) {
       // q = A p and p.q
-      for (int g = 0; g < gang.ngroups; ++g) {
-        const GangTile t = gang_tile(md, first_tile, g, worker);
+      for (int i4 = worker; i4 < 4; i4 += W) {
+        const GangTile t = gang_tile(md, gang.member, i4);
         float pq[K];
 #pragma unroll
         for (int c = 0; c < K; ++c) pq[c] = 0.f;
@@ -229,10 +240,14 @@ __device__ __forceinline__ bool gang_solve(GangShared& sh, const GangRows& gr, G
         }
         const float w = warp_sum_transposed<K>(pq, lane);
         const int idx = warp_sum_index<K>(lane);
-        if (warp_sum_writer<K>(lane) && idx < K) sh.red[g][worker][idx * kWarps + warp] = (double)w;
+        if (warp_sum_writer<K>(lane) && idx < K) sh.red[i4][idx * kWarps + warp] = to_double(w);
       }
-      if (!gang.meet_sums<K>(sh)) return false;
-      if (threadIdx.x < 32) finish_spmv(&sh.st, sh.st, K, sh.tot);
+      gang.post_sums<K>(sh);
+      if (!gang.collect_sums<K>(sh)) return false;
+      if (threadIdx.x < 32) {
+        finish_spmv_step(&sh.st, sh.st, K, sh.tot);
+        if (threadIdx.x < K) sh.alpha[threadIdx.x] = f64_to_f32_rn(sh.st.alpha[threadIdx.x]);
+      }
       __syncthreads();
       if (sh.st.done) break;
     }
@@ -243,11 +258,11 @@ __device__ __forceinline__ bool gang_solve(GangShared& sh, const GangRows& gr, G
       double inv[K];
 #pragma unroll
       for (int c = 0; c < K; ++c) {
-        alpha[c] = (float)sh.st.alpha[c];
+        alpha[c] = sh.alpha[c];
         inv[c] = inner ? 0.0 : 1.0 / sh.st.scale[c];
       }
-      for (int g = 0; g < gang.ngroups; ++g) {
-        const GangTile t = gang_tile(md, first_tile, g, worker);
+      for (int i4 = worker; i4 < 4; i4 += W) {
+        const GangTile t = gang_tile(md, gang.member, i4);
         float acc[2 * K];
 #pragma unroll
         for (int i = 0; i < 2 * K; ++i) acc[i] = 0.f;
@@ -270,58 +285,78 @@ __device__ __forceinline__ bool gang_solve(GangShared& sh, const GangRows& gr, G
         }
         const float w = warp_sum_transposed<2 * K>(acc, lane);
         const int idx = warp_sum_index<2 * K>(lane);
-        if (warp_sum_writer<2 * K>(lane) && idx < 2 * K) sh.red[g][worker][idx * kWarps + warp] = (double)w;
+        if (warp_sum_writer<2 * K>(lane) && idx < 2 * K) sh.red[i4][idx * kWarps + warp] = to_double(w);
       }
     }
-    if (!gang.meet_sums<2 * K>(sh)) return false;
+    gang.post_sums<2 * K>(sh);
+    if (inner) {
+      // x += alpha p while the sums are on their way
+      float alpha[K];
+#pragma unroll
+      for (int c = 0; c < K; ++c) alpha[c] = sh.alpha[c];
+      for (int i4 = worker; i4 < 4; i4 += W) {
+        const GangTile t = gang_tile(md, gang.member, i4);
+        for (int o = tid; o < t.rows; o += kBlock) {
+          float pi[K];
+          load_row32<K>(p, t.t0 + o, pi);
+#pragma unroll
+          for (int c = 0; c < K; ++c) {
+            float* x = gr.x + c * rp + t.local + o;
+            *x = fmaf(alpha[c], pi[c], *x);
+          }
+        }
+      }
+    }
+    if (!gang.collect_sums<2 * K>(sh)) return false;
     if (threadIdx.x < 32) {
-      if (inner) finish_update_mixed(&sh.st, sh.st, K, sh.tot);
-      else finish_restart(&sh.st, sh.st, K, sh.tot);
+      if (inner) finish_update_mixed_step(&sh.st, sh.st, K, sh.tot);
+      else finish_restart_step(&sh.st, sh.st, K, sh.tot);
+      if (threadIdx.x < K) sh.beta[threadIdx.x] = f64_to_f32_rn(sh.st.beta[threadIdx.x]);
     }
     __syncthreads();
     if (sh.st.done) break;
-    // x += alpha p (after an iteration); Inner: p = D^-1 r + beta p; Apply: x64 += ||r64|| x
-    {
-      const bool step = sh.st.inner_iter > 0, next = sh.st.phase == kPhaseInner;
-      float alpha[K], beta[K];
-      double sc[K];
+    if (sh.st.phase == kPhaseInner) {
+      // p = D^-1 r + beta p
+      float beta[K];
 #pragma unroll
-      for (int c = 0; c < K; ++c) {
-        alpha[c] = (float)sh.st.alpha[c];
-        beta[c] = (float)sh.st.beta[c];
-        sc[c] = sh.st.scale[c];
-      }
-      for (int g = 0; g < gang.ngroups; ++g) {
-        const GangTile t = gang_tile(md, first_tile, g, worker);
+      for (int c = 0; c < K; ++c) beta[c] = sh.beta[c];
+      for (int i4 = worker; i4 < 4; i4 += W) {
+        const GangTile t = gang_tile(md, gang.member, i4);
         for (int o = tid; o < t.rows; o += kBlock) {
           const int i = t.local + o;
-          const long row = t.t0 + o;
-          float pi[K], pn[K];
-          load_row32<K>(p, row, pi);
+          float pi[K];
+          load_row32<K>(p, t.t0 + o, pi);
           const float d = gr.d[i];
 #pragma unroll
-          for (int c = 0; c < K; ++c) {
-            float xv = gr.x[c * rp + i];
-            if (step) {
-              xv = fmaf(alpha[c], pi[c], xv);
-              gr.x[c * rp + i] = xv;
-            }
-            if (next) pn[c] = fmaf(beta[c], pi[c], d * gr.r[c * rp + i]);
-            else x64[c * nn + row] = fma(sc[c], (double)xv, x64[c * nn + row]);
-          }
-          if (next) store_row32<K>(p, row, pn);
+          for (int c = 0; c < K; ++c) pi[c] = fmaf(beta[c], pi[c], d * gr.r[c * rp + i]);
+          store_row32<K>(p, t.t0 + o, pi);
         }
       }
-      if (next && !gang.meet_writes()) return false;
+      if (!gang.meet_writes()) return false;
+    } else {
+      // x64 += ||r64|| x
+      double sc[K];
+#pragma unroll
+      for (int c = 0; c < K; ++c) sc[c] = sh.st.scale[c];
+      for (int i4 = worker; i4 < 4; i4 += W) {
+        const GangTile t = gang_tile(md, gang.member, i4);
+        for (int o = tid; o < t.rows; o += kBlock) {
+          const long row = t.t0 + o;
+#pragma unroll
+          for (int c = 0; c < K; ++c)
+            x64[c * nn + row] = fma(sc[c], (double)gr.x[c * rp + t.local + o], x64[c * nn + row]);
+        }
+      }
     }
   }
   return true;
 }
 
-template <int K>
-__global__ void __launch_bounds__(kGangThreads, 1) solve_gang_kernel(const MeshDev* __restrict__ mds,
-                                                                     const int4* __restrict__ plan, int nplan,
-                                                                     int tickets, unsigned* ticket, int cap) {
+template <int K, int W>
+__global__ void __launch_bounds__(W * kBlock, W == 4 ? 1 : 2) solve_gang_kernel(const MeshDev* __restrict__ mds,
+                                                                                const int4* __restrict__ plan, int nplan,
+                                                                                int tickets, unsigned* ticket, int cap) {
+  constexpr int kGangThreads = W * kBlock;
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ GangShared sh;
   for (;;) {
@@ -335,7 +370,7 @@ __global__ void __launch_bounds__(kGangThreads, 1) solve_gang_kernel(const MeshD
       if (__ldg(&plan[mid].y) <= sh.ticket) lo = mid;
       else hi = mid - 1;
     }
-    const int4 e = __ldg(plan + lo);  // mesh, first ticket, CTAs, groups per CTA
+    const int4 e = __ldg(plan + lo);  // mesh, first ticket, CTAs
     for (int j = threadIdx.x; j < (int)(sizeof(MeshDev) / 4); j += kGangThreads)
       reinterpret_cast<unsigned*>(&sh.md)[j] = __ldg(reinterpret_cast<const unsigned*>(mds + e.x) + j);
     __syncthreads();
@@ -345,10 +380,6 @@ __global__ void __launch_bounds__(kGangThreads, 1) solve_gang_kernel(const MeshD
     Gang gang;
     gang.member = sh.ticket - e.y;
     gang.nct = e.z;
-    gang.groups_per_cta = e.w;
-    gang.total = (md.ntiles32 + 3) / 4;
-    gang.first = gang.member * e.w;
-    gang.ngroups = min(e.w, gang.total - gang.first);
     gang.slots = reinterpret_cast<Slot*>(md.meet) + 1;
     const unsigned long long launches = __ldcg(reinterpret_cast<const unsigned long long*>(md.meet));
     gang.number = launches << 32;
@@ -357,10 +388,10 @@ __global__ void __launch_bounds__(kGangThreads, 1) solve_gang_kernel(const MeshD
 
     // the rows on chip
     GangRows gr;
-    const int first_row = 4 * gang.first * md.tile_rows32;
-    const int held = min(4 * gang.ngroups * md.tile_rows32, md.n - first_row);
-    gr.rp = 4 * e.w * md.tile_rows32;
-    gr.aw = gang_slots(gr.rp, K, md.sell_wmax);
+    const int first_row = 4 * gang.member * md.tile_rows32;
+    gr.rp = 4 * md.tile_rows32;
+    const int held = min(gr.rp, md.n - first_row);
+    gr.aw = gang_slots(kGangBytes<W>, gr.rp, K, md.sell_wmax);
     gr.r = reinterpret_cast<float*>(dyn);
     gr.x = gr.r + K * gr.rp;
     gr.q = gr.x + K * gr.rp;
@@ -380,7 +411,7 @@ __global__ void __launch_bounds__(kGangThreads, 1) solve_gang_kernel(const MeshD
     }
     __syncthreads();
 
-    const bool met = gang_solve<K>(sh, gr, gang, cap);
+    const bool met = gang_solve<K, W>(sh, gr, gang, cap);
     __syncthreads();
     if (gang.member == 0) {
       if (threadIdx.x == 0 && !met) {  // a CTA stayed away past the limit: report a failed solve
@@ -395,23 +426,22 @@ __global__ void __launch_bounds__(kGangThreads, 1) solve_gang_kernel(const MeshD
   }
 }
 
-static_assert(sizeof(GangShared) <= 8 * 1024 - 256, "shared memory of a gang CTA");
+// (1 KB of an SM's shared memory is the system's for each CTA)
+static_assert(sizeof(GangShared) <= 4 * 1024, "shared memory of a gang CTA");
 
-template <int K>
-bool launch(Group& g, int cap, cudaStream_t st) {
-  auto kern = solve_gang_kernel<K>;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGangBytes) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  if (cudaMemsetAsync(g.gang_ticket, 0, sizeof(unsigned), st) != cudaSuccess) {
+template <int K, int W>
+bool launch_w(Group& g, int cap, cudaStream_t st) {
+  auto kern = solve_gang_kernel<K, W>;
+  const int ctas = g.num_sms * (W == 4 ? 1 : 2);
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGangBytes<W>) != cudaSuccess ||
+      cudaMemsetAsync(g.gang_ticket, 0, sizeof(unsigned), st) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(g.gang_tickets < g.num_sms ? g.gang_tickets : g.num_sms, 1, 1);
-  cfg.blockDim = dim3(kGangThreads, 1, 1);
-  cfg.dynamicSmemBytes = kGangBytes;
+  cfg.gridDim = dim3(g.gang_tickets < ctas ? g.gang_tickets : ctas, 1, 1);
+  cfg.blockDim = dim3(W * kBlock, 1, 1);
+  cfg.dynamicSmemBytes = kGangBytes<W>;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeCooperative;
@@ -426,33 +456,38 @@ bool launch(Group& g, int cap, cudaStream_t st) {
   return true;
 }
 
+template <int K>
+bool launch(Group& g, int cap, cudaStream_t st) {
+  return g.gang_workers == 2 ? launch_w<K, 2>(g, cap, st) : launch_w<K, 4>(g, cap, st);
+}
+
 }  // namespace
 
-// The gangs of a group: mesh, first ticket, CTAs and groups of tiles per CTA, the largest first. One
-// group of tiles per CTA when the whole group of meshes then fits on the SMs at once, else two
-// (where they fit on chip): fewer CTAs per mesh leave less of an iteration to its meetings, and more
-// meshes run beside each other. Empty when some mesh is too large.
-std::vector<int4> gang_plan(const MeshDev* mds, int nmesh, int num_sms, int* tickets) {
+// The gangs of a group: mesh, first ticket, CTAs; empty when some mesh is too large. The meshes with the
+// longest solves come first, so that none of them is still running when the rest is done: iterations
+// grow with the square root of the time step over the squared edge length, that is of t n on meshes of
+// one size (t null: equal steps). CTAs of two workers (two per SM) when there are more of them than
+// SMs and their tiles are small enough.
+std::vector<int4> gang_plan(const MeshDev* mds, const double* t, int nmesh, int num_sms, int* tickets, int* workers) {
   std::vector<int4> plan;
-  long groups = 0;
+  std::vector<double> work((size_t)nmesh);
+  int rows = 0;
   for (int i = 0; i < nmesh; ++i) {
     const int g = (mds[i].ntiles32 + 3) / 4;
     if (!mds[i].meet || g > num_sms || g > kResMaxCtas || 4 * mds[i].tile_rows32 > kGangMaxRows) return {};
-    groups += g;
-  }
-  for (int i = 0; i < nmesh; ++i) {
-    const int g = (mds[i].ntiles32 + 3) / 4;
-    const int per = groups > num_sms && 4 * kGangGroups * mds[i].tile_rows32 <= kGangMaxRows ? kGangGroups : 1;
-    plan.push_back(make_int4(i, 0, (g + per - 1) / per, per));
+    rows = std::max(rows, 4 * mds[i].tile_rows32);
+    work[(size_t)i] = (t ? t[i] : 1.0) * mds[i].n;
+    plan.push_back(make_int4(i, 0, g, 0));
   }
   std::stable_sort(plan.begin(), plan.end(),
-                   [mds](const int4& a, const int4& b) { return mds[a.x].n > mds[b.x].n; });
-  int t = 0;
+                   [&work](const int4& a, const int4& b) { return work[(size_t)a.x] > work[(size_t)b.x]; });
+  int first = 0;
   for (int4& e : plan) {
-    e.y = t;
-    t += e.z;
+    e.y = first;
+    first += e.z;
   }
-  *tickets = t;
+  *tickets = first;
+  *workers = first > num_sms && rows <= kGangMaxRows / 2 - 32 ? 2 : 4;
   return plan;
 }
 
