@@ -117,16 +117,34 @@ ig_status bad_arg(ig_ctx* ctx, const char* msg) {
   return IG_ERR_INVALID_ARG;
 }
 
-template <typename T>
-cudaError_t mesh_alloc(ig_mesh* mesh, T** out, size_t count) {
+// The arrays of the next mesh_alloc calls come out of one allocation of `bytes` (padded sizes).
+cudaError_t mesh_reserve(ig_mesh* mesh, size_t bytes) {
   void* p = nullptr;
-  const size_t bytes = sizeof(T) * (count > 0 ? count : 1);
   cudaError_t e = cudaMalloc(&p, bytes);
   if (e != cudaSuccess) return e;
   mesh->allocs.push_back(p);
+  mesh->slab = Slab{static_cast<char*>(p), bytes, 0};
+  return cudaSuccess;
+}
+
+template <typename T>
+cudaError_t mesh_alloc(ig_mesh* mesh, T** out, size_t count) {
+  const size_t bytes = sizeof(T) * (count > 0 ? count : 1);
+  void* p = mesh->slab.take(bytes);
+  if (!p) {
+    cudaError_t e = cudaMalloc(&p, bytes);
+    if (e != cudaSuccess) return e;
+    mesh->allocs.push_back(p);
+  }
   mesh->bytes += (int64_t)bytes;
   *out = static_cast<T*>(p);
   return cudaSuccess;
+}
+
+// Padded bytes of `count` values of T, for mesh_reserve.
+template <typename T>
+size_t room(size_t count) {
+  return Slab::padded(sizeof(T) * (count > 0 ? count : 1));
 }
 
 void mesh_release(ig_mesh* mesh) {
@@ -157,19 +175,20 @@ const char* err_bits_message(int bits) {
 
 // Device temporaries released when the owner goes out of scope.
 struct TmpAllocs {
-  std::vector<void*> v;
+  Slab slab;
   ~TmpAllocs() {
-    for (void* p : v) cudaFree(p);
+    if (slab.base) cudaFree(slab.base);
+  }
+  cudaError_t reserve(size_t bytes) {
+    void* p = nullptr;
+    cudaError_t e = cudaMalloc(&p, bytes);
+    if (e == cudaSuccess) slab = Slab{static_cast<char*>(p), bytes, 0};
+    return e;
   }
   template <typename T>
   cudaError_t get(T** out, size_t count) {
-    void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, sizeof(T) * (count > 0 ? count : 1));
-    if (e == cudaSuccess) {
-      v.push_back(p);
-      *out = static_cast<T*>(p);
-    }
-    return e;
+    *out = static_cast<T*>(slab.take(sizeof(T) * count));
+    return *out ? cudaSuccess : cudaErrorMemoryAllocation;
   }
 };
 
@@ -230,6 +249,10 @@ cudaError_t mesh_ensure_mixed(ig_mesh* mesh, cudaStream_t st) {
   if (md.A32) return cudaSuccess;
   const size_t nv = (size_t)mesh->n * kMaxK;
   cudaError_t e;
+  const size_t ns = (size_t)md.nnz_sell;
+  if ((e = mesh_reserve(mesh, room<float>(ns) + room<float>((size_t)mesh->n) + 4 * room<float>(nv) +
+                                  (mesh->c16_fits ? room<short>(ns) : 0))) != cudaSuccess)
+    return e;
   if ((e = mesh_alloc(mesh, &md.A32, (size_t)md.nnz_sell)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(md.A32, 0, sizeof(float) * (size_t)md.nnz_sell, st)) != cudaSuccess) return e;
   if ((e = mesh_alloc(mesh, &md.Dinv32, (size_t)mesh->n)) != cudaSuccess) return e;
@@ -238,18 +261,11 @@ cudaError_t mesh_ensure_mixed(ig_mesh* mesh, cudaStream_t st) {
   if ((e = mesh_alloc(mesh, &md.p32, nv)) != cudaSuccess) return e;
   if ((e = mesh_alloc(mesh, &md.q32, nv)) != cudaSuccess) return e;
   if ((e = cudaMemsetAsync(md.p32, 0, sizeof(float) * nv, st)) != cudaSuccess) return e;
-  if (md.sell_ptr) {
-    // 16-bit column offsets, kept when every slice's columns fit (one-time check on the host)
+  if (mesh->c16_fits) {
     short* c16 = nullptr;
-    int* nfar = nullptr;
-    if ((e = mesh_alloc(mesh, &c16, (size_t)md.nnz_sell)) != cudaSuccess) return e;
-    if ((e = mesh_alloc(mesh, &nfar, 1)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(nfar, 0, sizeof(int), st)) != cudaSuccess) return e;
-    if ((e = launch_sell_c16(md.sell_ptr, md.sell_col, mesh->n, c16, nfar, st)) != cudaSuccess) return e;
-    int far = 1;
-    if ((e = cudaMemcpyAsync(&far, nfar, sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess) return e;
-    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return e;
-    md.sell_c16 = far == 0 ? c16 : nullptr;
+    if ((e = mesh_alloc(mesh, &c16, ns)) != cudaSuccess) return e;
+    if ((e = launch_sell_c16(md.sell_ptr, md.sell_col, mesh->n, c16, nullptr, st)) != cudaSuccess) return e;
+    md.sell_c16 = c16;
   }
   mesh->group.host_mds[0] = md;
   return group_upload_mds(mesh->group, st);
@@ -263,6 +279,7 @@ cudaError_t mesh_ensure_geom32(ig_mesh* mesh, cudaStream_t st) {
   MeshDev& md = mesh->md;
   if (md.vsplit) return cudaSuccess;
   const size_t n = (size_t)mesh->n;
+  if ((e = mesh_reserve(mesh, 3 * room<float>(8 * n) + room<float>(n))) != cudaSuccess) return e;
   if ((e = mesh_alloc(mesh, &md.vsplit, 8 * n)) != cudaSuccess) return e;
   if ((e = mesh_alloc(mesh, &md.usplit, 8 * n)) != cudaSuccess) return e;
   if ((e = mesh_alloc(mesh, &md.lsplit, 8 * n)) != cudaSuccess) return e;
@@ -385,6 +402,16 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
   } while (0)
 
   const size_t scan_ints = scan_scratch_ints(std::max(ni, 3 * mi) + 1);
+  const size_t nv = (size_t)n * kMaxK, nslices = ((size_t)n + 31) / 32;
+  UP_CK(mesh_reserve(M, room<int>(3 * (size_t)m) + 2 * room<int>((size_t)n + 1) + room<int>((size_t)n) +
+                            room<int2>(3 * (size_t)m) + room<int>(1) + room<int>(nslices + 1) +
+                            room<unsigned>((nslices + 31) / 32) + room<double>(4 * (size_t)m) +
+                            2 * room<double>((size_t)n) + 6 * room<double>(nv) + room<double>(9 * (size_t)m) +
+                            room<SolveScal>(1)),
+        "alloc mesh");
+  UP_CK(tmp.reserve(3 * room<int>((size_t)n) + room<int>(3 * (size_t)m) + room<int>(6 * (size_t)m + (size_t)n) +
+                    room<int>(scan_ints) + room<int>(2) + room<int>(nslices) + room<int>(3 + kPatW)),
+        "alloc tmp");
   UP_CK(mesh_alloc(M, &F, 3 * (size_t)m), "alloc F");
   UP_CK(mesh_alloc(M, &incptr, (size_t)n + 1), "alloc incptr");
   UP_CK(mesh_alloc(M, &rowptr, (size_t)n + 1), "alloc rowptr");
@@ -465,16 +492,20 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
   UP_CK(launch_sell_fill(rowptr, col, ni, sell_ptr, sell_col, st), "sell fill");
 
   // the column pattern that most slices share, if any
-  int host_pat[2 + kPatW] = {};  // found, offsets, slices that follow it
+  int host_pat[3 + kPatW] = {};  // found, offsets, slices that follow it, slices with far columns
   unsigned* patbit = nullptr;
   {
     int* pat = nullptr;
-    UP_CK(tmp.get(&pat, 2 + kPatW), "alloc tmp");
+    UP_CK(tmp.get(&pat, 3 + kPatW), "alloc tmp");
     UP_CK(mesh_alloc(M, &patbit, (size_t)(nsl + 31) / 32), "alloc pattern");
     UP_CK(launch_sell_pattern(sell_ptr, sell_col, rowptr, ni, pat, patbit, pat + 1 + kPatW, st), "sell pattern");
+    UP_CK(cudaMemsetAsync(pat + 2 + kPatW, 0, sizeof(int), st), "memset");
+    UP_CK(launch_sell_c16(sell_ptr, sell_col, ni, nullptr, pat + 2 + kPatW, st), "sell columns");
     UP_CK(cudaMemcpyAsync(host_pat, pat, sizeof(host_pat), cudaMemcpyDeviceToHost, st), "read pattern");
     UP_CK(cudaStreamSynchronize(st), "sell pattern");
   }
+
+  M->c16_fits = host_pat[2 + kPatW] == 0;
 
   // operator and solver workspace
   MeshDev& md = M->md;
@@ -588,15 +619,12 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
   md.incptr = incptr;
   md.inc = inc;
   md.err = err;
-  const size_t nv = (size_t)n * kMaxK;
   // partial sums: the loop kernels' tiles (and the geodesic warm start's, of kTileRows rows), and the
   // VJP's per-face-tile sums of dl/dt
   const size_t npart = std::max(std::max(std::max((size_t)md.ntiles, (size_t)std::max(md.ntiles32, md.ntiles32s)),
                                          (size_t)(ni + kTileRows - 1) / kTileRows) * kPartStride,
                                 (size_t)(mi + 255) / 256) + 8;
   UP_CK(mesh_alloc(M, &md.facew, 4 * (size_t)m), "alloc");
-  UP_CK(mesh_alloc(M, &md.A, (size_t)nnz_sell), "alloc");
-  UP_CK(cudaMemsetAsync(md.A, 0, sizeof(double) * (size_t)nnz_sell, st), "memset");
   UP_CK(mesh_alloc(M, &md.M, (size_t)n), "alloc");
   UP_CK(mesh_alloc(M, &md.Dinv, (size_t)n), "alloc");
   UP_CK(mesh_alloc(M, &md.x, nv), "alloc");
@@ -607,17 +635,22 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
   md.rhs = md.q;  // the FP64 q vector is unused in mixed precision, where it keeps the rhs
   UP_CK(mesh_alloc(M, &md.lam, nv), "alloc");
   UP_CK(mesh_alloc(M, &md.gface, 9 * (size_t)m), "alloc");
-  UP_CK(mesh_alloc(M, &md.part, npart), "alloc");
   UP_CK(mesh_alloc(M, &md.s, 1), "alloc");
-  md.resident = resident;
   const bool gang = (md.ntiles32 + 3) / 4 <= ctx->num_sms && 4 * md.tile_rows32 <= kGangMaxRows;
-  if (resident || gang) {
-    const size_t bytes = meet_bytes(std::max(resident ? md.ntiles : 0, gang ? (md.ntiles32 + 3) / 4 : 0));
+  const size_t nmeet = resident || gang
+                           ? meet_bytes(std::max(resident ? md.ntiles : 0, gang ? (md.ntiles32 + 3) / 4 : 0))
+                           : 0;
+  UP_CK(mesh_reserve(M, room<double>((size_t)nnz_sell) + room<double>(npart) + room<char>(nmeet)), "alloc");
+  UP_CK(mesh_alloc(M, &md.A, (size_t)nnz_sell), "alloc");
+  UP_CK(mesh_alloc(M, &md.part, npart), "alloc");
+  md.resident = resident;
+  if (nmeet) {
     unsigned char* meet = nullptr;
-    UP_CK(mesh_alloc(M, &meet, bytes), "alloc");
-    UP_CK(cudaMemsetAsync(meet, 0, bytes, st), "memset");
+    UP_CK(mesh_alloc(M, &meet, nmeet), "alloc");
+    UP_CK(cudaMemsetAsync(meet, 0, nmeet, st), "memset");
     md.meet = meet;
   }
+  UP_CK(cudaMemsetAsync(md.A, 0, sizeof(double) * (size_t)nnz_sell, st), "memset");
   UP_CK(cudaMemsetAsync(md.s, 0, sizeof(SolveScal), st), "memset");
   UP_CK(cudaMemsetAsync(md.p, 0, sizeof(double) * nv, st), "memset");
   UP_CK(cudaMemsetAsync(md.q, 0, sizeof(double) * nv, st), "memset");

@@ -170,8 +170,8 @@ ig_status ig_batch_assemble(ig_batch* b, const double* const* V_dev, const doubl
     calls[i].t = t[i];
   }
   BT_CK(ctx, refresh(b, ctx->stream), "upload");
-  BT_CK(ctx, group_set_calls(b->group, calls.data(), ctx->stream), "upload");
   if (nm > 1) BT_CK(ctx, group_order_gangs(b->group, t, ctx->stream), "upload");
+  BT_CK(ctx, group_set_calls(b->group, calls.data(), ctx->stream), "upload");
   BT_CK(ctx, launch_assemble(b->group, precision, ctx->stream), "batch assemble");
   for (int i = 0; i < nm; ++i) {
     b->meshes[i]->assembled = precision + 1;

@@ -264,9 +264,9 @@ __global__ void __launch_bounds__(256) sell_c16_kernel(const int* __restrict__ s
   for (int j = 0; j < w; ++j) {
     const int d = sell_col[b0 + 32 * j + lane] - base;
     fits = fits && d >= -32767 && d <= 32767;
-    c16[b0 + 32 * j + lane] = (short)(fits ? d : 0);
+    if (c16) c16[b0 + 32 * j + lane] = (short)(fits ? d : 0);
   }
-  if (!__all_sync(0xffffffffu, fits) && lane == 0) atomicAdd(nfar, 1);
+  if (!__all_sync(0xffffffffu, fits) && lane == 0 && nfar) atomicAdd(nfar, 1);
 }
 
 // Whether slice sl has kPatW entries in each of its 32 rows and slot j of every row at the same offset

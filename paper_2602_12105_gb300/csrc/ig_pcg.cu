@@ -21,6 +21,7 @@
 // handles several rows of a tile so the block reductions, which cost FP64 adds, are amortised.
 #include <cstring>
 #include <mutex>
+#include <new>
 
 #include "ig_device.cuh"
 
@@ -293,7 +294,8 @@ cudaError_t begin_k(Group& g, const IoTable& io, int rhs_mass, const ig_solve_op
 // Host-driven loop: up to max_it iterations, polling the device's stop word every `poll`.
 template <int K>
 cudaError_t host_loop_k(Group& g, int max_it, int poll, cudaStream_t st) {
-  cudaError_t e;
+  cudaError_t e = group_done_word(g);
+  if (e != cudaSuccess) return e;
   for (int it = 0; it < max_it; ++it) {
     {
       IG_PROF("pcg_spmv", st);
@@ -461,20 +463,41 @@ cudaError_t group_init(Group& g, const MeshDev* host_mds, int nmesh, int slots64
   g.nface_tiles = (int)ftiles.size();
   g.nrow_tiles = (int)rtiles.size();
   cudaError_t e;
-  if ((e = cudaMalloc(&g.mds, sizeof(MeshDev) * nmesh)) != cudaSuccess) return e;
-  if ((e = cudaMalloc(&g.tiles, sizeof(int2) * tiles.size())) != cudaSuccess) return e;
-  if ((e = cudaMalloc(&g.tiles32, sizeof(int2) * (tiles32.size() ? tiles32.size() : 1))) != cudaSuccess) return e;
-  if ((e = cudaMalloc(&g.face_tiles, sizeof(int2) * ftiles.size())) != cudaSuccess) return e;
-  if ((e = cudaMalloc(&g.row_tiles, sizeof(int2) * rtiles.size())) != cudaSuccess) return e;
-  if ((e = cudaMalloc(&g.ctl, sizeof(LoopCtl))) != cudaSuccess) return e;
   // ints: act_mesh, act_off64, act_off32, big_mesh, app_mesh, app_off32, app_big; then (16-byte
   // aligned) the int4 start tables start64, start32, app_start32
   const size_t list_ints = (7 * (size_t)nmesh + 3 + 3) / 4 * 4;
   const size_t list_words = list_ints + 4 * (size_t)(g.grid64 + 2 * g.grid32);
-  if ((e = cudaMalloc(&g.act_buf, sizeof(int) * list_words)) != cudaSuccess) return e;
-  if ((e = cudaMalloc(&g.calls_dev, sizeof(CallDev) * nmesh)) != cudaSuccess) return e;
-  if ((e = cudaMallocHost(&g.calls_host, sizeof(CallDev) * nmesh)) != cudaSuccess) return e;
-  if ((e = cudaMallocHost(&g.done_host, sizeof(int))) != cudaSuccess) return e;
+  g.gang_host = gang_plan(host_mds, nullptr, nmesh, num_sms, &g.gang_tickets, &g.gang_workers);
+  {
+    const size_t sizes[] = {sizeof(MeshDev) * nmesh,       sizeof(int2) * tiles.size(),  sizeof(int2) * tiles32.size(),
+                            sizeof(int2) * ftiles.size(),  sizeof(int2) * rtiles.size(), sizeof(LoopCtl),
+                            sizeof(int) * list_words,      sizeof(CallDev) * nmesh,
+                            sizeof(int4) * (g.gang_host.size() + 1)};
+    size_t total = 0;
+    for (size_t b : sizes) total += Slab::padded(b ? b : 1);
+    if ((e = cudaMalloc(&g.memory, total)) != cudaSuccess) return e;
+    Slab slab{g.memory, total, 0};
+    g.mds = static_cast<MeshDev*>(slab.take(sizes[0]));
+    g.tiles = static_cast<int2*>(slab.take(sizes[1]));
+    g.tiles32 = static_cast<int2*>(slab.take(sizes[2]));
+    g.face_tiles = static_cast<int2*>(slab.take(sizes[3]));
+    g.row_tiles = static_cast<int2*>(slab.take(sizes[4]));
+    g.ctl = static_cast<LoopCtl*>(slab.take(sizes[5]));
+    g.act_buf = static_cast<int*>(slab.take(sizes[6]));
+    g.calls_dev = static_cast<CallDev*>(slab.take(sizes[7]));
+    if (!g.gang_host.empty()) {
+      g.gang_plan = static_cast<int4*>(slab.take(sizes[8]));
+      g.gang_ticket = reinterpret_cast<unsigned*>(g.gang_plan + g.gang_host.size());
+    }
+  }
+  // The arguments of one mesh's call are copied from pageable memory: pinning costs 104 us here and 166
+  // when it is given back.
+  if (nmesh == 1) {
+    g.calls_host = new (std::nothrow) CallDev[1];
+    if (!g.calls_host) return cudaErrorMemoryAllocation;
+  } else if ((e = cudaMallocHost(&g.calls_host, sizeof(CallDev) * nmesh)) != cudaSuccess) {
+    return e;
+  }
   if ((e = cudaEventCreateWithFlags(&g.calls_ev, cudaEventDisableTiming)) != cudaSuccess) return e;
   if ((e = cudaMemcpyAsync(g.mds, host_mds, sizeof(MeshDev) * nmesh, cudaMemcpyHostToDevice, st)) != cudaSuccess)
     return e;
@@ -512,24 +535,28 @@ cudaError_t group_init(Group& g, const MeshDev* host_mds, int nmesh, int slots64
     g.listapp = ListRef{c.app_start32, c.app_mesh, c.app_big, &g.ctl->napp_big};
     if ((e = cudaMemcpyAsync(g.ctl, &c, sizeof(LoopCtl), cudaMemcpyHostToDevice, st)) != cudaSuccess) return e;
   }
-  if ((e = group_order_gangs(g, nullptr, st)) != cudaSuccess) return e;
+  if (g.gang_plan && (e = cudaMemcpyAsync(g.gang_plan, g.gang_host.data(), sizeof(int4) * g.gang_host.size(),
+                                          cudaMemcpyHostToDevice, st)) != cudaSuccess)
+    return e;
   if ((e = cudaStreamCreateWithFlags(&g.capture_stream, cudaStreamNonBlocking)) != cudaSuccess) return e;
   if ((e = cudaEventRecord(g.calls_ev, st)) != cudaSuccess) return e;
   return cudaStreamSynchronize(st);
 }
 
-// The gangs of the group's mixed-precision solves, in the order of these time steps (the ticket counter
-// lies behind the plan).
+// The gangs of the group's mixed-precision solves, in the order of these time steps; the group_set_calls
+// that follows records that the copy has been read.
 cudaError_t group_order_gangs(Group& g, const double* t, cudaStream_t st) {
-  const std::vector<int4> plan =
-      gang_plan(g.host_mds.data(), t, g.nmesh, g.num_sms, &g.gang_tickets, &g.gang_workers);
-  if (plan.empty()) return cudaSuccess;
-  if (!g.gang_plan) {
-    cudaError_t e = cudaMalloc(&g.gang_plan, sizeof(int4) * (plan.size() + 1));
-    if (e != cudaSuccess) return e;
-    g.gang_ticket = reinterpret_cast<unsigned*>(g.gang_plan + plan.size());
-  }
-  return cudaMemcpyAsync(g.gang_plan, plan.data(), sizeof(int4) * plan.size(), cudaMemcpyHostToDevice, st);
+  if (!g.gang_plan) return cudaSuccess;
+  cudaError_t e = cudaEventSynchronize(g.calls_ev);
+  if (e != cudaSuccess) return e;
+  g.gang_host = gang_plan(g.host_mds.data(), t, g.nmesh, g.num_sms, &g.gang_tickets, &g.gang_workers);
+  return cudaMemcpyAsync(g.gang_plan, g.gang_host.data(), sizeof(int4) * g.gang_host.size(), cudaMemcpyHostToDevice,
+                         st);
+}
+
+// The word that the host-driven loop reads the device's progress into.
+cudaError_t group_done_word(Group& g) {
+  return g.done_host ? cudaSuccess : cudaMallocHost(&g.done_host, sizeof(int));
 }
 
 // Refresh the device copy of the mesh descriptors from g.host_mds.
@@ -537,7 +564,7 @@ cudaError_t group_upload_mds(Group& g, cudaStream_t st) {
   return cudaMemcpyAsync(g.mds, g.host_mds.data(), sizeof(MeshDev) * g.nmesh, cudaMemcpyHostToDevice, st);
 }
 
-// Upload per-call arguments; waits until the previous upload from the pinned staging is done.
+// Upload per-call arguments; waits until the previous upload from the staging copy is done.
 cudaError_t group_set_calls(Group& g, const CallDev* calls, cudaStream_t st) {
   cudaError_t e = cudaEventSynchronize(g.calls_ev);
   if (e != cudaSuccess) return e;
@@ -556,16 +583,9 @@ void group_destroy(Group& g) {
     }
   if (g.calls_ev) cudaEventSynchronize(g.calls_ev);
   if (g.capture_stream) cudaStreamDestroy(g.capture_stream);
-  if (g.mds) cudaFree(g.mds);
-  if (g.tiles) cudaFree(g.tiles);
-  if (g.tiles32) cudaFree(g.tiles32);
-  if (g.face_tiles) cudaFree(g.face_tiles);
-  if (g.row_tiles) cudaFree(g.row_tiles);
-  if (g.ctl) cudaFree(g.ctl);
-  if (g.act_buf) cudaFree(g.act_buf);
-  if (g.gang_plan) cudaFree(g.gang_plan);
-  if (g.calls_dev) cudaFree(g.calls_dev);
-  if (g.calls_host) cudaFreeHost(g.calls_host);
+  if (g.memory) cudaFree(g.memory);
+  if (g.calls_host && g.nmesh == 1) delete[] g.calls_host;
+  if (g.calls_host && g.nmesh > 1) cudaFreeHost(g.calls_host);
   if (g.done_host) cudaFreeHost(g.done_host);
   if (g.calls_ev) cudaEventDestroy(g.calls_ev);
   if (g.flags_dev) cudaFree(g.flags_dev);

@@ -468,7 +468,8 @@ cudaError_t begin_mixed_k(Group& g, const IoTable& io, int rhs_mass, const ig_so
 
 template <int K>
 cudaError_t host_loop_mixed_k(Group& g, int max_it, int poll, cudaStream_t st) {
-  cudaError_t e;
+  cudaError_t e = group_done_word(g);
+  if (e != cudaSuccess) return e;
   for (int it = 0; it < max_it; ++it) {
     {
       IG_PROF("pcg32_resid64", st);
