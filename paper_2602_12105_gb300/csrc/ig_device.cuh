@@ -3,6 +3,7 @@
 #pragma once
 
 #include "ig_f32.cuh"
+#include "ig_fixed.cuh"
 #include "ig_internal.cuh"
 
 namespace ig {
@@ -270,13 +271,15 @@ struct GatherAoS64 {
 };
 
 // ------------------------------------------------------------------------------- warp and tile sums
-// The orders of the FP64 sums over warps and tiles. The FP64 solver adds in trees (the resident solves
-// run these sums in every CTA, where each FP64 step counts). The mixed-precision solver's products and
-// updates do too, with the tiles in groups of four (a CTA of its resident solve takes four at a time).
+// The orders of the FP64 sums over warps and tiles. The FP64 solver's (kFixed) take the shortest chain,
+// since its resident solve runs them in every CTA: in fixed point (ig_fixed.cuh) over at most kFixedTiles
+// tiles, and within a tile for one or two values; else in trees. Sums outside the loops are trees. The
+// mixed-precision solver's products and updates are too, with the tiles in groups of four (a CTA of its
+// resident solve takes four at a time).
 // Its residual norms are added in warp and tile order: the scale of the inner right-hand sides comes
 // from them, and FP32 face geometry rounds what depends on that scale, so that one bit of it shows
 // in the gradient.
-enum SumOrder { kTree, kGroups, kInOrder };
+enum SumOrder { kTree, kGroups, kInOrder, kFixed };
 
 // Transposed warp sum. In a plain butterfly every lane adds every value at each of the five
 // levels; here, at the first levels, a lane keeps half of its values and sends the other half to
@@ -410,13 +413,48 @@ __device__ __forceinline__ void add_warps_to(const double* red, double* out) {
   if ((lane & 3) == 0 && v < NV) out[v] = a;
 }
 
+// kFixed: up to two values are added in fixed point within the tile too; for more the transposed tree is
+// shorter, whose additions serve several values at once (163,842 rows, k = 3: 26 us an iteration with
+// trees, 27.5 without; 5,917 rows, k = 1: 7.3 with trees, 6.2 without).
+template <int NV>
+constexpr bool kFixedWarps = NV <= 2;
+template <int NV>
+__device__ __forceinline__ void warp_totals_fixed(double (&v)[NV], double* red) {
+  if constexpr (kFixedWarps<NV>) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int i = 0; i < NV; ++i) {
+      const double one[1] = {v[i]};
+      const double a = warp_sum_fixed<1>(one);
+      if (lane == 0) red[i * kWarps + warp] = a;
+    }
+  } else {
+    warp_totals<NV>(v, red);
+  }
+}
+// The sum of value v's warp totals, on one warp (every lane).
+__device__ __forceinline__ double add_warps_fixed(const double* red, int v) {
+  const int lane = threadIdx.x & 31;
+  const double one[1] = {lane < kWarps ? red[v * kWarps + lane] : 0.0};
+  return warp_sum_fixed<1>(one);
+}
+
 // Sum the per-thread values v[0..NV) over the CTA into out[0..NV). A caller that sums consecutive
 // tiles alternates between two red buffers, so that one barrier per tile suffices (a warp can reach
 // the buffer again only after the next tile's barrier, which warp 0 passes after its reads).
 template <int NV, SumOrder ORDER, typename T>
 __device__ __forceinline__ void tile_reduce(T (&v)[NV], double* red, double* out) {
-  warp_totals<NV>(v, red);
+  if constexpr (ORDER == kFixed) warp_totals_fixed<NV>(v, red);
+  else warp_totals<NV>(v, red);
   __syncthreads();
+  if constexpr (ORDER == kFixed && kFixedWarps<NV>) {
+    const int warp = threadIdx.x >> 5;
+    if (warp < NV) {
+      const double a = add_warps_fixed(red, warp);
+      if ((threadIdx.x & 31) == 0) out[warp] = a;
+    }
+    return;
+  }
   if (threadIdx.x < NV) out[threadIdx.x] = add_warps_of<ORDER>(red + threadIdx.x * kWarps);
 }
 
@@ -479,6 +517,23 @@ __device__ __noinline__ void combine_partials(const double* __restrict__ part, i
   }
 }
 
+// kFixed, at most kFixedTiles tiles: a warp to a value, its loads all in flight.
+constexpr int kFixedTiles = 32 * ((kResMaxCtas + 31) / 32);
+template <int NV>
+__device__ __noinline__ void combine_fixed(const double* __restrict__ part, int ntiles, double* tot) {
+  constexpr int J = kFixedTiles / 32;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (warp < NV) {
+    double x[J];
+#pragma unroll
+    for (int j = 0; j < J; ++j)
+      x[j] = lane + 32 * j < ntiles ? __ldcg(part + (long)(lane + 32 * j) * kPartStride + warp) : 0.0;
+    const double a = warp_sum_fixed<J>(x);
+    if (lane == 0) tot[warp] = a;
+  }
+  __syncthreads();
+}
+
 // In tile order: thread j of the CTA adds tiles j, j + kBlock, ... into out[0..NV) (the CTA then adds
 // its threads' sums by warp and in warp order). Loads go in batches of four tiles; kept out of line:
 // only the last CTA of a reduction runs it.
@@ -503,6 +558,18 @@ __device__ __noinline__ void gather_in_order(const double* __restrict__ part, in
   }
 #pragma unroll
   for (int i = 0; i < NV; ++i) out[i] = v[i];
+}
+
+// (The tree for more tiles: all warps share the loads. 608 tiles took 1.8 us longer a sum in parts of
+// kFixedTiles by a warp to a value.)
+template <int NV, SumOrder ORDER>
+__device__ __forceinline__ void combine_tiles(const double* part, int ntiles, double* red, double* tot) {
+  if constexpr (ORDER == kFixed) {
+    if (ntiles <= kFixedTiles) combine_fixed<NV>(part, ntiles, tot);
+    else combine_partials<NV, kTree>(part, ntiles, red, tot);
+  } else {
+    combine_partials<NV, ORDER>(part, ntiles, red, tot);
+  }
 }
 
 // Sum v over the tile, publish the tile's partials, and return true in the last CTA of the mesh,
@@ -535,7 +602,7 @@ __device__ __forceinline__ bool reduce_tiles(double (&v)[NV], double* part, int 
     return true;
   }
   tile_reduce<NV, ORDER>(v, red, part + (long)tile * kPartStride);
-  if (threadIdx.x < 32) __threadfence();
+  if (threadIdx.x < 64) __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -545,7 +612,7 @@ __device__ __forceinline__ bool reduce_tiles(double (&v)[NV], double* part, int 
   __syncthreads();
   if (!s_last) return false;
   __threadfence();
-  combine_partials<NV, ORDER>(part, ntiles, red, tot);
+  combine_tiles<NV, ORDER>(part, ntiles, red, tot);
   __syncthreads();
 #pragma unroll
   for (int i = 0; i < NV; ++i) v[i] = tot[i];
@@ -624,7 +691,7 @@ __device__ __forceinline__ void flush_tiles(TileCtx& tc, int tiling, unsigned ru
                                             const Finish& finish) {
   const int ntiles = tile_count(tc.md, tiling);
   unsigned int* cnt = &tc.md.s->cnt[cnt_idx];
-  if (threadIdx.x < 32) __threadfence();  // the tile sums this warp wrote, before the count
+  if (threadIdx.x < 64) __threadfence();  // the tile sums this warp wrote, before the count
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
@@ -642,7 +709,7 @@ __device__ __forceinline__ void flush_tiles(TileCtx& tc, int tiling, unsigned ru
           __ldcg(reinterpret_cast<const unsigned*>(tc.md.s) + threadIdx.x);
     // (the barriers in here also publish cur)
     if constexpr (ORDER != kInOrder) {
-      combine_partials<NV, ORDER>(tc.md.part, ntiles, tc.red[0], tc.tot);
+      combine_tiles<NV, ORDER>(tc.md.part, ntiles, tc.red[0], tc.tot);
     } else {
       double v[NV];
       gather_in_order<NV>(tc.md.part, ntiles, v);

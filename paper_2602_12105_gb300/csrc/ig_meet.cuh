@@ -38,16 +38,17 @@ __device__ __forceinline__ bool peek(const Slot* s, unsigned long long number, d
   value = __longlong_as_double((long long)a);
   return b == number;
 }
-// The sum of one value over `count` posted partials, on the kWarps warps of a CTA (PartialMap: a lane
-// takes a few of them, all polled together): buf[8 * i + value]. late is set when a wait ran out.
+// `count` posted partials buf[8 * i + value], on the kWarps warps of a CTA (PartialMap: a lane takes a few
+// tiles of one value, all polled together, 0 past the last). late is set when a wait ran out.
+template <int NV>
+constexpr int kLaneTiles = (kResMaxCtas + PartialMap<NV>::kStride - 1) / PartialMap<NV>::kStride;
 template <int NV, bool ACQUIRE>
-__device__ __forceinline__ double collect_sum(const Slot* buf, int count, unsigned long long number, long long patience,
-                                              bool& late) {
+__device__ __forceinline__ void collect(const Slot* buf, int count, unsigned long long number, long long patience,
+                                        double (&b)[kLaneTiles<NV>], bool& late) {
   using Map = PartialMap<NV>;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, val = Map::value(lane);
   const int first = Map::first(warp, lane);
-  constexpr int J = (kResMaxCtas + Map::kStride - 1) / Map::kStride;
-  double b[J];
+  constexpr int J = kLaneTiles<NV>;
   unsigned want = 0;
 #pragma unroll
   for (int j = 0; j < J; ++j) {
@@ -70,7 +71,15 @@ __device__ __forceinline__ double collect_sum(const Slot* buf, int count, unsign
         want &= ~(1u << j);
       }
   }
-  const int steps = (count + Map::kStride - 1) / Map::kStride;
+}
+// The lane's sum of them.
+template <int NV, bool ACQUIRE>
+__device__ __forceinline__ double collect_sum(const Slot* buf, int count, unsigned long long number, long long patience,
+                                              bool& late) {
+  constexpr int J = kLaneTiles<NV>;
+  double b[J];
+  collect<NV, ACQUIRE>(buf, count, number, patience, b, late);
+  const int steps = (count + PartialMap<NV>::kStride - 1) / PartialMap<NV>::kStride;
   double a = 0.0;
 #pragma unroll
   for (int j = 0; j < J; ++j)

@@ -68,7 +68,7 @@ __global__ void __launch_bounds__(kBlock) init_kernel(const MeshDev* __restrict_
       acc[K + c] = fma(b, b, acc[K + c]);
     }
   }
-  if (reduce_tiles<2 * K, kTree>(acc, md.part, tl.y, md.ntiles, &md.s->cnt[2]) && threadIdx.x == 0)
+  if (reduce_tiles<2 * K, kFixed>(acc, md.part, tl.y, md.ntiles, &md.s->cnt[2]) && threadIdx.x == 0)
     finish_init(md.s, K, acc, tol, max_iter);
 }
 
@@ -110,7 +110,7 @@ __device__ __forceinline__ void spmv_tile(const MeshDev& md, int tile, const Sca
     }
     store_row<K>(p, row, pi);
   }
-  tile_reduce<K, kTree>(pq, red, out);
+  tile_reduce<K, kFixed>(pq, red, out);
 }
 
 template <int K>
@@ -118,7 +118,7 @@ __global__ void __launch_bounds__(kBlock, 4) spmv_kernel(const MeshDev* __restri
   __shared__ TileCtx tc;
   __shared__ int s_stop;  // the loop has stopped: a launch after that (second half of a graph pass) does nothing
   if (threadIdx.x == 0) s_stop = __ldcg(&ctl->all_done);
-  tile_loop<K, kTree>(
+  tile_loop<K, kFixed>(
       mds, L, 0, 0, tc, [&](const ScalSnap& x) { return !x.done && !s_stop; },
       [&](const MeshDev& md, int tile, double* red, double* out) { spmv_tile<K>(md, tile, tc.sn, red, out); },
       [](const MeshDev& md, const SolveScal& cur, const double* v) { finish_spmv(md.s, cur, K, v); });
@@ -167,7 +167,7 @@ __device__ __forceinline__ void update_tile(const MeshDev& md, int tile, const S
     }
     store_row<K>(zv, row, zo);
   }
-  tile_reduce<2 * K, kTree>(acc, red, out);
+  tile_reduce<2 * K, kFixed>(acc, red, out);
 }
 
 template <int K>
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(kBlock, 4) update_kernel(const MeshDev* __rest
   }
   if (threadIdx.x == 0) tc.last = 0;
   __syncthreads();
-  tile_loop<2 * K, kTree>(
+  tile_loop<2 * K, kFixed>(
       mds, L, 0, 1, tc, [&](const ScalSnap& x) { return !x.done && !s_stop; },
       [&](const MeshDev& md, int tile, double* red, double* out) { update_tile<K>(md, tile, tc.sn, red, out); },
       [&](const MeshDev& md, const SolveScal& cur, const double* v) {

@@ -10,7 +10,7 @@
 // so no step waits for one last CTA, and no kernel boundary or graph node lies in the loop.
 //
 // Measured, per iteration (the two-kernel graph loop before, and this): 163,842 rows k = 3 41 -> 26 us
-// and k = 4 47 -> 31 us, 66,049 rows k = 1 23 -> 8.5 us, 5,917 rows k = 1 20.6 -> 8.5 us, 642 rows k = 3
+// and k = 4 47 -> 31 us, 66,049 rows k = 1 23 -> 7.4 us, 5,917 rows k = 1 20.6 -> 6.3 us, 642 rows k = 3
 // (a cluster of 6 CTAs; three CTAs of 256 rows before) 10 -> 6 us.
 //
 // What bounds it: on large meshes FP64 instructions and the gathers of z together. A warp's FP64
@@ -18,8 +18,8 @@
 // (three columns) take 11.7 us on 163,842 rows; eight row warps are enough to issue them, and fewer
 // threads leave fewer sums to add (the sums of 32 warps would take 2.2 us of FP64 issue in the
 // update alone, those of 8 a quarter). On small meshes the chain of an iteration: two gathers, two
-// meetings of about 1 us (a store to L2, then a load that sees it), and sums and divisions whose every
-// FP64 step costs 64 cycles.
+// meetings of about 1 us (a store to L2, then a load that sees it), and sums (in fixed point where that is
+// shorter) and divisions whose every FP64 step costs 64 cycles.
 #include "ig_meet.cuh"
 
 namespace ig {
@@ -50,7 +50,6 @@ struct ResShared {
   MeshDev md;
   SolveScal st;
   double red[8 * kWarps];
-  double red2[8 * kWarps];
   double tot[8];
   double box[2][8];          // cluster: this CTA's posted sums, by parity of the meeting
   int width[kResMaxRows / 32];
@@ -60,62 +59,79 @@ constexpr int kResThreads = kBlock + 32;  // eight warps take the rows; the nint
 
 // Where the CTAs meet. CLUSTER: all of them form one thread-block cluster (at most 16 CTAs).
 //
-// A meeting adds per-thread sums over all tiles, in three steps between CTA barriers: the row warps
-// leave their warps' totals in red; the ninth warp adds them and posts the tile's sums; the row warps
-// collect every tile's sums, a few per lane, into red2. The caller's ninth warp then adds red2.
+// A meeting adds per-thread sums over all tiles, a warp to a value, in fixed point: the row warps
+// leave their totals in red; after a barrier the tile's sums are added and posted; the row warps collect every
+// tile's; after another barrier warp v adds those of value v into tot[v].
 template <bool CLUSTER>
 struct Meeting {
   Slot* slots;
+  double* gathered;  // [value][tile]
   int nct;
   unsigned long long number;
 
-  // ninth warp: the tile's sums, posted. RELEASE: what the CTA wrote to global memory before is
-  // visible to the CTAs that collect them. (The product's meeting needs no order beyond its data:
-  // its sums depend on every z the CTA gathered, and the z written next depends on the sums.)
+  // One meeting up to the barrier after which tot is complete; true when a wait ran out. RELEASE: what a
+  // CTA wrote to global memory before is visible to all CTAs after it. (The product's meeting needs no order
+  // beyond its data: its sums depend on every z the CTA gathered, and the z written next depends on
+  // the sums.)
   template <int NV, bool RELEASE>
-  __device__ __forceinline__ void post_sums(ResShared& sh) {
-    const int lane = threadIdx.x & 31;
-    const double a = add_warps<NV>(sh.red);
-    const bool writer = (lane & 3) == 0 && (lane >> 2) < NV;
-    if constexpr (CLUSTER) {
-      if (writer) sh.box[number & 1][lane >> 2] = a;
-    } else {
-      if (RELEASE) fence_gpu();
-      if (writer) post(slots + (number & 1) * (8 * (size_t)nct) + 8 * (size_t)blockIdx.x + (lane >> 2), a, number);
-    }
-  }
-
-  // row warps: every tile's sums into red2 (ACQUIRE: with what their CTAs released). Returns true
-  // when a wait ran out.
-  template <int NV, bool ACQUIRE>
-  __device__ __forceinline__ bool collect(ResShared& sh) {
-    using Map = PartialMap<NV>;
-    double a = 0.0;
-    bool late = false;
-    if constexpr (CLUSTER) {
-      const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, val = Map::value(lane);
-      for (int t = Map::first(warp, lane); t < nct; t += Map::kStride)
-        if (val < NV) a += peer_load(&sh.box[number & 1][val], t);
-    } else {
-      a = collect_sum<NV, ACQUIRE>(slots + (number & 1) * (8 * (size_t)nct), nct, number, kSpinLimit, late);
-    }
-    Map::to_warp_total(a, sh.red2);
-    return late;
-  }
-
-  // One meeting up to the barrier after which red2 is complete; true when a wait ran out.
-  template <int NV, bool RELEASE>
-  __device__ __forceinline__ bool meet(ResShared& sh, double (&v)[NV], bool row_warp, bool has_rows) {
+  __device__ __forceinline__ bool meet(ResShared& sh, double (&v)[NV], bool row_warp) {
     ++number;
-    if (row_warp) {
-      if (has_rows) warp_totals<NV>(v, sh.red);
-      else if ((threadIdx.x & 31) < NV) sh.red[(threadIdx.x & 31) * kWarps + (threadIdx.x >> 5)] = 0.0;
-    }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (row_warp) warp_totals_fixed<NV>(v, sh.red);
     __syncthreads();
-    if (!row_warp) post_sums<NV, RELEASE>(sh);
-    if constexpr (CLUSTER) cluster_sync_all();
     bool late = false;
-    if (row_warp) late = collect<NV, RELEASE>(sh);
+    const int parity = (int)(number & 1);
+    Slot* const box = slots + (size_t)parity * 8 * (size_t)nct;
+    double a = 0.0;
+    int value = NV;  // the lane's value to post
+    if constexpr (kFixedWarps<NV>) {
+      if (warp < NV) {
+        a = add_warps_fixed(sh.red, warp);
+        if (lane == 0) value = warp;
+      }
+    } else if (!row_warp) {
+      a = add_warps<NV>(sh.red);
+      if ((lane & 3) == 0) value = lane >> 2;
+    }
+    if constexpr (CLUSTER) {
+      if (value < NV) sh.box[parity][value] = a;
+    } else {
+      if (RELEASE && (kFixedWarps<NV> ? warp < NV : !row_warp)) fence_gpu();
+      if (value < NV) post(box + 8 * (size_t)blockIdx.x + value, a, number);
+    }
+    constexpr int S = kFixedTiles;
+    if constexpr (CLUSTER) {
+      cluster_sync_all();
+    } else {
+      // eight lanes take a tile's values, which share a 128-byte line: a warp to a value would ask for
+      // 32 lines with each load (26 -> 28 us an iteration on 163,842 rows)
+      if (row_warp) {
+        using Map = PartialMap<NV>;
+        double b[kLaneTiles<NV>];
+        collect<NV, RELEASE>(box, nct, number, kSpinLimit, b, late);
+        const int val = Map::value(lane), first = Map::first(warp, lane);
+        if (val < NV) {
+#pragma unroll
+          for (int j = 0; j < kLaneTiles<NV>; ++j)
+            if (first + j * Map::kStride < S) gathered[val * S + first + j * Map::kStride] = b[j];
+        }
+      }
+      __syncthreads();
+    }
+    if (warp < NV) {
+      constexpr int J = CLUSTER ? 1 : S / 32;
+      double x[J];
+#pragma unroll
+      for (int j = 0; j < J; ++j) x[j] = 0.0;
+      if constexpr (CLUSTER) {
+        if (lane < nct) x[0] = peer_load(&sh.box[parity][warp], lane);
+      } else {
+#pragma unroll
+        for (int j = 0; j < J; ++j) x[j] = gathered[warp * S + 32 * j + lane];
+      }
+      const double b = warp_sum_fixed<J>(x);
+      if (lane == 0) sh.tot[warp] = b;
+    }
     return __syncthreads_or(late) != 0;
   }
 };
@@ -190,7 +206,6 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
   const long t0 = (long)blockIdx.x * md.tile_rows;
   // the ninth warp has no rows
   const int rows = !row_warp ? 0 : (int)(nn - t0 < md.tile_rows ? nn - t0 : md.tile_rows);
-  const bool has_rows = (tid & ~31) < rows;  // this warp has a row
   const int rp = lay.rp, aw = lay.aw;
   double* q = reinterpret_cast<double*>(dyn);
   double* p = q + K * rp;
@@ -198,7 +213,8 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
   double* dinv = r + K * rp;
   double* sa = dinv + rp;
   double* xs = sa + (size_t)aw * rp;
-  int* sc = reinterpret_cast<int*>(xs + (lay.x_on ? K * rp : 0));
+  double* sums = xs + (lay.x_on ? K * rp : 0);
+  int* sc = reinterpret_cast<int*>(sums + 2 * K * kFixedTiles);
   double* x = lay.x_on ? xs : md.x + t0;   // component c of row i at x[c * xn + i]
   const long xn = lay.x_on ? rp : nn;
   double* z = md.z;
@@ -219,6 +235,7 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
 
   Meeting<CLUSTER> mt;
   mt.slots = reinterpret_cast<Slot*>(md.meet) + 1;
+  mt.gathered = sums;
   mt.nct = gridDim.x;
   // numbers of this launch: above those of every launch before it (the word ahead of the slots
   // counts launches; CTA 0 advances it at the end, when every CTA has long read it)
@@ -250,12 +267,8 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
       }
       store_row<K>(z, row, zo);
     }
-    late = mt.template meet<2 * K, true>(sh, acc, row_warp, has_rows);
-    if (!row_warp) {
-      add_warps_to<2 * K>(sh.red2, sh.tot);
-      __syncwarp();
-      if (tid == kBlock) finish_init(&sh.st, K, sh.tot, tol, max_iter);
-    }
+    late = mt.template meet<2 * K, true>(sh, acc, row_warp);
+    if (tid == kBlock) finish_init(&sh.st, K, sh.tot, tol, max_iter);
   }
 
   for (int it = 0; it < cap && !late; ++it) {
@@ -317,13 +330,9 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
       }
       if (waiting) __syncthreads();
       if (sh.st.done) break;
-      late = mt.template meet<K, false>(sh, pq, row_warp, has_rows);
+      late = mt.template meet<K, false>(sh, pq, row_warp);
       if (late) break;
-      if (!row_warp) {
-        add_warps_to<K>(sh.red2, sh.tot);
-        __syncwarp();
-        finish_spmv_step(&sh.st, sh.st, K, sh.tot);
-      }
+      if (!row_warp) finish_spmv_step(&sh.st, sh.st, K, sh.tot);
       __syncthreads();
     }
     // x += alpha p, r -= alpha q, z = D^-1 r, r.z and r.r
@@ -352,13 +361,9 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
           acc[K + c] = fma(rn[c], rn[c], acc[K + c]);
         }
       }
-      late = mt.template meet<2 * K, true>(sh, acc, row_warp, has_rows);
+      late = mt.template meet<2 * K, true>(sh, acc, row_warp);
       if (late) break;
-      if (!row_warp) {
-        add_warps_to<2 * K>(sh.red2, sh.tot);
-        __syncwarp();
-        finish_update_step(&sh.st, sh.st, K, sh.tot);
-      }
+      if (!row_warp) finish_update_step(&sh.st, sh.st, K, sh.tot);
     }
   }
   for (int i = tid; i < rows; i += kBlock) {
@@ -383,7 +388,7 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
 template <int K>
 ResLayout layout(int rp, int wmax) {
   const int room = 227 * 1024 - (int)sizeof(ResShared) - 256;
-  const int fixed = rp * 8 * (3 * K + 1);
+  const int fixed = rp * 8 * (3 * K + 1) + 2 * K * kFixedTiles * 8;
   ResLayout l{};
   l.rp = rp;
   l.x_on = fixed + rp * 8 * K + 12 * rp * wmax <= room;
