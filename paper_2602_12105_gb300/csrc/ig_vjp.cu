@@ -7,19 +7,18 @@
 //   E_f = w_a * area_f + sum_c omega_c * cot_c,
 //   w_a     = (1/3) sum_{v in f} <Lambda_v, B_v - U_v>,
 //   omega_c = -(t/2) <Lambda_a - Lambda_b, U_a - U_b>   ((a, b) the edge opposite corner c),
-// with the coefficients held fixed. Writing d_c for the edge opposite corner c (d_0 = p2 - p1,
-// d_1 = p0 - p2, d_2 = p1 - p0), N = d_1 x d_2, s = |N|, dot_c = d_{c+1}.d_{c+2} (so
-// cot_c = -dot_c / s) and P = -sum_c omega_c dot_c, E_f = P / s + w_a s / 2 and
-//   grad_{p_c} E_f = [ -omega_c (d_{c+2} - d_{c+1}) + (omega_{c+1} - omega_{c+2}) d_c ] / s
-//                    + (w_a / 2 - P / s^2) (N x d_c) / s.
-// N x d_c = dot_{c+2} d_{c+2} - dot_{c+1} d_{c+1}, and d_c = -d_{c+1} - d_{c+2}, so with
-// W_c = omega_c / s and k_c = (w_a / 2 - P / s^2) dot_c / s each corner's gradient is a combination of
-// two edges,
-//   grad_{p_c} E_f = (W_c + e_c - k_{c+1}) d_{c+1} + (e_c - W_c + k_{c+2}) d_{c+2},
-//   e_c = W_{c+2} - W_{c+1},
-// and the third is minus the sum of the other two (E_f does not change when the face moves). The
-// FP64 kernel is bound by FP64 instructions (2 per clock per SM): this form takes about 104 per face
-// (k = 3) where the cross products corner by corner took about 140.
+// with the coefficients held fixed. With the edges u = p0 - p2 and v = p1 - p0 (opposite corners 1 and 2)
+// and s = |u x v|, the cotangents at corners 0, 1, 2 are -u.v / s, (u.v + v.v) / s and (u.u + u.v) / s, so
+//   E_f = P / s + w_a s / 2,   P = omega_2 u.u + (omega_1 + omega_2 - omega_0) u.v + omega_1 v.v.
+// With Lambda and U differenced along u and v (x_u, x_v, y_u, y_v), omega_1 and omega_2 are -t/2 times
+// x_u.y_u and x_v.y_v, and the middle coefficient t/2 (x_u.y_v + x_v.y_u): the third edge's product
+// is not needed. s^2 = u.u v.v - (u.v)^2, so with k = (P / s^2 - w_a / 2) / s
+//   dE/du = A u + X v,  dE/dv = X u + C v,
+//   A = 2 omega_2 / s - k v.v,  C = 2 omega_1 / s - k u.u,
+//   X = (omega_1 + omega_2 - omega_0) / s + k u.v,
+// and the corners get dE/du - dE/dv, dE/dv and -dE/du. The FP64 kernel is bound by FP64 instructions (2 per
+// clock per SM): this form takes about 90 per face (k = 3; 2,095,106 faces 346 us), combinations of
+// two edges corner by corner took 103 (424 us), cross products corner by corner about 140 (578 us).
 // (The CPU oracle reaches the same numbers through the per-corner cotangent gradients.)
 //
 // A loss may also depend on V through the mass directly (the M-norm loss of the inverse-fairing
@@ -78,74 +77,96 @@ __global__ void __launch_bounds__(256) vjp_face_kernel(const MeshDev* __restrict
 #pragma unroll
       for (int d = 0; d < 3; ++d) P[c][d] = __ldg(V + 3 * (long)vid[c] + d);
     }
-    double dd[3][3];
+    double u[3], v[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      dd[0][d] = P[2][d] - P[1][d];
-      dd[1][d] = P[0][d] - P[2][d];
-      dd[2][d] = P[1][d] - P[0][d];
+      u[d] = P[0][d] - P[2][d];
+      v[d] = P[1][d] - P[0][d];
     }
     double N[3];
-    N[0] = dd[1][1] * dd[2][2] - dd[1][2] * dd[2][1];
-    N[1] = dd[1][2] * dd[2][0] - dd[1][0] * dd[2][2];
-    N[2] = dd[1][0] * dd[2][1] - dd[1][1] * dd[2][0];
+    N[0] = u[1] * v[2] - u[2] * v[1];
+    N[1] = u[2] * v[0] - u[0] * v[2];
+    N[2] = u[0] * v[1] - u[1] * v[0];
     const double s2 = N[0] * N[0] + N[1] * N[1] + N[2] * N[2];
     const double inv_s = rsqrt(s2);
-    double dot[3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const int a = (c + 1) % 3, b = (c + 2) % 3;
-      dot[c] = dd[a][0] * dd[b][0] + dd[a][1] * dd[b][1] + dd[a][2] * dd[b][2];
-    }
-    // per-vertex <Lambda_v, B_v - U_v> and the per-corner <dLambda, dU>; with mass weights w,
-    // d(sum_i M_i w_i)/dV adds sum_f ((1/3) sum_{v in f} w_v) grad area_f, i.e. w_v to the sum
+    const double uu = u[0] * u[0] + u[1] * u[1] + u[2] * u[2];
+    const double uv = u[0] * v[0] + u[1] * v[1] + u[2] * v[2];
+    const double vv = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+    // per-vertex <Lambda_v, B_v - U_v> and the products of the differences along u and v; with mass
+    // weights w, d(sum_i M_i w_i)/dV adds sum_f ((1/3) sum_{v in f} w_v) grad area_f, i.e. w_v to the sum
     double wa = 0.0;
-    double W[3] = {0.0, 0.0, 0.0};  // omega_c / s
+    double A = 0.0, X = 0.0, C = 0.0, S = 0.0;  // the solve terms' parts; S = P / s
     if constexpr (MODE != 2) {
       // <Lambda_v, B_v - U_v> of the three vertices, formed once per vertex by vjp_vertex_kernel
       wa = (__ldg(wvert + vid[0]) + __ldg(wvert + vid[1])) + __ldg(wvert + vid[2]);
-      double L[3][K], Uv[3][K];
+      double xu[K], xv[K], yu[K], yv[K];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-          L[c][k] = lam[(long)vid[c] * K + k];
-          Uv[c][k] = U[(long)vid[c] * K + k];
-        }
+      for (int k = 0; k < K; ++k) {
+        const double l0 = lam[(long)vid[0] * K + k], u0 = U[(long)vid[0] * K + k];
+        xu[k] = l0 - lam[(long)vid[2] * K + k];
+        xv[k] = lam[(long)vid[1] * K + k] - l0;
+        yu[k] = u0 - U[(long)vid[2] * K + k];
+        yv[k] = U[(long)vid[1] * K + k] - u0;
       }
-      const double mt2 = -0.5 * tval * inv_s;
+      double lu = xu[0] * yu[0], lv = xv[0] * yv[0], lx = xu[0] * yv[0];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const int a = (c + 1) % 3, b = (c + 2) % 3;
-        double lu = (L[a][0] - L[b][0]) * (Uv[a][0] - Uv[b][0]);
+      for (int k = 1; k < K; ++k) {
+        lu = fma(xu[k], yu[k], lu);
+        lv = fma(xv[k], yv[k], lv);
+        lx = fma(xu[k], yv[k], lx);
+      }
 #pragma unroll
-        for (int k = 1; k < K; ++k) lu = fma(L[a][k] - L[b][k], Uv[a][k] - Uv[b][k], lu);
-        // dl/dt = -<Lambda, L U> = -sum_c (cot_c / 2) lu_c = sum_c (dot_c / s / 2) lu_c
-        if (CLAMP && clamp_on && -dot[c] * inv_s < clamp_min) {
-          // a clamped corner holds cot = clamp_min: no term in dl/dV, clamp_min in dl/dt
-          W[c] = 0.0;
+      for (int k = 0; k < K; ++k) lx = fma(xv[k], yu[k], lx);
+      if (CLAMP && clamp_on) {
+        // a clamped corner holds cot = clamp_min: no term in dl/dV, clamp_min in dl/dt. The corners'
+        // products are formed from their own two edges: at a right angle (a flat grid) the rounding of
+        // u.v + v.v could fall on the other side of a clamp at 0 than the assembly's.
+        double w[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) w[d] = P[2][d] - P[1][d];
+        const double dot1 = v[0] * w[0] + v[1] * w[1] + v[2] * w[2];
+        const double dot2 = w[0] * u[0] + w[1] * u[1] + w[2] * u[2];
+        double l0 = (lu + lv) + lx;
+        bool clamped = false;
+        if (-uv * inv_s < clamp_min) {
+          if (gt) gt_part = fma(-0.5 * clamp_min, l0, gt_part);
+          l0 = 0.0;
+          clamped = true;
+        }
+        if (-dot1 * inv_s < clamp_min) {
           if (gt) gt_part = fma(-0.5 * clamp_min, lu, gt_part);
-        } else {
-          W[c] = mt2 * lu;
-          if (gt) gt_part = fma(0.5 * dot[c] * inv_s, lu, gt_part);
+          lu = 0.0;
+          clamped = true;
         }
+        if (-dot2 * inv_s < clamp_min) {
+          if (gt) gt_part = fma(-0.5 * clamp_min, lv, gt_part);
+          lv = 0.0;
+          clamped = true;
+        }
+        if (clamped) lx = (l0 - lu) - lv;
       }
+      // dl/dt = -<Lambda, L U> = -sum_c (cot_c / 2) lu_c
+      const double Q = fma(lv, uu, fma(lu, vv, -(lx * uv)));
+      if (gt) gt_part = fma(-0.5 * inv_s, Q, gt_part);
+      const double mt = -tval * inv_s, h = 0.5 * mt;
+      S = h * Q;
+      A = mt * lv;
+      C = mt * lu;
+      X = -(h * lx);
     }
     if constexpr (MODE != 0) wa += (__ldg(cl.wm + vid[0]) + __ldg(cl.wm + vid[1])) + __ldg(cl.wm + vid[2]);
-    wa *= (1.0 / 6.0);  // w_a / 2
-    const double S = fma(W[0], dot[0], fma(W[1], dot[1], W[2] * dot[2]));
-    const double coef = inv_s * fma(inv_s, S, wa);
+    const double kk = inv_s * fma(inv_s, S, wa * (-1.0 / 6.0));
+    A = fma(-kk, vv, A);
+    C = fma(-kk, uu, C);
+    X = fma(kk, uv, X);
     double g[9];
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const int a = (c + 1) % 3, b = (c + 2) % 3;
-      const double e = W[b] - W[a];
-      const double ca = fma(-coef, dot[a], W[c] + e), cb = fma(coef, dot[b], e - W[c]);
-#pragma unroll
-      for (int d = 0; d < 3; ++d) g[3 * c + d] = fma(ca, dd[a][d], cb * dd[b][d]);
+    for (int d = 0; d < 3; ++d) {
+      const double gu = fma(A, u[d], X * v[d]), gv = fma(X, u[d], C * v[d]);
+      g[d] = gu - gv;
+      g[3 + d] = gv;
+      g[6 + d] = -gu;
     }
-#pragma unroll
-    for (int d = 0; d < 3; ++d) g[6 + d] = -(g[d] + g[3 + d]);
     double* out = md.gface + 9 * (long)f;
 #pragma unroll
     for (int i = 0; i < 9; ++i) out[i] = g[i];
