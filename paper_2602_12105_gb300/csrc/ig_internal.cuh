@@ -465,6 +465,14 @@ cudaError_t launch_operator32_csr(const MeshDev& md, float* Acsr, cudaStream_t s
 
 // ig_pcg.cu: see Group above
 
+// The launches in one are not recorded in a caller's capture (nor is one that cannot tell).
+inline bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;
+  cudaGetLastError();
+  return true;
+}
+
 // ig_resident.cu: a whole FP64 solve of a group of one mesh in one launch; false, with nothing
 // launched, when the mesh does not qualify or the device refuses the launch
 bool launch_resident(Group& g, int k, const double* in, double* out, int rhs_mass, const ig_solve_opts& o,

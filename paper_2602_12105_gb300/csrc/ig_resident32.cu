@@ -492,7 +492,7 @@ std::vector<int4> gang_plan(const MeshDev* mds, const double* t, int nmesh, int 
 }
 
 bool launch_gang(Group& g, int k, int cap, cudaStream_t st) {
-  if (!g.gang_plan) return false;
+  if (!g.gang_plan || capturing(st)) return false;
   switch (k) {
     case 1: return launch<1>(g, cap, st);
     case 2: return launch<2>(g, cap, st);
