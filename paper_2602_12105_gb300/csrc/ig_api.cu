@@ -564,11 +564,14 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
   // below which an iteration gets no shorter (2,025 rows, k = 3: 6.8 us an iteration in tiles of 128,
   // 7.8 in tiles of 64, 7.9 in tiles of 256). Above kResSmall rows the tiles have 256 rows at least,
   // for the sake of the batches, whose CTAs take 256 rows at a time (5,917 rows, k = 3: 9.0 us in
-  // tiles of 256 against 8.2 in tiles of 128).
+  // tiles of 256 against 8.2 in tiles of 128). For the same reason a tile of more than one such pass has
+  // two whole ones: 40,962 rows alone take 13.8 us an iteration in tiles of 288 and 14.4 in tiles of 512,
+  // a batch of 256 meshes 62.3 and 54.2 ms (58.3 in tiles of 256, too many for one to an SM).
   const bool resident = ctx->num_sms >= 1 && ctx->num_sms <= kResMaxCtas && ni <= (long)ctx->num_sms * kResMaxRows;
   if (resident) {
     const int rows = (ni + ctx->num_sms - 1) / ctx->num_sms;
     md.tile_rows = ni <= kResSmall ? 128 : (std::max(rows, kResMinRows) + 31) / 32 * 32;
+    if (md.tile_rows > kBlock && md.tile_rows < 2 * kBlock) md.tile_rows = 2 * kBlock;
     md.ntiles = (ni + md.tile_rows - 1) / md.tile_rows;
   } else {
     choose_tiles64(ctx->solver_slots, md.tile_rows, md.ntiles);

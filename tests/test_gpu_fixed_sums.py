@@ -25,8 +25,9 @@ def _t(a, dtype=torch.float64):
     (19, 7, 1),       # two tiles
     (64, 32, 4),      # a cluster of 16 tiles, eight sums
     (241, 17, 2),     # 17 tiles through global memory: one more than half a warp's addends
-    (257, 160, 1),    # 147 tiles: five addends to most lanes
-    (257, 160, 3),
+    (256, 152, 1),    # 152 tiles: five addends to most lanes
+    (256, 152, 3),
+    (257, 160, 3),    # 81 tiles of two passes
     (450, 420, 1),    # larger than a resident solve: a tree over the tiles
 ])
 def test_scales(api, nx, ny, k, launch):
