@@ -175,9 +175,9 @@ def algorithmic(kernel, n, m, nnz, k, prec, idx32=4):
     kp). FP64 path (pcg_*): two kernels per iteration. The SpMV gathers z = D^-1 r, forms
     p = z + beta p and q = A z + beta q (the recurrence q = A p) and the sum p.q; the update writes
     x, r and z. Mixed path (pcg32_*): 4-byte values and vectors, three kernels per iteration (SpMV
-    q = A p, update, p-update reading D^-1 and r), and the SpMV reads idx32-byte column indices
-    (2 where every slice of 32 rows keeps its columns as 16-bit offsets, as on the grid
-    workloads)."""
+    q = A p; update of r; p-update reading D^-1 and r, which also adds alpha p to x), and the SpMV
+    reads idx32-byte column indices (none where the slices of 32 rows share one column pattern, as
+    on the grid workloads)."""
     kp = 4 if k == 3 else k
     if kernel.startswith("pcg32_"):
         sv, si = 4, idx32
@@ -186,9 +186,9 @@ def algorithmic(kernel, n, m, nnz, k, prec, idx32=4):
             return (float(2 * k * nnz + 2 * k * n),
                     float(nnz * (sv + si) + 4 * (n + 1) + sv * kp * n + sv * k * n))
         if kernel == "update":
-            return float(11 * k * n), float(sv * (n + 3 * k * n + kp * n) + 2 * sv * k * n)
+            return float(7 * k * n), float(sv * (n + 2 * k * n) + sv * k * n)
         if kernel == "pupdate":
-            return float(3 * k * n), float(sv * (n + k * n + kp * n) + sv * kp * n)
+            return float(5 * k * n), float(sv * (n + 2 * k * n + kp * n) + sv * (k * n + kp * n))
         return None, None
     sv = 8
     if kernel == "pcg_spmv":
@@ -212,7 +212,7 @@ def algorithmic(kernel, n, m, nnz, k, prec, idx32=4):
     elif kernel == "vjp_face":
         # faces, V, U and Lambda at the vertices (each once from DRAM), the per-vertex weights;
         # the per-corner gradients written
-        flops = 300 * m
+        flops = 140 * m
         byts = 12 * m + 24 * n + 2 * 8 * k * n + 8 * n + 72 * m
     elif kernel == "vjp_gather":
         # incidence offsets and entries, the per-corner gradients (24 B each), M; gV written
@@ -381,9 +381,9 @@ def run_ours(args, rank, world, local_rank):
     alu = measure_alu_peaks(_native, local_rank, stream.cuda_stream)
     its_f, its_a = finfo["iterations"], ainfo["iterations"]
     rl_all, roofline = kernel_roofline(prof, p.n, p.m, mesh.nnz, k, precision, clocks, args.workload, alu,
-                                       idx32=2 if args.workload.startswith("grid") else 4)
+                                       idx32=0 if args.workload.startswith("grid") else 4)
     step_roof = step_hbm(prof, 3, total_ms / args.steps, p.n, p.m, mesh.nnz, k, precision,
-                         idx32=2 if args.workload.startswith("grid") else 4) if prof else None
+                         idx32=0 if args.workload.startswith("grid") else 4) if prof else None
 
     # the CPU oracle on the same workload (bounded sample)
     cpu = None
@@ -648,7 +648,7 @@ def variant_mixed_grid(api, _native, dev, p, tol, steps, fp64_U, fp64_gV, clocks
     """The headline grid in mixed precision (FP32 PCG inside FP64 refinement)."""
     r = single_mesh(api, _native, dev, p, "mixed", tol, steps, 3)
     table, roof = kernel_roofline(r["prof"], p.n, p.m, r["mesh"].nnz, p.B.shape[1], "mixed", clocks, p.name + "_mixed",
-                                  alu, idx32=2)
+                                  alu, idx32=0)
     out = {"workload": f"{p.name} mixed: FP32 Jacobi-PCG (FP32 CSR values) inside FP64 residual refinement to {tol:g}",
            "value": round(r["solves_per_s"], 3), "unit": UNIT, "ms_per_step": round(r["ms_per_step"], 4),
            "steps": steps, "iterations": {"forward": r["finfo"]["iterations"], "adjoint": r["ainfo"]["iterations"]},
