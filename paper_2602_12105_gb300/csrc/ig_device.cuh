@@ -683,7 +683,7 @@ __device__ __forceinline__ void load_mesh(const MeshDev* __restrict__ mds, int i
 // The loop kernels run one CTA per resident slot; CTA b takes the flat tiles b, b + G, b + 2G, ...
 // (G = gridDim.x). A tile's sums go to the mesh's part[tile]; each CTA counts the tiles it did
 // per run of consecutive tiles of one mesh and adds that count to the mesh's counter with one
-// atomic. The CTA whose addition completes the mesh adds the partials in tile order
+// atomic. The CTA whose addition completes the mesh adds the partials in ORDER
 // (deterministic, independent of G and of any batch) and calls finish(md, scalars, totals) on
 // warp 0, with a shared-memory copy of the mesh's scalars to read (writes go to md.s).
 template <int NV, SumOrder ORDER, typename Finish>

@@ -10,7 +10,7 @@
 //            -> last tile of the mesh: convergence test, beta = rz_new / rz
 //            -> last CTA of the launch: loop control (all meshes done or the cap reached)
 // Reductions are deterministic: every CTA writes its partial sums, the last CTA of a mesh (found
-// with a counter) adds the partials in tile order. No atomics touch floating-point data, so a mesh
+// with a counter) adds the partials in a fixed order. No atomics touch floating-point data, so a mesh
 // gives the same bits alone and inside a batch.
 //
 // The loop runs on the device: a CUDA graph holds a WHILE node whose body is one iteration; the

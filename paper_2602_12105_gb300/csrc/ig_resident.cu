@@ -3,17 +3,18 @@
 // sums, so the same bits).
 //
 // A mesh of at most kResMaxRows rows per SM gets one tile per CTA and at most one CTA per SM
-// (choose_tiles64 in ig_api.cu). Its CTAs keep their rows' operator, direction, residual and solution
+// (the tile rule in ig_api.cu). Its CTAs keep their rows' operator, direction, residual and solution
 // on chip through the whole solve; only z = D^-1 r, which the neighbours' rows gather, goes through
 // global memory (L2). Per iteration the CTAs meet twice, to add p.q and then r.z and r.r; every CTA adds
-// all the tiles' partials in tile order and runs the finish step on its own copy of the solve state,
+// all the tiles' partials and runs the finish step on its own copy of the solve state,
 // so no step waits for one last CTA, and no kernel boundary or graph node lies in the loop.
 //
 // Measured, per iteration (the two-kernel graph loop before, and this): 163,842 rows k = 3 41 -> 26 us
 // and k = 4 47 -> 31 us, 66,049 rows k = 1 23 -> 7.4 us, 5,917 rows k = 1 20.6 -> 6.3 us, 642 rows k = 3
 // (a cluster of 6 CTAs; three CTAs of 256 rows before) 10 -> 6 us.
 //
-// What bounds it: on large meshes FP64 instructions and the gathers of z together. A warp's FP64
+// What bounds it: on large meshes FP64 instructions (of 26 us, 163,842 rows, k = 3: 3 go without the
+// gathers, 11 without the SpMV's multiplications, 5.5 without the update; 7.7 are the two meetings). A warp's FP64
 // instruction occupies its SM sub-partition for 64 cycles (16 per SM), so the 45 per row and iteration
 // (three columns) take 11.7 us on 163,842 rows; eight row warps are enough to issue them, and fewer
 // threads leave fewer sums to add (the sums of 32 warps would take 2.2 us of FP64 issue in the
@@ -55,7 +56,7 @@ struct ResShared {
   int width[kResMaxRows / 32];
 };
 
-constexpr int kResThreads = kBlock + 32;  // eight warps take the rows; the ninth posts and finishes
+constexpr int kResThreads = kBlock + 32;  // eight warps take the rows; the ninth finishes a meeting
 
 // Where the CTAs meet. CLUSTER: all of them form one thread-block cluster (at most 16 CTAs).
 //
