@@ -7,8 +7,8 @@
 //   E_f = w_a * area_f + sum_c omega_c * cot_c,
 //   w_a     = (1/3) sum_{v in f} <Lambda_v, B_v - U_v>,
 //   omega_c = -(t/2) <Lambda_a - Lambda_b, U_a - U_b>   ((a, b) the edge opposite corner c),
-// with the coefficients held fixed. With the edges u = p0 - p2 and v = p1 - p0 (opposite corners 1 and 2)
-// and s = |u x v|, the cotangents at corners 0, 1, 2 are -u.v / s, (u.v + v.v) / s and (u.u + u.v) / s, so
+// with the coefficients held fixed. Number the vertices, in their cyclic order, from the one opposite the
+// longest edge. With the edges u = p0 - p2 and v = p1 - p0 (opposite corners 1 and 2) and s = |u x v|, the cotangents at corners 0, 1, 2 are -u.v / s, (u.v + v.v) / s and (u.u + u.v) / s, so
 //   E_f = P / s + w_a s / 2,   P = omega_2 u.u + (omega_1 + omega_2 - omega_0) u.v + omega_1 v.v.
 // With Lambda and U differenced along u and v (x_u, x_v, y_u, y_v), omega_1 and omega_2 are -t/2 times
 // x_u.y_u and x_v.y_v, and the middle coefficient t/2 (x_u.y_v + x_v.y_u): the third edge's product
@@ -17,8 +17,9 @@
 //   A = 2 omega_2 / s - k v.v,  C = 2 omega_1 / s - k u.u,
 //   X = (omega_1 + omega_2 - omega_0) / s + k u.v,
 // and the corners get dE/du - dE/dv, dE/dv and -dE/du. The FP64 kernel is bound by FP64 instructions (2 per
-// clock per SM): this form takes about 90 per face (k = 3; 2,095,106 faces 346 us), combinations of
-// two edges corner by corner took 103 (424 us), cross products corner by corner about 140 (578 us).
+// clock per SM): this form takes about 93 per face (k = 3; three of them choose the edge left out, 3% of
+// the kernel's time), combinations of two edges corner by corner took 103, cross products corner by corner
+// about 140.
 // (The CPU oracle reaches the same numbers through the per-corner cotangent gradients.)
 //
 // A loss may also depend on V through the mass directly (the M-norm loss of the inverse-fairing
@@ -77,11 +78,31 @@ __global__ void __launch_bounds__(256) vjp_face_kernel(const MeshDev* __restrict
 #pragma unroll
       for (int d = 0; d < 3; ++d) P[c][d] = __ldg(V + 3 * (long)vid[c] + d);
     }
+    // Everything along the edge left out is a sum of the other two's, so that is the longest edge: with a
+    // shorter one left out the sums cancel, by (long / short)^2 on a needle (dl/dV of a 1000 : 1 face
+    // 6e-10 off where its short edge was the one left out, 4e-15 with this choice; the per-corner form
+    // 9e-13). The lengths are compared by the largest component's upper word, in integers.
+    double e[3][3];
+    int len[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int a = (c + 1) % 3, b = (c + 2) % 3;
+      len[c] = 0;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        e[c][d] = P[b][d] - P[a][d];
+        len[c] = max(len[c], __double2hiint(e[c][d]) & 0x7fffffff);
+      }
+    }
+    const int r = len[0] >= len[1] ? (len[0] >= len[2] ? 0 : 2) : (len[1] >= len[2] ? 1 : 2);
+    const int v0 = r == 0 ? vid[0] : (r == 1 ? vid[1] : vid[2]);
+    const int v1 = r == 0 ? vid[1] : (r == 1 ? vid[2] : vid[0]);
+    const int v2 = r == 0 ? vid[2] : (r == 1 ? vid[0] : vid[1]);
     double u[3], v[3];
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-      u[d] = P[0][d] - P[2][d];
-      v[d] = P[1][d] - P[0][d];
+      u[d] = r == 0 ? e[1][d] : (r == 1 ? e[2][d] : e[0][d]);
+      v[d] = r == 0 ? e[2][d] : (r == 1 ? e[0][d] : e[1][d]);
     }
     double N[3];
     N[0] = u[1] * v[2] - u[2] * v[1];
@@ -98,15 +119,15 @@ __global__ void __launch_bounds__(256) vjp_face_kernel(const MeshDev* __restrict
     double A = 0.0, X = 0.0, C = 0.0, S = 0.0;  // the solve terms' parts; S = P / s
     if constexpr (MODE != 2) {
       // <Lambda_v, B_v - U_v> of the three vertices, formed once per vertex by vjp_vertex_kernel
-      wa = (__ldg(wvert + vid[0]) + __ldg(wvert + vid[1])) + __ldg(wvert + vid[2]);
+      wa = (__ldg(wvert + v0) + __ldg(wvert + v1)) + __ldg(wvert + v2);
       double xu[K], xv[K], yu[K], yv[K];
 #pragma unroll
       for (int k = 0; k < K; ++k) {
-        const double l0 = lam[(long)vid[0] * K + k], u0 = U[(long)vid[0] * K + k];
-        xu[k] = l0 - lam[(long)vid[2] * K + k];
-        xv[k] = lam[(long)vid[1] * K + k] - l0;
-        yu[k] = u0 - U[(long)vid[2] * K + k];
-        yv[k] = U[(long)vid[1] * K + k] - u0;
+        const double l0 = lam[(long)v0 * K + k], u0 = U[(long)v0 * K + k];
+        xu[k] = l0 - lam[(long)v2 * K + k];
+        xv[k] = lam[(long)v1 * K + k] - l0;
+        yu[k] = u0 - U[(long)v2 * K + k];
+        yv[k] = U[(long)v1 * K + k] - u0;
       }
       double lu = xu[0] * yu[0], lv = xv[0] * yv[0], lx = xu[0] * yv[0];
 #pragma unroll
@@ -123,22 +144,29 @@ __global__ void __launch_bounds__(256) vjp_face_kernel(const MeshDev* __restrict
         // u.v + v.v could fall on the other side of a clamp at 0 than the assembly's.
         double w[3];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) w[d] = P[2][d] - P[1][d];
+        for (int d = 0; d < 3; ++d) w[d] = r == 0 ? e[0][d] : (r == 1 ? e[1][d] : e[2][d]);
+        double inv_c = inv_s;
+        if (clamp_min != 0.0 && r != 0) {  // and the assembly's area, from its two edges
+          const double n0 = e[1][1] * e[2][2] - e[1][2] * e[2][1];
+          const double n1 = e[1][2] * e[2][0] - e[1][0] * e[2][2];
+          const double n2 = e[1][0] * e[2][1] - e[1][1] * e[2][0];
+          inv_c = rsqrt(n0 * n0 + n1 * n1 + n2 * n2);
+        }
         const double dot1 = v[0] * w[0] + v[1] * w[1] + v[2] * w[2];
         const double dot2 = w[0] * u[0] + w[1] * u[1] + w[2] * u[2];
         double l0 = (lu + lv) + lx;
         bool clamped = false;
-        if (-uv * inv_s < clamp_min) {
+        if (-uv * inv_c < clamp_min) {
           if (gt) gt_part = fma(-0.5 * clamp_min, l0, gt_part);
           l0 = 0.0;
           clamped = true;
         }
-        if (-dot1 * inv_s < clamp_min) {
+        if (-dot1 * inv_c < clamp_min) {
           if (gt) gt_part = fma(-0.5 * clamp_min, lu, gt_part);
           lu = 0.0;
           clamped = true;
         }
-        if (-dot2 * inv_s < clamp_min) {
+        if (-dot2 * inv_c < clamp_min) {
           if (gt) gt_part = fma(-0.5 * clamp_min, lv, gt_part);
           lv = 0.0;
           clamped = true;
@@ -154,22 +182,22 @@ __global__ void __launch_bounds__(256) vjp_face_kernel(const MeshDev* __restrict
       C = mt * lu;
       X = -(h * lx);
     }
-    if constexpr (MODE != 0) wa += (__ldg(cl.wm + vid[0]) + __ldg(cl.wm + vid[1])) + __ldg(cl.wm + vid[2]);
+    if constexpr (MODE != 0) wa += (__ldg(cl.wm + v0) + __ldg(cl.wm + v1)) + __ldg(cl.wm + v2);
     const double kk = inv_s * fma(inv_s, S, wa * (-1.0 / 6.0));
     A = fma(-kk, vv, A);
     C = fma(-kk, uu, C);
     X = fma(kk, uv, X);
-    double g[9];
+    double* out = md.gface + 9 * (long)f;
+    double* out0 = out + 3 * r;
+    double* out1 = out + (r == 2 ? 0 : 3 * r + 3);
+    double* out2 = out + (r == 0 ? 6 : 3 * r - 3);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       const double gu = fma(A, u[d], X * v[d]), gv = fma(X, u[d], C * v[d]);
-      g[d] = gu - gv;
-      g[3 + d] = gv;
-      g[6 + d] = -gu;
+      out0[d] = gu - gv;
+      out1[d] = gv;
+      out2[d] = -gu;
     }
-    double* out = md.gface + 9 * (long)f;
-#pragma unroll
-    for (int i = 0; i < 9; ++i) out[i] = g[i];
   }
   if (gt == nullptr) return;
   // deterministic reduction of dl/dt: warp shuffle, CTA partial, last CTA adds partials in order
