@@ -335,6 +335,7 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
       if (late) break;
       if (!row_warp) finish_spmv_step(&sh.st, sh.st, K, sh.tot);
       __syncthreads();
+      if (sh.st.done) break;  // a breakdown: no update, as in the multi-CTA loop
     }
     // x += alpha p, r -= alpha q, z = D^-1 r, r.z and r.r
     {
