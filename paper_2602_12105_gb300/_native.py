@@ -29,6 +29,7 @@ IG_PRECISION_MIXED = 1
 IG_PRECISION_MIXED_GEOM32 = 2
 IG_LAUNCH_GRAPH = 0
 IG_LAUNCH_HOST = 1
+ROUTES = ("none", "host", "graph", "one_launch")  # IG_ROUTE_*
 
 
 class NativeLibraryError(RuntimeError):
@@ -78,6 +79,8 @@ SIGNATURES = {
     "ig_mesh_pattern": (_i32, [_vp, _vp, _vp]),
     "ig_assemble": (_i32, [_vp, _vp, _dbl, _i32]),
     "ig_check": (_i32, [_vp]),
+    "ig_mesh_route": (_i32, [_vp, _P(_i32), _P(_i32)]),
+    "ig_batch_route": (_i32, [_vp, _P(_i32)]),
     "ig_operator": (_i32, [_vp, _vp, _vp]),
     "ig_operator32": (_i32, [_vp, _vp]),
     "ig_solve": (_i32, [_vp, _vp, _i32, _vp, _P(SolveOpts), _P(SolveInfo)]),

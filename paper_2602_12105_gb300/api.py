@@ -143,6 +143,14 @@ class Mesh:
     def check(self):
         self.ctx.check(self.ctx.lib.ig_check(self.h))
 
+    def route(self):
+        """How the last solve's loop was run ("none", "host", "graph" or "one_launch") and the number of
+        CTAs that shared it in one launch (ig_mesh_route). Synchronises."""
+        r, c = ctypes.c_int(), ctypes.c_int()
+        self.ctx.sync_stream()
+        self.ctx.check(self.ctx.lib.ig_mesh_route(self.h, ctypes.byref(r), ctypes.byref(c)))
+        return N.ROUTES[r.value], c.value
+
     def operator(self):
         A = torch.empty(self.nnz, dtype=torch.float64, device=self.ctx.device)
         M = torch.empty(self.n, dtype=torch.float64, device=self.ctx.device)
@@ -558,6 +566,12 @@ class Batch:
 
     def __len__(self):
         return len(self.meshes)
+
+    def route(self):
+        """How the batch's last solve's loop was run (ig_batch_route)."""
+        r = ctypes.c_int()
+        self.ctx.check(self.ctx.lib.ig_batch_route(self.h, ctypes.byref(r)))
+        return N.ROUTES[r.value]
 
     def close(self):
         if self.h:

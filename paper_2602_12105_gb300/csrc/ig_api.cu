@@ -750,6 +750,18 @@ ig_status ig_check(ig_mesh* mesh) {
   return err_bits_to_status(bits);
 }
 
+ig_status ig_mesh_route(ig_mesh* mesh, int* route, int* ctas) {
+  IG_NVTX("ig_mesh_route");
+  if (!mesh || !route) return IG_ERR_INVALID_ARG;
+  ig_ctx* ctx = mesh->ctx;
+  DeviceGuard guard(ctx->device);
+  *route = mesh->group.route;
+  if (!ctas) return IG_OK;
+  IG_CK(ctx, cudaMemcpyAsync(ctas, &mesh->md.s->members, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream), "read state");
+  IG_CK(ctx, cudaStreamSynchronize(ctx->stream), "route");
+  return IG_OK;
+}
+
 ig_status ig_operator(ig_mesh* mesh, double* Aval_dev, double* M_dev) {
   IG_NVTX("ig_operator");
   if (!mesh) return IG_ERR_INVALID_ARG;

@@ -265,6 +265,12 @@ ig_status ig_batch_adjoint(ig_batch* b, const double* const* V_dev, const double
   return batch_info(b, k, infos);
 }
 
+ig_status ig_batch_route(ig_batch* b, int* route) {
+  if (!b || !route) return IG_ERR_INVALID_ARG;
+  *route = b->group.route;
+  return IG_OK;
+}
+
 ig_status ig_batch_iterate(ig_batch* b, int k, int max_iters, int* done_host) {
   IG_NVTX("ig_batch_iterate");
   if (!b) return IG_ERR_INVALID_ARG;

@@ -1120,6 +1120,7 @@ __device__ __noinline__ void finish_init(SolveScal* s, int k, const double* acc,
   s->iter = 0;
   s->refine = 0;
   s->phase = 0;
+  s->members = 0;
   s->tol2 = tol * tol;
   s->max_iter = max_iter;
   s->status = bad ? IG_ERR_NONFINITE : IG_OK;

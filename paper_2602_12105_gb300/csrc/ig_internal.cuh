@@ -109,6 +109,8 @@ struct SolveScal {
   int refine;            // mixed precision: refinements so far
   int phase;             // mixed precision: kPhaseInner / kPhaseApply / kPhaseRestart
   int max_iter, max_refine;
+  int members;           // CTAs that shared the solve in one launch (0: another route)
+  int pad;
   double tol2, inner_tol2;  // squares of the tolerances
   unsigned int cnt[4];   // last-CTA counters (spmv, update, init/residual, vjp)
 };
@@ -364,6 +366,7 @@ struct Group {
   int4* gang_plan = nullptr;      // device: the gangs of a mixed-precision solve (null: not one), in mesh order of size
   int gang_tickets = 0, gang_workers = 4;
   unsigned* gang_ticket = nullptr;
+  int route = IG_ROUTE_NONE;      // of the last solve
   int* done_host = nullptr;       // pinned host word for the host-driven loop (on its first use)
   SolvePlan plans[2][kMaxK + 1];  // [mixed][k]
   cudaStream_t capture_stream = nullptr;

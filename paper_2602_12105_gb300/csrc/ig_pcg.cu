@@ -328,8 +328,10 @@ cudaError_t loop_k(Group& g, const ig_solve_opts& o, cudaStream_t st) {
       cudaError_t e = build_plan<K>(g, pl);
       if (e != cudaSuccess) return e;
     }
+    g.route = IG_ROUTE_GRAPH;
     return cudaGraphLaunch(pl.exec, st);
   }
+  g.route = IG_ROUTE_HOST;
   return host_loop_k<K>(g, o.max_iter + 2, 16, st);
 }
 
@@ -342,8 +344,10 @@ cudaError_t end_k(Group& g, const IoTable& io, cudaStream_t st) {
 
 template <int K>
 cudaError_t solve_k(Group& g, const IoTable& io, int rhs_mass, const ig_solve_opts& o, cudaStream_t st) {
-  if (o.launch == IG_LAUNCH_GRAPH && !prof_on() && launch_resident(g, K, io.in[0], io.out[0], rhs_mass, o, st))
+  if (o.launch == IG_LAUNCH_GRAPH && !prof_on() && launch_resident(g, K, io.in[0], io.out[0], rhs_mass, o, st)) {
+    g.route = IG_ROUTE_ONE_LAUNCH;
     return cudaSuccess;
+  }
   cudaError_t e = begin_k<K>(g, io, rhs_mass, o, st);
   if (e == cudaSuccess) e = loop_k<K>(g, o, st);
   if (e == cudaSuccess) e = end_k<K>(g, io, st);

@@ -507,6 +507,7 @@ cudaError_t solve_mixed_k(Group& g, const IoTable& io, int rhs_mass, const ig_so
   if (graph && g.gang_plan) {
     if ((e = init_mixed_k<K>(g, io, rhs_mass, o, st)) != cudaSuccess) return e;
     if (launch_gang(g, K, slot_cap(o), st)) {
+      g.route = IG_ROUTE_ONE_LAUNCH;
       finalize_kernel<K><<<g.ntiles, kBlock, 0, st>>>(g.mds, g.tiles, io);
       return cudaGetLastError();
     }
@@ -519,8 +520,10 @@ cudaError_t solve_mixed_k(Group& g, const IoTable& io, int rhs_mass, const ig_so
       e = build_plan_mixed<K>(g, pl);
       if (e != cudaSuccess) return e;
     }
+    g.route = IG_ROUTE_GRAPH;
     e = cudaGraphLaunch(pl.exec, st);
   } else {
+    g.route = IG_ROUTE_HOST;
     e = host_loop_mixed_k<K>(g, slot_cap(o), 16, st);
   }
   if (e != cudaSuccess) return e;

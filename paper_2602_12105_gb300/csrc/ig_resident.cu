@@ -376,6 +376,7 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
     sh.st.status = IG_ERR_CUDA;
     sh.st.done = 1;
   }
+  if (tid == 0) sh.st.members = (int)gridDim.x;
   __syncthreads();
   if (blockIdx.x == 0) {
     for (int j = tid; j < (int)(sizeof(SolveScal) / 4); j += kResThreads)

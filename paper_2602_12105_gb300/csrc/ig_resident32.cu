@@ -418,6 +418,7 @@ __global__ void __launch_bounds__(W * kBlock, W == 4 ? 1 : 2) solve_gang_kernel(
         sh.st.status = IG_ERR_CUDA;
         sh.st.done = 1;
       }
+      if (threadIdx.x == 0) sh.st.members = gang.nct;
       __syncthreads();
       for (int j = threadIdx.x; j < (int)(sizeof(SolveScal) / 4); j += kGangThreads)
         reinterpret_cast<unsigned*>(md.s)[j] = reinterpret_cast<const unsigned*>(&sh.st)[j];
