@@ -154,6 +154,7 @@ void mesh_release(ig_mesh* mesh) {
 }
 
 ig_status err_bits_to_status(int bits) {
+  if (bits & kErrStopped) return IG_ERR_CUDA;
   if (bits & (kErrIndex | kErrBounds)) return IG_ERR_INDEX_OUT_OF_RANGE;
   if (bits & kErrRepeated) return IG_ERR_DEGENERATE_FACE;
   if (bits & kErrNonfinite) return IG_ERR_NONFINITE;
@@ -163,6 +164,7 @@ ig_status err_bits_to_status(int bits) {
 }
 
 const char* err_bits_message(int bits) {
+  if (bits & kErrStopped) return "a solve in one launch was given up: a CTA waited past the limit for another";
   if (bits & kErrBounds) return "an index read from device data was out of range (bounds-checked build)";
   if (bits & kErrIndex) return "a face index is outside [0, n)";
   if (bits & kErrRepeated) return "a face repeats a vertex";
@@ -361,6 +363,14 @@ ig_status ig_destroy(ig_ctx* ctx) {
   if (!ctx) return IG_ERR_INVALID_ARG;
   if (ctx->live_meshes != 0) return bad_arg(ctx, "meshes still alive on this context");
   delete ctx;
+  return IG_OK;
+}
+
+ig_status ig_set_wait_limits(ig_ctx* ctx, int meet_polls) {
+  if (!ctx) return IG_ERR_INVALID_ARG;
+  if (meet_polls < -1) return bad_arg(ctx, "meet_polls must be >= 0, or -1 for the default");
+  ctx->waits = WaitLimits{};
+  if (meet_polls >= 0) ctx->waits.meet = meet_polls;
   return IG_OK;
 }
 
@@ -658,6 +668,7 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
   UP_CK(cudaMemsetAsync(md.p, 0, sizeof(double) * nv, st), "memset");
   UP_CK(cudaMemsetAsync(md.q, 0, sizeof(double) * nv, st), "memset");
   UP_CK(cudaMemsetAsync(md.z, 0, sizeof(double) * nv, st), "memset");
+  M->group.waits = &ctx->waits;
   UP_CK(group_init(M->group, &md, 1, ctx->solver_slots, ctx->solver_slots32, ctx->num_sms, st), "group");
   UP_CK(cudaStreamSynchronize(st), "upload");
 #undef UP_CK
@@ -1326,6 +1337,7 @@ ig_status ig_rgd_admm(ig_mesh* mesh, const double* V_dev, const int32_t* sources
   }
   if (worst != IG_OK) {
     set_error(ctx, worst == IG_ERR_NOT_CONVERGED ? "a u-step solve reached max_iter above rel_tol"
+                   : worst == IG_ERR_CUDA        ? err_bits_message(kErrStopped)
                                                  : "a u-step solve met a non-finite value");
     return (ig_status)worst;
   }

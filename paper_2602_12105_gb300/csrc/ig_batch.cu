@@ -76,8 +76,9 @@ ig_status batch_info(ig_batch* b, int k, ig_solve_info* infos) {
   for (size_t i = 0; i < nm; ++i) {
     ig_status st = (ig_status)ss[i].status;
     if (bits[i])
-      st = (bits[i] & kErrBounds) ? IG_ERR_INDEX_OUT_OF_RANGE
-                                  : ((bits[i] & kErrNonfinite) ? IG_ERR_NONFINITE : IG_ERR_DEGENERATE_FACE);
+      st = (bits[i] & kErrStopped)  ? IG_ERR_CUDA
+           : (bits[i] & kErrBounds) ? IG_ERR_INDEX_OUT_OF_RANGE
+                                    : ((bits[i] & kErrNonfinite) ? IG_ERR_NONFINITE : IG_ERR_DEGENERATE_FACE);
     if (st != IG_OK && worst == IG_OK) worst = st;
     if (infos) {
       ig_solve_info& inf = infos[i];
@@ -121,6 +122,7 @@ ig_status ig_batch_create(ig_ctx* ctx, ig_mesh* const* meshes, int count, ig_bat
   if (!b) return IG_ERR_OOM;
   b->ctx = ctx;
   b->meshes.assign(meshes, meshes + count);
+  b->group.waits = &ctx->waits;
   std::vector<MeshDev> mds(count);
   for (int i = 0; i < count; ++i) mds[i] = meshes[i]->md;
   cudaError_t e = group_init(b->group, mds.data(), count, ctx->solver_slots, ctx->solver_slots32,

@@ -59,6 +59,7 @@ enum : int {
   kErrDegenerate = 16,
   kErrNonfinite = 32,
   kErrBounds = 64,  // bounds-checked build only: an index read from device data was out of range
+  kErrStopped = 128,  // a one-launch solve gave up on a wait: its result is NaN
 };
 
 // Bounds-checked build (compiled with -DIG_CHECK, a separate library): the indices the kernels
@@ -243,6 +244,13 @@ struct ProfScope {
 
 // ---------------------------------------------------------------------------------------------
 // Opaque types of the C ABI.
+namespace ig {
+// Polls of a wait in a one-launch solve before it is given up (ig_set_wait_limits; about a second).
+struct WaitLimits {
+  int meet = 1 << 21;
+};
+}  // namespace ig
+
 struct ig_ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -250,6 +258,7 @@ struct ig_ctx {
   int solver_slots = 0;    // CTAs of the FP64 solver kernels resident at once on the device
   int solver_slots32 = 0;  // same for the mixed-precision solver kernels
   int live_meshes = 0;
+  ig::WaitLimits waits;
   std::string last_error;
 };
 
@@ -367,6 +376,7 @@ struct Group {
   int gang_tickets = 0, gang_workers = 4;
   unsigned* gang_ticket = nullptr;
   int route = IG_ROUTE_NONE;      // of the last solve
+  const WaitLimits* waits = nullptr;  // the context's
   int* done_host = nullptr;       // pinned host word for the host-driven loop (on its first use)
   SolvePlan plans[2][kMaxK + 1];  // [mixed][k]
   cudaStream_t capture_stream = nullptr;

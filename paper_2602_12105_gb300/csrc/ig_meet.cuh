@@ -13,7 +13,21 @@ struct __align__(16) Slot {
   double value;
   unsigned long long number;
 };
-constexpr int kSpinLimit = 1 << 21;  // polls of one wait (about a second); then the solve fails
+
+// Ahead of a mesh's slots: the one-launch solves of the mesh so far (times 2^16) plus the CTAs of the
+// current one that have begun. The last of them moves it on to the next solve: by then every CTA has its
+// number, whenever it began.
+struct __align__(16) MeetHead {
+  unsigned long long word, unused;
+};
+static_assert(sizeof(MeetHead) == sizeof(Slot), "one slot");
+// This CTA (one of count) begins; the solve's number.
+__device__ __forceinline__ unsigned long long begin_solve(MeetHead* h, int count) {
+  const unsigned long long w = atomicAdd(&h->word, 1ull);
+  if ((int)(w & 0xffffu) == count - 1) atomicExch(&h->word, ((w >> 16) + 1ull) << 16);
+  return w >> 16;
+}
+__device__ __forceinline__ double not_a_number() { return __longlong_as_double(0x7ff8000000000000ll); }
 
 __device__ __forceinline__ void post(Slot* s, double value, unsigned long long number) {
   asm volatile("{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(s),

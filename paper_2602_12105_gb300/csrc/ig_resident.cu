@@ -53,6 +53,7 @@ struct ResShared {
   double red[8 * kWarps];
   double tot[8];
   double box[2][8];          // cluster: this CTA's posted sums, by parity of the meeting
+  unsigned long long solve;  // number of this solve of the mesh
   int width[kResMaxRows / 32];
 };
 
@@ -68,6 +69,7 @@ struct Meeting {
   Slot* slots;
   double* gathered;  // [value][tile]
   int nct;
+  int patience;  // polls of a wait before the solve is given up
   unsigned long long number;
 
   // One meeting up to the barrier after which tot is complete; true when a wait ran out. RELEASE: what a
@@ -109,7 +111,7 @@ struct Meeting {
       if (row_warp) {
         using Map = PartialMap<NV>;
         double b[kLaneTiles<NV>];
-        collect<NV, RELEASE>(box, nct, number, kSpinLimit, b, late);
+        collect<NV, RELEASE>(box, nct, number, patience, b, late);
         const int val = Map::value(lane), first = Map::first(warp, lane);
         if (val < NV) {
 #pragma unroll
@@ -188,7 +190,7 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
                                                                         const double* __restrict__ in,
                                                                         double* __restrict__ out, int rhs_mass,
                                                                         double tol, int max_iter, int cap,
-                                                                        ResLayout lay) {
+                                                                        int patience, ResLayout lay) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ ResShared sh;
   {
@@ -220,6 +222,9 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
   const long xn = lay.x_on ? rp : nn;
   double* z = md.z;
 
+  // (the ninth warp, while the others load)
+  if (!CLUSTER && tid == kBlock) sh.solve = begin_solve(reinterpret_cast<MeetHead*>(md.meet), gridDim.x);
+
   // the rows' operator on chip; slices of 32 rows, one per warp and step
   for (int i = tid; i < rows; i += kBlock) {
     const long row = t0 + i;
@@ -238,11 +243,8 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
   mt.slots = reinterpret_cast<Slot*>(md.meet) + 1;
   mt.gathered = sums;
   mt.nct = gridDim.x;
-  // numbers of this launch: above those of every launch before it (the word ahead of the slots
-  // counts launches; CTA 0 advances it at the end, when every CTA has long read it)
-  unsigned long long launches = 0;
-  if constexpr (!CLUSTER) launches = __ldcg(reinterpret_cast<const unsigned long long*>(md.meet));
-  mt.number = launches << 32;
+  mt.patience = patience;
+  mt.number = 0;
 
   // start: rhs = M * in or in; r = rhs, z = D^-1 r, p = q = x = 0; r.z and |rhs|^2
   bool late;
@@ -267,6 +269,10 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
         acc[K + c] = fma(b, b, acc[K + c]);
       }
       store_row<K>(z, row, zo);
+    }
+    if constexpr (!CLUSTER) {
+      __syncthreads();
+      mt.number = sh.solve << 32;  // above those of every solve of the mesh before
     }
     late = mt.template meet<2 * K, true>(sh, acc, row_warp);
     if (tid == kBlock) finish_init(&sh.st, K, sh.tot, tol, max_iter);
@@ -370,9 +376,10 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
   }
   for (int i = tid; i < rows; i += kBlock) {
 #pragma unroll
-    for (int c = 0; c < K; ++c) out[(t0 + i) * K + c] = x[c * xn + i];
+    for (int c = 0; c < K; ++c) out[(t0 + i) * K + c] = late ? not_a_number() : x[c * xn + i];
   }
-  if (late && tid == kBlock) {  // a CTA stayed away past the limit: report a failed solve
+  if (late && tid == kBlock) {  // a CTA stayed away past the limit: a failed solve, for every caller to see
+    atomicOr(md.err, kErrStopped);
     sh.st.status = IG_ERR_CUDA;
     sh.st.done = 1;
   }
@@ -381,7 +388,6 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
   if (blockIdx.x == 0) {
     for (int j = tid; j < (int)(sizeof(SolveScal) / 4); j += kResThreads)
       reinterpret_cast<unsigned*>(md.s)[j] = reinterpret_cast<const unsigned*>(&sh.st)[j];
-    if (!CLUSTER && tid == 0) *reinterpret_cast<unsigned long long*>(md.meet) = launches + 1;
   }
   if constexpr (CLUSTER) cluster_sync_all();  // no CTA leaves while another reads its sums
 }
@@ -436,7 +442,7 @@ bool launch_k(Group& g, const double* in, double* out, int rhs_mass, const ig_so
     }
   }
   if (cudaLaunchKernelEx(&cfg, kern, (const MeshDev*)g.mds, in, out, rhs_mass, o.rel_tol, o.max_iter, o.max_iter + 2,
-                         lay) != cudaSuccess) {
+                         g.waits->meet, lay) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }

@@ -52,6 +52,7 @@ struct GangShared {
   double tot[8];
   float alpha[kMaxK], beta[kMaxK];         // as floats (a conversion in every warp costs FP64 issue)
   int ticket;
+  unsigned long long solve;                // number of this solve of the mesh
   int width[kGangMaxRows / 32];
 };
 
@@ -355,7 +356,8 @@ __device__ __forceinline__ bool gang_solve(GangShared& sh, const GangRows& gr, G
 template <int K, int W>
 __global__ void __launch_bounds__(W * kBlock, W == 4 ? 1 : 2) solve_gang_kernel(const MeshDev* __restrict__ mds,
                                                                                 const int4* __restrict__ plan, int nplan,
-                                                                                int tickets, unsigned* ticket, int cap) {
+                                                                                int tickets, unsigned* ticket, int cap,
+                                                                                long long patience) {
   constexpr int kGangThreads = W * kBlock;
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ GangShared sh;
@@ -381,10 +383,8 @@ __global__ void __launch_bounds__(W * kBlock, W == 4 ? 1 : 2) solve_gang_kernel(
     gang.member = sh.ticket - e.y;
     gang.nct = e.z;
     gang.slots = reinterpret_cast<Slot*>(md.meet) + 1;
-    const unsigned long long launches = __ldcg(reinterpret_cast<const unsigned long long*>(md.meet));
-    gang.number = launches << 32;
-    // a wait for the rest of the gang lasts as long as the solve of a mesh drawn before
-    gang.patience = kSpinLimit + 256ll * cap;
+    gang.patience = patience;
+    if (threadIdx.x == kGangThreads - 32) sh.solve = begin_solve(reinterpret_cast<MeetHead*>(md.meet), gang.nct);
 
     // the rows on chip
     GangRows gr;
@@ -410,11 +410,18 @@ __global__ void __launch_bounds__(W * kBlock, W == 4 ? 1 : 2) solve_gang_kernel(
       gr.d[i] = __ldg(md.Dinv32 + row);
     }
     __syncthreads();
+    gang.number = sh.solve << 32;  // above those of every solve of the mesh before
 
     const bool met = gang_solve<K, W>(sh, gr, gang, cap);
     __syncthreads();
+    if (!met) {  // a CTA stayed away past the limit: a failed solve, for every caller to see
+      for (int i = threadIdx.x; i < held; i += kGangThreads)
+#pragma unroll
+        for (int c = 0; c < K; ++c) md.x[(long)c * md.n + first_row + i] = not_a_number();
+      if (threadIdx.x == 0) atomicOr(md.err, kErrStopped);
+    }
     if (gang.member == 0) {
-      if (threadIdx.x == 0 && !met) {  // a CTA stayed away past the limit: report a failed solve
+      if (threadIdx.x == 0 && !met) {
         sh.st.status = IG_ERR_CUDA;
         sh.st.done = 1;
       }
@@ -422,7 +429,6 @@ __global__ void __launch_bounds__(W * kBlock, W == 4 ? 1 : 2) solve_gang_kernel(
       __syncthreads();
       for (int j = threadIdx.x; j < (int)(sizeof(SolveScal) / 4); j += kGangThreads)
         reinterpret_cast<unsigned*>(md.s)[j] = reinterpret_cast<const unsigned*>(&sh.st)[j];
-      if (threadIdx.x == 0) *reinterpret_cast<unsigned long long*>(md.meet) = launches + 1;
     }
   }
 }
@@ -449,8 +455,10 @@ bool launch_w(Group& g, int cap, cudaStream_t st) {
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  // a wait for the rest of a gang lasts as long as the solve of a mesh drawn before
+  const long long patience = g.waits->meet + (g.waits->meet == WaitLimits{}.meet ? 256ll * cap : 0ll);
   if (cudaLaunchKernelEx(&cfg, kern, (const MeshDev*)g.mds, (const int4*)g.gang_plan, g.nmesh, g.gang_tickets,
-                         g.gang_ticket, cap) != cudaSuccess) {
+                         g.gang_ticket, cap, patience) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }

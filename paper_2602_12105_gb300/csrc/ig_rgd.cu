@@ -513,7 +513,7 @@ __global__ void __launch_bounds__(kBlock) rgd_axpy_kernel(double* __restrict__ u
 
 // The worst status of the solves so far (codes grow with severity: 0 ok, NOT_CONVERGED, NONFINITE).
 __global__ void rgd_note_status_kernel(const MeshDev* __restrict__ mds, int* worst) {
-  const int st = mds[0].s->status;
+  const int st = (*mds[0].err & kErrStopped) ? IG_ERR_CUDA : mds[0].s->status;
   if (st > *worst) *worst = st;
 }
 
