@@ -107,12 +107,14 @@ ig_status ig_set_stream(ig_ctx* ctx, void* cuda_stream);
 /* Destroy a context. Every mesh created on it must have been freed first. */
 ig_status ig_destroy(ig_ctx* ctx);
 
-/* How often a CTA of a solve in one launch (IG_ROUTE_ONE_LAUNCH) looks for what another has to post before
- * it gives the solve up: meet_polls, or -1 for the default (2^21, about a second). A solve that was given up
- * has NaN in its result, and IG_ERR_CUDA is reported by its ig_solve_info and by the next ig_check (until
- * the mesh is assembled again). For later solves of the context's meshes and batches; results do not
- * depend on it otherwise. Errors: IG_ERR_INVALID_ARG (NULL context, meet_polls < -1). */
-ig_status ig_set_wait_limits(ig_ctx* ctx, int meet_polls);
+/* How often a CTA of a solve in one launch (IG_ROUTE_ONE_LAUNCH) looks before it stops waiting; -1 for the
+ * defaults. begin_polls (default 2^9, some 0.2 ms): for the other CTAs to begin; the solve then goes
+ * on with those that have (other work on the GPU may hold the rest's SMs), with the same results.
+ * meet_polls (default 2^21, about a second): for what another of them has to post; the solve is then given
+ * up: it has NaN in its result, and IG_ERR_CUDA is reported by its ig_solve_info and by the next ig_check
+ * (until the mesh is assembled again). For later solves of the context's meshes and batches; results do not
+ * depend on the limits otherwise. Errors: IG_ERR_INVALID_ARG (NULL context, a limit < -1). */
+ig_status ig_set_wait_limits(ig_ctx* ctx, int begin_polls, int meet_polls);
 
 /* Last error message recorded on ctx (empty string if none). */
 const char* ig_last_error(ig_ctx* ctx);

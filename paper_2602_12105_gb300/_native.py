@@ -72,7 +72,7 @@ SIGNATURES = {
     "ig_create": (_i32, [_P(_vp), _i32, _vp]),
     "ig_set_stream": (_i32, [_vp, _vp]),
     "ig_destroy": (_i32, [_vp]),
-    "ig_set_wait_limits": (_i32, [_vp, _i32]),
+    "ig_set_wait_limits": (_i32, [_vp, _i32, _i32]),
     "ig_last_error": (ctypes.c_char_p, [_vp]),
     "ig_mesh_upload": (_i32, [_vp, _vp, _i64, _i64, _P(_vp)]),
     "ig_mesh_free": (_i32, [_vp]),

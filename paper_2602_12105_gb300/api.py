@@ -61,9 +61,9 @@ class Context:
     def check(self, status):
         N.check(status, self.h)
 
-    def set_wait_limits(self, meet: int = -1):
+    def set_wait_limits(self, begin: int = -1, meet: int = -1):
         """How long the CTAs of a solve in one launch wait for one another (ig_set_wait_limits)."""
-        self.check(self.lib.ig_set_wait_limits(self.h, int(meet)))
+        self.check(self.lib.ig_set_wait_limits(self.h, int(begin), int(meet)))
 
     def close(self):
         if self.h:

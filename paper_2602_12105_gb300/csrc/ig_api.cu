@@ -366,10 +366,11 @@ ig_status ig_destroy(ig_ctx* ctx) {
   return IG_OK;
 }
 
-ig_status ig_set_wait_limits(ig_ctx* ctx, int meet_polls) {
+ig_status ig_set_wait_limits(ig_ctx* ctx, int begin_polls, int meet_polls) {
   if (!ctx) return IG_ERR_INVALID_ARG;
-  if (meet_polls < -1) return bad_arg(ctx, "meet_polls must be >= 0, or -1 for the default");
+  if (begin_polls < -1 || meet_polls < -1) return bad_arg(ctx, "a limit must be >= 0, or -1 for the default");
   ctx->waits = WaitLimits{};
+  if (begin_polls >= 0) ctx->waits.begin = begin_polls;
   if (meet_polls >= 0) ctx->waits.meet = meet_polls;
   return IG_OK;
 }
@@ -632,9 +633,10 @@ ig_status ig_mesh_upload(ig_ctx* ctx, const int32_t* F_dev, int64_t m, int64_t n
   md.incptr = incptr;
   md.inc = inc;
   md.err = err;
-  // partial sums: the loop kernels' tiles (and the geodesic warm start's, of kTileRows rows), and the
-  // VJP's per-face-tile sums of dl/dt
-  const size_t npart = std::max(std::max(std::max((size_t)md.ntiles, (size_t)std::max(md.ntiles32, md.ntiles32s)),
+  // partial sums: the loop kernels' tiles (and the geodesic warm start's, of kTileRows rows; the product's
+  // and the update's side by side for one-launch solves with fewer CTAs than tiles), and the VJP's
+  // per-face-tile sums of dl/dt
+  const size_t npart = std::max(std::max(std::max((size_t)md.ntiles * (resident ? 2 : 1), (size_t)std::max(md.ntiles32, md.ntiles32s)),
                                          (size_t)(ni + kTileRows - 1) / kTileRows) * kPartStride,
                                 (size_t)(mi + 255) / 256) + 8;
   UP_CK(mesh_alloc(M, &md.facew, 4 * (size_t)m), "alloc");

@@ -245,9 +245,10 @@ struct ProfScope {
 // ---------------------------------------------------------------------------------------------
 // Opaque types of the C ABI.
 namespace ig {
-// Polls of a wait in a one-launch solve before it is given up (ig_set_wait_limits; about a second).
+// Polls of the waits in a one-launch solve (ig_set_wait_limits): for its CTAs to begin, after which it goes
+// on with those that have (some 0.2 ms), and for a post, after which it is given up (a second).
 struct WaitLimits {
-  int meet = 1 << 21;
+  int begin = 1 << 9, meet = 1 << 21;
 };
 }  // namespace ig
 

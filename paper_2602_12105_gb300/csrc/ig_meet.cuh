@@ -14,11 +14,12 @@ struct __align__(16) Slot {
   unsigned long long number;
 };
 
-// Ahead of a mesh's slots: the one-launch solves of the mesh so far (times 2^16) plus the CTAs of the
+// Ahead of a mesh's slots. word: the one-launch solves of the mesh so far (times 2^16) plus the CTAs of the
 // current one that have begun. The last of them moves it on to the next solve: by then every CTA has its
-// number, whenever it began.
+// number, whenever it began. team: the solve (its number + 1, times 2^16) that was settled last and how many
+// CTAs share it.
 struct __align__(16) MeetHead {
-  unsigned long long word, unused;
+  unsigned long long word, team;
 };
 static_assert(sizeof(MeetHead) == sizeof(Slot), "one slot");
 // This CTA (one of count) begins; the solve's number.
@@ -27,6 +28,46 @@ __device__ __forceinline__ unsigned long long begin_solve(MeetHead* h, int count
   if ((int)(w & 0xffffu) == count - 1) atomicExch(&h->word, ((w >> 16) + 1ull) << 16);
   return w >> 16;
 }
+
+// The CTAs of a solve wait for one another, so those that share it must all run at once, and nothing makes
+// sure that a grid starts as a whole when other work holds some of the SMs. So they settle who takes part:
+// the last of them to begin settles on all; one that has waited `patience` polls settles on those that
+// have begun by then (they run and will see it), and a CTA that begins after that leaves at once. One
+// word decides (compare-and-swap), so all read the same.
+struct Team {
+  unsigned long long solve;  // number of the solve
+  int rank;                  // in the order of beginning; takes part if below size
+  int size;                  // CTAs that share the solve (-1: not settled within the limits)
+};
+__device__ __forceinline__ unsigned long long load_relaxed(const unsigned long long* p) {
+  unsigned long long v;
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ Team join_team(MeetHead* h, int count, int patience, int limit) {
+  const unsigned long long w = atomicAdd(&h->word, 1ull);
+  Team t{w >> 16, (int)(w & 0xffffu), -1};
+  const unsigned long long mark = t.solve + 1ull;
+  unsigned long long s = load_relaxed(&h->team);
+  auto settle = [&](unsigned long long size) {  // a failed swap found this solve settled already
+    const unsigned long long was = atomicCAS(&h->team, s, mark << 16 | size);
+    s = was == s ? (mark << 16 | size) : was;
+  };
+  if (t.rank == count - 1) {
+    if (s >> 16 != mark) settle((unsigned long long)count);
+    __threadfence();
+    atomicExch(&h->word, mark << 16);
+  } else {
+    for (int spins = 0; s >> 16 != mark && (spins < patience || spins - patience < limit); ++spins) {
+      const unsigned long long now = spins >= patience ? load_relaxed(&h->word) : 0ull;
+      if (spins >= patience && now >> 16 == t.solve) settle(now & 0xffffu);
+      else s = load_relaxed(&h->team);
+    }
+  }
+  if (s >> 16 == mark) t.size = (int)(s & 0xffffu);
+  return t;
+}
+
 __device__ __forceinline__ double not_a_number() { return __longlong_as_double(0x7ff8000000000000ll); }
 
 __device__ __forceinline__ void post(Slot* s, double value, unsigned long long number) {
@@ -57,7 +98,7 @@ __device__ __forceinline__ bool peek(const Slot* s, unsigned long long number, d
 template <int NV>
 constexpr int kLaneTiles = (kResMaxCtas + PartialMap<NV>::kStride - 1) / PartialMap<NV>::kStride;
 template <int NV, bool ACQUIRE>
-__device__ __forceinline__ void collect(const Slot* buf, int count, unsigned long long number, long long patience,
+__device__ __forceinline__ void collect(const Slot* buf, int count, unsigned long long number, int patience,
                                         double (&b)[kLaneTiles<NV>], bool& late) {
   using Map = PartialMap<NV>;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, val = Map::value(lane);
@@ -70,7 +111,7 @@ __device__ __forceinline__ void collect(const Slot* buf, int count, unsigned lon
     if (val < NV && first + j * Map::kStride < count) want |= 1u << j;
   }
   // all the missing slots of a round are loaded before any is looked at
-  for (long long spins = 0; want != 0 && !late; late = ++spins > patience) {
+  for (int spins = 0; want != 0 && !late; late = ++spins > patience) {
     double x[J];
     bool there[J];
 #pragma unroll
@@ -88,7 +129,7 @@ __device__ __forceinline__ void collect(const Slot* buf, int count, unsigned lon
 }
 // The lane's sum of them.
 template <int NV, bool ACQUIRE>
-__device__ __forceinline__ double collect_sum(const Slot* buf, int count, unsigned long long number, long long patience,
+__device__ __forceinline__ double collect_sum(const Slot* buf, int count, unsigned long long number, int patience,
                                               bool& late) {
   constexpr int J = kLaneTiles<NV>;
   double b[J];

@@ -9,6 +9,12 @@
 // all the tiles' partials and runs the finish step on its own copy of the solve state,
 // so no step waits for one last CTA, and no kernel boundary or graph node lies in the loop.
 //
+// A CTA of a large mesh takes all of an SM's shared memory, so other kernels on the GPU (another stream's)
+// can keep some of the CTAs from starting. The solve waits some 0.2 ms for them and then goes on with those
+// that have begun (join_team, solve_shared), from global memory. 184,470 rows, k = 4, while another kernel
+// holds SMs for 10 ms: 1.8 ms with none held, 2.8 with one held and 3.1 with 30 (the two-kernel graph loop
+// 2.6 in all of these; a cooperative launch, which starts only as a whole, 11.4).
+//
 // Measured, per iteration (the two-kernel graph loop before, and this): 163,842 rows k = 3 41 -> 26 us
 // and k = 4 47 -> 31 us, 66,049 rows k = 1 23 -> 7.4 us, 5,917 rows k = 1 20.6 -> 6.3 us, 642 rows k = 3
 // (a cluster of 6 CTAs; three CTAs of 256 rows before) 10 -> 6 us.
@@ -22,6 +28,7 @@
 // meetings of about 1 us (a store to L2, then a load that sees it), and sums (in fixed point where that is
 // shorter) and divisions whose every FP64 step costs 64 cycles.
 #include "ig_meet.cuh"
+#include "ig_tiles64.cuh"
 
 namespace ig {
 
@@ -53,7 +60,7 @@ struct ResShared {
   double red[8 * kWarps];
   double tot[8];
   double box[2][8];          // cluster: this CTA's posted sums, by parity of the meeting
-  unsigned long long solve;  // number of this solve of the mesh
+  Team team;                 // the CTAs that share the solve
   int width[kResMaxRows / 32];
 };
 
@@ -185,12 +192,122 @@ __device__ __forceinline__ void wide_slots(const MeshDev& md, const double* sa, 
   }
 }
 
+// The solve by fewer CTAs than the mesh has tiles (the others had not begun in time: join_team): a CTA takes
+// the tiles rank, rank + size, ... with the rows in global memory, through the tile bodies of the loop
+// kernels, and adds all the tiles' sums itself. The same arithmetic and order, the same bits. Only the
+// eight row warps come here. Two meetings per iteration, each after a half of the partial sums is
+// complete: a half is written again only after the meeting of the other.
+struct SharedScratch {  // at the start of the dynamic shared memory
+  ScalSnap sn;
+  double red[2][8 * kWarps];
+  double tot[8];
+};
+static_assert(sizeof(SharedScratch) <= 128 * 4 * 8, "fits where the smallest tile's rows would be");
+template <int K>
+__device__ __noinline__ void solve_shared(ResShared& sh, SharedScratch& w, Slot* slots, const double* in, double* out,
+                                          int rhs_mass, double tol, int max_iter, int cap, int patience) {
+  const MeshDev& md = sh.md;
+  const int tid = threadIdx.x, nt = md.ntiles, size = sh.team.size, rank = sh.team.rank;
+  const long nn = md.n;
+  double* const part_spmv = md.part;
+  double* const part_update = md.part + (long)nt * kPartStride;
+  unsigned long long number = sh.team.solve << 32;
+  bool late = false;
+  auto meet = [&]() {  // what any of the CTAs wrote before is visible to all of them after
+    ++number;
+    Slot* const box = slots + (size_t)(number & 1) * 8 * (size_t)nt;
+    __syncthreads();
+    if (tid == 0) {
+      fence_gpu();
+      post(box + 8 * (size_t)rank, 0.0, number);
+    }
+    bool mine = false;
+    if (tid < size) {
+      double x;
+      for (int spins = 0; !peek<true>(box + 8 * (size_t)tid, number, x) && !mine; mine = ++spins > patience) {
+      }
+    }
+    late = __syncthreads_or(mine) != 0;
+    return !late;
+  };
+  int b = 0;
+  for (int tile = rank; tile < nt; tile += size, b ^= 1) {
+    const long t0 = (long)tile * md.tile_rows, t1 = t0 + md.tile_rows < nn ? t0 + md.tile_rows : nn;
+    double acc[2 * K];
+#pragma unroll
+    for (int i = 0; i < 2 * K; ++i) acc[i] = 0.0;
+    for (long row = t0 + tid; row < t1; row += kBlock) {
+      const double dinv = md.Dinv[row], mass = rhs_mass ? md.M[row] : 1.0;
+      double zo[K], zero[K];
+#pragma unroll
+      for (int c = 0; c < K; ++c) {
+        const double v = rhs_mass ? mass * in[row * K + c] : in[row * K + c];
+        zo[c] = dinv * v;
+        zero[c] = 0.0;
+        md.x[c * nn + row] = 0.0;
+        md.r[c * nn + row] = v;
+        md.q[c * nn + row] = 0.0;
+        acc[c] = fma(v, zo[c], acc[c]);
+        acc[K + c] = fma(v, v, acc[K + c]);
+      }
+      store_row<K>(md.z, row, zo);
+      store_row<K>(md.p, row, zero);
+    }
+    tile_reduce<2 * K, kFixed>(acc, w.red[b], part_update + (long)tile * kPartStride);
+  }
+  if (meet()) {
+    combine_tiles<2 * K, kFixed>(part_update, nt, w.red[0], w.tot);
+    if (tid == 0) finish_init(&sh.st, K, w.tot, tol, max_iter);
+    __syncthreads();
+  }
+  for (int it = 0; it < cap && !late && !sh.st.done; ++it) {
+    if (tid < kMaxK) w.sn.beta[tid] = sh.st.beta[tid];
+    __syncthreads();
+    for (int tile = rank; tile < nt; tile += size, b ^= 1)
+      spmv_tile<K>(md, tile, w.sn, w.red[b], part_spmv + (long)tile * kPartStride);
+    if (!meet()) break;
+    combine_tiles<K, kFixed>(part_spmv, nt, w.red[0], w.tot);
+    if (tid < 32) finish_spmv_step(&sh.st, sh.st, K, w.tot);
+    __syncthreads();
+    if (sh.st.done) break;
+    if (tid < kMaxK) w.sn.alpha[tid] = sh.st.alpha[tid];
+    __syncthreads();
+    for (int tile = rank; tile < nt; tile += size, b ^= 1)
+      update_tile<K>(md, tile, w.sn, w.red[b], part_update + (long)tile * kPartStride);
+    if (!meet()) break;
+    combine_tiles<2 * K, kFixed>(part_update, nt, w.red[0], w.tot);
+    if (tid < 32) finish_update_step(&sh.st, sh.st, K, w.tot);
+    __syncthreads();
+  }
+  for (int tile = rank; tile < nt; tile += size) {
+    const long t0 = (long)tile * md.tile_rows, t1 = t0 + md.tile_rows < nn ? t0 + md.tile_rows : nn;
+    for (long row = t0 + tid; row < t1; row += kBlock) {
+#pragma unroll
+      for (int c = 0; c < K; ++c) out[row * K + c] = late ? not_a_number() : md.x[c * nn + row];
+    }
+  }
+  if (tid == 0) {
+    if (late) {
+      atomicOr(md.err, kErrStopped);
+      sh.st.status = IG_ERR_CUDA;
+      sh.st.done = 1;
+    }
+    sh.st.members = size;
+  }
+  __syncthreads();
+  if (rank == 0) {
+    for (int j = tid; j < (int)(sizeof(SolveScal) / 4); j += kBlock)
+      reinterpret_cast<unsigned*>(md.s)[j] = reinterpret_cast<const unsigned*>(&sh.st)[j];
+  }
+}
+
 template <int K, bool CLUSTER>
 __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const MeshDev* __restrict__ mds,
                                                                         const double* __restrict__ in,
                                                                         double* __restrict__ out, int rhs_mass,
                                                                         double tol, int max_iter, int cap,
-                                                                        int patience, ResLayout lay) {
+                                                                        int begin_patience, int patience,
+                                                                        ResLayout lay) {
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ ResShared sh;
   {
@@ -223,7 +340,8 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
   double* z = md.z;
 
   // (the ninth warp, while the others load)
-  if (!CLUSTER && tid == kBlock) sh.solve = begin_solve(reinterpret_cast<MeetHead*>(md.meet), gridDim.x);
+  if (!CLUSTER && tid == kBlock)
+    sh.team = join_team(reinterpret_cast<MeetHead*>(md.meet), (int)gridDim.x, begin_patience, patience);
 
   // the rows' operator on chip; slices of 32 rows, one per warp and step
   for (int i = tid; i < rows; i += kBlock) {
@@ -245,6 +363,25 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
   mt.nct = gridDim.x;
   mt.patience = patience;
   mt.number = 0;
+
+  if constexpr (!CLUSTER) {
+    __syncthreads();  // nothing is written to global memory before it is settled who takes part
+    if (__builtin_expect(sh.team.size != (int)gridDim.x, 0)) {
+      if (!row_warp || sh.team.rank >= sh.team.size) {
+        if (sh.team.size < 0) {  // not settled: a failed solve
+          for (int i = tid; i < rows; i += kBlock)
+#pragma unroll
+            for (int c = 0; c < K; ++c) out[(t0 + i) * K + c] = not_a_number();
+          if (tid == 0) atomicOr(md.err, kErrStopped);
+        }
+        return;
+      }
+      solve_shared<K>(sh, *reinterpret_cast<SharedScratch*>(dyn), mt.slots, in, out, rhs_mass, tol, max_iter, cap,
+                      patience);
+      return;
+    }
+    mt.number = sh.team.solve << 32;  // above those of every solve of the mesh before
+  }
 
   // start: rhs = M * in or in; r = rhs, z = D^-1 r, p = q = x = 0; r.z and |rhs|^2
   bool late;
@@ -269,10 +406,6 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
         acc[K + c] = fma(b, b, acc[K + c]);
       }
       store_row<K>(z, row, zo);
-    }
-    if constexpr (!CLUSTER) {
-      __syncthreads();
-      mt.number = sh.solve << 32;  // above those of every solve of the mesh before
     }
     late = mt.template meet<2 * K, true>(sh, acc, row_warp);
     if (tid == kBlock) finish_init(&sh.st, K, sh.tot, tol, max_iter);
@@ -428,12 +561,10 @@ bool launch_k(Group& g, const double* in, double* out, int rhs_mass, const ig_so
     attr[0].val.clusterDim.x = md.ntiles;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
-  } else {
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
   }
+  // (Not a cooperative launch: that starts as a whole, once no other work holds any SM it needs. See join_team.)
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = CLUSTER ? 1 : 0;
   if (CLUSTER) {
     int clusters = 0;
     if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters < 1) {
@@ -442,7 +573,7 @@ bool launch_k(Group& g, const double* in, double* out, int rhs_mass, const ig_so
     }
   }
   if (cudaLaunchKernelEx(&cfg, kern, (const MeshDev*)g.mds, in, out, rhs_mass, o.rel_tol, o.max_iter, o.max_iter + 2,
-                         g.waits->meet, lay) != cudaSuccess) {
+                         g.waits->begin, g.waits->meet, lay) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }

@@ -67,7 +67,7 @@ struct Gang {
   Slot* slots;
   int member, nct;     // this CTA and the CTAs of the gang: as many as the mesh has groups of four tiles
   unsigned long long number;
-  long long patience;  // polls before a wait is given up
+  int patience;        // polls before a wait is given up
 
   __device__ __forceinline__ Slot* buffer() const { return slots + (number & 1) * (8 * (size_t)nct); }
 
@@ -114,7 +114,7 @@ struct Gang {
     if ((int)threadIdx.x < nct) {
       const Slot* theirs = buffer() + 8 * (size_t)threadIdx.x;
       double x;
-      for (long long spins = 0; !peek<true>(theirs, number, x) && !late; late = ++spins > patience) {
+      for (int spins = 0; !peek<true>(theirs, number, x) && !late; late = ++spins > patience) {
       }
     }
     return __syncthreads_or(late) == 0;
@@ -357,7 +357,7 @@ template <int K, int W>
 __global__ void __launch_bounds__(W * kBlock, W == 4 ? 1 : 2) solve_gang_kernel(const MeshDev* __restrict__ mds,
                                                                                 const int4* __restrict__ plan, int nplan,
                                                                                 int tickets, unsigned* ticket, int cap,
-                                                                                long long patience) {
+                                                                                int patience) {
   constexpr int kGangThreads = W * kBlock;
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ GangShared sh;
@@ -456,7 +456,8 @@ bool launch_w(Group& g, int cap, cudaStream_t st) {
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   // a wait for the rest of a gang lasts as long as the solve of a mesh drawn before
-  const long long patience = g.waits->meet + (g.waits->meet == WaitLimits{}.meet ? 256ll * cap : 0ll);
+  const long long longest = g.waits->meet + (g.waits->meet == WaitLimits{}.meet ? 256ll * cap : 0ll);
+  const int patience = (int)std::min<long long>(longest, INT32_MAX - 1);
   if (cudaLaunchKernelEx(&cfg, kern, (const MeshDev*)g.mds, (const int4*)g.gang_plan, g.nmesh, g.gang_tickets,
                          g.gang_ticket, cap, patience) != cudaSuccess) {
     cudaGetLastError();
