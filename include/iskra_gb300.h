@@ -167,11 +167,13 @@ ig_status ig_mesh_set_cot_clamp(ig_mesh* mesh, int enable, double clamp_min);
 /* How the loop of the last solve of this mesh (ig_mesh_route: solves of the mesh itself, also inside
  * ig_adjoint, ig_fairing_step, ig_eigs and ig_rgd_*) or batch was run: IG_ROUTE_NONE before the first,
  * IG_ROUTE_HOST launched by the host (also while profiling), IG_ROUTE_GRAPH a CUDA graph, IG_ROUTE_ONE_LAUNCH
- * one launch with the rows on chip. A diagnostic: the results do not depend on it. *ctas (may be NULL)
- * receives the CTAs that shared the mesh's last solve in one launch, 0 when it ran otherwise; it is read
- * from the device, which synchronises.
+ * one launch with the rows on chip, IG_ROUTE_OFF_CHIP (only told with ctas) in a launch of which not every
+ * CTA could start, with the rows in global memory. A diagnostic: the results do not depend on it. *ctas
+ * (may be NULL) receives the CTAs that shared the mesh's last solve in one launch, 0 when it ran otherwise
+ * (of a mesh solved in a batch too, whose route is then the batch's); it is read from the device, which
+ * synchronises.
  * Errors: IG_ERR_INVALID_ARG (NULL mesh, batch or route), IG_ERR_CUDA. */
-enum { IG_ROUTE_NONE = 0, IG_ROUTE_HOST = 1, IG_ROUTE_GRAPH = 2, IG_ROUTE_ONE_LAUNCH = 3 };
+enum { IG_ROUTE_NONE = 0, IG_ROUTE_HOST = 1, IG_ROUTE_GRAPH = 2, IG_ROUTE_ONE_LAUNCH = 3, IG_ROUTE_OFF_CHIP = 4 };
 ig_status ig_mesh_route(ig_mesh* mesh, int* route, int* ctas);
 ig_status ig_batch_route(ig_batch* batch, int* route);
 

@@ -29,7 +29,7 @@ IG_PRECISION_MIXED = 1
 IG_PRECISION_MIXED_GEOM32 = 2
 IG_LAUNCH_GRAPH = 0
 IG_LAUNCH_HOST = 1
-ROUTES = ("none", "host", "graph", "one_launch")  # IG_ROUTE_*
+ROUTES = ("none", "host", "graph", "one_launch", "off_chip")  # IG_ROUTE_*
 
 
 class NativeLibraryError(RuntimeError):

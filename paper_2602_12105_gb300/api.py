@@ -148,7 +148,8 @@ class Mesh:
         self.ctx.check(self.ctx.lib.ig_check(self.h))
 
     def route(self):
-        """How the last solve's loop was run ("none", "host", "graph" or "one_launch") and the number of
+        """How the last solve's loop was run ("none", "host", "graph", "one_launch" or
+        "off_chip") and the number of
         CTAs that shared it in one launch (ig_mesh_route). Synchronises."""
         r, c = ctypes.c_int(), ctypes.c_int()
         self.ctx.sync_stream()

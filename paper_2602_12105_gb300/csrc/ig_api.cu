@@ -770,8 +770,11 @@ ig_status ig_mesh_route(ig_mesh* mesh, int* route, int* ctas) {
   DeviceGuard guard(ctx->device);
   *route = mesh->group.route;
   if (!ctas) return IG_OK;
-  IG_CK(ctx, cudaMemcpyAsync(ctas, &mesh->md.s->members, sizeof(int), cudaMemcpyDeviceToHost, ctx->stream), "read state");
+  SolveScal s;
+  IG_CK(ctx, cudaMemcpyAsync(&s, mesh->md.s, sizeof(SolveScal), cudaMemcpyDeviceToHost, ctx->stream), "read state");
   IG_CK(ctx, cudaStreamSynchronize(ctx->stream), "route");
+  *ctas = s.members;
+  if (s.off_chip) *route = IG_ROUTE_OFF_CHIP;
   return IG_OK;
 }
 

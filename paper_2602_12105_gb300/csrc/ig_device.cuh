@@ -1121,6 +1121,7 @@ __device__ __noinline__ void finish_init(SolveScal* s, int k, const double* acc,
   s->refine = 0;
   s->phase = 0;
   s->members = 0;
+  s->off_chip = 0;
   s->tol2 = tol * tol;
   s->max_iter = max_iter;
   s->status = bad ? IG_ERR_NONFINITE : IG_OK;

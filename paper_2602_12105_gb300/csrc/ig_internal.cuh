@@ -111,7 +111,7 @@ struct SolveScal {
   int phase;             // mixed precision: kPhaseInner / kPhaseApply / kPhaseRestart
   int max_iter, max_refine;
   int members;           // CTAs that shared the solve in one launch (0: another route)
-  int pad;
+  int off_chip;          // one launch: not every CTA could start, the rows are in global memory
   double tol2, inner_tol2;  // squares of the tolerances
   unsigned int cnt[4];   // last-CTA counters (spmv, update, init/residual, vjp)
 };
@@ -492,10 +492,10 @@ inline bool capturing(cudaStream_t st) {
 bool launch_resident(Group& g, int k, const double* in, double* out, int rhs_mass, const ig_solve_opts& o,
                      cudaStream_t st);
 size_t meet_bytes(int parts);  // for meetings that post up to `parts` partial sums
-// ig_resident32.cu: the loop of a mixed-precision solve of a whole group in one launch (between its
-// init and finalize kernels); false, with nothing launched, when the group does not qualify or the
-// device refuses the launch
-bool launch_gang(Group& g, int k, int cap, cudaStream_t st);
+// ig_resident32.cu: the loop of a mixed-precision solve of a whole group in one launch (after its init
+// kernel) and the solutions in io.out; false, with nothing launched, when the group does not qualify or the
+// device refuses the launch. e: of the launch that writes the solutions
+bool launch_gang(Group& g, int k, int cap, const IoTable& io, cudaStream_t st, cudaError_t& e);
 std::vector<int4> gang_plan(const MeshDev* mds, const double* t, int nmesh, int num_sms, int* tickets, int* workers);
 cudaError_t group_order_gangs(Group& g, const double* t, cudaStream_t st);  // before group_set_calls
 

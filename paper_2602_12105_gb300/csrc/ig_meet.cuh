@@ -22,18 +22,12 @@ struct __align__(16) MeetHead {
   unsigned long long word, team;
 };
 static_assert(sizeof(MeetHead) == sizeof(Slot), "one slot");
-// This CTA (one of count) begins; the solve's number.
-__device__ __forceinline__ unsigned long long begin_solve(MeetHead* h, int count) {
-  const unsigned long long w = atomicAdd(&h->word, 1ull);
-  if ((int)(w & 0xffffu) == count - 1) atomicExch(&h->word, ((w >> 16) + 1ull) << 16);
-  return w >> 16;
-}
 
 // The CTAs of a solve wait for one another, so those that share it must all run at once, and nothing makes
 // sure that a grid starts as a whole when other work holds some of the SMs. So they settle who takes part:
-// the last of them to begin settles on all; one that has waited `patience` polls settles on those that
-// have begun by then (they run and will see it), and a CTA that begins after that leaves at once. One
-// word decides (compare-and-swap), so all read the same.
+// the last of them to begin settles on all; one that has waited long enough (enough(polls)) settles on
+// those that have begun by then (they run and will see it), and a CTA that begins after that leaves at
+// once. One word decides (compare-and-swap), so all read the same. ALL: all or none.
 struct Team {
   unsigned long long solve;  // number of the solve
   int rank;                  // in the order of beginning; takes part if below size
@@ -44,7 +38,8 @@ __device__ __forceinline__ unsigned long long load_relaxed(const unsigned long l
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
-__device__ __forceinline__ Team join_team(MeetHead* h, int count, int patience, int limit) {
+template <bool ALL = false, typename Enough>
+__device__ __forceinline__ Team join_team(MeetHead* h, int count, long long limit, const Enough& enough) {
   const unsigned long long w = atomicAdd(&h->word, 1ull);
   Team t{w >> 16, (int)(w & 0xffffu), -1};
   const unsigned long long mark = t.solve + 1ull;
@@ -58,9 +53,10 @@ __device__ __forceinline__ Team join_team(MeetHead* h, int count, int patience, 
     __threadfence();
     atomicExch(&h->word, mark << 16);
   } else {
-    for (int spins = 0; s >> 16 != mark && (spins < patience || spins - patience < limit); ++spins) {
-      const unsigned long long now = spins >= patience ? load_relaxed(&h->word) : 0ull;
-      if (spins >= patience && now >> 16 == t.solve) settle(now & 0xffffu);
+    for (long long spins = 0; s >> 16 != mark && spins < limit; ++spins) {
+      const bool now = enough(spins);
+      const unsigned long long begun = now ? load_relaxed(&h->word) : 0ull;
+      if (now && begun >> 16 == t.solve) settle(ALL ? 0ull : begun & 0xffffu);
       else s = load_relaxed(&h->team);
     }
   }

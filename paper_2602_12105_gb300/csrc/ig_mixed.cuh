@@ -36,6 +36,7 @@ __device__ __noinline__ void finish_init_mixed(SolveScal* s, int k, const double
   s->inner_cap = max_iter < 4000 ? max_iter : 4000;
   s->phase = kPhaseRestart;
   s->members = 0;
+  s->off_chip = 0;
   s->tol2 = tol * tol;
   s->inner_tol2 = inner_tol * inner_tol;
   s->max_iter = max_iter;

@@ -506,10 +506,9 @@ cudaError_t solve_mixed_k(Group& g, const IoTable& io, int rhs_mass, const ig_so
   cudaError_t e;
   if (graph && g.gang_plan) {
     if ((e = init_mixed_k<K>(g, io, rhs_mass, o, st)) != cudaSuccess) return e;
-    if (launch_gang(g, K, slot_cap(o), st)) {
+    if (launch_gang(g, K, slot_cap(o), io, st, e)) {
       g.route = IG_ROUTE_ONE_LAUNCH;
-      finalize_kernel<K><<<g.ntiles, kBlock, 0, st>>>(g.mds, g.tiles, io);
-      return cudaGetLastError();
+      return e;
     }
   }
   e = begin_mixed_k<K>(g, io, rhs_mass, o, st);

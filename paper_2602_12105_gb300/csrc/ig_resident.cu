@@ -293,6 +293,7 @@ __device__ __noinline__ void solve_shared(ResShared& sh, SharedScratch& w, Slot*
       sh.st.done = 1;
     }
     sh.st.members = size;
+    sh.st.off_chip = 1;
   }
   __syncthreads();
   if (rank == 0) {
@@ -341,7 +342,8 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
 
   // (the ninth warp, while the others load)
   if (!CLUSTER && tid == kBlock)
-    sh.team = join_team(reinterpret_cast<MeetHead*>(md.meet), (int)gridDim.x, begin_patience, patience);
+    sh.team = join_team(reinterpret_cast<MeetHead*>(md.meet), (int)gridDim.x, (long long)begin_patience + patience,
+                        [&](long long polls) { return polls >= begin_patience; });
 
   // the rows' operator on chip; slices of 32 rows, one per warp and step
   for (int i = tid; i < rows; i += kBlock) {

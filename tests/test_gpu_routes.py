@@ -1,5 +1,9 @@
 """Which meshes and batches are solved in one launch, by which solves of the public interface, and what a
 caller's stream capture gets."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -108,15 +112,9 @@ def test_route_batches(api):
     assert api.Batch([ms[0][0]]).route() == "none"
 
 
-@pytest.mark.parametrize("nx,ny,precision,works", [
-    (40, 30, "fp64", True),    # one cluster: a plain kernel
-    (100, 90, "fp64", False),  # the graph of the loop holds a conditional node, which no capture takes
-    (40, 30, "mixed", False),
-])
-def test_solve_under_a_capture(api, nx, ny, precision, works):
-    """A captured solve replays with the solve's bits, or the capture is refused; the mesh solves as before
-    after either (the refused launch's error may be reported once more first)."""
+def _captured(nx, ny, precision, works):
     from paper_2602_12105_gb300 import _native as N
+    from paper_2602_12105_gb300 import api
     mesh, V, t = _mesh(api, nx, ny)
     B = V.clone()
     s = torch.cuda.Stream()
@@ -149,3 +147,19 @@ def test_solve_under_a_capture(api, nx, ny, precision, works):
                 assert e.status == N.IG_ERR_CUDA
         assert torch.equal(mesh.solve(B), U0)
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("nx,ny,precision,works", [
+    (40, 30, "fp64", True),    # one cluster: a plain kernel
+    (100, 90, "fp64", False),  # the graph of the loop holds a conditional node, which no capture takes
+    (40, 30, "mixed", False),
+])
+def test_solve_under_a_capture(api, nx, ny, precision, works):
+    """A captured solve replays with the solve's bits, or the capture is refused; the mesh solves as before
+    after either (the refused launch's error may be reported once more first). In a process of its own:
+    after a refused capture torch's generator stays in its capture state."""
+    code = f"import test_gpu_routes as t; t._captured({nx}, {ny}, {precision!r}, {works})"
+    here = os.path.dirname(os.path.abspath(__file__))
+    res = subprocess.run([sys.executable, "-c", code], cwd=here, capture_output=True, text=True, timeout=300,
+                         env={**os.environ, "PYTHONPATH": os.pathsep.join([here, os.path.dirname(here)])})
+    assert res.returncode == 0, res.stderr[-2000:]

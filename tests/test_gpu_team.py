@@ -46,7 +46,7 @@ def _hold(streams):
 
 def _compare(api, nx, ny, k, precision):
     """With little waiting for the others to begin, and with SMs held by other kernels: the team is whoever
-    has begun by then. Returns the teams' sizes and the whole one's."""
+    has begun by then. Returns the sizes of the teams with rows off chip and the whole team's."""
     ctx = api.Context(0)
     mesh, V, t = _mesh(api, ctx, nx, ny)
     B = _t(np.random.default_rng(5).uniform(-1.0, 1.0, (mesh.n, k)))
@@ -62,11 +62,12 @@ def _compare(api, nx, ny, k, precision):
                 route, ctas = mesh.route()
             torch.cuda.synchronize()
             assert torch.equal(U, Uh) and i == ih
-            assert route == "one_launch" and ctas > 0
             if (begin, held) == (-1, 0):
+                assert route == "one_launch"
                 full = ctas
-            sizes.add(ctas)
-    assert max(sizes) == full
+            assert route in ("one_launch", "off_chip") and 0 < ctas <= full
+            if route == "off_chip":
+                sizes.add(ctas)
     mesh.close()
     return sizes, full
 
@@ -82,7 +83,50 @@ def test_fewer_ctas_than_tiles_fp64(api, nx, ny, k):
     sizes, full = _compare(api, nx, ny, k, "fp64")
     print(f"{nx}x{ny} k {k}: teams of {sorted(sizes)} of {full} CTAs")
     if ny == 429 and full == torch.cuda.get_device_properties(0).multi_processor_count:
-        assert min(sizes) < full  # a CTA takes an SM's whole shared memory: held SMs are missing
+        assert sizes and max(sizes) < full  # a CTA takes an SM's whole shared memory: held SMs are missing
+
+
+@pytest.mark.parametrize("nx,ny,k,precision", [
+    (64, 17, 4, "mixed"),      # two groups of four tiles
+    (205, 5, 2, "mixed32"),    # 1,025 rows: a second group of one row
+    (300, 211, 3, "mixed"),
+    (591, 592, 1, "mixed"), (591, 592, 2, "mixed"), (591, 592, 3, "mixed32"), (591, 592, 4, "mixed"),
+    (0, 5000, 3, "mixed"),     # a row of 5,001 entries
+])
+def test_fewer_ctas_than_groups_mixed(api, nx, ny, k, precision):
+    sizes, full = _compare(api, nx, ny, k, precision)
+    print(f"{nx}x{ny} k {k}: teams of {sorted(sizes)} of {full} CTAs")
+    if ny == 592 and full == torch.cuda.get_device_properties(0).multi_processor_count:
+        assert sizes
+
+
+@pytest.mark.parametrize("k", [1, 3])
+@pytest.mark.parametrize("large", [False, True])
+def test_batches_of_which_not_every_cta_starts(api, k, large):
+    """Batches in CTAs of four workers (a mesh of more than 155,000 rows) and of two, with SMs held: every
+    mesh has the bits it has alone."""
+    ctx = api.Context(0)
+    sizes = [(61 + 3 * i, 40 + i) for i in range(24)] + [(200, 150)] * 6 + ([(450, 430)] * 2 if large else [])
+    ms = [_mesh(api, ctx, nx, ny) for nx, ny in sizes]
+    batch = api.Batch([m for m, _, _ in ms])
+    Vs, ts = [V for _, V, _ in ms], [t for _, _, t in ms]
+    Bs = [V[:, :k].contiguous() for V in Vs]
+    batch.assemble(Vs, ts, "mixed")
+    U0, i0 = batch.solve(Bs, opts=api.make_opts(launch="host"), info=True)
+    others, main = [torch.cuda.Stream() for _ in range(30)], torch.cuda.Stream()
+    routes = set()
+    for begin, held in ((-1, 0), (0, 0), (0, 9), (1, 30), (-1, 30), (-1, 0)):
+        ctx.set_wait_limits(begin=begin)
+        _hold(others[:held])
+        with torch.cuda.stream(main):
+            U, i = batch.solve(Bs, info=True)
+            routes |= {m.route() for m, _, _ in ms}
+        torch.cuda.synchronize()
+        assert batch.route() == "one_launch"
+        assert all(torch.equal(a, b) for a, b in zip(U, U0)) and i == i0
+    print(f"large {large} k {k}: {sorted(routes)}")
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        assert any(ctas > 0 for _, ctas in routes)
 
 
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
