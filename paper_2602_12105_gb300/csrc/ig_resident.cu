@@ -302,6 +302,12 @@ __device__ __noinline__ void solve_shared(ResShared& sh, SharedScratch& w, Slot*
   }
 }
 
+// The calling thread settles who takes part (out of line: the kernel's own code is scheduled as without it).
+__device__ __noinline__ void resident_join(ResShared& sh, int begin, int patience) {
+  sh.team = join_team(reinterpret_cast<MeetHead*>(sh.md.meet), (int)gridDim.x, (long long)begin + patience,
+                      [=](long long polls) { return polls >= begin; });
+}
+
 template <int K, bool CLUSTER>
 __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const MeshDev* __restrict__ mds,
                                                                         const double* __restrict__ in,
@@ -342,8 +348,7 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
 
   // (the ninth warp, while the others load)
   if (!CLUSTER && tid == kBlock)
-    sh.team = join_team(reinterpret_cast<MeetHead*>(md.meet), (int)gridDim.x, (long long)begin_patience + patience,
-                        [&](long long polls) { return polls >= begin_patience; });
+    resident_join(sh, begin_patience, patience);
 
   // the rows' operator on chip; slices of 32 rows, one per warp and step
   for (int i = tid; i < rows; i += kBlock) {
@@ -527,11 +532,13 @@ __global__ void __launch_bounds__(kResThreads, 1) solve_resident_kernel(const Me
   if constexpr (CLUSTER) cluster_sync_all();  // no CTA leaves while another reads its sums
 }
 
+constexpr int kResBytes = 227 * 1024 - (int)sizeof(ResShared) - 256;  // most dynamic shared memory of a CTA
+
 // Shared memory of a CTA of rp rows: everything, less the solution, then less operator slots, as far
 // as the SM's 227 KB demand.
 template <int K>
 ResLayout layout(int rp, int wmax) {
-  const int room = 227 * 1024 - (int)sizeof(ResShared) - 256;
+  const int room = kResBytes;
   const int fixed = rp * 8 * (3 * K + 1) + 2 * K * kFixedTiles * 8;
   ResLayout l{};
   l.rp = rp;
@@ -547,7 +554,9 @@ bool launch_k(Group& g, const double* in, double* out, int rhs_mass, const ig_so
   const MeshDev& md = g.host_mds[0];
   auto kern = solve_resident_kernel<K, CLUSTER>;
   const ResLayout lay = layout<K>(md.tile_rows, md.sell_wmax);
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, lay.bytes) != cudaSuccess ||
+  // (the same limit whatever the mesh: it is the kernel's, and a thread with a smaller mesh could lower it
+  // between another's call here and its launch)
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kResBytes) != cudaSuccess ||
       (CLUSTER && cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess)) {
     cudaGetLastError();
     return false;

@@ -172,3 +172,40 @@ def test_streams_and_threads(api, precision):
         th.join()
     torch.cuda.synchronize()
     assert not failed, failed
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_threads_keep_their_route(api, precision):
+    """Two threads whose meshes take different amounts of shared memory: no launch is refused for the other
+    thread's limit."""
+    import ctypes
+    jobs = [_mesh(api, api.Context(0), nx, ny) for nx, ny in ((430, 429), (241, 17))]
+    for mesh, V, t in jobs:
+        mesh.assemble(V, t, precision)
+        mesh.solve(V)
+    torch.cuda.synchronize()
+    routes, go = {0: {}, 1: {}}, threading.Barrier(2)
+
+    def work(i):  # calls of the library alone, so that two of them overlap
+        mesh, V, _ = jobs[i]
+        opts, U, lib = api.make_opts(max_iter=2, max_refine=1), torch.empty_like(V), mesh.ctx.lib
+        B, out, po = ctypes.c_void_p(V.data_ptr()), ctypes.c_void_p(U.data_ptr()), ctypes.byref(opts)
+        r, k, n = ctypes.c_int(), mesh.h, {}
+        with torch.cuda.stream(torch.cuda.Stream()):
+            mesh.ctx.sync_stream()
+            go.wait()
+            for j in range(6000):
+                lib.ig_solve(k, B, 3, out, po, None)
+                lib.ig_mesh_route(k, ctypes.byref(r), None)
+                n[r.value] = n.get(r.value, 0) + 1
+                if j % 200 == 199:
+                    torch.cuda.current_stream().synchronize()
+        routes[i] = n
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in (0, 1)]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    torch.cuda.synchronize()
+    assert all(set(r) == {3} for r in routes.values()), routes  # IG_ROUTE_ONE_LAUNCH
