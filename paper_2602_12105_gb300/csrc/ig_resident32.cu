@@ -26,6 +26,7 @@
 // chain of an iteration (three meetings, their FP64 sums and divisions), then the latency of the
 // gathers; the L1 data path is busy 36% of the time, DRAM not at all.
 #include <algorithm>
+#include <cmath>
 
 #include "ig_meet.cuh"
 #include "ig_mixed.cuh"
@@ -783,6 +784,14 @@ bool launch(Group& g, int cap, const IoTable& io, cudaStream_t st, cudaError_t& 
 // grow with the square root of the time step over the squared edge length, that is of t n on meshes of
 // one size (t null: equal steps). CTAs of two workers (two per SM) when there are more of them than
 // SMs and their tiles are small enough.
+//
+// Empty too for batches that the multi-CTA loop solves sooner. A CTA of four workers has an SM to itself, and
+// gangs of more than half the SMs run one after another, so the chain of an iteration (some 12.5 us in any
+// gang) is not hidden: n gangs at a time take 12.5 / n us an iteration and mesh, the loop 40 us an
+// iteration and 40 us per million rows (fitted to 102 batches, leaning to the gangs; weights: iterations as
+// the square root of the rows). 163,842 rows each, k = 3: 4 meshes 5.6 ms in gangs and 6.4 in the loop, 8
+// 11.2 and 10.7, 16 22.2 and 19.6; one of these and 40 of 40,962 rows 10.9 and 9.5; of 250,000 rows each, 8
+// 7.0 and 7.9, 32 27.7 and 25.7. In CTAs of two workers no batch was slower than in the loop by more than 2%.
 std::vector<int4> gang_plan(const MeshDev* mds, const double* t, int nmesh, int num_sms, int* tickets, int* workers) {
   std::vector<int4> plan;
   std::vector<double> work((size_t)nmesh);
@@ -803,6 +812,17 @@ std::vector<int4> gang_plan(const MeshDev* mds, const double* t, int nmesh, int 
   }
   *tickets = first;
   *workers = first > num_sms && rows <= kGangMaxRows / 2 - 32 ? 2 : 4;
+  if (first > num_sms && *workers == 4) {
+    int most = 1;
+    for (int i = 0; i < nmesh; ++i) most = std::max(most, mds[i].n);
+    double gangs = 0.0, loop = 40.0;  // us per iteration of the largest mesh
+    for (const int4& e : plan) {
+      const double n = mds[e.x].n, w = std::sqrt(n / most);
+      gangs += w * 12.5 / (num_sms / e.z);
+      loop += w * 40.0 * 1e-6 * n;
+    }
+    if (gangs > loop) return {};
+  }
   return plan;
 }
 

@@ -112,6 +112,30 @@ def test_route_batches(api):
     assert api.Batch([ms[0][0]]).route() == "none"
 
 
+@pytest.mark.parametrize("sizes,route", [
+    ([(405, 405)] * 4, "one_launch"),             # a few large meshes: gangs one after another
+    ([(405, 405)] * 10, "graph"),                 # many: the multi-CTA loop
+    ([(405, 405)] + [(220, 186)] * 8, "one_launch"),
+    ([(405, 405)] + [(220, 186)] * 40, "graph"),  # CTAs of four workers for all: 41 of them a mesh
+    ([(220, 186)] * 60, "one_launch"),            # CTAs of two workers
+    ([(590, 590)] * 12, "one_launch"),
+])
+def test_route_of_large_mixed_batches(api, sizes, route):
+    """Batches that the multi-CTA loop solves sooner go there, with the same bits as each mesh alone."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the sizes are those of 152 SMs")
+    ms = [_mesh(api, nx, ny) for nx, ny in sizes]
+    batch = api.Batch([m for m, _, _ in ms])
+    Bs = [V.clone() for _, V, _ in ms]
+    batch.assemble([V for _, V, _ in ms], [t for _, _, t in ms], "mixed")
+    opts = api.make_opts(max_iter=12)
+    Us = batch.solve(Bs, opts=opts)
+    assert batch.route() == route
+    for i in (0, len(ms) - 1):
+        U = ms[i][0].solve(Bs[i], opts=opts)
+        assert ms[i][0].route()[0] == "one_launch" and torch.equal(U, Us[i])
+
+
 def _captured(nx, ny, precision, works):
     from paper_2602_12105_gb300 import _native as N
     from paper_2602_12105_gb300 import api
