@@ -38,20 +38,28 @@ __device__ __forceinline__ unsigned long long load_relaxed(const unsigned long l
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
+struct Arrival {  // the words as a CTA that begins finds them
+  unsigned long long word, team;
+};
+__device__ __forceinline__ Arrival arrive(MeetHead* h, int count) {
+  if (count == 1) return {atomicAdd(&h->word, 1ull << 16), 0ull};
+  const unsigned long long s = load_relaxed(&h->team);
+  return {atomicAdd(&h->word, 1ull), s};
+}
 template <bool ALL = false, typename Enough>
-__device__ __forceinline__ Team join_team(MeetHead* h, int count, long long limit, const Enough& enough) {
-  const unsigned long long w = atomicAdd(&h->word, 1ull);
-  Team t{w >> 16, (int)(w & 0xffffu), -1};
+__device__ __forceinline__ Team join_team(MeetHead* h, int count, const Arrival& a, long long limit,
+                                          const Enough& enough) {
+  if (count == 1) return Team{a.word >> 16, 0, 1};
+  unsigned long long s = a.team;
+  Team t{a.word >> 16, (int)(a.word & 0xffffu), -1};
   const unsigned long long mark = t.solve + 1ull;
-  unsigned long long s = load_relaxed(&h->team);
   auto settle = [&](unsigned long long size) {  // a failed swap found this solve settled already
     const unsigned long long was = atomicCAS(&h->team, s, mark << 16 | size);
     s = was == s ? (mark << 16 | size) : was;
   };
   if (t.rank == count - 1) {
     if (s >> 16 != mark) settle((unsigned long long)count);
-    __threadfence();
-    atomicExch(&h->word, mark << 16);
+    atomicExch(&h->word, mark << 16);  // (one that sees this first looks at team again)
   } else {
     for (long long spins = 0; s >> 16 != mark && spins < limit; ++spins) {
       const bool now = enough(spins);

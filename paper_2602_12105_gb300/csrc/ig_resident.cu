@@ -304,7 +304,8 @@ __device__ __noinline__ void solve_shared(ResShared& sh, SharedScratch& w, Slot*
 
 // The calling thread settles who takes part (out of line: the kernel's own code is scheduled as without it).
 __device__ __noinline__ void resident_join(ResShared& sh, int begin, int patience) {
-  sh.team = join_team(reinterpret_cast<MeetHead*>(sh.md.meet), (int)gridDim.x, (long long)begin + patience,
+  MeetHead* h = reinterpret_cast<MeetHead*>(sh.md.meet);
+  sh.team = join_team(h, (int)gridDim.x, arrive(h, (int)gridDim.x), (long long)begin + patience,
                       [=](long long polls) { return polls >= begin; });
 }
 

@@ -365,11 +365,12 @@ __device__ __forceinline__ bool gang_solve(GangShared& sh, const GangRows& gr, G
 // The calling thread waits for the rest of the gang of the CTA's mesh: CTAs at work on meshes drawn before for
 // as long as such a solve takes, but not those that have not been able to start. (Out of line, like
 // gang_failed: the loop has all the registers.)
-__device__ __noinline__ void gang_join(GangShared& sh, const unsigned* started, unsigned ctas, int begin, int patience,
-                                       long long longest) {
-  sh.team = join_team<true>(reinterpret_cast<MeetHead*>(sh.md.meet), sh.groups, longest + patience, [=](long long polls) {
-    return polls >= longest || (polls >= begin && __ldcg(started) < ctas);
-  });
+__device__ __noinline__ void gang_join(GangShared& sh, Arrival a, const unsigned* started, unsigned ctas, int begin,
+                                       int patience, long long longest) {
+  sh.team = join_team<true>(reinterpret_cast<MeetHead*>(sh.md.meet), sh.groups, a, longest + patience,
+                            [=](long long polls) {
+                              return polls >= longest || (polls >= begin && __ldcg(started) < ctas);
+                            });
 }
 // A wait ran out: a failed solve, for every caller to see.
 template <int K>
@@ -393,10 +394,10 @@ __global__ void __launch_bounds__(W * kBlock, W == 4 ? 1 : 2) solve_gang_kernel(
                                                                                 int begin, int patience,
                                                                                 long long longest) {
   constexpr int kGangThreads = W * kBlock;
-  constexpr int kLoaders = kGangThreads - 32;  // the last warp waits for the gang meanwhile
   extern __shared__ __align__(16) unsigned char dyn[];
   __shared__ GangShared sh;
-  if (threadIdx.x == 0) atomicAdd(ticket + 1, 1u);  // a CTA of the launch has started
+  // ticket[0]: the next ticket, [1]: CTAs of the launch that have started, [2]: a mesh is left to finish_gang_kernel
+  if (threadIdx.x == 0) atomicAdd(ticket + 1, 1u);
   for (;;) {
     __syncthreads();  // every thread is done with the mesh before
     if (threadIdx.x == 0) sh.ticket = (int)atomicAdd(ticket, 1u);
@@ -424,7 +425,8 @@ __global__ void __launch_bounds__(W * kBlock, W == 4 ? 1 : 2) solve_gang_kernel(
     gang.nct = e.z;
     gang.slots = reinterpret_cast<Slot*>(md.meet) + 1;
     gang.patience = patience;
-    if (threadIdx.x == kLoaders) gang_join(sh, ticket + 1, gridDim.x, begin, patience, longest);
+    Arrival arrival{};
+    if (threadIdx.x == kGangThreads - 32) arrival = arrive(reinterpret_cast<MeetHead*>(md.meet), gang.nct);
 
     // the rows on chip
     GangRows gr;
@@ -438,7 +440,7 @@ __global__ void __launch_bounds__(W * kBlock, W == 4 ? 1 : 2) solve_gang_kernel(
     gr.d = gr.q + K * gr.rp;
     gr.a = gr.d + gr.rp;
     gr.c = reinterpret_cast<int*>(gr.a + gr.aw * gr.rp);
-    for (int i = threadIdx.x; i < held && threadIdx.x < kLoaders; i += kLoaders) {
+    for (int i = threadIdx.x; i < held; i += kGangThreads) {
       const int row = first_row + i, sl = row >> 5;
       const int b0 = __ldg(md.sell_ptr + sl), w = (__ldg(md.sell_ptr + sl + 1) - b0) >> 5;
       if ((i & 31) == 0) sh.width[i >> 5] = w;
@@ -449,9 +451,13 @@ __global__ void __launch_bounds__(W * kBlock, W == 4 ? 1 : 2) solve_gang_kernel(
       }
       gr.d[i] = __ldg(md.Dinv32 + row);
     }
+    if (threadIdx.x == kGangThreads - 32) gang_join(sh, arrival, ticket + 1, gridDim.x, begin, patience, longest);
     __syncthreads();
     if (sh.team.size == 0) {  // left to finish_gang_kernel
-      if (threadIdx.x == 0) md.s->off_chip = 1;
+      if (threadIdx.x == 0) {
+        md.s->off_chip = 1;
+        ticket[2] = 1u;
+      }
       continue;
     }
     gang.number = sh.team.solve << 32;  // above those of every solve of the mesh before
@@ -692,12 +698,14 @@ __device__ __noinline__ bool gang_solve_shared(GangShared& sh, int cap, int pati
 template <int K>
 __global__ void __launch_bounds__(kBlock) finish_gang_kernel(const MeshDev* __restrict__ mds,
                                                              const int2* __restrict__ tiles, IoTable io, int cap,
-                                                             int begin, int patience) {
+                                                             int begin, int patience,
+                                                             const unsigned* __restrict__ left) {
+  const unsigned any = __ldcg(left);  // whether some mesh is left (beside the loads that follow)
   const int2 tl = tiles[blockIdx.x];
   const MeshDev& gmd = mds[tl.x];
   const long nn = gmd.n;
   double* __restrict__ out = io.out[tl.x];
-  if (!gmd.s->off_chip) {
+  if (any == 0u || !gmd.s->off_chip) {
     const long t0 = (long)tl.y * gmd.tile_rows, t1 = t0 + gmd.tile_rows < nn ? t0 + gmd.tile_rows : nn;
     for (long row = t0 + threadIdx.x; row < t1; row += kBlock) {
 #pragma unroll
@@ -714,7 +722,8 @@ __global__ void __launch_bounds__(kBlock) finish_gang_kernel(const MeshDev* __re
     reinterpret_cast<unsigned*>(&sh.st)[j] = __ldcg(reinterpret_cast<const unsigned*>(gmd.s) + j);
   if (threadIdx.x == 0) {
     sh.groups = groups;
-    sh.team = join_team(reinterpret_cast<MeetHead*>(gmd.meet), count, (long long)begin + patience,
+    MeetHead* h = reinterpret_cast<MeetHead*>(gmd.meet);
+    sh.team = join_team(h, count, arrive(h, count), (long long)begin + patience,
                         [&](long long polls) { return polls >= begin; });
   }
   __syncthreads();
@@ -750,7 +759,7 @@ bool launch_w(Group& g, int cap, cudaStream_t st) {
   auto kern = solve_gang_kernel<K, W>;
   const int ctas = g.num_sms * (W == 4 ? 1 : 2);
   if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kGangBytes<W>) != cudaSuccess ||
-      cudaMemsetAsync(g.gang_ticket, 0, 2 * sizeof(unsigned), st) != cudaSuccess) {
+      cudaMemsetAsync(g.gang_ticket, 0, 3 * sizeof(unsigned), st) != cudaSuccess) {
     cudaGetLastError();
     return false;
   }
@@ -772,7 +781,8 @@ bool launch_w(Group& g, int cap, cudaStream_t st) {
 template <int K>
 bool launch(Group& g, int cap, const IoTable& io, cudaStream_t st, cudaError_t& e) {
   if (!(g.gang_workers == 2 ? launch_w<K, 2>(g, cap, st) : launch_w<K, 4>(g, cap, st))) return false;
-  finish_gang_kernel<K><<<g.ntiles, kBlock, 0, st>>>(g.mds, g.tiles, io, cap, g.waits->begin, g.waits->meet);
+  finish_gang_kernel<K><<<g.ntiles, kBlock, 0, st>>>(g.mds, g.tiles, io, cap, g.waits->begin, g.waits->meet,
+                                                   g.gang_ticket + 2);
   e = cudaGetLastError();
   return true;
 }
