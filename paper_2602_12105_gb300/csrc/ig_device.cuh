@@ -11,9 +11,11 @@ namespace {
 
 constexpr int kWarps = kBlock / 32;
 
-// a / b to within one unit in the last place for operands of ordinary magnitude: a third-order
-// (hyperpower) iteration on the hardware's reciprocal estimate (about 20 bits, whose error e becomes
-// e^3), then one correction of the quotient by its residual. Six FP64 instructions in line, about 450
+// a / b for operands of ordinary magnitude: a third-order (hyperpower) iteration on the hardware's
+// reciprocal estimate (about 20 bits, whose error e becomes e^3, below 2^-57), then one correction of the
+// quotient by its residual, which is off by less than 2^-50 units in the last place before the one
+// rounding. So it is the division's result unless the exact quotient lies that close to the middle of two
+// doubles (1 / (2 - 2^-52), say), and then one of the two. Six FP64 instructions in line, about 450
 // cycles; the compiler's division, a call, took 660 to 1,650 in the finish steps, which every CTA of
 // a resident solve waits for. Other operands (zero, subnormal, infinite, NaN, or 2^400 from 1) take the
 // plain division.
