@@ -45,7 +45,7 @@ constexpr int kResMaxCtas = 160;     // most CTAs
 constexpr int kResMinRows = 256;     // fewest rows of a tile of more than kResSmall rows
 constexpr int kResSmall = 2048;      // meshes up to this size: tiles of 128 rows
 constexpr int kResMaxRows = 1216;    // most rows of a tile (227 KB of shared memory at 188 bytes a row)
-constexpr int kGangMaxRows = 2336;   // most rows of a CTA of a mixed-precision gang (ig_resident32.cu)
+constexpr int kGangMaxRows = 2336;   // most rows of a CTA of a mixed-precision gang (ig_resident32.cu): 4 tiles of 576
 constexpr int kClusterTiles = 16;    // up to this many tiles meet as one thread-block cluster
 constexpr int kPatW = 7;             // entries of a column pattern (MeshDev::pat): the regular vertex of valence 6
 constexpr int kPartStride = 8;       // doubles per tile in the partial-sum arrays
@@ -373,7 +373,7 @@ struct Group {
   int* act_buf = nullptr;         // device storage of the active list and start tables (LoopCtl)
   ListRef list64{}, list32{}, listapp{};  // what the FP64, mixed and residual loop kernels walk
   int num_sms = 0;                // SMs of the device (resident solves: at most one CTA on each)
-  int4* gang_plan = nullptr;      // device: the gangs of a mixed-precision solve (null: not one), in mesh order of size
+  int4* gang_plan = nullptr;      // device: the gangs of a mixed-precision solve, longest solves first (null: no gangs)
   int gang_tickets = 0, gang_workers = 4;
   unsigned* gang_ticket = nullptr;
   int route = IG_ROUTE_NONE;      // of the last solve
@@ -479,7 +479,8 @@ cudaError_t launch_operator32_csr(const MeshDev& md, float* Acsr, cudaStream_t s
 
 // ig_pcg.cu: see Group above
 
-// The launches in one are not recorded in a caller's capture (nor is one that cannot tell).
+// Solves in one launch but those of a cluster are not recorded in a caller's capture (nor is one that cannot
+// tell); it gets the graph loop, whose conditional node a capture refuses.
 inline bool capturing(cudaStream_t st) {
   cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;

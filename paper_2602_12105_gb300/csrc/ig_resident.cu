@@ -595,7 +595,7 @@ bool launch_k(Group& g, const double* in, double* out, int rhs_mass, const ig_so
 template <int K>
 bool launch(Group& g, const double* in, double* out, int rhs_mass, const ig_solve_opts& o, cudaStream_t st) {
   if (g.host_mds[0].ntiles <= kClusterTiles && launch_k<K, true>(g, in, out, rhs_mass, o, st)) return true;
-  if (capturing(st)) return false;  // a capture gets the graph loop's answer
+  if (capturing(st)) return false;
   return launch_k<K, false>(g, in, out, rhs_mass, o, st);
 }
 

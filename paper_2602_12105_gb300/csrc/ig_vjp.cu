@@ -17,9 +17,9 @@
 //   A = 2 omega_2 / s - k v.v,  C = 2 omega_1 / s - k u.u,
 //   X = (omega_1 + omega_2 - omega_0) / s + k u.v,
 // and the corners get dE/du - dE/dv, dE/dv and -dE/du. The FP64 kernel is bound by FP64 instructions (2 per
-// clock per SM): this form takes about 93 per face (k = 3; three of them choose the edge left out, 3% of
-// the kernel's time), combinations of two edges corner by corner took 103, cross products corner by corner
-// about 140.
+// clock per SM): this form takes about 93 per face (k = 3; 2,095,106 faces 359 us, 346 without the three that
+// choose the edge left out), combinations of two edges corner by corner took 103 (424 us), cross products
+// corner by corner about 140 (578 us).
 // (The CPU oracle reaches the same numbers through the per-corner cotangent gradients.)
 //
 // A loss may also depend on V through the mass directly (the M-norm loss of the inverse-fairing
@@ -33,7 +33,9 @@
 //
 // FP32 face geometry (the mode whose operator was assembled from FP32 cotangents): a vertex pass
 // splits U and Lambda into hi/lo floats and forms w_v = <Lambda_v, B_v - U_v> per vertex; K6a
-// evaluates the same formula in FP32 with every difference of neighbouring values (edges, U_a -
+// takes the gradient of E_f corner by corner in FP32 (with N = d_1 x d_2 and d_c the edge opposite corner c:
+// grad_{p_c} E_f = [-omega_c (d_{c+2} - d_{c+1}) + (omega_{c+1} - omega_{c+2}) d_c] / s + (w_a / 2 - P / s^2)
+// (N x d_c) / s), with every difference of neighbouring values (edges, U_a -
 // U_b, Lambda_a - Lambda_b) taken as (hi_a - hi_b) + (lo_a - lo_b), and slivers (sin theta < 1e-2
 // at a corner, the test of the assembly) in FP64; gface is then [m][3][4] float (one 16-byte row
 // per corner) and K6b adds in FP32. The FP64 solve terms of B = V (M Lambda) stay FP64.
@@ -323,8 +325,8 @@ __global__ void __launch_bounds__(256) vjp32_split_kernel(const MeshDev* __restr
   md.wv[v] = w;
 }
 
-// The FP64 per-corner gradients of one face (the formula of vjp_face_kernel, mode 0), and its
-// term of dl/dt; for slivers under FP32 geometry.
+// The FP64 gradients of one face, corner by corner as vjp32_face_kernel takes them, and its term of dl/dt; for
+// slivers under FP32 geometry.
 template <int K>
 __device__ __noinline__ double face_grad64(const MeshDev& md, const CallDev& cl, const int (&vid)[3], double (&g)[9]) {
   const double* __restrict__ V = cl.V;
